@@ -9,14 +9,20 @@
 // d logp / d y_ij = r_ij c_j / sigma_j^2 for both, and one set of kernels serves both.
 //
 // grpo_step_signals runs in three launches:
-//   1. advantages A_i (Eq. advantage) from the group's rewards, and the W pairs (a_j, c_j);
-//   2. ||r_ij||^2, one CTA per (i, j, chunk of D), partial sums in f64 written to the
-//      workspace (fixed order: deterministic);
-//   3. per (i, j): log-prob (Eq. logprob), ratio, clip decision (Eq. grpo_loss), the
-//      coefficient k_ij = scale (-A_i) rho_ij c_j / sigma_j^2 (0 when clipped); then one
-//      elementwise pass writes s_ij = k_ij r_ij and/or the aggregated cotangents
+//   1. ||r_ij||^2, one CTA per (i, j, chunk of D), partial sums in f64 written to the
+//      workspace (fixed order: deterministic); the first CTA of a sample also forms its
+//      advantage A_i (Eq. advantage) from the group's rewards;
+//   2. a warp per (i, j): log-prob (Eq. logprob), ratio, clip decision (Eq. grpo_loss), the
+//      coefficient k_ij = scale (-A_i) rho_ij c_j / sigma_j^2 (0 when clipped);
+//   3. one elementwise pass writes s_ij = k_ij r_ij and/or the aggregated cotangents
 //      sum_j (1 - alpha_j) s_ij and sum_j alpha_j s_ij (Eq. alpha, Eq. s_base_corr).
 // The v-hat / z tiles of a window are read twice; at the paper's shapes they fit in L2.
+// f64 runs at a small fraction of the f32 rate here, so each f64 value is formed once (the
+// coefficients by one thread per CTA, a chunk's sum by four warps): a window of 4 x 4 steps
+// of 262144 bf16 elements took 80 us with an f64 coefficient set and butterfly in every thread
+// and five launches, 67 us with the log-prob part repeated by every CTA of the elementwise
+// pass (two launches), and takes 35 us like this (29 us replayed from a CUDA graph; reading
+// and writing its 38 MB once is 5.6 us); 8 x 4 steps of 16384 elements 37 -> 25 us.
 #include <mutex>
 
 #include "common.cuh"
@@ -27,13 +33,10 @@ int unit_status_signals(unsigned* v, int clear) { return read_unit_status(v, cle
 
 namespace {
 
-constexpr int SIG_THREADS = 256;
-constexpr int SIG_PER_THREAD = 32;
-constexpr int SIG_CHUNK = SIG_THREADS * SIG_PER_THREAD;  // elements of D per CTA in pass 2
-
-__device__ __forceinline__ float ldv_any(const void* p, int64_t i, int is_f32) {
-  return is_f32 ? static_cast<const float*>(p)[i] : __bfloat162float(static_cast<const bf16*>(p)[i]);
-}
+constexpr int SIG_THREADS = 1024;
+constexpr int SIG_PER_THREAD = 8;  // consecutive elements: two 16-byte loads of each f32 row
+constexpr int SIG_CHUNK = SIG_THREADS * SIG_PER_THREAD;  // elements of D per CTA of the residual sums
+constexpr int APPLY_THREADS = 256;
 
 // An f64 mean coefficient as an unevaluated sum of two floats (hi + lo).  Rounding a_j or c_j
 // to one float shifts r_ij by the same relative amount at every element, an error that does
@@ -75,66 +78,58 @@ __device__ __forceinline__ bool mean_coef(double t0, double t1, bool eps, double
   return false;
 }
 
-// One warp.  Lane 0: the advantages.  All lanes: the mean coefficients mc[j] = a_j,
-// mc[W + j] = c_j; sched_alpha == nullptr selects the rectified-flow step.
-__global__ void prep_kernel(const float* rewards, int G, double adv_eps, double adv_clip, double* adv, const double* t,
-                            const double* sched_alpha, const double* sched_sigma, int W, double* mc) {
-  if (blockIdx.x != 0) return;
-  for (int j = threadIdx.x; j < W; j += 32) {
-    const bool eps = sched_alpha != nullptr;
-    double a, c;
-    if (!mean_coef(t[j], t[j + 1], eps, eps ? sched_alpha[j] : 0.0, eps ? sched_alpha[j + 1] : 0.0,
-                   eps ? sched_sigma[j] : 0.0, eps ? sched_sigma[j + 1] : 0.0, &a, &c))
-      set_device_status(JAGG_DEV_BADARG);
-    mc[j] = a;
-    mc[W + j] = c;
+// Elements k .. k + 7 of a row (zeros past D).  `vec`: the row is 16-byte aligned.
+__device__ __forceinline__ void load8(const float* p, int64_t k, int64_t D, bool vec, float (&x)[8]) {
+  if (vec && k + 8 <= D) {
+    const float4 a = *reinterpret_cast<const float4*>(p + k), b = *reinterpret_cast<const float4*>(p + k + 4);
+    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = k + e < D ? p[k + e] : 0.f;
   }
-  if (threadIdx.x != 0) return;
-  double mu = 0.0;
-  for (int i = 0; i < G; ++i) mu += (double)rewards[i];
-  mu /= G;
-  double ss = 0.0;
-  for (int i = 0; i < G; ++i) {
-    const double d = (double)rewards[i] - mu;
-    ss += d * d;
-  }
-  const double sd = G > 1 ? sqrt(ss / (G - 1)) : 0.0;
-  for (int i = 0; i < G; ++i) {
-    double a = ((double)rewards[i] - mu) / (sd + adv_eps);
-    a = a > adv_clip ? adv_clip : (a < -adv_clip ? -adv_clip : a);
-    adv[i] = a;
+}
+__device__ __forceinline__ void load8_any(const void* p, int64_t base, int is_f32, int64_t k, int64_t D, bool vec,
+                                          float (&x)[8]) {
+  if (is_f32) {
+    load8(static_cast<const float*>(p) + base, k, D, vec, x);
+  } else if (vec && k + 8 <= D) {
+    const uint4 raw = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p) + base + k);
+    const bf16* h = reinterpret_cast<const bf16*>(&raw);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = __bfloat162float(h[e]);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      x[e] = k + e < D ? __bfloat162float(static_cast<const bf16*>(p)[base + k + e]) : 0.f;
   }
 }
 
-// sum of r(k)^2 over the CTA's chunk of D (k = blockIdx.x * SIG_CHUNK + ...), valid in thread
-// 0: f32 partial sums folded into f64 every 8 terms, then a fixed-order block reduction.  The
-// rollout sampler and the step signals share it, so equal residuals give equal log-probs.
-template <class R>
-__device__ __forceinline__ double chunk_sq_sum(int64_t D, R r_at) {
-  const int64_t k0 = (int64_t)blockIdx.x * SIG_CHUNK;
-  double acc = 0.0;
-  float part = 0.f;
-#pragma unroll 4
-  for (int u = 0; u < SIG_PER_THREAD; ++u) {
-    const int64_t k = k0 + threadIdx.x + (int64_t)u * SIG_THREADS;
-    if (k < D) {
-      const float r = r_at(k);
-      part = fmaf(r, r, part);
-    }
-    if ((u & 7) == 7) {  // fold every 8 terms into the f64 accumulator
-      acc += (double)part;
-      part = 0.f;
-    }
-  }
-  acc += (double)part;
-  acc = warp_sum(acc);
-  __shared__ double red[SIG_THREADS / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = acc;
+// sum over the CTA's chunk of D of one f32 value per thread (the sum of r^2 over the thread's
+// 8 consecutive elements, blockIdx.x * SIG_CHUNK + 8 threadIdx.x + ...) in f64, in a fixed
+// order; valid in thread 0.  The f32 values meet in shared memory and 128 threads fold 8
+// each, so f64 adds run on full warps.  The rollout sampler and the step signals share it
+// and the element-to-thread map, so equal residuals give equal log-probs.
+__device__ __forceinline__ double chunk_sum(float part) {
+  __shared__ float vals[SIG_THREADS];
+  __shared__ double red[4];
+  vals[threadIdx.x] = part;
   __syncthreads();
+  if (threadIdx.x < 128) {
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < SIG_THREADS / 128; ++q) s += (double)vals[q * 128 + threadIdx.x];
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = s;
+  }
+  __syncthreads();
+  return threadIdx.x == 0 ? (red[0] + red[1]) + (red[2] + red[3]) : 0.0;
+}
+// sum of a row's chunk partials by one warp, in a fixed order (every lane gets it).
+__device__ __forceinline__ double sum_partials(const double* partial, int chunks) {
   double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < SIG_THREADS / 32; ++w) s += red[w];
-  return s;
+  for (int c = threadIdx.x & 31; c < chunks; c += 32) s += partial[c];
+  return warp_sum(s);
 }
 
 // Eq. logprob from the squared residual norm.  Written with explicitly rounded operations so
@@ -146,78 +141,177 @@ __device__ __forceinline__ double gauss_logp(double rr, double sg, int64_t D) {
   return __dsub_rn(-quad, norm);
 }
 
-// grid: (chunks, G*W)
-__global__ void __launch_bounds__(SIG_THREADS) resid_norm_kernel(const void* v, int v_f32, const float* z,
-                                                                 const double* mc, int W, int64_t D, double* partial) {
-  const int ij = blockIdx.y;
-  const int i = ij / W, j = ij % W;
-  const Coef2 a = split_coef(mc[j]), c = split_coef(mc[W + j]);
-  const float* z0 = z + ((int64_t)i * (W + 1) + j) * D;
-  const float* z1 = z0 + D;
-  const int64_t vb = ((int64_t)i * W + j) * D;
-  const double s =
-      chunk_sq_sum(D, [&](int64_t k) { return resid(z1[k], z0[k], ldv_any(v, vb + k, v_f32), a, c); });
-  if (threadIdx.x == 0) partial[(int64_t)ij * gridDim.x + blockIdx.x] = s;
+// The inputs of one window's step signals; sched_alpha == nullptr selects the rectified-flow
+// step.  vec: every row of v and z starts on a 16-byte boundary.
+struct Window {
+  const void* v;
+  int v_f32, vec;
+  const float* z;
+  const double* t;
+  const double* sched_alpha;
+  const double* sched_sigma;
+  int G, W;
+  int64_t D;
+};
+
+// The mean coefficients of step j of the window (false: a bad schedule).
+__device__ __forceinline__ bool window_coef(const Window& w, int j, double* a, double* c) {
+  const bool eps = w.sched_alpha != nullptr;
+  return mean_coef(w.t[j], w.t[j + 1], eps, eps ? w.sched_alpha[j] : 0.0, eps ? w.sched_alpha[j + 1] : 0.0,
+                   eps ? w.sched_sigma[j] : 0.0, eps ? w.sched_sigma[j + 1] : 0.0, a, c);
 }
 
-// One thread per (i, j).
-__global__ void logprob_kernel(const double* partial, int chunks, const double* mc, const double* sigma,
-                               const double* logp_old, const double* adv, int G, int W, int64_t D, double clip_eps,
-                               double scale, double* logp_new, double* ratio, uint8_t* clipped, float* coef) {
-  const int ij = blockIdx.x * blockDim.x + threadIdx.x;
-  if (ij >= G * W) return;
-  const int i = ij / W, j = ij % W;
-  double rr = 0.0;
-  for (int c = 0; c < chunks; ++c) rr += partial[(int64_t)ij * chunks + c];
+// Advantage of sample i by one warp: A_i = clamp((r_i - mean) / (std + eps), +-clip).
+__device__ __forceinline__ void advantage(const float* rewards, int G, int i, double adv_eps, double adv_clip,
+                                          double* adv) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int g = lane; g < G; g += 32) s += (double)rewards[g];
+  const double mu = warp_sum(s) / G;
+  s = 0.0;
+  for (int g = lane; g < G; g += 32) {
+    const double d = (double)rewards[g] - mu;
+    s += d * d;
+  }
+  s = warp_sum(s);
+  if (lane != 0) return;
+  const double sd = G > 1 ? sqrt(s / (G - 1)) : 0.0;
+  const double a = ((double)rewards[i] - mu) / (sd + adv_eps);
+  adv[i] = a > adv_clip ? adv_clip : (a < -adv_clip ? -adv_clip : a);
+}
+
+// grid: (chunks, G*W).  Bound by reading v and z once from DRAM; every load of a thread is
+// issued before the first use.
+__global__ void __launch_bounds__(SIG_THREADS) resid_norm_kernel(Window w, const float* rewards, double adv_eps,
+                                                                 double adv_clip, double* adv, double* partial) {
+  const int ij = blockIdx.y;
+  const int i = ij / w.W, j = ij % w.W;
+  const float* z0 = w.z + ((int64_t)i * (w.W + 1) + j) * w.D;
+  const int64_t vb = ((int64_t)i * w.W + j) * w.D;
+  const int64_t k = (int64_t)blockIdx.x * SIG_CHUNK + (int64_t)threadIdx.x * SIG_PER_THREAD;
+  float x0[8], x1[8], y[8];
+  load8(z0, k, w.D, w.vec, x0);
+  load8(z0 + w.D, k, w.D, w.vec, x1);
+  load8_any(w.v, vb, w.v_f32, k, w.D, w.vec, y);
+  __shared__ Coef2 coef[2];
+  if (threadIdx.x == 0) {
+    double ad, cd;
+    if (!window_coef(w, j, &ad, &cd) && blockIdx.x == 0) set_device_status(JAGG_DEV_BADARG);
+    coef[0] = split_coef(ad);
+    coef[1] = split_coef(cd);
+  }
+  __syncthreads();
+  const Coef2 a = coef[0], c = coef[1];
+  float part = 0.f;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {  // elements past D loaded as zeros: r = 0
+    const float r = resid(x1[e], x0[e], y[e], a, c);
+    part = fmaf(r, r, part);
+  }
+  const double s = chunk_sum(part);
+  if (threadIdx.x == 0) partial[(int64_t)ij * gridDim.x + blockIdx.x] = s;
+  if (blockIdx.x == 0 && j == 0 && threadIdx.x < 32) advantage(rewards, w.G, i, adv_eps, adv_clip, adv);
+}
+
+// One warp per (i, j).  What the elementwise pass needs of a step goes back into the workspace:
+// mc[j] = the mean coefficients (a.hi, a.lo, c.hi, c.lo), and the signal's coefficient and
+// the aggregation weight (k, alpha) over the first of the step's own partial sums.
+__global__ void __launch_bounds__(32) logprob_kernel(Window w, double* partial, int chunks, const double* sigma,
+                                                     const double* logp_old, const double* adv, double clip_eps,
+                                                     double scale, int aggregate, double* logp_new, double* ratio,
+                                                     uint8_t* clipped, float4* mc) {
+  const int ij = blockIdx.x;
+  const int i = ij / w.W, j = ij % w.W;
+  const double rr = sum_partials(partial + (int64_t)ij * chunks, chunks);
+  if (threadIdx.x != 0) return;
+  double am, c;
+  window_coef(w, j, &am, &c);
   const double sg = sigma[j];
-  const double c = mc[W + j];
-  const double lp = gauss_logp(rr, sg, D);
+  const double lp = gauss_logp(rr, sg, w.D);
   const double rho = exp(lp - logp_old[ij]);
   const double a = adv[i];
   const bool clip = (a > 0.0 && rho > 1.0 + clip_eps) || (a < 0.0 && rho < 1.0 - clip_eps);
   logp_new[ij] = lp;
   ratio[ij] = rho;
   clipped[ij] = clip ? 1 : 0;
-  coef[ij] = clip ? 0.f : (float)(scale * (-a) * rho * c / (sg * sg));
+  float2 q = make_float2(clip ? 0.f : (float)(scale * (-a) * rho * c / (sg * sg)), 0.f);
+  if (aggregate) {
+    const double den = w.t[0] - w.t[w.W - 1];
+    if (den != 0.0)
+      q.y = (float)((w.t[0] - w.t[j]) / den);
+    else
+      set_device_status(JAGG_DEV_BADARG);
+  }
+  *reinterpret_cast<float2*>(partial + (int64_t)ij * chunks) = q;
+  if (i == 0) {
+    const Coef2 ca = split_coef(am), cc = split_coef(c);
+    mc[j] = make_float4(ca.hi, ca.lo, cc.hi, cc.lo);
+  }
 }
 
-// grid: (ceil(D / SIG_THREADS / 4), G).  Each thread: 4 consecutive elements of D.
-__global__ void __launch_bounds__(SIG_THREADS) apply_kernel(const void* v, int v_f32, const float* z, const double* t,
-                                                            const double* mc, const float* coef, int G, int W,
-                                                            int64_t D, float* s_out, float* cot_out) {
+// grid: (ceil(D / 4 / APPLY_THREADS), G).  Each thread: 4 consecutive elements of D over every
+// step.
+__global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(Window w, const double* partial, int chunks,
+                                                              const float4* mc, float* s_out, float* cot_out,
+                                                              int vec_out) {
   const int i = blockIdx.y;
-  const int64_t kbase = ((int64_t)blockIdx.x * SIG_THREADS + threadIdx.x) * 4;
+  const int64_t D = w.D;
+  const int64_t kbase = ((int64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) * 4;
   if (kbase >= D) return;
-  const double den = t[0] - t[W - 1];
+  const bool full = kbase + 4 <= D;
+  auto load4 = [&](const float* p, bool vec, float (&x)[4]) {
+    if (vec && full) {
+      const float4 f = *reinterpret_cast<const float4*>(p + kbase);
+      x[0] = f.x; x[1] = f.y; x[2] = f.z; x[3] = f.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = kbase + e < D ? p[kbase + e] : 0.f;
+    }
+  };
+  auto store4 = [&](float* p, const float (&x)[4]) {
+    if (vec_out && full) {
+      *reinterpret_cast<float4*>(p + kbase) = make_float4(x[0], x[1], x[2], x[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (kbase + e < D) p[kbase + e] = x[e];
+    }
+  };
   float base[4] = {0.f, 0.f, 0.f, 0.f}, corr[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int j = 0; j < W; ++j) {
-    const Coef2 ma = split_coef(mc[j]), mcj = split_coef(mc[W + j]);
-    const float c = coef[i * W + j];
-    const float al = cot_out ? (den != 0.0 ? (float)((t[0] - t[j]) / den) : 0.f) : 0.f;
-    const float* z0 = z + ((int64_t)i * (W + 1) + j) * D;
-    const float* z1 = z0 + D;
-    const int64_t vb = ((int64_t)i * W + j) * D;
+  float x0[4];
+  load4(w.z + (int64_t)i * (w.W + 1) * D, w.vec, x0);
+#pragma unroll 4
+  for (int j = 0; j < w.W; ++j) {
+    const int64_t vb = ((int64_t)i * w.W + j) * D;
+    float x1[4], y[4], s[4];
+    load4(w.z + ((int64_t)i * (w.W + 1) + j + 1) * D, w.vec, x1);
+    if (w.v_f32) {
+      load4(static_cast<const float*>(w.v) + vb, w.vec, y);
+    } else if (w.vec && full) {
+      const uint2 raw = *reinterpret_cast<const uint2*>(static_cast<const bf16*>(w.v) + vb + kbase);
+      const bf16* h = reinterpret_cast<const bf16*>(&raw);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) y[e] = __bfloat162float(h[e]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        y[e] = kbase + e < D ? __bfloat162float(static_cast<const bf16*>(w.v)[vb + kbase + e]) : 0.f;
+    }
+    const float2 q = *reinterpret_cast<const float2*>(partial + ((int64_t)i * w.W + j) * chunks);
+    const float4 m = mc[j];
+    const Coef2 a{m.x, m.y}, c{m.z, m.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int64_t k = kbase + e;
-      if (k < D) {
-        const float r = resid(z1[k], z0[k], ldv_any(v, vb + k, v_f32), ma, mcj);
-        const float s = c * r;
-        if (s_out) s_out[vb + k] = s;
-        base[e] += (1.f - al) * s;
-        corr[e] += al * s;
-      }
+      s[e] = q.x * resid(x1[e], x0[e], y[e], a, c);
+      base[e] += (1.f - q.y) * s[e];
+      corr[e] += q.y * s[e];
+      x0[e] = x1[e];
     }
+    if (s_out) store4(s_out + vb, s);
   }
   if (cot_out) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int64_t k = kbase + e;
-      if (k < D) {
-        cot_out[(int64_t)i * D + k] = base[e];
-        cot_out[((int64_t)G + i) * D + k] = corr[e];
-      }
-    }
+    store4(cot_out + (int64_t)i * D, base);
+    store4(cot_out + ((int64_t)w.G + i) * D, corr);
   }
 }
 
@@ -225,7 +319,7 @@ __global__ void __launch_bounds__(SIG_THREADS) apply_kernel(const void* v, int v
 // and stored, then its residual against the mean enters the same chunk sums as the signals.
 struct RolloutStep {
   const void* y;
-  int y_f32;
+  int y_f32, vec;  // vec: every row of y, z, xi and z_model starts on a 16-byte boundary
   const float* z_cur;
   const float* xi;
   float* z_next;
@@ -239,41 +333,70 @@ struct RolloutStep {
 
 __global__ void __launch_bounds__(SIG_THREADS) rollout_step_kernel(RolloutStep p) {
   const int i = blockIdx.y;
-  double ad, cd;
-  if (!mean_coef(p.t0, p.t1, p.eps != 0, p.a0, p.a1, p.s0, p.s1, &ad, &cd) && blockIdx.x == 0 && i == 0 &&
-      threadIdx.x == 0)
-    set_device_status(JAGG_DEV_BADARG);
-  const Coef2 a = split_coef(ad), c = split_coef(cd);
+  const int64_t D = p.D;
+  const int64_t k = (int64_t)blockIdx.x * SIG_CHUNK + (int64_t)threadIdx.x * SIG_PER_THREAD;
+  float zc[8], y[8], xi[8];
+  load8(p.z_cur + (int64_t)i * p.z_ld, k, D, p.vec, zc);
+  load8_any(p.y, (int64_t)i * p.y_ld, p.y_f32, k, D, p.vec, y);
+  load8(p.xi + (int64_t)i * p.xi_ld, k, D, p.vec, xi);
+  __shared__ Coef2 coef[2];
+  if (threadIdx.x == 0) {
+    double ad, cd;
+    if (!mean_coef(p.t0, p.t1, p.eps != 0, p.a0, p.a1, p.s0, p.s1, &ad, &cd) && blockIdx.x == 0 && i == 0)
+      set_device_status(JAGG_DEV_BADARG);
+    coef[0] = split_coef(ad);
+    coef[1] = split_coef(cd);
+  }
+  __syncthreads();
+  const Coef2 a = coef[0], c = coef[1];
   const float sg = (float)p.sigma;
-  const float* z0 = p.z_cur + (int64_t)i * p.z_ld;
+  float zn[8];
+  float part = 0.f;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {  // elements past D loaded as zeros: z_next = r = 0 there
+    float m = fmaf(a.lo, zc[e], c.lo * y[e]);
+    m = fmaf(c.hi, y[e], m);
+    m = fmaf(a.hi, zc[e], m);
+    zn[e] = fmaf(sg, xi[e], m);
+    const float r = resid(zn[e], zc[e], y[e], a, c);
+    part = fmaf(r, r, part);
+  }
   float* z1 = p.z_next + (int64_t)i * p.z_ld;
-  const float* xi = p.xi + (int64_t)i * p.xi_ld;
-  const int64_t yb = (int64_t)i * p.y_ld;
-  const double s = chunk_sq_sum(p.D, [&](int64_t k) {
-    const float zk = z0[k], yk = ldv_any(p.y, yb + k, p.y_f32);
-    float m = fmaf(a.lo, zk, c.lo * yk);
-    m = fmaf(c.hi, yk, m);
-    m = fmaf(a.hi, zk, m);
-    const float zn = fmaf(sg, xi[k], m);
-    z1[k] = zn;
-    if (p.z_model) {
-      if (p.zm_f32)
-        static_cast<float*>(p.z_model)[(int64_t)i * p.D + k] = zn;
-      else
-        static_cast<bf16*>(p.z_model)[(int64_t)i * p.D + k] = __float2bfloat16_rn(zn);
+  float* zmf = p.zm_f32 ? static_cast<float*>(p.z_model) : nullptr;
+  bf16* zmb = p.zm_f32 ? nullptr : static_cast<bf16*>(p.z_model);
+  if (p.vec && k + 8 <= D) {
+    const float4 lo = make_float4(zn[0], zn[1], zn[2], zn[3]), hi = make_float4(zn[4], zn[5], zn[6], zn[7]);
+    *reinterpret_cast<float4*>(z1 + k) = lo;
+    *reinterpret_cast<float4*>(z1 + k + 4) = hi;
+    if (zmf) {
+      *reinterpret_cast<float4*>(zmf + (int64_t)i * D + k) = lo;
+      *reinterpret_cast<float4*>(zmf + (int64_t)i * D + k + 4) = hi;
+    } else if (zmb) {
+      uint4 raw;
+      __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&raw);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) h[e] = __floats2bfloat162_rn(zn[2 * e], zn[2 * e + 1]);
+      *reinterpret_cast<uint4*>(zmb + (int64_t)i * D + k) = raw;
     }
-    return resid(zn, zk, yk, a, c);
-  });
+  } else {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (k + e >= D) break;
+      z1[k + e] = zn[e];
+      if (zmf) zmf[(int64_t)i * D + k + e] = zn[e];
+      if (zmb) zmb[(int64_t)i * D + k + e] = __float2bfloat16_rn(zn[e]);
+    }
+  }
+  const double s = chunk_sum(part);
   if (threadIdx.x == 0) p.partial[(int64_t)i * gridDim.x + blockIdx.x] = s;
 }
 
-__global__ void rollout_logp_kernel(const double* partial, int chunks, double sigma, int G, int64_t D,
-                                    double* logp, int64_t logp_ld) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= G) return;
-  double rr = 0.0;
-  for (int c = 0; c < chunks; ++c) rr += partial[(int64_t)i * chunks + c];
-  logp[(int64_t)i * logp_ld] = gauss_logp(rr, sigma, D);
+// One warp per sample.
+__global__ void __launch_bounds__(32) rollout_logp_kernel(const double* partial, int chunks, double sigma, int64_t D,
+                                                          double* logp, int64_t logp_ld) {
+  const int i = blockIdx.x;
+  const double rr = sum_partials(partial + (int64_t)i * chunks, chunks);
+  if (threadIdx.x == 0) logp[(int64_t)i * logp_ld] = gauss_logp(rr, sigma, D);
 }
 
 __global__ void check_alpha_kernel(const double* t, int W) {
@@ -411,7 +534,7 @@ __global__ void grad_reduce_final(const double* partial, double* out3) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// The (a_j, c_j) pairs at the head of the signals workspace, padded to 16 bytes.
+// The mean coefficients (a_j, c_j as hi, lo floats) at the head of the signals workspace.
 int64_t mean_coef_bytes(int W) { return ((int64_t)2 * W * 8 + 15) / 16 * 16; }
 
 }  // namespace
@@ -448,27 +571,22 @@ int step_signals(const char* name, const void* v_hat, int v_dtype, const float* 
   }
   JAGG_CHECK_ARG(aligned16(ws), "%s: workspace not 16-byte aligned", name);
   const int chunks = (int)((D + SIG_CHUNK - 1) / SIG_CHUNK);
-  double* mc = static_cast<double*>(ws);
+  float4* mc = static_cast<float4*>(ws);
   double* partial = reinterpret_cast<double*>(static_cast<char*>(ws) + mean_coef_bytes(W));
-  float* coef = reinterpret_cast<float*>(partial + (int64_t)G * W * chunks);
   const int vf32 = v_dtype == JAGG_DTYPE_F32;
+  // 16-byte rows: z rows of D floats and v rows of D elements from aligned bases
+  const bool vec = D % 8 == 0 && aligned16(v_hat) && aligned16(z);
+  const bool vec_out = D % 4 == 0 && (!s_out || aligned16(s_out)) && (!cot_out || aligned16(cot_out));
+  const Window win{v_hat, vf32, vec ? 1 : 0, z, t, sched_alpha, sched_sigma, G, W, D};
   const int tok = prof_start(stream);
-  prep_kernel<<<1, 32, 0, stream>>>(rewards, G, adv_eps, adv_clip, adv_out, t, sched_alpha, sched_sigma, W, mc);
+  resid_norm_kernel<<<dim3(chunks, G * W), SIG_THREADS, 0, stream>>>(win, rewards, adv_eps, adv_clip, adv_out, partial);
   JAGG_LAUNCHED();
-  resid_norm_kernel<<<dim3(chunks, G * W), SIG_THREADS, 0, stream>>>(v_hat, vf32, z, mc, W, D, partial);
-  JAGG_LAUNCHED();
-  logprob_kernel<<<ceil_div((int64_t)G * W, 128), 128, 0, stream>>>(partial, chunks, mc, sigma, logp_old, adv_out, G,
-                                                                     W, D, clip_eps, scale, logp_new, ratio, clipped,
-                                                                     coef);
+  logprob_kernel<<<G * W, 32, 0, stream>>>(win, partial, chunks, sigma, logp_old, adv_out, clip_eps, scale,
+                                           cot_out ? 1 : 0, logp_new, ratio, clipped, mc);
   JAGG_LAUNCHED();
   if (s_out || cot_out) {
-    if (cot_out) {
-      check_alpha_kernel<<<1, 32, 0, stream>>>(t, W);
-      JAGG_LAUNCHED();
-    }
-    const int gx = ceil_div(D, (int64_t)SIG_THREADS * 4);
-    apply_kernel<<<dim3(gx, G), SIG_THREADS, 0, stream>>>(v_hat, vf32, z, t, mc, coef, G, W, D, s_out,
-                                                          cot_out);
+    const int gx = ceil_div(D, (int64_t)APPLY_THREADS * 4);
+    apply_kernel<<<dim3(gx, G), APPLY_THREADS, 0, stream>>>(win, partial, chunks, mc, s_out, cot_out, vec_out ? 1 : 0);
     JAGG_LAUNCHED();
   }
   // algorithmic bytes: v-hat and the W + 1 latents of every sample read once, the signals
@@ -530,14 +648,15 @@ extern "C" int jagg_rollout_step(const void* y_hat, int y_dtype, int64_t y_sampl
   }
   JAGG_CHECK_ARG(aligned16(ws), "jagg_rollout_step: workspace not 16-byte aligned");
   const int chunks = (int)((D + SIG_CHUNK - 1) / SIG_CHUNK);
-  RolloutStep p{y_hat, y_dtype == JAGG_DTYPE_F32, z_cur, xi, z_next, z_model, z_model_dtype == JAGG_DTYPE_F32,
+  const bool vec = D % 8 == 0 && zl % 4 == 0 && yl % 8 == 0 && xl % 4 == 0 && aligned16(y_hat) && aligned16(z_cur) &&
+                   aligned16(z_next) && aligned16(xi) && (!z_model || aligned16(z_model));
+  RolloutStep p{y_hat, y_dtype == JAGG_DTYPE_F32, vec ? 1 : 0, z_cur, xi, z_next, z_model, z_model_dtype == JAGG_DTYPE_F32,
                 D, zl, yl, xl, t_cur, t_next, sigma,
                 sched ? sched[0] : 0.0, sched ? sched[1] : 0.0, sched ? sched[2] : 0.0, sched ? sched[3] : 0.0,
                 sched ? 1 : 0, static_cast<double*>(ws)};
   rollout_step_kernel<<<dim3(chunks, G), SIG_THREADS, 0, stream>>>(p);
   JAGG_LAUNCHED();
-  rollout_logp_kernel<<<ceil_div((int64_t)G, 128), 128, 0, stream>>>(static_cast<double*>(ws), chunks, sigma, G, D,
-                                                                      logp, logp_stride);
+  rollout_logp_kernel<<<G, 32, 0, stream>>>(static_cast<double*>(ws), chunks, sigma, D, logp, logp_stride);
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
