@@ -446,12 +446,18 @@ __global__ void aggregate_span_kernel(const float* s, int64_t ld, const double* 
 }
 
 // ------------------------------------------------------------------ grad_reduce
-constexpr int GR_BLOCKS = 1024;
+constexpr int GR_BLOCKS = 1024;  // the most CTAs (rows of partial sums in the workspace)
 constexpr int GR_THREADS = 256;
+constexpr int GR_UNROLL = 4;
+constexpr int GR_RUN = GR_THREADS * GR_UNROLL;  // float4 of a vector per CTA and iteration
 
 // HAS_B: a second vector b (else <a, b> = |b|^2 = |a|^2 and b is not read); HAS_ACC: the
-// update acc += alpha a.  Each thread loads a run of 8 float4 of each input before using any
-// of them, so 8 (16) loads per thread are in flight; f32 sums over a run fold into f64.
+// update acc += alpha a.  A CTA walks runs of GR_RUN consecutive float4 of each vector; each
+// thread issues its GR_UNROLL loads of every input before using any, as streaming accesses
+// (the vectors are read once); f32 sums over 16 terms fold into f64.  Bound by DRAM: with a,
+// b and acc of 130 M elements 305 us (6.8 TB/s, the copy rate); 427 us when a thread's eight
+// loads were a grid apart, 1024 CTAs ran in more than one wave and one thread per sum
+// added the partials.
 template <bool HAS_B, bool HAS_ACC>
 __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a, const float* b, int64_t P,
                                                                  float alpha, float* acc, double* partial) {
@@ -460,34 +466,29 @@ __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a,
   const float4* a4 = reinterpret_cast<const float4*>(a);
   const float4* b4 = reinterpret_cast<const float4*>(b);
   float4* c4 = reinterpret_cast<float4*>(acc);
-  const int64_t stride = (int64_t)GR_BLOCKS * GR_THREADS;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int64_t idx = (int64_t)blockIdx.x * GR_THREADS + threadIdx.x; idx < nvec; idx += 8 * stride) {
-    float4 x[8], y[8];
+  for (int64_t i0 = (int64_t)blockIdx.x * GR_RUN + threadIdx.x; i0 < nvec; i0 += (int64_t)gridDim.x * GR_RUN) {
+    float4 x[GR_UNROLL], y[GR_UNROLL], c[GR_UNROLL];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int64_t q = idx + (int64_t)r * stride;
-      x[r] = q < nvec ? a4[q] : zero;
-      if constexpr (HAS_B) y[r] = q < nvec ? b4[q] : zero;
+    for (int r = 0; r < GR_UNROLL; ++r) {
+      const int64_t q = i0 + r * GR_THREADS;
+      const bool in = q < nvec;
+      x[r] = in ? __ldcs(a4 + q) : zero;
+      if constexpr (HAS_B) y[r] = in ? __ldcs(b4 + q) : zero;
+      if constexpr (HAS_ACC) c[r] = in ? __ldcs(c4 + q) : zero;
     }
     float fab = 0.f, faa = 0.f, fbb = 0.f;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
+    for (int r = 0; r < GR_UNROLL; ++r) {
       faa += x[r].x * x[r].x + x[r].y * x[r].y + x[r].z * x[r].z + x[r].w * x[r].w;
       if constexpr (HAS_B) {
         fab += x[r].x * y[r].x + x[r].y * y[r].y + x[r].z * y[r].z + x[r].w * y[r].w;
         fbb += y[r].x * y[r].x + y[r].y * y[r].y + y[r].z * y[r].z + y[r].w * y[r].w;
       }
-    }
-    if constexpr (HAS_ACC) {
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int64_t q = idx + (int64_t)r * stride;
-        if (q < nvec) {
-          float4 c = c4[q];
-          c.x += alpha * x[r].x; c.y += alpha * x[r].y; c.z += alpha * x[r].z; c.w += alpha * x[r].w;
-          c4[q] = c;
-        }
+      if constexpr (HAS_ACC) {
+        const int64_t q = i0 + r * GR_THREADS;
+        c[r].x += alpha * x[r].x; c[r].y += alpha * x[r].y; c[r].z += alpha * x[r].z; c[r].w += alpha * x[r].w;
+        if (q < nvec) __stcs(c4 + q, c[r]);
       }
     }
     if constexpr (!HAS_B) fab = fbb = faa;
@@ -524,12 +525,14 @@ __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a,
   }
 }
 
-__global__ void grad_reduce_final(const double* partial, double* out3) {
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int i = 0; i < GR_BLOCKS; ++i) s += partial[(int64_t)i * 3 + threadIdx.x];
-    out3[threadIdx.x] = s;
-  }
+// Three warps: the sums over the CTAs' partials of <a, b>, |a|^2, |b|^2.
+__global__ void __launch_bounds__(96) grad_reduce_final(const double* partial, int blocks, double* out3) {
+  const int w = threadIdx.x / 32;
+  double s = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 31; i < blocks; i += 32) s += partial[(int64_t)i * 3 + w];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) out3[w] = s;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -731,17 +734,21 @@ extern "C" int grad_reduce(const float* a, const float* b, int64_t P, float alph
   }
   const int tok = prof_start(stream);
   double* part = out3 ? static_cast<double*>(ws) : nullptr;
+  // as many CTAs as stay resident at 3 per SM, fewer for a short vector
+  const int64_t runs = (P / 4 + GR_RUN - 1) / GR_RUN;
+  const int most = 3 * sm_count() < GR_BLOCKS ? 3 * sm_count() : GR_BLOCKS;
+  const int blocks = runs < 1 ? 1 : (runs < most ? (int)runs : most);
   if (b && acc)
-    grad_reduce_kernel<true, true><<<GR_BLOCKS, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    grad_reduce_kernel<true, true><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
   else if (b)
-    grad_reduce_kernel<true, false><<<GR_BLOCKS, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    grad_reduce_kernel<true, false><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
   else if (acc)
-    grad_reduce_kernel<false, true><<<GR_BLOCKS, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    grad_reduce_kernel<false, true><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
   else
-    grad_reduce_kernel<false, false><<<GR_BLOCKS, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    grad_reduce_kernel<false, false><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
   JAGG_LAUNCHED();
   if (out3) {
-    grad_reduce_final<<<1, 32, 0, stream>>>(static_cast<const double*>(ws), out3);
+    grad_reduce_final<<<1, 96, 0, stream>>>(static_cast<const double*>(ws), blocks, out3);
     JAGG_LAUNCHED();
   }
   // algorithmic bytes: a (and b) read, acc read and written
