@@ -93,6 +93,7 @@ __device__ __forceinline__ void load_tile(bf16* sm, const SegRows& sr, int b, in
 // ------------------------------------------------------------------ bf16 forward
 template <int D>
 __global__ void __launch_bounds__(128) fa_fwd_kernel(AttnArgs a) {
+  pdl_wait();
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int P = D + 8;
   bf16* sQ = reinterpret_cast<bf16*>(smem);
@@ -215,6 +216,7 @@ __global__ void __launch_bounds__(128) fa_fwd_kernel(AttnArgs a) {
 // ------------------------------------------------------------------ bf16 backward
 template <int D>
 __global__ void __launch_bounds__(128) fa_bwd_kernel(AttnBwdArgs a) {
+  pdl_wait();
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int P = D + 8;
   constexpr int PS = TILE + 8;
@@ -407,6 +409,7 @@ __global__ void __launch_bounds__(128) fa_bwd_kernel(AttnBwdArgs a) {
 // ------------------------------------------------------------------ SIMT (any dtype)
 template <int D>
 __global__ void attn_fwd_simt(AttnArgs a) {
+  pdl_wait();
   const int bh = blockIdx.y, b = bh / a.heads, h = bh % a.heads;
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   const int N = a.N;
@@ -437,6 +440,7 @@ __global__ void attn_fwd_simt(AttnArgs a) {
 
 template <int D>
 __global__ void attn_bwd_simt(AttnBwdArgs a) {
+  pdl_wait();
   const AttnArgs& f = a.f;
   const int bh = blockIdx.y, b = bh / f.heads, h = bh % f.heads;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -481,6 +485,7 @@ __global__ void attn_bwd_simt(AttnBwdArgs a) {
 // One thread per (row, 8 columns); the D/8 threads of a head are adjacent lanes and
 // combine their partial dots with shuffles.
 __global__ void rowdot_zero_kernel(AttnBwdArgs a) {
+  pdl_wait();
   const AttnArgs& f = a.f;
   const int d = f.heads * f.dh;
   const int cpr = d / 8;  // 8-column chunks per row
@@ -519,6 +524,7 @@ __global__ void rowdot_zero_kernel(AttnBwdArgs a) {
 
 // dq (storage type, segment rows) <- dq_acc (f32); one thread per (row, 8 columns).
 __global__ void dq_store_kernel(AttnBwdArgs a) {
+  pdl_wait();
   const AttnArgs& f = a.f;
   const int d = f.heads * f.dh;
   const int cpr = d / 8;
@@ -554,7 +560,7 @@ int fwd_tc(const AttnArgs& a, cudaStream_t s) {
   }
   dim3 grid(ceil_div(a.N, TILE), a.B * a.heads);
   const int tok = prof_start(s);
-  fa_fwd_kernel<D><<<grid, 128, smem, s>>>(a);
+  JAGG_CUDA_TRY(launch(fa_fwd_kernel<D>, grid, 128, smem, s, a));
   JAGG_LAUNCHED();
   // QK^T and PV: 2 N^2 d multiply-adds per (sequence, head)
   prof_stop(tok, s, PROF_ATTN_FWD, 4.0 * a.B * a.heads * (double)a.N * a.N * D,
@@ -571,7 +577,7 @@ int bwd_tc(const AttnBwdArgs& a, cudaStream_t s) {
   }
   dim3 grid(ceil_div(a.f.N, TILE), a.f.B * a.f.heads);
   const int tok = prof_start(s);
-  fa_bwd_kernel<D><<<grid, 128, smem, s>>>(a);
+  JAGG_CUDA_TRY(launch(fa_bwd_kernel<D>, grid, 128, smem, s, a));
   JAGG_LAUNCHED();
   // dV = P^T dO, dP = dO V^T, dQ = dS K, dK = dS^T Q: 4 N^2 d multiply-adds per (sequence,
   // head); the recomputation of S is not counted
@@ -583,14 +589,14 @@ int bwd_tc(const AttnBwdArgs& a, cudaStream_t s) {
 template <int D>
 int fwd_simt(const AttnArgs& a, cudaStream_t s) {
   dim3 grid(ceil_div(a.N, 64), a.B * a.heads);
-  attn_fwd_simt<D><<<grid, 64, 0, s>>>(a);
+  JAGG_CUDA_TRY(launch(attn_fwd_simt<D>, grid, 64, 0, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 template <int D>
 int bwd_simt(const AttnBwdArgs& a, cudaStream_t s) {
   dim3 grid(ceil_div(a.f.N, 64), a.f.B * a.f.heads);
-  attn_bwd_simt<D><<<grid, 64, 0, s>>>(a);
+  JAGG_CUDA_TRY(launch(attn_bwd_simt<D>, grid, 64, 0, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -644,7 +650,7 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
   const int64_t chunks = (int64_t)f.B * f.N * f.heads * f.dh / 8;
   JAGG_CHECK_ARG(chunks < (1ll << 31), "attention: too many rows");
   int tok = prof_start(s);
-  rowdot_zero_kernel<<<(int)((chunks + 255) / 256), 256, 0, s>>>(a);
+  JAGG_CUDA_TRY(launch(rowdot_zero_kernel, (int)((chunks + 255) / 256), 256, 0, s, a));
   JAGG_LAUNCHED();
   prof_stop(tok, s, PROF_ATTN_AUX, 0.0, 4.0 * f.B * f.N * f.heads * f.dh * 1.5);
   int st = JAGG_ERR_UNSUPPORTED;
@@ -674,7 +680,7 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
   }
   const int64_t total = (int64_t)f.B * f.N * f.heads * f.dh;
   tok = prof_start(s);
-  dq_store_kernel<<<(int)((chunks + 255) / 256), 256, 0, s>>>(a);
+  JAGG_CUDA_TRY(launch(dq_store_kernel, (int)((chunks + 255) / 256), 256, 0, s, a));
   JAGG_LAUNCHED();
   prof_stop(tok, s, PROF_ATTN_AUX, 0.0, 6.0 * total);
   return JAGG_OK;

@@ -198,6 +198,7 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
@@ -650,6 +651,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
@@ -1012,6 +1014,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
@@ -1313,7 +1316,7 @@ int launch_v3(const AttnBwdArgs& a, cudaStream_t s) {
   }
   const int units = ceil_div(N, C::BK) * f.B * f.heads;
   const int nsm = sm_count();
-  kernel<<<units < nsm ? units : nsm, FB2_THREADS, C::SMEM, s>>>(maps, p);
+  JAGG_CUDA_TRY(launch(kernel, units < nsm ? units : nsm, FB2_THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -1349,7 +1352,7 @@ int launch_fwd(const AttnArgs& f, cudaStream_t s) {
   }
   const int units = ceil_div(N, C::BQ) * f.B * f.heads;
   const int nsm = sm_count();
-  fa_fwd_tc_kernel<D><<<units < nsm ? units : nsm, FF_THREADS, C::SMEM, s>>>(maps, p);
+  JAGG_CUDA_TRY(launch(fa_fwd_tc_kernel<D>, units < nsm ? units : nsm, FF_THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -1403,7 +1406,7 @@ int launch_fwd128(const AttnArgs& f, cudaStream_t s) {
   }
   const int units = ceil_div(ceil_div(N, C::BQ), 2) * f.B * f.heads;
   const int nsm = sm_count();
-  fa_fwd_tc128_kernel<<<units < nsm ? units : nsm, FF2_THREADS, C::SMEM, s>>>(maps, p);
+  JAGG_CUDA_TRY(launch(fa_fwd_tc128_kernel, units < nsm ? units : nsm, FF2_THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }

@@ -27,6 +27,7 @@ int grid_for(int64_t n, int threads) {
 
 // ------------------------------------------------------------------ layouts
 __global__ void patchify_kernel(const void* z, int in_f32, void* xp, int out_f32, int B, int C, int H, int W, int p) {
+  pdl_wait();
   const int gw = W / p, gh = H / p;
   const int pd = C * p * p;
   const int64_t total = (int64_t)B * gh * gw * pd;
@@ -43,6 +44,7 @@ __global__ void patchify_kernel(const void* z, int in_f32, void* xp, int out_f32
 }
 
 __global__ void unpatchify_kernel(const void* xp, void* z, int is_f32, int B, int C, int H, int W, int p) {
+  pdl_wait();
   const int gw = W / p, gh = H / p;
   const int pd = C * p * p;
   const int64_t total = (int64_t)B * C * H * W;
@@ -58,6 +60,7 @@ __global__ void unpatchify_kernel(const void* xp, void* z, int is_f32, int B, in
 }
 
 __global__ void temb_kernel(const float* t, float* phi, int B, int dim) {
+  pdl_wait();
   const int half = dim / 2;
   const int total = B * half;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
@@ -71,15 +74,18 @@ __global__ void temb_kernel(const float* t, float* phi, int B, int dim) {
 }
 
 __global__ void silu_kernel(const float* in, float* out, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = silu_f(in[i]);
 }
 __global__ void mul_silu_grad_kernel(float* g, const float* x, int64_t n) {
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     g[i] *= silu_grad_f(x[i]);
 }
 
 __global__ void pos_embed_kernel(float* h, int B, int rows_per_seq, int row0, int gh, int gw, int d) {
+  pdl_wait();
   const int q = d / 4;
   const int64_t total = (int64_t)B * gh * gw * d;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -103,6 +109,7 @@ __global__ void pos_embed_kernel(float* h, int B, int rows_per_seq, int row0, in
 constexpr int LN_MAXV = 24;  // d <= 3072
 
 __global__ void ln_mod_fwd_kernel(LnModFwd a) {
+  pdl_wait();
   const int warps = blockDim.x / 32;
   const int m = blockIdx.x * warps + threadIdx.x / 32;
   const int lane = threadIdx.x & 31;
@@ -199,6 +206,7 @@ constexpr int LNF_ROWS = 8 * LNF_R;
 #endif
 template <int NVT>
 __global__ void __launch_bounds__(256, LNF_MIN_BLOCKS) ln_gate_fused_kernel(LnGateBwd a) {
+  pdl_wait();
   extern __shared__ float part[];  // [4 quantities][4][d/4]
   const int d = a.d, d4 = a.d / 4;
   const int chunks = (a.rows_per_seq + LNF_ROWS - 1) / LNF_ROWS;
@@ -347,6 +355,7 @@ __global__ void __launch_bounds__(256, LNF_MIN_BLOCKS) ln_gate_fused_kernel(LnGa
 // (at most a few sequence segments), so every CTA finishes at the same time.
 template <int NV, bool GATE, bool YBF>
 __global__ void __launch_bounds__(256, 2) ln_gate_rowreg_kernel(LnGateBwd a) {
+  pdl_wait();
   extern __shared__ float part[];  // [8 warps][4 quantities][d], then scale[d], gate[d]
   constexpr int d = 128 * NV;
   const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
@@ -464,6 +473,7 @@ __global__ void __launch_bounds__(256, 2) ln_gate_rowreg_kernel(LnGateBwd a) {
 // at each sequence boundary.
 template <int NV4, bool LN, bool GATE>
 __global__ void __launch_bounds__(256, 2) ln_gate_rowcta_kernel(LnGateBwd a) {
+  pdl_wait();
   constexpr int d = 1024 * NV4;
   __shared__ float red[2][2][8];  // [row parity][s1, s2][warp]
   __shared__ __align__(16) float sc_s[LN ? d : 4], gt_s[GATE ? d : 4];  // 1 + scale, gate of the sequence
@@ -595,7 +605,7 @@ int launch_ln_gate_rowcta_t(const LnGateBwd& a, cudaStream_t s) {
   // equal row shares of at least 8 rows per CTA, at most one wave of resident CTAs
   const int cap = per_sm * sm_count();
   const int want = ceil_div(a.M, 8);
-  ln_gate_rowcta_kernel<NV4, LN, GATE><<<want < cap ? want : cap, 256, 0, s>>>(a);
+  JAGG_CUDA_TRY(launch(ln_gate_rowcta_kernel<NV4, LN, GATE>, want < cap ? want : cap, 256, 0, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -625,7 +635,7 @@ int launch_ln_gate_rowreg_t(const LnGateBwd& a, cudaStream_t s) {
   // equal row shares of at least 16 rows per CTA, at most one wave of resident CTAs
   const int cap = per_sm * sm_count();
   const int want = ceil_div(a.M, 16);
-  ln_gate_rowreg_kernel<NV, GATE, YBF><<<want < cap ? want : cap, 256, smem, s>>>(a);
+  JAGG_CUDA_TRY(launch(ln_gate_rowreg_kernel<NV, GATE, YBF>, want < cap ? want : cap, 256, smem, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -646,7 +656,7 @@ int launch_ln_gate_nv(const LnGateBwd& a, int smem, cudaStream_t s) {
   }
   const int units = (a.M / a.rows_per_seq) * ceil_div(a.rows_per_seq, LNF_ROWS);
   const int cap = per_sm * sm_count();
-  ln_gate_fused_kernel<NVT><<<units < cap ? units : cap, 256, smem, s>>>(a);
+  JAGG_CUDA_TRY(launch(ln_gate_fused_kernel<NVT>, units < cap ? units : cap, 256, smem, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -654,6 +664,7 @@ int launch_ln_gate_nv(const LnGateBwd& a, int smem, cudaStream_t s) {
 // ------------------------------------------------------------------ reductions / copies
 constexpr int CS_ROWS = 64;
 __global__ void colsum_kernel(const void* X, int x_f32, int rows, int cols, int64_t ld, float* db) {
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int r0 = blockIdx.y * CS_ROWS;
   if (c >= cols) return;
@@ -668,6 +679,7 @@ __global__ void colsum_kernel(const void* X, int x_f32, int rows, int cols, int6
 // and each column gets one atomic add per block.
 constexpr int CSV_ROWS = 256;
 __global__ void __launch_bounds__(256) colsum_bf16x8_kernel(const bf16* X, int rows, int cols, int64_t ld, float* db) {
+  pdl_wait();
   __shared__ float part[8][257];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int c0 = (blockIdx.x * 32 + tx) * 8;
@@ -697,6 +709,7 @@ __global__ void __launch_bounds__(256) colsum_bf16x8_kernel(const bf16* X, int r
 
 __global__ void gather_rows_kernel(const float* in, int64_t ld_in, int seg, int seg_off, int64_t seg_stride, void* out,
                                    int out_f32, int rows, int cols) {
+  pdl_wait();
   const int64_t total = (int64_t)rows * cols;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int r = (int)(i / cols), c = (int)(i % cols);
@@ -707,6 +720,7 @@ __global__ void gather_rows_kernel(const float* in, int64_t ld_in, int seg, int 
 template <typename E>
 __global__ void copy_rows_kernel(const E* in, int64_t ld_in, int is, int io, int64_t iss, E* out, int64_t ld_out,
                                  int os, int oo, int64_t oss, int rows, int cols) {
+  pdl_wait();
   const int64_t total = (int64_t)rows * cols;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int r = (int)(i / cols), c = (int)(i % cols);
@@ -718,6 +732,7 @@ __global__ void copy_rows_kernel(const E* in, int64_t ld_in, int is, int io, int
 // bases 16-byte aligned).
 __global__ void copy_rows_v16_kernel(const uint8_t* in, int64_t ld_in_b, int is, int io, int64_t iss, uint8_t* out,
                                      int64_t ld_out_b, int os, int oo, int64_t oss, int rows, int nvec) {
+  pdl_wait();
   for (int r = blockIdx.x; r < rows; r += gridDim.x) {
     const uint4* src = reinterpret_cast<const uint4*>(in + seg_row(r, is, io, iss) * ld_in_b);
     uint4* dst = reinterpret_cast<uint4*>(out + seg_row(r, os, oo, oss) * ld_out_b);
@@ -727,6 +742,7 @@ __global__ void copy_rows_v16_kernel(const uint8_t* in, int64_t ld_in_b, int is,
 
 __global__ void attn_rowdot_kernel(const void* dO, const void* O, int64_t ld, float* Dv, int B, int N, int heads,
                                    int dh, int is_f32) {
+  pdl_wait();
   // one warp per (row, head)
   const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
   const int lane = threadIdx.x & 31;
@@ -770,6 +786,7 @@ __device__ __forceinline__ void rope_angle(int n, int n_txt, int gw, int dh, int
 constexpr int QKN_THREADS = 256, QKN_WARPS = QKN_THREADS / 32;
 
 __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_kernel(QkNormRope a) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int dh = a.d / a.heads;
   const int is_f32 = a.dtype == JAGG_DTYPE_F32;
@@ -815,6 +832,7 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_kernel(QkNormRop
 // sums in registers (q / k x text / image), the block adds its warps' partials in shared
 // memory and issues one atomic per element.
 __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_bwd_kernel(QkNormRopeBwd b) {
+  pdl_wait();
   const QkNormRope& a = b.f;
   __shared__ float part[QKN_WARPS][4][128];
   const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
@@ -951,6 +969,7 @@ __device__ __forceinline__ void rope_lane(const QkNormRope& a, const float2* tab
 }
 
 __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_v_kernel(QkNormRope a) {
+  pdl_wait();
   extern __shared__ __align__(16) float2 rope_tab[];  // [side][32] when a.rope
   if (a.rope) rope_table_fill(a, rope_tab);
   __syncthreads();
@@ -1004,6 +1023,7 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_v_kernel(QkNormR
 }
 
 __global__ void __launch_bounds__(QKN_THREADS, 3) qk_norm_rope_bwd_v_kernel(QkNormRopeBwd b) {
+  pdl_wait();
   const QkNormRope& a = b.f;
   __shared__ float part[QKN_WARPS][4][128];
   extern __shared__ __align__(16) float2 rope_tab[];  // [side][32] when a.rope
@@ -1096,33 +1116,35 @@ int launch_patchify(const void* z, int in_f32, void* xp, int out_f32, int dtype,
                     cudaStream_t s) {
   (void)dtype;
   const int64_t n = (int64_t)B * C * H * W;
-  patchify_kernel<<<grid_for(n, 256), 256, 0, s>>>(z, in_f32, xp, out_f32, B, C, H, W, p);
+  JAGG_CUDA_TRY(launch(patchify_kernel, grid_for(n, 256), 256, 0, s, z, in_f32, xp, out_f32, B, C, H, W, p));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 int launch_unpatchify(const void* xp, void* z, int dtype, int B, int C, int H, int W, int p, cudaStream_t s) {
   const int64_t n = (int64_t)B * C * H * W;
-  unpatchify_kernel<<<grid_for(n, 256), 256, 0, s>>>(xp, z, dtype == JAGG_DTYPE_F32, B, C, H, W, p);
+  JAGG_CUDA_TRY(launch(unpatchify_kernel, grid_for(n, 256), 256, 0, s, xp, z, dtype == JAGG_DTYPE_F32, B, C, H, W,
+                       p));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 int launch_timestep_embedding(const float* t, float* phi, int B, int dim, cudaStream_t s) {
-  temb_kernel<<<grid_for((int64_t)B * dim / 2, 256), 256, 0, s>>>(t, phi, B, dim);
+  JAGG_CUDA_TRY(launch(temb_kernel, grid_for((int64_t)B * dim / 2, 256), 256, 0, s, t, phi, B, dim));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 int launch_silu(const float* in, float* out, int64_t n, cudaStream_t s) {
-  silu_kernel<<<grid_for(n, 256), 256, 0, s>>>(in, out, n);
+  JAGG_CUDA_TRY(launch(silu_kernel, grid_for(n, 256), 256, 0, s, in, out, n));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 int launch_mul_silu_grad(float* g, const float* x, int64_t n, cudaStream_t s) {
-  mul_silu_grad_kernel<<<grid_for(n, 256), 256, 0, s>>>(g, x, n);
+  JAGG_CUDA_TRY(launch(mul_silu_grad_kernel, grid_for(n, 256), 256, 0, s, g, x, n));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 int launch_add_pos_embed(float* h, int B, int rows_per_seq, int row0, int gh, int gw, int d, cudaStream_t s) {
-  pos_embed_kernel<<<grid_for((int64_t)B * gh * gw * d, 256), 256, 0, s>>>(h, B, rows_per_seq, row0, gh, gw, d);
+  JAGG_CUDA_TRY(launch(pos_embed_kernel, grid_for((int64_t)B * gh * gw * d, 256), 256, 0, s, h, B, rows_per_seq,
+                       row0, gh, gw, d));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -1130,7 +1152,7 @@ int launch_ln_mod_fwd(const LnModFwd& a, cudaStream_t s) {
   JAGG_CHECK_ARG(a.d % 4 == 0 && a.d <= 128 * LN_MAXV, "ln_mod: hidden %d unsupported", a.d);
   const int warps = 8;
   const int tok = prof_start(s);
-  ln_mod_fwd_kernel<<<ceil_div(a.M, warps), warps * 32, 0, s>>>(a);
+  JAGG_CUDA_TRY(launch(ln_mod_fwd_kernel, ceil_div(a.M, warps), warps * 32, 0, s, a));
   JAGG_LAUNCHED();
   // algorithmic bytes: h read (f32), the modulated output written (storage type), statistics
   prof_stop(tok, s, PROF_LN_FWD, 0.0,
@@ -1180,21 +1202,22 @@ int launch_colsum(const void* X, int x_f32, int dtype, int rows, int cols, int64
   const double bytes = (double)rows * cols * (x_f32 ? 4 : 2) + 8.0 * cols;
   if (!x_f32 && cols % 8 == 0 && ld % 8 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
     dim3 grid(ceil_div(cols, 256), ceil_div(rows, CSV_ROWS));
-    colsum_bf16x8_kernel<<<grid, 256, 0, s>>>(static_cast<const bf16*>(X), rows, cols, ld, db);
+    JAGG_CUDA_TRY(launch(colsum_bf16x8_kernel, grid, 256, 0, s, static_cast<const bf16*>(X), rows, cols, ld, db));
     JAGG_LAUNCHED();
     prof_stop(tok, s, PROF_COLSUM, 0.0, bytes);
     return JAGG_OK;
   }
   dim3 grid(ceil_div(cols, 256), ceil_div(rows, CS_ROWS));
-  colsum_kernel<<<grid, 256, 0, s>>>(X, x_f32, rows, cols, ld, db);
+  JAGG_CUDA_TRY(launch(colsum_kernel, grid, 256, 0, s, X, x_f32, rows, cols, ld, db));
   JAGG_LAUNCHED();
   prof_stop(tok, s, PROF_COLSUM, 0.0, bytes);
   return JAGG_OK;
 }
 int launch_gather_rows(const float* in, int64_t ld_in, int seg, int seg_off, int64_t seg_stride, void* out,
                        int dtype, int rows, int cols, cudaStream_t s) {
-  gather_rows_kernel<<<grid_for((int64_t)rows * cols, 256), 256, 0, s>>>(in, ld_in, seg, seg_off, seg_stride, out,
-                                                                         dtype == JAGG_DTYPE_F32, rows, cols);
+  JAGG_CUDA_TRY(launch(gather_rows_kernel, grid_for((int64_t)rows * cols, 256), 256, 0, s, in, ld_in, seg, seg_off,
+                       seg_stride, out,
+                                                                         dtype == JAGG_DTYPE_F32, rows, cols));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -1208,17 +1231,20 @@ int launch_copy_rows(const void* in, int64_t ld_in, int in_seg, int in_seg_off, 
   const int g = grid_for((int64_t)rows * cols, 256);
   if (v16 && rows > 0) {
     const int nb = rows < 8 * sm_count() ? rows : 8 * sm_count();
-    copy_rows_v16_kernel<<<nb, 256, 0, s>>>(static_cast<const uint8_t*>(in), ld_in * elem_bytes, in_seg, in_seg_off,
+    JAGG_CUDA_TRY(launch(copy_rows_v16_kernel, nb, 256, 0, s, static_cast<const uint8_t*>(in), ld_in * elem_bytes,
+                         in_seg, in_seg_off,
                                             in_seg_stride, static_cast<uint8_t*>(out), ld_out * elem_bytes, out_seg,
-                                            out_seg_off, out_seg_stride, rows, (int)(row_b / 16));
+                                            out_seg_off, out_seg_stride, rows, (int)(row_b / 16)));
   } else if (elem_bytes == 4)
-    copy_rows_kernel<float><<<g, 256, 0, s>>>(static_cast<const float*>(in), ld_in, in_seg, in_seg_off, in_seg_stride,
+    JAGG_CUDA_TRY(launch(copy_rows_kernel<float>, g, 256, 0, s, static_cast<const float*>(in), ld_in, in_seg,
+                         in_seg_off, in_seg_stride,
                                              static_cast<float*>(out), ld_out, out_seg, out_seg_off, out_seg_stride,
-                                             rows, cols);
+                                             rows, cols));
   else
-    copy_rows_kernel<uint16_t><<<g, 256, 0, s>>>(static_cast<const uint16_t*>(in), ld_in, in_seg, in_seg_off,
+    JAGG_CUDA_TRY(launch(copy_rows_kernel<uint16_t>, g, 256, 0, s, static_cast<const uint16_t*>(in), ld_in, in_seg,
+                         in_seg_off,
                                                 in_seg_stride, static_cast<uint16_t*>(out), ld_out, out_seg,
-                                                out_seg_off, out_seg_stride, rows, cols);
+                                                out_seg_off, out_seg_stride, rows, cols));
   JAGG_LAUNCHED();
   prof_stop(tok, s, PROF_COPY, 0.0, 2.0 * rows * cols * elem_bytes);
   return JAGG_OK;
@@ -1226,8 +1252,8 @@ int launch_copy_rows(const void* in, int64_t ld_in, int in_seg, int in_seg_off, 
 int launch_attn_rowdot(const void* dO, const void* O, int64_t ld, float* Dv, int B, int N, int heads, int dh,
                        int dtype, cudaStream_t s) {
   const int64_t warps = (int64_t)B * N * heads;
-  attn_rowdot_kernel<<<grid_for(warps * 32, 256), 256, 0, s>>>(dO, O, ld, Dv, B, N, heads, dh,
-                                                              dtype == JAGG_DTYPE_F32);
+  JAGG_CUDA_TRY(launch(attn_rowdot_kernel, grid_for(warps * 32, 256), 256, 0, s, dO, O, ld, Dv, B, N, heads, dh,
+                                                              dtype == JAGG_DTYPE_F32));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -1255,9 +1281,10 @@ int launch_qk_norm_rope_fwd(const QkNormRope& a, cudaStream_t s) {
   if (qkn_vector(a)) {
     const int64_t vb = ceil_div((int64_t)a.M, (int64_t)QKN_WARPS);
     const int cap = 3 * sm_count();  // the resident blocks (77 registers, 3 per SM)
-    qk_norm_rope_fwd_v_kernel<<<(int)(vb < cap ? vb : cap), QKN_THREADS, qkn_table_bytes(a), s>>>(a);
+    JAGG_CUDA_TRY(launch(qk_norm_rope_fwd_v_kernel, (int)(vb < cap ? vb : cap), QKN_THREADS, qkn_table_bytes(a), s,
+                         a));
   } else {
-    qk_norm_rope_fwd_kernel<<<(int)(blocks < 65536 ? blocks : 65536), QKN_THREADS, 0, s>>>(a);
+    JAGG_CUDA_TRY(launch(qk_norm_rope_fwd_kernel, (int)(blocks < 65536 ? blocks : 65536), QKN_THREADS, 0, s, a));
   }
   JAGG_LAUNCHED();
   // algorithmic bytes: raw q, k read, transformed q, k written (storage type), 1/rms of both
@@ -1279,9 +1306,10 @@ int launch_qk_norm_rope_bwd(const QkNormRopeBwd& a, cudaStream_t s) {
     // a few blocks per SM: each block ends in 4 x 128 scale-gradient atomics
     const int64_t vb = ceil_div((int64_t)f.M, (int64_t)QKN_WARPS);
     const int vcap = 3 * sm_count();  // the resident blocks (80 registers, 3 per SM)
-    qk_norm_rope_bwd_v_kernel<<<(int)(vb < vcap ? vb : vcap), QKN_THREADS, qkn_table_bytes(f), s>>>(a);
+    JAGG_CUDA_TRY(launch(qk_norm_rope_bwd_v_kernel, (int)(vb < vcap ? vb : vcap), QKN_THREADS, qkn_table_bytes(f), s,
+                         a));
   } else {
-    qk_norm_rope_bwd_kernel<<<(int)(blocks < cap ? blocks : cap), QKN_THREADS, 0, s>>>(a);
+    JAGG_CUDA_TRY(launch(qk_norm_rope_bwd_kernel, (int)(blocks < cap ? blocks : cap), QKN_THREADS, 0, s, a));
   }
   JAGG_LAUNCHED();
   // algorithmic bytes: dq, dk read and rewritten in place, raw q, k read (storage type), 1/rms

@@ -275,6 +275,7 @@ __global__ void __launch_bounds__(tc_threads(EW), 1)
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_wait();
 
   const int total = p.tiles_m * p.tiles_n * p.splits;
   // tile index -> (m tile, n tile, split), the faster of m and n chosen by the host.
@@ -738,6 +739,7 @@ struct SimtParams {
 
 template <int BM, int BN>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(SimtParams p) {
+  pdl_wait();
   constexpr int BK = 16;
   constexpr int TM = BM / 16, TN = BN / 16;
   __shared__ float As[BK][BM + 1];
@@ -1002,7 +1004,8 @@ int launch_tc(const GemmArgs& g, cudaStream_t stream) {
     attr_set = true;
   }
   const int tok = prof_start(stream);
-  gemm_tc_kernel<BN, A_MN, B_MN, AUX, EW><<<grid, tc_threads(EW), Cfg::SMEM_BYTES, stream>>>(ta, tb, tc, tx, p);
+  JAGG_CUDA_TRY(launch(gemm_tc_kernel<BN, A_MN, B_MN, AUX, EW>, grid, tc_threads(EW), Cfg::SMEM_BYTES, stream, ta,
+                       tb, tc, tx, p));
   JAGG_LAUNCHED();
   prof_stop(tok, stream, PROF_GEMM_TC, 2.0 * g.M * g.N * g.K,
             2.0 * ((double)g.M * g.K + (double)g.N * g.K) + (double)g.M * g.N * (g.c_dtype == JAGG_DTYPE_F32 ? 4 : 2),
@@ -1111,9 +1114,9 @@ int gemm_simt(const GemmArgs& g, cudaStream_t stream) {
   dim3 grid(tiles, splits);
   const int tok = prof_start(stream);
   if (skinny)
-    gemm_simt_kernel<16, 64><<<grid, 256, 0, stream>>>(p);
+    JAGG_CUDA_TRY(launch(gemm_simt_kernel<16, 64>, grid, 256, 0, stream, p));
   else
-    gemm_simt_kernel<64, 64><<<grid, 256, 0, stream>>>(p);
+    JAGG_CUDA_TRY(launch(gemm_simt_kernel<64, 64>, grid, 256, 0, stream, p));
   JAGG_LAUNCHED();
   prof_stop(tok, stream, PROF_GEMM_SIMT, 2.0 * g.M * g.N * g.K, 0.0, g.M, g.N, g.K);
   return JAGG_OK;

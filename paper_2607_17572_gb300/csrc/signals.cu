@@ -184,6 +184,7 @@ __device__ __forceinline__ void advantage(const float* rewards, int G, int i, do
 // issued before the first use.
 __global__ void __launch_bounds__(SIG_THREADS) resid_norm_kernel(Window w, const float* rewards, double adv_eps,
                                                                  double adv_clip, double* adv, double* partial) {
+  pdl_wait();
   const int ij = blockIdx.y;
   const int i = ij / w.W, j = ij % w.W;
   const float* z0 = w.z + ((int64_t)i * (w.W + 1) + j) * w.D;
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(32) logprob_kernel(Window w, double* partial, 
                                                      const double* logp_old, const double* adv, double clip_eps,
                                                      double scale, int aggregate, double* logp_new, double* ratio,
                                                      uint8_t* clipped, float4* mc) {
+  pdl_wait();
   const int ij = blockIdx.x;
   const int i = ij / w.W, j = ij % w.W;
   const double rr = sum_partials(partial + (int64_t)ij * chunks, chunks);
@@ -254,6 +256,7 @@ __global__ void __launch_bounds__(32) logprob_kernel(Window w, double* partial, 
 __global__ void __launch_bounds__(APPLY_THREADS) apply_kernel(Window w, const double* partial, int chunks,
                                                               const float4* mc, float* s_out, float* cot_out,
                                                               int vec_out) {
+  pdl_wait();
   const int i = blockIdx.y;
   const int64_t D = w.D;
   const int64_t kbase = ((int64_t)blockIdx.x * APPLY_THREADS + threadIdx.x) * 4;
@@ -332,6 +335,7 @@ struct RolloutStep {
 };
 
 __global__ void __launch_bounds__(SIG_THREADS) rollout_step_kernel(RolloutStep p) {
+  pdl_wait();
   const int i = blockIdx.y;
   const int64_t D = p.D;
   const int64_t k = (int64_t)blockIdx.x * SIG_CHUNK + (int64_t)threadIdx.x * SIG_PER_THREAD;
@@ -394,16 +398,19 @@ __global__ void __launch_bounds__(SIG_THREADS) rollout_step_kernel(RolloutStep p
 // One warp per sample.
 __global__ void __launch_bounds__(32) rollout_logp_kernel(const double* partial, int chunks, double sigma, int64_t D,
                                                           double* logp, int64_t logp_ld) {
+  pdl_wait();
   const int i = blockIdx.x;
   const double rr = sum_partials(partial + (int64_t)i * chunks, chunks);
   if (threadIdx.x == 0) logp[(int64_t)i * logp_ld] = gauss_logp(rr, sigma, D);
 }
 
 __global__ void check_alpha_kernel(const double* t, int W) {
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0 && !(t[0] - t[W - 1] != 0.0)) set_device_status(JAGG_DEV_BADARG);
 }
 
 __global__ void aggregate_kernel(const float* s, const double* t, int G, int W, int64_t D, float* cot) {
+  pdl_wait();
   const int i = blockIdx.y;
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= D) return;
@@ -423,6 +430,7 @@ __global__ void aggregate_kernel(const float* s, const double* t, int G, int W, 
 
 __global__ void aggregate_span_kernel(const float* s, int64_t ld, const double* t, double t_first, double t_last, int G,
                                       int n, int64_t D, float* cot, int accumulate) {
+  pdl_wait();
   const int i = blockIdx.y;
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= D) return;
@@ -461,6 +469,7 @@ constexpr int GR_RUN = GR_THREADS * GR_UNROLL;  // float4 of a vector per CTA an
 template <bool HAS_B, bool HAS_ACC>
 __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a, const float* b, int64_t P,
                                                                  float alpha, float* acc, double* partial) {
+  pdl_wait();
   double sab = 0.0, saa = 0.0, sbb = 0.0;
   const int64_t nvec = P / 4;
   const float4* a4 = reinterpret_cast<const float4*>(a);
@@ -527,6 +536,7 @@ __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a,
 
 // Three warps: the sums over the CTAs' partials of <a, b>, |a|^2, |b|^2.
 __global__ void __launch_bounds__(96) grad_reduce_final(const double* partial, int blocks, double* out3) {
+  pdl_wait();
   const int w = threadIdx.x / 32;
   double s = 0.0;
 #pragma unroll 4
@@ -582,14 +592,17 @@ int step_signals(const char* name, const void* v_hat, int v_dtype, const float* 
   const bool vec_out = D % 4 == 0 && (!s_out || aligned16(s_out)) && (!cot_out || aligned16(cot_out));
   const Window win{v_hat, vf32, vec ? 1 : 0, z, t, sched_alpha, sched_sigma, G, W, D};
   const int tok = prof_start(stream);
-  resid_norm_kernel<<<dim3(chunks, G * W), SIG_THREADS, 0, stream>>>(win, rewards, adv_eps, adv_clip, adv_out, partial);
+  JAGG_CUDA_TRY(launch(resid_norm_kernel, dim3(chunks, G * W), SIG_THREADS, 0, stream, win, rewards, adv_eps,
+                       adv_clip, adv_out, partial));
   JAGG_LAUNCHED();
-  logprob_kernel<<<G * W, 32, 0, stream>>>(win, partial, chunks, sigma, logp_old, adv_out, clip_eps, scale,
-                                           cot_out ? 1 : 0, logp_new, ratio, clipped, mc);
+  JAGG_CUDA_TRY(launch(logprob_kernel, G * W, 32, 0, stream, win, partial, chunks, sigma, logp_old, adv_out,
+                       clip_eps, scale,
+                                           cot_out ? 1 : 0, logp_new, ratio, clipped, mc));
   JAGG_LAUNCHED();
   if (s_out || cot_out) {
     const int gx = ceil_div(D, (int64_t)APPLY_THREADS * 4);
-    apply_kernel<<<dim3(gx, G), APPLY_THREADS, 0, stream>>>(win, partial, chunks, mc, s_out, cot_out, vec_out ? 1 : 0);
+    JAGG_CUDA_TRY(launch(apply_kernel, dim3(gx, G), APPLY_THREADS, 0, stream, win, partial, chunks, mc, s_out,
+                         cot_out, vec_out ? 1 : 0));
     JAGG_LAUNCHED();
   }
   // algorithmic bytes: v-hat and the W + 1 latents of every sample read once, the signals
@@ -657,9 +670,10 @@ extern "C" int jagg_rollout_step(const void* y_hat, int y_dtype, int64_t y_sampl
                 D, zl, yl, xl, t_cur, t_next, sigma,
                 sched ? sched[0] : 0.0, sched ? sched[1] : 0.0, sched ? sched[2] : 0.0, sched ? sched[3] : 0.0,
                 sched ? 1 : 0, static_cast<double*>(ws)};
-  rollout_step_kernel<<<dim3(chunks, G), SIG_THREADS, 0, stream>>>(p);
+  JAGG_CUDA_TRY(launch(rollout_step_kernel, dim3(chunks, G), SIG_THREADS, 0, stream, p));
   JAGG_LAUNCHED();
-  rollout_logp_kernel<<<G, 32, 0, stream>>>(static_cast<double*>(ws), chunks, sigma, D, logp, logp_stride);
+  JAGG_CUDA_TRY(launch(rollout_logp_kernel, G, 32, 0, stream, static_cast<double*>(ws), chunks, sigma, D, logp,
+                       logp_stride));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -669,9 +683,9 @@ extern "C" int jagg_aggregate(const float* s, const double* t_window, int G, int
   JAGG_CHECK_ARG(s && t_window && cot, "jagg_aggregate: null pointer");
   JAGG_CHECK_ARG(G > 0 && G <= 65535 && D > 0, "jagg_aggregate: bad G=%d or D=%lld", G, (long long)D);
   JAGG_CHECK_ARG(W >= 2, "jagg_aggregate: W=%d, the endpoints must differ (W >= 2)", W);
-  check_alpha_kernel<<<1, 32, 0, stream>>>(t_window, W);
+  JAGG_CUDA_TRY(launch(check_alpha_kernel, 1, 32, 0, stream, t_window, W));
   JAGG_LAUNCHED();
-  aggregate_kernel<<<dim3(ceil_div(D, 256), G), 256, 0, stream>>>(s, t_window, G, W, D, cot);
+  JAGG_CUDA_TRY(launch(aggregate_kernel, dim3(ceil_div(D, 256), G), 256, 0, stream, s, t_window, G, W, D, cot));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -685,8 +699,9 @@ extern "C" int jagg_aggregate_span(const float* s, int64_t s_sample_stride, cons
   JAGG_CHECK_ARG(t_first != t_last, "jagg_aggregate_span: the window endpoints must differ");
   const int64_t ld = s_sample_stride ? s_sample_stride : (int64_t)n * D;
   JAGG_CHECK_ARG(ld >= (int64_t)n * D, "jagg_aggregate_span: sample stride %lld below n * D", (long long)ld);
-  aggregate_span_kernel<<<dim3(ceil_div(D, 256), G), 256, 0, stream>>>(s, ld, t_steps, t_first, t_last, G, n, D, cot,
-                                                                       accumulate);
+  JAGG_CUDA_TRY(launch(aggregate_span_kernel, dim3(ceil_div(D, 256), G), 256, 0, stream, s, ld, t_steps, t_first,
+                       t_last, G, n, D, cot,
+                                                                       accumulate));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -739,16 +754,16 @@ extern "C" int grad_reduce(const float* a, const float* b, int64_t P, float alph
   const int most = 3 * sm_count() < GR_BLOCKS ? 3 * sm_count() : GR_BLOCKS;
   const int blocks = runs < 1 ? 1 : (runs < most ? (int)runs : most);
   if (b && acc)
-    grad_reduce_kernel<true, true><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    JAGG_CUDA_TRY(launch(grad_reduce_kernel<true, true>, blocks, GR_THREADS, 0, stream, a, b, P, alpha, acc, part));
   else if (b)
-    grad_reduce_kernel<true, false><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    JAGG_CUDA_TRY(launch(grad_reduce_kernel<true, false>, blocks, GR_THREADS, 0, stream, a, b, P, alpha, acc, part));
   else if (acc)
-    grad_reduce_kernel<false, true><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    JAGG_CUDA_TRY(launch(grad_reduce_kernel<false, true>, blocks, GR_THREADS, 0, stream, a, b, P, alpha, acc, part));
   else
-    grad_reduce_kernel<false, false><<<blocks, GR_THREADS, 0, stream>>>(a, b, P, alpha, acc, part);
+    JAGG_CUDA_TRY(launch(grad_reduce_kernel<false, false>, blocks, GR_THREADS, 0, stream, a, b, P, alpha, acc, part));
   JAGG_LAUNCHED();
   if (out3) {
-    grad_reduce_final<<<1, 96, 0, stream>>>(static_cast<const double*>(ws), blocks, out3);
+    JAGG_CUDA_TRY(launch(grad_reduce_final, 1, 96, 0, stream, static_cast<const double*>(ws), blocks, out3));
     JAGG_LAUNCHED();
   }
   // algorithmic bytes: a (and b) read, acc read and written
