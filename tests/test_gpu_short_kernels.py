@@ -1,0 +1,84 @@
+"""GPU tests of the short, latency-bound kernels at the edges of their tiles: the f32 products
+and attention, the LayerNorm + modulation forward at every compiled width, the position table
+and the bias column sums."""
+import math
+
+import pytest
+import torch
+
+import synth
+from gpu_cases import GpuModel, model_inputs, rel_l2
+from oracle import dit
+from test_gpu_kernels import _desc, _rel
+
+pytestmark = pytest.mark.gpu
+
+jg = pytest.importorskip("paper_2607_17572_gb300")
+
+
+@pytest.mark.parametrize("a_mn,b_mn", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("M,N,K,pad", [(1, 1, 1, 0), (32, 32, 64, 0), (33, 31, 65, 0), (70, 36, 130, 4), (192, 64, 256, 1)])
+def test_f32_product_tiles(M, N, K, pad, a_mn, b_mn):
+    """Whole and ragged 32 x 32 x 64 tiles, aligned and unaligned row pitches, with the bias and
+    with accumulation.  Bound: f32 sums of K products, far below 1e-5 relative."""
+    torch.manual_seed(M + N + K)
+    A = torch.randn(K if a_mn else M, (M if a_mn else K) + pad, device="cuda")
+    B = torch.randn(K if b_mn else N, (N if b_mn else K) + pad, device="cuda")
+    a = A[:, :M].t() if a_mn else A[:, :K]
+    b = B[:, :N].t() if b_mn else B[:, :K]
+    bias = torch.randn(N, device="cuda")
+    C = torch.full((M, N + 3), 7.0, device="cuda")
+    jg.test_gemm(_desc(M, N, K, A, A.shape[1], a_mn, B, B.shape[1], b_mn, jg.DTYPE_F32, C, N + 3, jg.DTYPE_F32,
+                       bias=bias))
+    ref = a.double() @ b.double().t()
+    assert _rel(C[:, :N], ref + bias.double()) < 1e-5 and (C[:, N:] == 7.0).all()
+    jg.test_gemm(_desc(M, N, K, A, A.shape[1], a_mn, B, B.shape[1], b_mn, jg.DTYPE_F32, C, N + 3, jg.DTYPE_F32, epi=4))
+    assert _rel(C[:, :N], 2 * ref + bias.double()) < 1e-5 and (C[:, N:] == 7.0).all()
+
+
+@pytest.mark.parametrize("dh", [16, 32, 64, 128])
+@pytest.mark.parametrize("N", [1, 31, 32, 33, 70])
+def test_f32_attention_tiles(N, dh):
+    """One key, one tile less a row, whole tiles and remainders against float64."""
+    torch.manual_seed(N + dh)
+    B, H = 2, 3
+    d = H * dh
+    qkv = torch.randn(B * N, 3 * d, device="cuda") * 2
+    dO = torch.randn(B * N, d, device="cuda")
+    o, lse, dqkv = torch.empty_like(dO), torch.empty(B, H, N, device="cuda"), torch.empty_like(qkv)
+    jg.test_attention_fwd(qkv, B, N, H, dh, o, lse)
+    jg.test_attention_bwd(qkv, o, lse, dO, B, N, H, dh, dqkv)
+    x = qkv.double().requires_grad_()
+    q, k, v = x.view(B, N, 3, H, dh).permute(2, 0, 3, 1, 4)
+    s = q @ k.transpose(-1, -2) / math.sqrt(dh)
+    ref = (torch.softmax(s, -1) @ v).transpose(1, 2).reshape(B * N, d)
+    ref.backward(dO.double())
+    assert _rel(o, ref) < 1e-5
+    assert (lse - torch.logsumexp(s, -1)).abs().max().item() < 1e-5
+    # with one key dS vanishes: dK, dQ are rounding noise beside dV, so the whole is compared
+    assert _rel(dqkv, x.grad) < 2e-5
+
+
+@pytest.mark.parametrize("hidden,heads", [(512, 8), (768, 12), (1024, 16), (2048, 16), (3072, 24), (320, 5)])
+def test_layernorm_forward_widths(hidden, heads):
+    """A one-block f32 forward at every width with its own LayerNorm kernel (and one without),
+    rows not a multiple of the rows per CTA, a grid that is not square."""
+    wl = synth.small_variant(synth.WORKLOADS["tiny_dit_f32"], name="ln_width", hidden=hidden, heads=heads, mlp=64,
+                             depth=1, latent_h=3, latent_w=5, txt_len=2)
+    params = synth.make_params(wl)
+    z, t, txt = model_inputs(wl, 3, 11)
+    v, _, _ = GpuModel(jg, wl, params).forward(z, t, txt)
+    ref, _ = dit.Backbone(wl, params).forward(z, t, txt)
+    assert rel_l2(v.float().cpu().numpy(), ref) < 1e-5
+    assert jg.device_status() == 0
+
+
+@pytest.mark.parametrize("rows", [1, 7, 8, 9, 1225, 5328])
+@pytest.mark.parametrize("cols", [8, 264, 3072])
+def test_colsum_row_blocks(rows, cols):
+    """Every choice of rows per block, from one partly filled block to the cap."""
+    torch.manual_seed(rows + cols)
+    X = torch.randn(rows, cols, device="cuda").bfloat16()
+    db = torch.full((cols,), 0.5, device="cuda")
+    jg.test_colsum(X, db)
+    assert _rel(db, X.double().sum(0) + 0.5) < 1e-5
