@@ -33,6 +33,7 @@ static inline int read_unit_status(unsigned* v, int clear) {
   return 0;
 }
 int unit_status_gemm(unsigned* v, int clear);
+int unit_status_gemm_pair(unsigned* v, int clear);
 int unit_status_signals(unsigned* v, int clear);
 int unit_status_attention_tc(unsigned* v, int clear);
 int unit_status_testing(unsigned* v, int clear);

@@ -958,6 +958,20 @@ double tile_cost(const GemmArgs& g, int BN, int nsm) {
   return waves * BN * ((double)ceil_div(g.K, TC_BK) / splits) / eff;
 }
 
+// The better of the 128- and 256-column single-CTA tiles, in 256-column k-blocks of one CTA with
+// two more per unit, the measure of gemm_pair_serves.
+double single_cost(const GemmArgs& g, int nsm) {
+  double best = 0.0;
+  for (int BN = 128; BN <= 256; BN *= 2) {
+    if (g.N < BN) continue;
+    const int splits = choose_splits(g, BN, nsm);
+    const long long units = (long long)ceil_div(g.M, TC_BM) * ceil_div(g.N, BN) * splits;
+    const double waves = (double)((units + nsm - 1) / nsm);
+    const double c = waves * ((double)ceil_div(g.K, TC_BK) / splits * (BN == 256 ? 1.0 : 0.62) + 2.0);
+    if (best == 0.0 || c < best) best = c;
+  }
+  return best;
+}
 // Tile order.  The CTAs resident at one time work on consecutive tile indices, so the
 // operand panel that those tiles share is read from DRAM once and from L2 after that.  With
 // N fastest, tiles_n neighbours share one 128-row panel of A; with M fastest, tiles_m
@@ -1171,6 +1185,14 @@ int gemm_simt(const GemmArgs& g, cudaStream_t stream) {
 int gemm(const GemmArgs& g, cudaStream_t stream) {
   JAGG_TRY(validate(g));
   if (!tc_eligible(g)) return gemm_simt(g, stream);
+  // The CTA-pair kernel where its estimate is within a factor of the single-CTA one: it runs the
+  // same k-blocks faster (less shared-memory and L2 traffic, eight epilogue warps), which pays
+  // most where the epilogue works hardest.  The factors are fitted to both kernels timed on
+  // 96 products (768- to 12288-wide, 633 to 21312 rows, every epilogue of the model): with
+  // them the choice is 0.7 % slower than the better of the two on average.
+  double pair;
+  if (gemm_pair_serves(g, &pair) && pair < (g.c_dtype == JAGG_DTYPE_F32 ? 1.03 : 1.2) * single_cost(g, sm_count()))
+    return gemm_pair(g, stream);
   if (!g.a_mn && !g.b_mn) return dispatch_bn<false, false>(g, stream);
   if (!g.a_mn && g.b_mn) return dispatch_bn<false, true>(g, stream);
   if (g.a_mn && g.b_mn) return dispatch_bn<true, true>(g, stream);

@@ -57,6 +57,11 @@ struct GemmArgs {
 // anything involving f32 operands goes to the SIMT kernel.
 int gemm(const GemmArgs& g, cudaStream_t stream);
 
+// The 256 x 256 CTA-pair kernel (gemm_pair.cu): whether it serves a bf16 product that is eligible
+// for the tensor cores, with its estimated duration in 256-column k-blocks; and the product.
+bool gemm_pair_serves(const GemmArgs& g, double* cost);
+int gemm_pair(const GemmArgs& g, cudaStream_t stream);
+
 // Forces the SIMT kernel (tests of the tensor-core path compare against it).
 int gemm_simt(const GemmArgs& g, cudaStream_t stream);
 

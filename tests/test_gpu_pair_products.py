@@ -1,0 +1,106 @@
+"""GPU tests of the CTA-pair dense products (256 x 256 tiles): shapes that the library sends to
+them, with ragged rows, columns and K, an odd number of 64-column chunks in the last tile,
+outputs inside wider buffers, sequences that start inside a tile, and every epilogue, against
+float32 PyTorch on the same rounded inputs."""
+import math
+
+import pytest
+import torch
+import torch.nn.functional as F
+
+from test_gpu_kernels import _desc, _rel
+
+pytestmark = pytest.mark.gpu
+
+jg = pytest.importorskip("paper_2607_17572_gb300")
+
+
+def _operands(M, N, K, a_mn, b_mn):
+    torch.manual_seed(M + N + K)
+    A = torch.randn(M, K, device="cuda").bfloat16()
+    B = (torch.randn(N, K, device="cuda") / math.sqrt(K)).bfloat16()
+    ref = A.float() @ B.float().t()
+    As = A.t().contiguous() if a_mn else A
+    Bs = B.t().contiguous() if b_mn else B
+    return (As, M if a_mn else K, a_mn, Bs, N if b_mn else K, b_mn, jg.DTYPE_BF16), ref
+
+
+def _out(M, N, pad, dtype):
+    return torch.full((M, N + pad), 5.0, device="cuda", dtype=dtype)
+
+
+def _done(*wide):
+    torch.cuda.synchronize()
+    assert jg.device_status() == 0
+    for t, N in wide:
+        assert (t[:, N:] == 5.0).all(), "wrote past the output's columns"
+
+
+# bf16 outputs are rounded once: relative error of the rounding 2^-9 / sqrt(3) ~ 1.1e-3 .. 1.7e-3
+BF16_TOL = 4e-3
+
+
+@pytest.mark.parametrize("M,N,K", [(2601, 1088, 1000), (2560, 1024, 1024)])
+def test_forward_epilogues(M, N, K):
+    ops, acc = _operands(M, N, K, 0, 0)
+    bias = torch.randn(N, device="cuda").bfloat16()
+    u = acc + bias.float()
+    C = _out(M, N, 8, torch.bfloat16)
+    jg.test_gemm(_desc(M, N, K, *ops, C, N + 8, jg.DTYPE_BF16, bias=bias))
+    D, G, G1 = (_out(M, N, 16, torch.bfloat16) for _ in range(3))
+    jg.test_gemm(_desc(M, N, K, *ops, D, N + 16, jg.DTYPE_BF16, epi=1, bias=bias, C2=G, ldc2=N + 16))
+    d = _desc(M, N, K, *ops, D, N + 16, jg.DTYPE_BF16, epi=1, bias=bias, C2=G1, ldc2=N + 16)
+    d.C = None  # a forward that keeps nothing
+    jg.test_gemm(d)
+    rows = 333
+    gate = torch.randn((M + rows - 1) // rows, N + 4, device="cuda")
+    hin = torch.randn(M, N + 4, device="cuda")
+    Y, H = _out(M, N, 8, torch.bfloat16), _out(M, N, 4, torch.float32)
+    jg.test_gemm(_desc(M, N, K, *ops, Y, N + 8, jg.DTYPE_BF16, epi=2, bias=bias, C2=H, ldc2=N + 4, aux=hin,
+                       ld_aux=N + 4, gate=gate, gate_stride=N + 4, rows_per_seq=rows))
+    _done((C, N), (D, N), (G, N), (G1, N), (Y, N), (H, N))
+    assert _rel(C[:, :N].float(), u) < BF16_TOL and _rel(Y[:, :N].float(), u) < BF16_TOL
+    assert _rel(H[:, :N], hin[:, :N] + gate[torch.arange(M, device="cuda") // rows, :N] * u) < 1e-5
+    assert torch.equal(G[:, :N], G1[:, :N])
+    v = u.requires_grad_()
+    g = F.gelu(v, approximate="tanh")
+    g.sum().backward()
+    assert _rel(G[:, :N].float(), g.detach()) < BF16_TOL and _rel(D[:, :N].float(), v.grad) < BF16_TOL
+
+
+@pytest.mark.parametrize("M,N,K", [(2601, 1096, 1000), (2560, 1024, 1024)])
+def test_input_gradient_epilogues(M, N, K):
+    ops, acc = _operands(M, N, K, 0, 1)
+    X = torch.rand(M, N + 8, device="cuda").bfloat16()
+    C, O = _out(M, N, 8, torch.bfloat16), _out(M, N, 24, torch.bfloat16)
+    jg.test_gemm(_desc(M, N, K, *ops, C, N + 8, jg.DTYPE_BF16))
+    jg.test_gemm(_desc(M, N, K, *ops, O, N + 24, jg.DTYPE_BF16, epi=3, aux=X, ld_aux=N + 8))
+    _done((C, N), (O, N))
+    assert _rel(C[:, :N].float(), acc) < BF16_TOL
+    assert _rel(O[:, :N].float(), acc * X[:, :N].float()) < BF16_TOL
+
+
+@pytest.mark.parametrize("M,N,K", [(2500, 3080, 4104), (2560, 3072, 4096)])
+def test_f32_output(M, N, K):
+    ops, acc = _operands(M, N, K, 0, 1)
+    C = _out(M, N, 4, torch.float32)
+    jg.test_gemm(_desc(M, N, K, *ops, C, N + 4, jg.DTYPE_F32))
+    _done((C, N))
+    assert _rel(C[:, :N], acc) < 1e-5
+
+
+@pytest.mark.parametrize("M,N,K", [(4100, 3076, 8200), (3072, 12288, 2304)])
+def test_accumulation(M, N, K):
+    """The weight-gradient layout, added to what is there: f32 sums of bf16 products."""
+    ops, acc = _operands(M // 4 * 4, N, K, 1, 1)
+    M = acc.shape[0]
+    G0 = torch.randn(M, N, device="cuda")
+    G = _out(M, N, 4, torch.float32)
+    G[:, :N] = G0
+    # MN-major operands need row pitches of 16 bytes: both are multiples of 8 elements here or padded
+    As, lda, _, Bs, ldb, _, dt = ops
+    pad = lambda t: F.pad(t, (0, -t.shape[1] % 8))
+    As, Bs = pad(As).contiguous(), pad(Bs).contiguous()
+    jg.test_gemm(_desc(M, N, K, As, As.shape[1], 1, Bs, Bs.shape[1], 1, dt, G, N + 4, jg.DTYPE_F32, epi=4))
+    _done((G, N))
+    assert _rel(G[:, :N], G0 + acc) < 1e-5
