@@ -44,12 +44,12 @@ struct AttnBwdArgs {
 };
 
 int attention_fwd(const AttnArgs& a, cudaStream_t s);
-// The tcgen05 forward (attention_tc.cu): bf16, head dim 64 / 128, stream boundary on a
-// multiple of 128 tokens, 16-byte aligned views.
+// The tcgen05 forward (attention_tc.cu): bf16, head dim 64 / 128, any stream boundary,
+// 16-byte aligned views.
 bool attention_fwd_tc_eligible(const AttnArgs& a);
 int attention_fwd_tc(const AttnArgs& a, cudaStream_t s);
-// The tcgen05 backward (attention_tc.cu): bf16, head dim 64 / 128, stream boundary on a
-// multiple of 128 tokens, 16-byte aligned views.
+// The tcgen05 backward (attention_tc.cu): bf16, head dim 64 / 128, any stream boundary,
+// 16-byte aligned views.
 bool attention_bwd_tc_eligible(const AttnBwdArgs& a);
 int attention_bwd_tc(const AttnBwdArgs& a, cudaStream_t s);
 // Scratch: Dv and dq_acc as described above.  dq_acc must be 16-byte aligned (it receives

@@ -17,6 +17,28 @@ int unit_status_attention_tc(unsigned* v, int clear) { return read_unit_status(v
 namespace {
 
 constexpr float kLog2eTc = 1.4426950408889634f;
+
+// Token tiles of a sequence whose first n0 tokens lie in one stream buffer and the other N - n0
+// in the second: each stream is cut into tiles of its own, the first stream's last tile
+// partly filled when n0 is not a multiple of the tile.  The order of the keys does not matter
+// to a softmax, so a partly filled tile in the middle of the sequence is masked like the one at
+// its end, and a stream boundary may lie on any token.
+struct TokTile {
+  int seg, row, valid, tok;  // stream, first row in it, tokens of the tile, first token of the sequence
+};
+__host__ __device__ __forceinline__ int tok_tiles(int N, int n0, int bt) {
+  return (n0 + bt - 1) / bt + (N - n0 + bt - 1) / bt;
+}
+__device__ __forceinline__ TokTile tok_tile(int j, int N, int n0, int bt) {
+  const int t0 = (n0 + bt - 1) / bt;
+  TokTile t;
+  t.seg = j < t0 ? 0 : 1;
+  t.row = (t.seg ? j - t0 : j) * bt;
+  t.valid = min(bt, (t.seg ? N - n0 : n0) - t.row);
+  t.tok = (t.seg ? n0 : 0) + t.row;
+  return t;
+}
+
 // Tensor maps of one backward call: per stream buffer (0: the first n0 tokens of every
 // sequence, 1: the rest) the query, key, value and output-gradient views, and the dQ
 // accumulator.
@@ -149,18 +171,16 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = p.N;
-  const int nkt = (N + BK - 1) / BK;
+  const int nkt = tok_tiles(N, p.n0, BK);
   const int units = nkt * p.B * p.heads;
-  const int nq = (N + BQ - 1) / BQ;
+  const int nq = tok_tiles(N, p.n0, BQ);
   // unit u: key tile u % nkt of sequence-head u / nkt
-  auto unit_of = [&](int u, int& k0, int& b, int& h) {
+  auto unit_of = [&](int u, TokTile& kt, int& b, int& h) {
     const int bh = u / nkt;
-    k0 = (u % nkt) * BK;
+    kt = tok_tile(u % nkt, N, p.n0, BK);
     b = bh / p.heads;
     h = bh % p.heads;
   };
-  auto seg_of = [&](int r) { return r < p.n0 ? 0 : 1; };
-  auto row_in = [&](int r) { return r < p.n0 ? r : r - p.n0; };
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -205,14 +225,15 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
     int i = 0;
     int i_last = -1, g_last = -1;  // the last unit whose K, V and the last tile whose Q, dO were issued
     for (int u = blockIdx.x; u < units && !*abort_flag; u += gridDim.x, ++i) {
-      int k0, b, h;
-      unit_of(u, k0, b, h);
+      TokTile kt;
+      int b, h;
+      unit_of(u, kt, b, h);
       const int bh = b * p.heads + h;
       bool ok = true;
       if (lane == 0) {
         ok = ptx::mbar_wait(kv_free, (i & 1) ^ 1);
         if (ok) {
-          const int sg = seg_of(k0), r = row_in(k0);
+          const int sg = kt.seg, r = kt.row;
           ptx::mbar_arrive_expect_tx(bar_kv, 2 * C::KV_BYTES);
 #pragma unroll
           for (int c = 0; c < D / 64; ++c) {
@@ -230,12 +251,12 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
         if (lane == 0) ok = ptx::mbar_wait(&empty[st], ((g / NS) & 1) ^ 1);
         ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
         if (!ok || *abort_flag) { *abort_flag = 1; break; }
-        const int q0 = j * BQ;
+        const TokTile qt = tok_tile(j, N, p.n0, BQ);
         // lse and rowsum(dO O) of the tile's queries by 4-byte copies the stage barrier tracks
-        // (their rows need not be 16-byte aligned); +inf / 0 past the last query
+        // (their rows need not be 16-byte aligned); +inf / 0 past the tile's last query: P = dS = 0
         for (int t = lane; t < BQ; t += 32) {
-          const int q = q0 + t;
-          if (q < N) {
+          const int q = qt.tok + t;
+          if (t < qt.valid) {
             ptx::cp_async4(sLse + st * BQ + t, p.lse + (int64_t)bh * N + q);
             ptx::cp_async4(sRd + st * BQ + t, p.Dv + (int64_t)bh * N + q);
           } else {
@@ -246,7 +267,7 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
         ptx::cp_async_arrive_noinc(&full[st]);
         __syncwarp();
         if (lane == 0) {
-          const int sg = seg_of(q0), r = row_in(q0);
+          const int sg = qt.seg, r = qt.row;
           ptx::mbar_arrive_expect_tx(&full[st], 2 * C::QT_BYTES);
 #pragma unroll
           for (int c = 0; c < D / 64; ++c) {
@@ -432,8 +453,9 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
     bool ok = true;
     int i = 0;
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++i) {
-      int k0, b, h;
-      unit_of(u, k0, b, h);
+      TokTile kt;
+      int b, h;
+      unit_of(u, kt, b, h);
       for (int j = 0; j < nq; ++j) {
         const int g = i * nq + j;
         const int bb = g & 1;
@@ -447,7 +469,7 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&dqfree[bb]);
-        const int q0 = j * BQ;
+        const TokTile qt = tok_tile(j, N, p.n0, BQ);
         // dQ^T: lane = head-dim index, columns = the tile's 64 queries; two 32 x 32 boxes
         // (box rows = queries) through one staging box (head dim 64: lane quarters 0, 1 only)
         if (quarter * 32 >= D) continue;
@@ -462,9 +484,10 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
           ptx::fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            const int row = q0 + hh * 32;
-            if (row < N) {
-              ptx::tma_reduce_add_3d(&maps.dq, stg, h * D + quarter * 32, row, b);
+            // rows past the tile's last query add the zeros of P = dS = 0 (a box inside the
+            // sequence) or are dropped (past its end)
+            if (hh * 32 < qt.valid) {
+              ptx::tma_reduce_add_3d(&maps.dq, stg, h * D + quarter * 32, qt.tok + hh * 32, b);
               ptx::bulk_commit();
             }
           }
@@ -475,14 +498,15 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
       ok = __all_sync(0xffffffffu, ptx::mbar_wait(bar_fin, i & 1));
       if (!ok || *abort_flag) { ok = false; *abort_flag = 1; break; }
       ptx::tc_fence_after();
-      const int key = k0 + quarter * 32 + lane;
+      const int key = kt.tok + quarter * 32 + lane;
+      const bool key_live = quarter * 32 + lane < kt.valid;
 #pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t rv[32], rk[32];
         ptx::tmem_ld_32x32b_x32(trow + C::T_DV + c * 32, rv);
         ptx::tmem_ld_32x32b_x32(trow + C::T_DK + c * 32, rk);
         ptx::tmem_ld_wait();
-        if (key < N) {
+        if (key_live) {
           bf16* dv = static_cast<bf16*>(p.dv.base(key)) + p.dv.off(b, key, N, p.dv_col0 + h * D + c * 32);
           bf16* dk = static_cast<bf16*>(p.dk.base(key)) + p.dk.off(b, key, N, p.dk_col0 + h * D + c * 32);
 #pragma unroll
@@ -604,18 +628,16 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = p.N;
-  const int nk = (N + BK - 1) / BK;
-  const int nq = (N + BQ - 1) / BQ;
+  const int nk = tok_tiles(N, p.n0, BK);
+  const int nq = tok_tiles(N, p.n0, BQ);
   const int units = nq * p.B * p.heads;
   // unit u: query tile u % nq of sequence-head u / nq
-  auto unit_of = [&](int u, int& q0, int& b, int& h) {
+  auto unit_of = [&](int u, TokTile& qt, int& b, int& h) {
     const int bh = u / nq;
-    q0 = (u % nq) * BQ;
+    qt = tok_tile(u % nq, N, p.n0, BQ);
     b = bh / p.heads;
     h = bh % p.heads;
   };
-  auto seg_of = [&](int r) { return r < p.n0 ? 0 : 1; };
-  auto row_in = [&](int r) { return r < p.n0 ? r : r - p.n0; };
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -659,20 +681,21 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
       int g = 0, i = 0, iq_last = -1;  // g: K / V tiles issued; iq_last: the last unit whose Q was issued
       bool ok = true;
       for (int u = blockIdx.x; u < units && ok && !abort_flag; u += gridDim.x, ++i) {
-        int q0, b, h;
-        unit_of(u, q0, b, h);
+        TokTile qt;
+        int b, h;
+        unit_of(u, qt, b, h);
         if (i > 0 && !ptx::mbar_wait(qfree, (i - 1) & 1)) { ok = false; break; }
         iq_last = i;
         ptx::mbar_arrive_expect_tx(qfull, C::Q_BYTES);
 #pragma unroll
         for (int c = 0; c < D / 64; ++c)
-          ptx::tma_load_3d(sQ + c * BQ * 128, &maps.q[seg_of(q0)], qfull, (int)(p.q_col0 + h * D + c * 64),
-                           row_in(q0), b);
+          ptx::tma_load_3d(sQ + c * BQ * 128, &maps.q[qt.seg], qfull, (int)(p.q_col0 + h * D + c * 64), qt.row, b);
         for (int pass = 0; pass < 2 && ok; ++pass) {
           for (int j = 0; j < nk; ++j, ++g) {
             const int st = g % NS;
             if (g >= NS && !ptx::mbar_wait(&empty[st], ((g / NS) & 1) ^ 1)) { ok = false; break; }
-            const int k0 = j * BK, sg = seg_of(k0), r = row_in(k0);
+            const TokTile kt = tok_tile(j, N, p.n0, BK);
+            const int sg = kt.seg, r = kt.row;
             ptx::mbar_arrive_expect_tx(&full[st], (pass + 1) * C::KV_BYTES);
 #pragma unroll
             for (int c = 0; c < D / 64; ++c) {
@@ -777,8 +800,9 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
     };
     int sc = 0, pc = 0, i = 0;
     for (int u = blockIdx.x; u < units; u += gridDim.x, ++i) {
-      int q0, b, h;
-      unit_of(u, q0, b, h);
+      TokTile qt;
+      int b, h;
+      unit_of(u, qt, b, h);
       // pass 1: the row maximum over the valid keys
       float m = -INFINITY;
       for (int j = 0; j < nk; ++j, ++sc) {
@@ -792,7 +816,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0 && ok) ptx::mbar_arrive(&sfree[sb]);
-        const int kv = N - (j * BK + half * 64);  // valid keys among this warp's 64
+        const int kv = tok_tile(j, N, p.n0, BK).valid - half * 64;  // valid keys among this warp's 64
 #pragma unroll
         for (int c = 0; c < 64; ++c)
           if (c < kv) m = fmaxf(m, __uint_as_float(rs[c]));
@@ -807,7 +831,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
         wait(&bar_s[sb], (sc >> 1) & 1);
         ptx::tc_fence_after();
         uint32_t hp[32];
-        const int kv = N - (j * BK + half * 64);
+        const int kv = tok_tile(j, N, p.n0, BK).valid - half * 64;
 #pragma unroll
         for (int cc = 0; cc < 2; ++cc) {
           uint32_t rs[32];
@@ -838,14 +862,15 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
       // the unit's output: O / l, and the log-sum-exp
       wait(bar_o, i & 1);
       ptx::tc_fence_after();
-      const int q = q0 + r;
+      const int q = qt.tok + r;
+      const bool q_live = r < qt.valid;
       const float inv = 1.f / l;
 #pragma unroll
       for (int cc = 0; cc < D / 64; ++cc) {
         uint32_t ro[32];
         ptx::tmem_ld_32x32b_x32(trow + C::T_O + half * (D / 2) + cc * 32, ro);
         ptx::tmem_ld_wait();
-        if (q < N && ok) {
+        if (q_live && ok) {
           bf16* o = static_cast<bf16*>(p.o.base(q)) + p.o.off(b, q, N, (int64_t)h * D + half * (D / 2) + cc * 32);
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
@@ -861,7 +886,7 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0 && ok) ptx::mbar_arrive(ofree);
-      if (half == 0 && q < N && ok) p.lse[((int64_t)b * p.heads + h) * N + q] = p.scale * m + logf(l);
+      if (half == 0 && q_live && ok) p.lse[((int64_t)b * p.heads + h) * N + q] = p.scale * m + logf(l);
     }
   }
   ptx::tc_fence_before();
@@ -966,19 +991,17 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int N = p.N;
-  const int nk = (N + BK - 1) / BK;
-  const int nq = (N + BQ - 1) / BQ;
+  const int nk = tok_tiles(N, p.n0, BK);
+  const int nq = tok_tiles(N, p.n0, BQ);
   const int npair = (nq + 1) / 2;
   const int units = npair * p.B * p.heads;
-  // unit u: query tiles 2 (u % npair) and + 1 of sequence-head u / npair
-  auto unit_of = [&](int u, int& q0, int& b, int& h) {
+  // unit u: query tiles j0 = 2 (u % npair) and j0 + 1 of sequence-head u / npair
+  auto unit_of = [&](int u, int& j0, int& b, int& h) {
     const int bh = u / npair;
-    q0 = (u % npair) * 2 * BQ;
+    j0 = (u % npair) * 2;
     b = bh / p.heads;
     h = bh % p.heads;
   };
-  auto seg_of = [&](int r) { return r < p.n0 ? 0 : 1; };
-  auto row_in = [&](int r) { return r < p.n0 ? r : r - p.n0; };
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -1022,21 +1045,22 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
       int gk = 0, gv = 0, i = 0, iq_last = -1;  // K / V tiles issued; the last unit whose Q was issued
       bool ok = true;
       for (int u = blockIdx.x; u < units && ok && !*abort_flag; u += gridDim.x, ++i) {
-        int q0, b, h;
-        unit_of(u, q0, b, h);
+        int j0, b, h;
+        unit_of(u, j0, b, h);
         if (!ptx::mbar_wait(qfree, (i & 1) ^ 1)) { ok = false; break; }
         iq_last = i;
         ptx::mbar_arrive_expect_tx(qfull, 2 * C::TILE);
         for (int x = 0; x < 2; ++x) {
-          // query tile B past the last query (odd tile count): a tile of zeros
-          const int qx = q0 + x * BQ < N ? q0 + x * BQ : q0;
+          // query tile B past the last tile (odd tile count): tile A again, not written
+          const TokTile qx = tok_tile(j0 + x < nq ? j0 + x : j0, N, p.n0, BQ);
 #pragma unroll
           for (int c = 0; c < D / 64; ++c)
-            ptx::tma_load_3d(sQ + x * C::TILE + c * BQ * 128, &maps.q[seg_of(qx)], qfull,
-                             (int)(p.q_col0 + h * D + c * 64), row_in(qx), b);
+            ptx::tma_load_3d(sQ + x * C::TILE + c * BQ * 128, &maps.q[qx.seg], qfull,
+                             (int)(p.q_col0 + h * D + c * 64), qx.row, b);
         }
         for (int j = 0; j < nk && ok; ++j, ++gk, ++gv) {
-          const int k0 = j * BK, sg = seg_of(k0), r = row_in(k0);
+          const TokTile kt = tok_tile(j, N, p.n0, BK);
+          const int sg = kt.seg, r = kt.row;
           const int ks = gk % NKS, vs = gv % NVS;
           if (!ptx::mbar_wait(&kempty[ks], ((gk / NKS) & 1) ^ 1)) { ok = false; break; }
           ptx::mbar_arrive_expect_tx(&kfull[ks], C::TILE);
@@ -1144,8 +1168,8 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
     int i = 0;
     uint32_t s_phase = 0, pv_phase = 0;  // bar_s[x] / bar_pv[x] phases consumed
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++i) {
-      int q0, b, h;
-      unit_of(u, q0, b, h);
+      int j0, b, h;
+      unit_of(u, j0, b, h);
       float m = -INFINITY, l = 0.f;
       for (int j = 0; j < nk; ++j) {
         ok = __all_sync(0xffffffffu, ptx::mbar_wait(&bar_s[x], s_phase));
@@ -1153,7 +1177,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
         if (!ok || *abort_flag) { ok = false; *abort_flag = 1; break; }
         ptx::tc_fence_after();
         // The row maximum: keys 0-63 (read again below), then 64-127 (kept in registers).
-        const int kv = N - j * BK;  // valid keys of the tile (at least one)
+        const int kv = tok_tile(j, N, p.n0, BK).valid;  // valid keys of the tile (at least one)
         const bool ragged = kv < BK;
         uint32_t rh[64];
         float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
@@ -1228,14 +1252,16 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
       pv_phase ^= 1u;
       if (!ok || *abort_flag) { ok = false; *abort_flag = 1; break; }
       ptx::tc_fence_after();
-      const int q = q0 + x * BQ + r;
+      const TokTile qt = tok_tile(j0 + x, N, p.n0, BQ);
+      const int q = qt.tok + r;
+      const bool q_live = j0 + x < nq && r < qt.valid;
       const float inv = 1.f / l;
 #pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t ro[32];
         ptx::tmem_ld_32x32b_x32(tO + c * 32, ro);
         ptx::tmem_ld_wait();
-        if (q < N) {
+        if (q_live) {
           bf16* o = static_cast<bf16*>(p.o.base(q)) + p.o.off(b, q, N, (int64_t)h * D + c * 32);
 #pragma unroll
           for (int v = 0; v < 4; ++v) {
@@ -1251,7 +1277,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&ofree[x]);
-      if (q < N) p.lse[((int64_t)b * p.heads + h) * N + q] = p.scale * m + logf(l);
+      if (q_live) p.lse[((int64_t)b * p.heads + h) * N + q] = p.scale * m + logf(l);
     }
   }
   ptx::tc_fence_before();
@@ -1314,7 +1340,7 @@ int launch_v3(const AttnBwdArgs& a, cudaStream_t s) {
     JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     attr = true;
   }
-  const int units = ceil_div(N, C::BK) * f.B * f.heads;
+  const int units = tok_tiles(N, p.n0, C::BK) * f.B * f.heads;
   const int nsm = sm_count();
   JAGG_CUDA_TRY(launch(kernel, units < nsm ? units : nsm, FB2_THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
@@ -1350,7 +1376,7 @@ int launch_fwd(const AttnArgs& f, cudaStream_t s) {
     JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_fwd_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     attr = true;
   }
-  const int units = ceil_div(N, C::BQ) * f.B * f.heads;
+  const int units = tok_tiles(N, p.n0, C::BQ) * f.B * f.heads;
   const int nsm = sm_count();
   JAGG_CUDA_TRY(launch(fa_fwd_tc_kernel<D>, units < nsm ? units : nsm, FF_THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
@@ -1359,13 +1385,13 @@ int launch_fwd(const AttnArgs& f, cudaStream_t s) {
 
 }  // namespace
 
-// Whether the tensor-core forward serves the call: bf16, head dim 64 / 128, the stream
-// boundary on a 128-token multiple, 16-byte aligned operands and output rows.
+// Whether the tensor-core forward serves the call: bf16, head dim 64 / 128, 16-byte aligned
+// operands and output rows.
 bool attention_fwd_tc_eligible(const AttnArgs& f) {
   if (f.dtype != JAGG_DTYPE_BF16 || (f.dh != 64 && f.dh != 128) || !f.lse) return false;
   const int n0 = f.q.n0;
   const bool single = n0 >= f.N;
-  if (!single && (n0 <= 0 || n0 % 128)) return false;
+  if (!single && n0 <= 0) return false;
   const SegRows* views[4] = {&f.q, &f.k, &f.v, &f.o};
   for (const SegRows* v : views) {
     if (v->n0 != n0) return false;
@@ -1404,7 +1430,7 @@ int launch_fwd128(const AttnArgs& f, cudaStream_t s) {
     JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_fwd_tc128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     attr = true;
   }
-  const int units = ceil_div(ceil_div(N, C::BQ), 2) * f.B * f.heads;
+  const int units = ceil_div(tok_tiles(N, p.n0, C::BQ), 2) * f.B * f.heads;
   const int nsm = sm_count();
   JAGG_CUDA_TRY(launch(fa_fwd_tc128_kernel, units < nsm ? units : nsm, FF2_THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
@@ -1415,14 +1441,14 @@ int attention_fwd_tc(const AttnArgs& f, cudaStream_t s) {
   return f.dh == 64 ? launch_fwd<64>(f, s) : launch_fwd128(f, s);
 }
 
-// Whether the tensor-core backward serves the call: bf16, head dim 64 / 128, the stream
-// boundary on a 128-token multiple, 16-byte aligned buffers with 16-byte row pitches.
+// Whether the tensor-core backward serves the call: bf16, head dim 64 / 128, 16-byte aligned
+// buffers with 16-byte row pitches.
 bool attention_bwd_tc_eligible(const AttnBwdArgs& a) {
   const AttnArgs& f = a.f;
   if (f.dtype != JAGG_DTYPE_BF16 || (f.dh != 64 && f.dh != 128)) return false;
   const int n0 = f.q.n0;
   const bool single = n0 >= f.N;
-  if (!single && (n0 <= 0 || n0 % 128)) return false;
+  if (!single && n0 <= 0) return false;
   const SegRows* views[4] = {&f.q, &f.k, &f.v, &a.dO};
   for (const SegRows* v : views) {
     if (v->n0 != n0) return false;
