@@ -1110,7 +1110,9 @@ int dispatch_bn(const GemmArgs& g, cudaStream_t stream) {
   return launch_tc<128, A_MN, B_MN, 0>(g, stream);
 }
 
-bool tc_eligible(const GemmArgs& g) {
+}  // namespace
+
+bool gemm_tc_eligible(const GemmArgs& g) {
   if (g.a_dtype != JAGG_DTYPE_BF16 || g.b_dtype != JAGG_DTYPE_BF16) return false;
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   if (!al16(g.A) || !al16(g.B)) return false;
@@ -1119,8 +1121,6 @@ bool tc_eligible(const GemmArgs& g) {
   if (g.lda % 8 || g.ldb % 8) return false;
   return true;
 }
-
-}  // namespace
 
 int encode_tmap(CUtensorMap* m, bool f32, int rank, const void* base, const uint64_t* dims, const uint64_t* strides,
                 const uint32_t* box, CUtensorMapSwizzle swz) {
@@ -1182,17 +1182,29 @@ int gemm_simt(const GemmArgs& g, cudaStream_t stream) {
   return JAGG_OK;
 }
 
+// The CTA-pair kernel where its estimate is within a factor of the single-CTA one: it runs the
+// same k-blocks faster (less shared-memory and L2 traffic, eight epilogue warps), which pays
+// most where the epilogue works hardest.  The factors and the costs in both estimates are fitted
+// to both kernels timed on 96 products (768 to 12288 columns, 633 to 21312 rows, every epilogue of
+// the model): with them the choice is 0.7 % slower than the better of the two on average.
+static bool takes_pair(const GemmArgs& g, double* cost) {
+  const double single = single_cost(g, sm_count());
+  double pair;
+  const bool take = gemm_pair_serves(g, &pair) && pair < (g.c_dtype == JAGG_DTYPE_F32 ? 1.1 : 1.3) * single;
+  *cost = take ? pair : single;
+  return take;
+}
+double gemm_best_cost(const GemmArgs& g) {
+  double cost;
+  takes_pair(g, &cost);
+  return cost;
+}
+
 int gemm(const GemmArgs& g, cudaStream_t stream) {
   JAGG_TRY(validate(g));
-  if (!tc_eligible(g)) return gemm_simt(g, stream);
-  // The CTA-pair kernel where its estimate is within a factor of the single-CTA one: it runs the
-  // same k-blocks faster (less shared-memory and L2 traffic, eight epilogue warps), which pays
-  // most where the epilogue works hardest.  The factors are fitted to both kernels timed on
-  // 96 products (768- to 12288-wide, 633 to 21312 rows, every epilogue of the model): with
-  // them the choice is 0.7 % slower than the better of the two on average.
-  double pair;
-  if (gemm_pair_serves(g, &pair) && pair < (g.c_dtype == JAGG_DTYPE_F32 ? 1.03 : 1.2) * single_cost(g, sm_count()))
-    return gemm_pair(g, stream);
+  if (!gemm_tc_eligible(g)) return gemm_simt(g, stream);
+  double cost;
+  if (takes_pair(g, &cost)) return gemm_pair(g, stream);
   if (!g.a_mn && !g.b_mn) return dispatch_bn<false, false>(g, stream);
   if (!g.a_mn && g.b_mn) return dispatch_bn<false, true>(g, stream);
   if (g.a_mn && g.b_mn) return dispatch_bn<true, true>(g, stream);

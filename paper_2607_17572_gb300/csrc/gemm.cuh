@@ -57,10 +57,19 @@ struct GemmArgs {
 // anything involving f32 operands goes to the SIMT kernel.
 int gemm(const GemmArgs& g, cudaStream_t stream);
 
-// The 256 x 256 CTA-pair kernel (gemm_pair.cu): whether it serves a bf16 product that is eligible
+// The CTA-pair kernel (gemm_pair.cu): whether it serves a bf16 product that is eligible
 // for the tensor cores, with its estimated duration in 256-column k-blocks; and the product.
 bool gemm_pair_serves(const GemmArgs& g, double* cost);
 int gemm_pair(const GemmArgs& g, cudaStream_t stream);
+
+// Two independent products of the same layout and epilogue (the text and image streams of a
+// dual-stream block), in one launch where the CTA-pair kernel serves both.
+int gemm_two(const GemmArgs& x, const GemmArgs& y, cudaStream_t stream);
+// The estimated duration of a bf16 product by the kernel that gemm() would choose, in k-blocks of a
+// 256-column tile.
+double gemm_best_cost(const GemmArgs& g);
+// bf16 operands that the tensor-core kernels can address.
+bool gemm_tc_eligible(const GemmArgs& g);
 
 // Forces the SIMT kernel (tests of the tensor-core path compare against it).
 int gemm_simt(const GemmArgs& g, cudaStream_t stream);

@@ -1,4 +1,4 @@
-// Dense products in 256 x 256 tiles on CTA pairs (tcgen05.mma.cta_group::2).
+// Dense products in tiles of 256 rows x up to 256 columns on CTA pairs (tcgen05.mma.cta_group::2).
 //
 // Bound by the tensor pipe on long products.  Rates in isolation, before (one CTA per 128 x 256
 // tile, four or eight epilogue warps) and now, of 1923 TFLOP/s (cuBLAS): 18432 x 9216 x 3072 stored
@@ -7,8 +7,8 @@
 // weight gradients of 18432 rows 1667-1735 -> 1847-1864.  Short K is bound by the epilogue: 21312 x
 // 3072 x 768 with GELU 837 -> 1110, 21312 x 768 x 768 with the gated residual 368 -> 500.
 //
-// A cluster of two CTAs (the two SMs of a TPC) owns one 256 x 256 tile: each CTA stages its 128
-// rows of A and its 128 of the 256 columns of B, so a k-block of 64 moves 32 KB into each SM where
+// A cluster of two CTAs (the two SMs of a TPC) owns one tile: each CTA stages its 128 rows of A
+// and its half of the columns of B, so at 256 columns a k-block of 64 moves 32 KB into each SM where
 // a CTA on its own moves 48 KB for a 128 x 256 tile, and the tensor core reads 64 instead of 96
 // bytes of shared memory per clock.  The leader's MMA thread issues for both; every CTA drains
 // the 128 rows of the accumulator that its tensor memory holds (two 256-column accumulators:
@@ -34,22 +34,23 @@ namespace {
 
 enum PairEpi : int { PE_STORE_BF16 = 0, PE_STORE_F32, PE_ACCUM, PE_MUL, PE_GELU, PE_GATE };
 
-constexpr int PT = 256;       // tile rows and columns
+constexpr int PT = 256;       // tile rows, and the most columns
 constexpr int PK = 64;        // k-block
 constexpr int P_EW = 8;       // epilogue warps
 constexpr int P_THREADS = 64 + 32 * P_EW;
-constexpr int P_BOX = 4096;   // one staging box: 32 rows x 128 bytes
 constexpr int P_HALF = 128 * PK * 2;      // bytes of a CTA's half of an operand tile
 constexpr int P_STAGE = 2 * P_HALF;
 
 template <int EPI>
 struct PairCfg {
-  // staging boxes per epilogue warp: one for a plain output, two where an input or a second output
-  // shares them.  The rest of shared memory is operand stages (six, or five): with four the
-  // products are 7 % slower (18432 x 3072 x 12288: 805 us against 748), since the loads of
-  // 4 x 0.27 us of tensor work no longer cover the L2 latency under load.
-  static constexpr int BOXES = EPI <= PE_ACCUM ? 1 : 2;
-  static constexpr int WARP_BYTES = BOXES * P_BOX;
+  // Staging boxes of 32 rows x 32 columns per epilogue warp: 8 KB where inputs or a second output
+  // share them, 4 KB otherwise.  The rest of shared memory is operand stages (five or six): with
+  // four the products are 7 % slower (18432 x 3072 x 12288: 805 us against 748), since the
+  // loads of 4 x 0.27 us of tensor work no longer cover the L2 latency under load.
+  static constexpr bool OUT_BF16 = EPI == PE_STORE_BF16 || EPI == PE_MUL || EPI == PE_GELU;
+  static constexpr int BOX = OUT_BF16 ? 2048 : 4096;
+  static constexpr int BOXES = EPI == PE_STORE_BF16 ? 2 : EPI <= PE_ACCUM ? 1 : EPI == PE_GATE ? 2 : 4;
+  static constexpr int WARP_BYTES = BOXES * BOX;
   static constexpr int EPI_BYTES = P_EW * WARP_BYTES;
   static constexpr int FIXED = 1024 /*align*/ + 512 /*barriers*/;
   static constexpr int STAGES = (232448 - FIXED - EPI_BYTES) / P_STAGE;
@@ -59,6 +60,7 @@ struct PairCfg {
 
 struct PairParams {
   int M, N;
+  int bn;               // tile columns: a multiple of 32 from 128 to 256
   int tiles_m, tiles_n, splits, k_blocks;
   const bf16* bias;     // [N] or null
   const float* gate;    // PE_GATE
@@ -75,18 +77,30 @@ struct PairMaps {
   CUtensorMap a, b, c, x, c2;
 };
 
+// One or two products of the same operand layout and epilogue in one launch (the text and image
+// streams of a dual-stream block): the units of the second follow those of the first, so the
+// small product fills the last wave of the large one instead of a wave of its own.
+struct PairGroup {
+  PairMaps maps[2];
+  PairParams p[2];
+  int total0, total;  // units of the first product, and of both
+};
+
 // Tiles walk groups of P_GROUP row tiles, the row tile fastest inside a group: the pairs at work
 // at one time cover about P_GROUP x 9 tiles, so an operand panel is read from DRAM once for
 // all of them.
 constexpr int P_GROUP = 8;
-__device__ __forceinline__ void pair_decode(const PairParams& p, int t, int& tm, int& tn, int& ks) {
+__device__ __forceinline__ void pair_decode(const PairGroup& g, int t, int& pr, int& tm, int& tn, int& ks) {
+  pr = t < g.total0 ? 0 : 1;
+  if (pr) t -= g.total0;
+  const PairParams& p = g.p[pr];
   const int per_split = p.tiles_m * p.tiles_n;
   ks = t / per_split;
   t -= ks * per_split;
   const int per_group = P_GROUP * p.tiles_n;
-  const int g = t / per_group, in = t - g * per_group;
-  const int gm = min(P_GROUP, p.tiles_m - g * P_GROUP);
-  tm = g * P_GROUP + in % gm;
+  const int grp = t / per_group, in = t - grp * per_group;
+  const int gm = min(P_GROUP, p.tiles_m - grp * P_GROUP);
+  tm = grp * P_GROUP + in % gm;
   tn = in / gm;
 }
 
@@ -115,7 +129,7 @@ __device__ __forceinline__ float2 unpack2(uint32_t w) {
 
 template <bool A_MN, bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
-    gemm_pair_kernel(const __grid_constant__ PairMaps maps, PairParams p) {
+    gemm_pair_kernel(const __grid_constant__ PairGroup g) {
   using Cfg = PairCfg<EPI>;
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ uint8_t smem_pair[];
@@ -148,11 +162,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
     ptx::mbar_init(drainbar, 1);
     ptx::mbar_init(never, 1);
     ptx::fence_mbar_init();
-    ptx::prefetch_tmap(&maps.a);
-    ptx::prefetch_tmap(&maps.b);
-    if (EPI != PE_GATE) ptx::prefetch_tmap(&maps.c);
-    if (EPI >= PE_MUL) ptx::prefetch_tmap(&maps.x);
-    if (EPI == PE_GATE) ptx::prefetch_tmap(&maps.c2);
+    for (int pr = 0; pr < (g.total > g.total0 ? 2 : 1); ++pr) {
+      ptx::prefetch_tmap(&g.maps[pr].a);
+      ptx::prefetch_tmap(&g.maps[pr].b);
+      if (EPI != PE_GATE) ptx::prefetch_tmap(&g.maps[pr].c);
+      if (EPI >= PE_MUL) ptx::prefetch_tmap(&g.maps[pr].x);
+      if (EPI == PE_GATE) ptx::prefetch_tmap(&g.maps[pr].c2);
+    }
   }
   if (warp == 1) {
     ptx::tmem_alloc_pair(tmem_slot, 512);
@@ -165,9 +181,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
   const uint32_t tmem = *tmem_slot;
   pdl_wait();
 
-  const int total = p.tiles_m * p.tiles_n * p.splits;
+  const int total = g.total;
   const int npairs = gridDim.x >> 1;
-  auto krange = [&](int ks, int& kb0, int& kb1) {
+  auto krange = [&](int pr, int ks, int& kb0, int& kb1) {
+    const PairParams& p = g.p[pr];
     kb0 = (int)((long long)p.k_blocks * ks / p.splits);
     kb1 = (int)((long long)p.k_blocks * (ks + 1) / p.splits);
   };
@@ -179,15 +196,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
       uint32_t phase = 0;
       uint32_t issued = 0, issued_parity = 0;
       for (int t = blockIdx.x >> 1; t < total && !abort_flag; t += npairs) {
-        int tm, tn, ks, kb0, kb1;
-        pair_decode(p, t, tm, tn, ks);
-        krange(ks, kb0, kb1);
-        const int ma = tm * PT + (int)rank * 128, nb = tn * PT + (int)rank * 128;
+        int pr, tm, tn, ks, kb0, kb1;
+        pair_decode(g, t, pr, tm, tn, ks);
+        krange(pr, ks, kb0, kb1);
+        const PairMaps& maps = g.maps[pr];
+        const int half_n = g.p[pr].bn >> 1;  // this CTA's columns of B
+        const int ma = tm * PT + (int)rank * 128, nb = tn * g.p[pr].bn + (int)rank * half_n;
+        // an MN-major B arrives in whole 64-column chunks (of the last, half_n % 64 are used)
+        const bool two_chunks = half_n > 64;
+        const uint32_t stage_bytes = 2u * (P_HALF + (B_MN ? (two_chunks ? P_HALF : P_HALF / 2) : half_n * PK * 2));
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!ptx::mbar_wait(&empty[stage], phase ^ 1)) { abort_flag = 1; break; }
           uint8_t* sA = smem + stage * P_STAGE;
           uint8_t* sB = sA + P_HALF;
-          if (rank == 0) ptx::mbar_arrive_expect_tx(&full[stage], 2 * P_STAGE);
+          if (rank == 0) ptx::mbar_arrive_expect_tx(&full[stage], stage_bytes);
           const uint32_t bar = ptx::mapa(ptx::smem_u32(&full[stage]), 0);
           if (!A_MN) {
             ptx::tma_load_2d_pair(sA, &maps.a, bar, kb * PK, ma);
@@ -199,7 +221,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
             ptx::tma_load_2d_pair(sB, &maps.b, bar, kb * PK, nb);
           } else {
             ptx::tma_load_2d_pair(sB, &maps.b, bar, nb, kb * PK);
-            ptx::tma_load_2d_pair(sB + P_HALF / 2, &maps.b, bar, nb + 64, kb * PK);
+            if (two_chunks) ptx::tma_load_2d_pair(sB + P_HALF / 2, &maps.b, bar, nb + 64, kb * PK);
           }
           issued |= 1u << stage;
           issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
@@ -221,16 +243,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
   } else if (warp == 1) {
     if (rank == 0 && ptx::elect_one()) {
       // ---------------- MMA issuer for both CTAs
-      constexpr uint32_t idesc = ptx::idesc_bf16(PT, PT, A_MN, B_MN);
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       for (int t = blockIdx.x >> 1; t < total && !abort_flag; t += npairs) {
-        int tm, tn, ks, kb0, kb1;
-        pair_decode(p, t, tm, tn, ks);
-        krange(ks, kb0, kb1);
+        int pr, tm, tn, ks, kb0, kb1;
+        pair_decode(g, t, pr, tm, tn, ks);
+        krange(pr, ks, kb0, kb1);
         if (!ptx::mbar_wait(&tempty[acc], acc_phase ^ 1)) { abort_flag = 1; break; }
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * PT;
+        const uint32_t idesc = ptx::idesc_bf16(PT, g.p[pr].bn, A_MN, B_MN);
         bool ok = true;
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!ptx::mbar_wait(&full[stage], phase)) { ok = false; break; }
@@ -263,31 +285,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
     const int q = warp & 3, half = (warp - 2) >> 2, ew = warp - 2;
     uint8_t* box = epi_smem + ew * Cfg::WARP_BYTES;
     uint64_t* aux = auxbar + Cfg::BOXES * ew;
-    constexpr bool WIDE = EPI == PE_STORE_BF16 || EPI == PE_MUL || EPI == PE_GELU;  // 64-column bf16 boxes
-    constexpr int CW = WIDE ? 64 : 32;
-    constexpr int CHUNKS = PT / CW / 2;  // chunks of this warp per tile
     const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
-    uint8_t* row0 = box + lane * 128;
-    const int sw = lane & 7;
+    // the 16-byte piece j of this lane's row in a box: 128-byte rows (f32) or 64-byte rows (bf16),
+    // swizzled as the tensor maps say
+    auto piece = [&](uint8_t* bx, int j) {
+      return Cfg::OUT_BF16 ? bx + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4) : bx + lane * 128 + ((j ^ (lane & 7)) << 4);
+    };
     int acc = 0, sb = 0;  // sb: the box of the next store (epilogues without an input)
     uint32_t acc_phase = 0, aux_phase = 0;  // aux_phase bit b: the phase box b's barrier waits for next
     for (int t = blockIdx.x >> 1; t < total; t += npairs) {
-      int tm, tn, ks;
-      pair_decode(p, t, tm, tn, ks);
+      int pr, tm, tn, ks;
+      pair_decode(g, t, pr, tm, tn, ks);
+      const PairParams& p = g.p[pr];
+      const PairMaps& maps = g.maps[pr];
       const int m0 = tm * PT + (int)rank * 128 + q * 32;
       const bool rows_live = m0 < p.M;
-      auto col = [&](int i) { return tn * PT + (half + 2 * i) * CW; };
+      auto col = [&](int i) { return tn * p.bn + (half + 2 * i) * 32; };
       const float* gate_row = nullptr;
       if constexpr (EPI == PE_GATE)
         gate_row = p.gate + (int64_t)(min(m0 + lane, p.M - 1) / p.rows_per_seq) * p.gate_stride;
       int live = 0;  // chunks with columns inside the output
       if (rows_live)
-        for (int i = 0; i < CHUNKS; ++i) live += col(i) < p.N ? 1 : 0;
+        for (int i = 0; (half + 2 * i) * 32 < p.bn; ++i) live += col(i) < p.N ? 1 : 0;
       // PE_MUL, PE_GATE: the first BOXES chunks' inputs, before the accumulator is waited for
       auto load_aux = [&](int i) {
         const int b = i % Cfg::BOXES;
-        ptx::mbar_arrive_expect_tx(&aux[b], P_BOX);
-        ptx::tma_load_2d(box + b * P_BOX, &maps.x, &aux[b], col(i), m0);
+        ptx::mbar_arrive_expect_tx(&aux[b], Cfg::BOX);
+        ptx::tma_load_2d(box + b * Cfg::BOX, &maps.x, &aux[b], col(i), m0);
       };
       int loaded = 0;  // chunks whose input has been requested
       if constexpr (EPI == PE_MUL || EPI == PE_GATE) {
@@ -309,21 +333,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
 #pragma unroll 1
       for (int i = 0; i < live; ++i) {
         const int n0 = col(i);
-        const uint32_t tcol = trow + acc * PT + (half + 2 * i) * CW;
+        // the chunk's box; PE_GELU: the box of GELU(u), that of GELU'(u) after it
         const int sl = EPI == PE_MUL || EPI == PE_GATE ? i % Cfg::BOXES : sb;
-        uint8_t* slot = box + sl * P_BOX;
-        uint8_t* row = row0 + sl * P_BOX;
+        uint8_t* slot = box + sl * Cfg::BOX;
         constexpr bool BIAS = EPI == PE_STORE_BF16 || EPI == PE_GELU || EPI == PE_GATE;
-        uint4 bq[BIAS ? CW / 8 : 1];  // the chunk's bias
+        uint4 bq[BIAS ? 4 : 1];  // the chunk's bias
         if constexpr (BIAS) {
           if (p.bias) {
 #pragma unroll
-            for (int j = 0; j < CW / 8; ++j) bq[j] = *reinterpret_cast<const uint4*>(p.bias + n0 + 8 * j);
+            for (int j = 0; j < 4; ++j) bq[j] = *reinterpret_cast<const uint4*>(p.bias + n0 + 8 * j);
           }
         }
-        uint32_t r[CW];
-        ptx::tmem_ld_32x32b_x32(tcol, *reinterpret_cast<uint32_t(*)[32]>(r));
-        if constexpr (CW == 64) ptx::tmem_ld_32x32b_x32(tcol + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
+        uint32_t r[32];
+        ptx::tmem_ld_32x32b_x32(trow + acc * PT + (half + 2 * i) * 32, r);
         float4 gq[EPI == PE_GATE ? 8 : 1];  // the gate of this lane's row
         if constexpr (EPI == PE_GATE) {
           // the next input first: into the previous chunk's box, once its store has read it
@@ -349,7 +371,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
           }
         } else {
           if (lane == 0) {  // the box's previous store has read it
-            if (Cfg::BOXES == 1 || (EPI == PE_GELU && p.gelu_d))
+            if constexpr (Cfg::BOXES == 1)
               ptx::bulk_wait_read<0>();
             else
               ptx::bulk_wait_read<1>();
@@ -368,52 +390,48 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
             r[8 * j + 2 * e + 1] = __float_as_uint(v.y);
           }
         };
+        auto f2 = [&](int c) { return make_float2(__uint_as_float(r[c]), __uint_as_float(r[c + 1])); };
         if constexpr (EPI == PE_STORE_BF16) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 0; j < 4; ++j) {
             add_bias(j);
-            *reinterpret_cast<uint4*>(row + ((j ^ sw) << 4)) =
-                make_uint4(pack2(__uint_as_float(r[8 * j]), __uint_as_float(r[8 * j + 1])),
-                           pack2(__uint_as_float(r[8 * j + 2]), __uint_as_float(r[8 * j + 3])),
-                           pack2(__uint_as_float(r[8 * j + 4]), __uint_as_float(r[8 * j + 5])),
-                           pack2(__uint_as_float(r[8 * j + 6]), __uint_as_float(r[8 * j + 7])));
+            uint32_t o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = pack2(f2(8 * j + 2 * e).x, f2(8 * j + 2 * e).y);
+            *reinterpret_cast<uint4*>(piece(slot, j)) = make_uint4(o[0], o[1], o[2], o[3]);
           }
         } else if constexpr (EPI == PE_STORE_F32 || EPI == PE_ACCUM) {
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<uint4*>(row + ((j ^ sw) << 4)) =
-                make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+            *reinterpret_cast<uint4*>(piece(slot, j)) = make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
         } else if constexpr (EPI == PE_MUL) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            uint4* at = reinterpret_cast<uint4*>(row + ((j ^ sw) << 4));
+          for (int j = 0; j < 4; ++j) {
+            uint4* at = reinterpret_cast<uint4*>(piece(slot, j));
             const uint4 x = *at;
             const uint32_t w[4] = {x.x, x.y, x.z, x.w};
             uint32_t o[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              const float2 v = ptx::mul2(make_float2(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1])),
-                                         unpack2(w[e]));
+              const float2 v = ptx::mul2(f2(8 * j + 2 * e), unpack2(w[e]));
               o[e] = pack2(v.x, v.y);
             }
             *at = make_uint4(o[0], o[1], o[2], o[3]);
           }
         } else if constexpr (EPI == PE_GELU) {
-          // GELU(u) into this chunk's box, or, with the derivative, GELU' into box 0 and GELU into 1
-          uint8_t* row_g = p.gelu_d ? row0 + P_BOX : row;
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 0; j < 4; ++j) {
             add_bias(j);
             uint32_t og[4], od[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              float2 g, dg;
-              gelu2(make_float2(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1])), g, dg);
-              og[e] = pack2(g.x, g.y);
+              float2 gl, dg;
+              gelu2(f2(8 * j + 2 * e), gl, dg);
+              og[e] = pack2(gl.x, gl.y);
               od[e] = pack2(dg.x, dg.y);
             }
-            *reinterpret_cast<uint4*>(row_g + ((j ^ sw) << 4)) = make_uint4(og[0], og[1], og[2], og[3]);
-            if (p.gelu_d) *reinterpret_cast<uint4*>(row0 + ((j ^ sw) << 4)) = make_uint4(od[0], od[1], od[2], od[3]);
+            *reinterpret_cast<uint4*>(piece(slot, j)) = make_uint4(og[0], og[1], og[2], og[3]);
+            if (p.gelu_d) *reinterpret_cast<uint4*>(piece(slot + Cfg::BOX, j)) = make_uint4(od[0], od[1], od[2], od[3]);
           }
         } else {  // PE_GATE: y straight to global memory (64 bytes of this lane's row), the residual in place
           bf16* yp = m0 + lane < p.M ? p.y + (int64_t)(m0 + lane) * p.ldy + n0 : nullptr;
@@ -424,11 +442,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
             add_bias(j);
             uint32_t y[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) y[e] = pack2(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1]));
+            for (int e = 0; e < 4; ++e) y[e] = pack2(f2(8 * j + 2 * e).x, f2(8 * j + 2 * e).y);
             if (yp) *reinterpret_cast<uint4*>(yp + 8 * j) = make_uint4(y[0], y[1], y[2], y[3]);
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-              float4* at = reinterpret_cast<float4*>(row + (((2 * j + hh) ^ sw) << 4));
+              float4* at = reinterpret_cast<float4*>(piece(slot, 2 * j + hh));
               float4 h = *at;
               h.x = fmaf(gv[4 * hh], __uint_as_float(r[8 * j + 4 * hh]), h.x);
               h.y = fmaf(gv[4 * hh + 1], __uint_as_float(r[8 * j + 4 * hh + 1]), h.y);
@@ -444,12 +462,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
           if constexpr (EPI == PE_ACCUM) {
             ptx::tma_reduce_add_2d(&maps.c, slot, n0, m0);
           } else if constexpr (EPI == PE_GELU) {
-            if (p.gelu_d) {
-              ptx::tma_store_2d(&maps.c, box, n0, m0);
-              ptx::tma_store_2d(&maps.x, box + P_BOX, n0, m0);
-            } else {
-              ptx::tma_store_2d(&maps.x, slot, n0, m0);
-            }
+            ptx::tma_store_2d(&maps.x, slot, n0, m0);
+            if (p.gelu_d) ptx::tma_store_2d(&maps.c, slot + Cfg::BOX, n0, m0);
           } else if constexpr (EPI == PE_GATE) {
             ptx::tma_store_2d(&maps.c2, slot, n0, m0);
           } else {
@@ -457,7 +471,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
           }
           ptx::bulk_commit();
         }
-        sb = (sb + 1) % Cfg::BOXES;
+        sb = (sb + (EPI == PE_GELU ? 2 : 1)) % Cfg::BOXES;
       }
       ptx::tc_fence_before();
       __syncwarp();
@@ -515,28 +529,26 @@ int pair_epi(const GemmArgs& g) {
 }
 
 template <bool A_MN, bool B_MN, int EPI>
-int launch_pair(const GemmArgs& g, int splits, int npairs, cudaStream_t s) {
-  using Cfg = PairCfg<EPI>;
-  PairMaps maps;
-  const auto swz = CU_TENSOR_MAP_SWIZZLE_128B;
+int fill_pair(const GemmArgs& g, int bn, int splits, PairMaps& maps, PairParams& p) {
+  const auto swz = CU_TENSOR_MAP_SWIZZLE_128B, swz_bf16 = CU_TENSOR_MAP_SWIZZLE_64B;
   JAGG_TRY(A_MN ? map2d(&maps.a, g.A, g.K, g.M, g.lda, 64, PK, false, swz)
                 : map2d(&maps.a, g.A, g.M, g.K, g.lda, PK, 128, false, swz));
   JAGG_TRY(B_MN ? map2d(&maps.b, g.B, g.K, g.N, g.ldb, 64, PK, false, swz)
-                : map2d(&maps.b, g.B, g.N, g.K, g.ldb, PK, 128, false, swz));
+                : map2d(&maps.b, g.B, g.N, g.K, g.ldb, PK, bn / 2, false, swz));
   maps.c = maps.x = maps.c2 = maps.a;  // unused ones
   if (EPI == PE_STORE_BF16 || EPI == PE_MUL || (EPI == PE_GELU && g.C))
-    JAGG_TRY(map2d(&maps.c, g.C, g.M, g.N, g.ldc, 64, 32, false, swz));
+    JAGG_TRY(map2d(&maps.c, g.C, g.M, g.N, g.ldc, 32, 32, false, swz_bf16));
   if (EPI == PE_STORE_F32 || EPI == PE_ACCUM) JAGG_TRY(map2d(&maps.c, g.C, g.M, g.N, g.ldc, 32, 32, true, swz));
-  if (EPI == PE_MUL) JAGG_TRY(map2d(&maps.x, g.aux, g.M, g.N, g.ld_aux, 64, 32, false, swz));
-  if (EPI == PE_GELU) JAGG_TRY(map2d(&maps.x, g.C2, g.M, g.N, g.ldc2, 64, 32, false, swz));
+  if (EPI == PE_MUL) JAGG_TRY(map2d(&maps.x, g.aux, g.M, g.N, g.ld_aux, 32, 32, false, swz_bf16));
+  if (EPI == PE_GELU) JAGG_TRY(map2d(&maps.x, g.C2, g.M, g.N, g.ldc2, 32, 32, false, swz_bf16));
   if (EPI == PE_GATE) {
     JAGG_TRY(map2d(&maps.x, g.aux, g.M, g.N, g.ld_aux, 32, 32, true, swz));
     JAGG_TRY(map2d(&maps.c2, g.C2, g.M, g.N, g.ldc2, 32, 32, true, swz));
   }
-  PairParams p;
   p.M = g.M; p.N = g.N;
   p.tiles_m = ceil_div(g.M, PT);
-  p.tiles_n = ceil_div(g.N, PT);
+  p.bn = bn;
+  p.tiles_n = ceil_div(g.N, bn);
   p.splits = splits;
   p.k_blocks = ceil_div(g.K, PK);
   p.bias = static_cast<const bf16*>(g.bias);
@@ -546,77 +558,168 @@ int launch_pair(const GemmArgs& g, int splits, int npairs, cudaStream_t s) {
   p.gelu_d = EPI == PE_GELU && g.C ? 1 : 0;
   p.y = static_cast<bf16*>(g.C);
   p.ldy = g.ldc;
+  return JAGG_OK;
+}
+
+// Tile columns and K splits of one product.
+struct PairPlan {
+  int bn, splits;
+};
+
+// The product `a` and, when given, `b` of the same layout and epilogue.
+template <bool A_MN, bool B_MN, int EPI>
+int launch_pair(const GemmArgs& a, const GemmArgs* b, const PairPlan (&plan)[2], int npairs, cudaStream_t s) {
+  using Cfg = PairCfg<EPI>;
+  PairGroup grp;
+  JAGG_TRY((fill_pair<A_MN, B_MN, EPI>(a, plan[0].bn, plan[0].splits, grp.maps[0], grp.p[0])));
+  if (b) {
+    JAGG_TRY((fill_pair<A_MN, B_MN, EPI>(*b, plan[1].bn, plan[1].splits, grp.maps[1], grp.p[1])));
+  } else {
+    grp.maps[1] = grp.maps[0];
+    grp.p[1] = grp.p[0];
+  }
+  auto units = [](const PairParams& p) { return p.tiles_m * p.tiles_n * p.splits; };
+  grp.total0 = units(grp.p[0]);
+  grp.total = grp.total0 + (b ? units(grp.p[1]) : 0);
   auto kernel = gemm_pair_kernel<A_MN, B_MN, EPI>;
   static bool attr = false;
   if (!attr) {
     JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM));
     attr = true;
   }
-  const int total = p.tiles_m * p.tiles_n * splits;
   const int tok = prof_start(s);
-  JAGG_CUDA_TRY(launch(kernel, 2 * (total < npairs ? total : npairs), P_THREADS, Cfg::SMEM, s, maps, p));
+  JAGG_CUDA_TRY(launch(kernel, 2 * (grp.total < npairs ? grp.total : npairs), P_THREADS, Cfg::SMEM, s, grp));
   JAGG_LAUNCHED();
-  prof_stop(tok, s, PROF_GEMM_TC, 2.0 * g.M * g.N * g.K,
-            2.0 * ((double)g.M * g.K + (double)g.N * g.K) + (double)g.M * g.N * (g.c_dtype == JAGG_DTYPE_F32 ? 4 : 2),
-            g.M, g.N, g.K);
+  double flops = 0.0, bytes = 0.0;
+  for (const GemmArgs* g : {&a, b}) {
+    if (!g) continue;
+    flops += 2.0 * g->M * g->N * g->K;
+    bytes += 2.0 * ((double)g->M * g->K + (double)g->N * g->K) + (double)g->M * g->N * (g->c_dtype == JAGG_DTYPE_F32 ? 4 : 2);
+  }
+  // a group's M (or, for weight gradients, K) is the sum over its products
+  const bool sum_k = A_MN && b;
+  prof_stop(tok, s, PROF_GEMM_TC, flops, bytes, a.M + (b && !sum_k ? b->M : 0), a.N, a.K + (sum_k ? b->K : 0));
   return JAGG_OK;
+}
+
+// The estimate behind the choice of tiles, in k-blocks of a 256-column tile.  A unit (a tile, or
+// one K split of it) costs its k-blocks times bn / 256, a little more for narrower tiles (whose
+// operand traffic per FLOP is larger), plus P_UNIT_OVERHEAD for its pipeline fill and epilogue;
+// units go round-robin to the pairs, so a product takes the units of the pair that gets most.
+// Narrower tiles pay where 256 columns would leave the last wave nearly empty: 4096 x 3072 x 12288 in f32 takes
+// 180 us at 256 columns (192 units on 76 pairs) and 171 at 224; 633 x 3072 x 3072 19.4 -> 13.1,
+// 1225 x 768 x 3072 20.7 -> 12.7, 2664 x 2304 x 768 13.6 -> 12.5.
+constexpr double P_UNIT_OVERHEAD = 5.0;
+constexpr int P_WIDTHS[] = {256, 224, 192, 160, 128};
+constexpr double P_LAUNCH = 12.0;
+constexpr double P_WIDTH_COST[] = {1.0, 1.05, 1.07, 1.10, 1.15};
+
+struct PairUnits {
+  long long n;
+  double cost;
+};
+PairUnits pair_units(const GemmArgs& g, int w, int splits) {
+  const int bn = P_WIDTHS[w];
+  return {(long long)ceil_div(g.M, PT) * ceil_div(g.N, bn) * splits,
+          ceil_div(ceil_div(g.K, PK), splits) * P_WIDTH_COST[w] * bn / 256.0 + P_UNIT_OVERHEAD};
+}
+// Duration of a's units followed by b's, dealt round-robin to np pairs.
+double pair_time(PairUnits a, PairUnits b, int np) {
+  const long long qa = a.n / np, ra = a.n % np, qb = b.n / np, rb = b.n % np;
+  // pairs before ra take one more unit of a; b's deal starts at pair ra
+  const double early = ra ? (qa + 1) * a.cost + (qb + (rb > np - ra ? 1 : 0)) * b.cost : 0.0;
+  const double late = qa * a.cost + (qb + (rb > 0 ? 1 : 0)) * b.cost;
+  return early > late ? early : late;
+}
+int most_splits(const GemmArgs& g) {
+  const int kb = ceil_div(g.K, PK);
+  return g.epi != EPI_ACCUM ? 1 : kb < 32 ? kb : 32;
+}
+double pair_plan(const GemmArgs& g, int np, PairPlan* plan) {
+  double best = 0.0;
+  int lo = 1, hi = most_splits(g);
+  if (g.epi == EPI_ACCUM && g.split_k > 0) lo = hi = g.split_k < ceil_div(g.K, PK) ? g.split_k : ceil_div(g.K, PK);
+  for (int w = 0; w < 5; ++w)
+    for (int s = lo; s <= hi; ++s) {
+      const double c = pair_time(pair_units(g, w, s), {0, 0.0}, np);
+      if (best == 0.0 || c < 0.999 * best) {
+        best = c;
+        *plan = {P_WIDTHS[w], s};
+      }
+    }
+  return best;
+}
+
+// Whether the kernel has an instance for the product.
+bool pair_instance(const GemmArgs& g) {
+  if (g.tile_n != 0 || g.M <= 128 || g.N < 128 || (g.a_mn && !g.b_mn)) return false;
+  const int epi = pair_epi(g);
+  if (epi < 0) return false;
+  if (g.a_mn) return epi == PE_ACCUM;
+  return g.b_mn ? epi == PE_STORE_BF16 || epi == PE_STORE_F32 || epi == PE_MUL
+                : epi == PE_STORE_BF16 || epi == PE_GELU || epi == PE_GATE;
+}
+
+int dispatch_pair(const GemmArgs& a, const GemmArgs* b, const PairPlan (&plan)[2], cudaStream_t s) {
+  const int np = sm_count() / 2, epi = pair_epi(a);
+  if (!a.a_mn && !a.b_mn) {
+    if (epi == PE_STORE_BF16) return launch_pair<false, false, PE_STORE_BF16>(a, b, plan, np, s);
+    if (epi == PE_GELU) return launch_pair<false, false, PE_GELU>(a, b, plan, np, s);
+    if (epi == PE_GATE) return launch_pair<false, false, PE_GATE>(a, b, plan, np, s);
+  } else if (!a.a_mn) {
+    if (epi == PE_STORE_BF16) return launch_pair<false, true, PE_STORE_BF16>(a, b, plan, np, s);
+    if (epi == PE_STORE_F32) return launch_pair<false, true, PE_STORE_F32>(a, b, plan, np, s);
+    if (epi == PE_MUL) return launch_pair<false, true, PE_MUL>(a, b, plan, np, s);
+  } else if (epi == PE_ACCUM) {
+    return launch_pair<true, true, PE_ACCUM>(a, b, plan, np, s);
+  }
+  set_last_error("gemm: the pair kernel does not serve this product");
+  return JAGG_ERR_UNSUPPORTED;
 }
 
 }  // namespace
 
-// Waves of units over the pairs times the k-blocks of a unit, plus P_UNIT_OVERHEAD k-blocks (fitted
-// to measurements) per unit for its pipeline fill and epilogue; the split count of an accumulating product is the
-// one with the least.
-constexpr double P_UNIT_OVERHEAD = 3.0;
-static double pair_cost(const GemmArgs& g, int npairs, int* splits) {
-  const int k_blocks = ceil_div(g.K, PK);
-  const long long tiles = (long long)ceil_div(g.M, PT) * ceil_div(g.N, PT);
-  *splits = 1;
-  double best = 0.0;
-  int lo = 1, hi = g.epi == EPI_ACCUM ? (k_blocks < 32 ? k_blocks : 32) : 1;
-  if (g.epi == EPI_ACCUM && g.split_k > 0) lo = hi = g.split_k < k_blocks ? g.split_k : k_blocks;
-  for (int s = lo; s <= hi; ++s) {
-    const double waves = (double)((tiles * s + npairs - 1) / npairs);
-    const double cost = waves * (ceil_div(k_blocks, s) + P_UNIT_OVERHEAD);
-    if (s == lo || cost < 0.999 * best) {
-      best = cost;
-      *splits = s;
-    }
-  }
-  return best;
-}
-
 bool gemm_pair_serves(const GemmArgs& g, double* cost) {
-  if (g.tile_n != 0 || g.M <= 128 || g.N < 192 || (g.a_mn && !g.b_mn)) return false;
-  const int epi = pair_epi(g);
-  if (epi < 0) return false;
-  const bool fwd = !g.a_mn && !g.b_mn, dx = !g.a_mn && g.b_mn;
-  if (fwd && !(epi == PE_STORE_BF16 || epi == PE_GELU || epi == PE_GATE)) return false;
-  if (dx && !(epi == PE_STORE_BF16 || epi == PE_STORE_F32 || epi == PE_MUL)) return false;
-  if (g.a_mn && epi != PE_ACCUM) return false;
-  int splits;
-  *cost = pair_cost(g, sm_count() / 2, &splits);
+  if (!pair_instance(g)) return false;
+  PairPlan plan;
+  *cost = pair_plan(g, sm_count() / 2, &plan);
   return true;
 }
 
 int gemm_pair(const GemmArgs& g, cudaStream_t s) {
-  const int npairs = sm_count() / 2;
-  int splits;
-  pair_cost(g, npairs, &splits);
-  const int epi = pair_epi(g);
-  if (!g.a_mn && !g.b_mn) {
-    if (epi == PE_STORE_BF16) return launch_pair<false, false, PE_STORE_BF16>(g, splits, npairs, s);
-    if (epi == PE_GELU) return launch_pair<false, false, PE_GELU>(g, splits, npairs, s);
-    if (epi == PE_GATE) return launch_pair<false, false, PE_GATE>(g, splits, npairs, s);
-  } else if (!g.a_mn) {
-    if (epi == PE_STORE_BF16) return launch_pair<false, true, PE_STORE_BF16>(g, splits, npairs, s);
-    if (epi == PE_STORE_F32) return launch_pair<false, true, PE_STORE_F32>(g, splits, npairs, s);
-    if (epi == PE_MUL) return launch_pair<false, true, PE_MUL>(g, splits, npairs, s);
-  } else if (epi == PE_ACCUM) {
-    return launch_pair<true, true, PE_ACCUM>(g, splits, npairs, s);
+  PairPlan plan[2] = {};
+  pair_plan(g, sm_count() / 2, &plan[0]);
+  return dispatch_pair(g, nullptr, plan, s);
+}
+
+int gemm_two(const GemmArgs& x, const GemmArgs& y, cudaStream_t s) {
+  const bool same = x.a_mn == y.a_mn && x.b_mn == y.b_mn && x.epi == y.epi && gemm_tc_eligible(x) &&
+                    gemm_tc_eligible(y) && pair_instance(x) && pair_instance(y) && pair_epi(x) == pair_epi(y);
+  if (same) {
+    // the longer units first, so that the short ones even out the end
+    const GemmArgs& a = x.K > y.K || (x.K == y.K && x.M >= y.M) ? x : y;
+    const GemmArgs& b = &a == &x ? y : x;
+    const int np = sm_count() / 2;
+    PairPlan plan[2] = {}, alone;
+    double best = 0.0;
+    const int sa_max = most_splits(a) < 8 ? most_splits(a) : 8, sb_max = most_splits(b) < 4 ? most_splits(b) : 4;
+    for (int wa = 0; wa < 5; ++wa)
+      for (int sa = 1; sa <= sa_max; ++sa)
+        for (int wb = 0; wb < 5; ++wb)
+          for (int sb = 1; sb <= sb_max; ++sb) {
+            const double c = pair_time(pair_units(a, wa, sa), pair_units(b, wb, sb), np);
+            if (best == 0.0 || c < 0.999 * best) {
+              best = c;
+              plan[0] = {P_WIDTHS[wa], sa};
+              plan[1] = {P_WIDTHS[wb], sb};
+            }
+          }
+    // against two launches of their own (the second's ramp is about P_LAUNCH k-blocks)
+    const double apart = gemm_best_cost(a) + gemm_best_cost(b) + P_LAUNCH;
+    if (best < apart) return dispatch_pair(a, &b, plan, s);
   }
-  set_last_error("gemm: the pair kernel does not serve this product");
-  return JAGG_ERR_UNSUPPORTED;
+  JAGG_TRY(gemm(x, s));
+  return gemm(y, s);
 }
 
 }  // namespace jagg

@@ -690,6 +690,10 @@ int zero_vjp_accumulators(const jagg_model& m, int B, const VjpWs& w, cudaStream
   return JAGG_OK;
 }
 
+// The products of a block, one per stream (one stream: a DiT or single block; two: the text and
+// image streams of an MMDiT double block, whose products of one step run as one launch).
+int gemm_streams(const GemmArgs* g, int n, cudaStream_t s) { return n == 2 ? gemm_two(g[0], g[1], s) : gemm(g[0], s); }
+
 // The MLP half of a block's backward, shared by DiT blocks and the streams of MMDiT
 // double blocks (Ms rows of Ns tokens per sequence): from dy = g2 dh (already formed)
 // through fc2, GELU, fc1 and LN2 + modulation, then the attention branch's gate, ending
@@ -697,61 +701,101 @@ int zero_vjp_accumulators(const jagg_model& m, int B, const VjpWs& w, cudaStream
 struct BranchW {
   int64_t proj_w, proj_b, fc1_w, fc1_b, fc2_w, fc2_b, mod_col;
 };
-int mlp_and_proj_bwd(const jagg_model& m, int Ms, int Ns, const DitSaved& k, const BranchW& bw, const float* mod,
-                     float* dmod, float* dh, void* dy, void* dO, const VjpWs& w, float* grad, cudaStream_t s) {
+struct StreamBwd {
+  int Ms, Ns;
+  const DitSaved* k;
+  BranchW bw;
+  const float* mod;
+  float* dmod;
+  float* dh;
+  void* dy;
+  void* dO;
+  void* du;     // [Ms, dm] scratch
+  float* dx32;  // [Ms, d] scratch
+};
+int mlp_and_proj_bwd(const jagg_model& m, const StreamBwd* st, int n, float* grad, cudaStream_t s) {
   const int dt = m.cfg.dtype, d = m.d, dmw = m.dm;
   const int64_t Lm = m.T.Lmod;
-  JAGG_TRY(gemm(dw_gemm(m, Ms, d, dmw, dy, d, k.gu, dmw, grad, bw.fc2_w), s));
-  {
-    GemmArgs g = dx_gemm(m, Ms, d, dmw, dy, d, bw.fc2_w);
-    g.epi = EPI_MUL_AUX; g.C = w.du; g.ldc = dmw; g.aux = k.gp; g.ld_aux = dmw;
-    JAGG_TRY(gemm(g, s));
+  GemmArgs g[2];
+  for (int i = 0; i < n; ++i)
+    g[i] = dw_gemm(m, st[i].Ms, d, dmw, st[i].dy, d, st[i].k->gu, dmw, grad, st[i].bw.fc2_w);
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i) {
+    g[i] = dx_gemm(m, st[i].Ms, d, dmw, st[i].dy, d, st[i].bw.fc2_w);
+    g[i].epi = EPI_MUL_AUX; g[i].C = st[i].du; g[i].ldc = dmw; g[i].aux = st[i].k->gp; g[i].ld_aux = dmw;
   }
-  JAGG_TRY(launch_colsum(w.du, dt == JAGG_DTYPE_F32, dt, Ms, dmw, dmw, grad + bw.fc1_b, s));
-  JAGG_TRY(gemm(dw_gemm(m, Ms, dmw, d, w.du, dmw, k.m, d, grad, bw.fc1_w), s));
-  {
-    GemmArgs g = dx_gemm(m, Ms, dmw, d, w.du, dmw, bw.fc1_w);
-    g.C = w.dx32; g.ldc = d; g.c_dtype = JAGG_DTYPE_F32;
-    JAGG_TRY(gemm(g, s));
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i)
+    JAGG_TRY(launch_colsum(st[i].du, dt == JAGG_DTYPE_F32, dt, st[i].Ms, dmw, dmw, grad + st[i].bw.fc1_b, s));
+  for (int i = 0; i < n; ++i)
+    g[i] = dw_gemm(m, st[i].Ms, dmw, d, st[i].du, dmw, st[i].k->m, d, grad, st[i].bw.fc1_w);
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i) {
+    g[i] = dx_gemm(m, st[i].Ms, dmw, d, st[i].du, dmw, st[i].bw.fc1_w);
+    g[i].C = st[i].dx32; g[i].ldc = d; g[i].c_dtype = JAGG_DTYPE_F32;
   }
-  {  // LN2 + modulation backward, then the attention branch's gate
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i) {  // LN2 + modulation backward, then the attention branch's gate
+    const StreamBwd& q = st[i];
     LnGateBwd a{};
-    a.M = Ms; a.d = d; a.rows_per_seq = Ns;
-    a.do_ln = 1; a.dm = w.dx32; a.dm_f32 = 1; a.h = k.h_mid; a.mean = k.st2; a.rstd = k.st2 + Ms;
-    a.scale = mod + 4 * d; a.mod_stride = Lm; a.dshift = dmod + 3 * d; a.dscale = dmod + 4 * d;
-    a.dmod_stride = Lm; a.dh_in = dh; a.dh_out = dh;
-    a.do_gate = 1; a.y = k.y1; a.gate = mod + 2 * d; a.dgate = dmod + 2 * d; a.dy = dy;
-    a.dbias = grad + bw.proj_b; a.dtype = dt;
+    a.M = q.Ms; a.d = d; a.rows_per_seq = q.Ns;
+    a.do_ln = 1; a.dm = q.dx32; a.dm_f32 = 1; a.h = q.k->h_mid; a.mean = q.k->st2; a.rstd = q.k->st2 + q.Ms;
+    a.scale = q.mod + 4 * d; a.mod_stride = Lm; a.dshift = q.dmod + 3 * d; a.dscale = q.dmod + 4 * d;
+    a.dmod_stride = Lm; a.dh_in = q.dh; a.dh_out = q.dh;
+    a.do_gate = 1; a.y = q.k->y1; a.gate = q.mod + 2 * d; a.dgate = q.dmod + 2 * d; a.dy = q.dy;
+    a.dbias = grad + q.bw.proj_b; a.dtype = dt;
     JAGG_TRY(launch_ln_gate_bwd(a, s));
   }
-  JAGG_TRY(gemm(dw_gemm(m, Ms, d, d, dy, d, k.o, d, grad, bw.proj_w), s));
-  GemmArgs g = dx_gemm(m, Ms, d, d, dy, d, bw.proj_w);
-  g.C = dO; g.ldc = d;
-  return gemm(g, s);
+  for (int i = 0; i < n; ++i) g[i] = dw_gemm(m, st[i].Ms, d, d, st[i].dy, d, st[i].k->o, d, grad, st[i].bw.proj_w);
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i) {
+    g[i] = dx_gemm(m, st[i].Ms, d, d, st[i].dy, d, st[i].bw.proj_w);
+    g[i].C = st[i].dO; g[i].ldc = d;
+  }
+  return gemm_streams(g, n, s);
 }
 
 // The qkv half of a block's backward after attention: qkv bias / weight gradients, the
 // gradient into the LN1 input, and LN1 + modulation backward (dh accumulates in place).
 // `gate`, when given, fuses the gate backward of the previous block's last branch.
-int qkv_and_ln1_bwd(const jagg_model& m, int Ms, int Ns, const void* dqkv, int64_t ld_dqkv, int n_out,
-                    int64_t w_off, int64_t b_off, const void* a_in, const float* h_in, const float* st1,
-                    const float* mod, float* dmod, float* dh, const LnGateBwd* gate, const VjpWs& w, float* grad,
+struct QkvBwd {
+  int Ms, Ns;
+  const void* dqkv;
+  const void* a_in;
+  const float* h_in;
+  const float* st1;
+  int64_t w_off, b_off;
+  const float* mod;
+  float* dmod;
+  float* dh;
+  float* dx32;  // [Ms, d] scratch
+  LnGateBwd gate;
+};
+int qkv_and_ln1_bwd(const jagg_model& m, const QkvBwd* st, int n, int64_t ld_dqkv, int n_out, float* grad,
                     cudaStream_t s) {
   const int dt = m.cfg.dtype, d = m.d;
   const int64_t Lm = m.T.Lmod;
-  JAGG_TRY(launch_colsum(dqkv, dt == JAGG_DTYPE_F32, dt, Ms, n_out, ld_dqkv, grad + b_off, s));
-  JAGG_TRY(gemm(dw_gemm(m, Ms, n_out, d, dqkv, ld_dqkv, a_in, d, grad, w_off), s));
-  {
-    GemmArgs g = dx_gemm(m, Ms, n_out, d, dqkv, ld_dqkv, w_off);
-    g.C = w.dx32; g.ldc = d; g.c_dtype = JAGG_DTYPE_F32;
-    JAGG_TRY(gemm(g, s));
+  GemmArgs g[2];
+  for (int i = 0; i < n; ++i) {
+    JAGG_TRY(launch_colsum(st[i].dqkv, dt == JAGG_DTYPE_F32, dt, st[i].Ms, n_out, ld_dqkv, grad + st[i].b_off, s));
+    g[i] = dw_gemm(m, st[i].Ms, n_out, d, st[i].dqkv, ld_dqkv, st[i].a_in, d, grad, st[i].w_off);
   }
-  LnGateBwd a = gate ? *gate : LnGateBwd{};
-  a.M = Ms; a.d = d; a.rows_per_seq = Ns;
-  a.do_ln = 1; a.dm = w.dx32; a.dm_f32 = 1; a.h = h_in; a.mean = st1; a.rstd = st1 + Ms;
-  a.scale = mod + d; a.mod_stride = Lm; a.dshift = dmod; a.dscale = dmod + d; a.dmod_stride = Lm;
-  a.dh_in = dh; a.dh_out = dh; a.dtype = dt;
-  return launch_ln_gate_bwd(a, s);
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i) {
+    g[i] = dx_gemm(m, st[i].Ms, n_out, d, st[i].dqkv, ld_dqkv, st[i].w_off);
+    g[i].C = st[i].dx32; g[i].ldc = d; g[i].c_dtype = JAGG_DTYPE_F32;
+  }
+  JAGG_TRY(gemm_streams(g, n, s));
+  for (int i = 0; i < n; ++i) {
+    const QkvBwd& q = st[i];
+    LnGateBwd a = q.gate;
+    a.M = q.Ms; a.d = d; a.rows_per_seq = q.Ns;
+    a.do_ln = 1; a.dm = q.dx32; a.dm_f32 = 1; a.h = q.h_in; a.mean = q.st1; a.rstd = q.st1 + q.Ms;
+    a.scale = q.mod + d; a.mod_stride = Lm; a.dshift = q.dmod; a.dscale = q.dmod + d; a.dmod_stride = Lm;
+    a.dh_in = q.dh; a.dh_out = q.dh; a.dtype = dt;
+    JAGG_TRY(launch_ln_gate_bwd(a, s));
+  }
+  return JAGG_OK;
 }
 
 // Gate backward of a branch y with gate mod[gcol]: dgate += sum dh y; dy = gate dh; dbias.
@@ -851,7 +895,8 @@ int vjp_dit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float* g
     const DitSaved& k = S.blk[l];
     const float* mod = S.mod + bw.mod_col;
     float* dmod = w.dmod + bw.mod_col;
-    JAGG_TRY(mlp_and_proj_bwd(m, M, N, k, branch_of(bw), mod, dmod, w.dh, w.dy, w.dO, w, grad, s));
+    const StreamBwd st{M, N, &k, branch_of(bw), mod, dmod, w.dh, w.dy, w.dO, w.du, w.dx32};
+    JAGG_TRY(mlp_and_proj_bwd(m, &st, 1, grad, s));
     AttnBwdArgs ab;
     ab.f = attn_args(m, B, seg_single(k.qkv, 3 * d, N), seg_single(k.qkv, 3 * d, N), seg_single(k.o, d, N), k.lse);
     ab.f.q_col0 = 0; ab.f.k_col0 = d; ab.f.v_col0 = 2 * d;
@@ -862,8 +907,8 @@ int vjp_dit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float* g
     JAGG_TRY(attention_bwd(ab, s));
     LnGateBwd prev{};
     if (l > 0) prev = mlp_gate(l - 1);
-    JAGG_TRY(qkv_and_ln1_bwd(m, M, N, w.dqkv, 3 * d, 3 * d, bw.qkv_w, bw.qkv_b, k.a, k.h_in, k.st1, mod, dmod, w.dh,
-                             l > 0 ? &prev : nullptr, w, grad, s));
+    const QkvBwd qb{M, N, w.dqkv, k.a, k.h_in, k.st1, bw.qkv_w, bw.qkv_b, mod, dmod, w.dh, w.dx32, prev};
+    JAGG_TRY(qkv_and_ln1_bwd(m, &qb, 1, 3 * d, 3 * d, grad, s));
   }
   return JAGG_OK;
 }
@@ -880,18 +925,24 @@ int forward_mmdit(const jagg_model& m, const Saved& S, int B, cudaStream_t s) {
   for (int l = 0; l < Ld; ++l) {
     const DoubleW& bw = m.T.doubles[l];
     const DoubleSaved& k = S.dbl[l];
+    GemmArgs g[2];
+    int Ns[2] = {Nt, Ni}, Ms[2] = {B * Nt, B * Ni};
     for (int si = 0; si < 2; ++si) {
       const StreamW& sw = bw.s[si];
       const DitSaved& q = k.s[si];
-      const int Ns = si ? Ni : Nt, Ms = B * Ns;
       const float* mod = S.mod + sw.mod_col;
-      LnModFwd ln{q.h_in, 0, 0, 0, Ms, d, Ns, mod, mod + d, Lm, q.a, dt, q.st1, q.st1 + Ms};
+      LnModFwd ln{q.h_in, 0, 0, 0, Ms[si], d, Ns[si], mod, mod + d, Lm, q.a, dt, q.st1, q.st1 + Ms[si]};
       JAGG_TRY(launch_ln_mod_fwd(ln, s));
-      GemmArgs g = fwd_gemm(m, Ms, 3 * d, d, q.a, d, sw.qkv_w, sw.qkv_b);
-      g.C = q.qkv; g.ldc = 3 * d;
-      JAGG_TRY(gemm(g, s));
+      g[si] = fwd_gemm(m, Ms[si], 3 * d, d, q.a, d, sw.qkv_w, sw.qkv_b);
+      g[si].C = q.qkv; g[si].ldc = 3 * d;
+    }
+    JAGG_TRY(gemm_streams(g, 2, s));
+    for (int si = 0; si < 2; ++si) {
+      const StreamW& sw = bw.s[si];
+      const DitSaved& q = k.s[si];
       // text tokens sit at RoPE position (0, 0): the whole text stream is unrotated
-      JAGG_TRY(launch_qk_norm_rope_fwd(qk_args(m, q.qkv, Ms, Ns, si ? 0 : Ns, sw.qn, sw.kn, q.qk, q.rq, q.rk), s));
+      JAGG_TRY(launch_qk_norm_rope_fwd(
+          qk_args(m, q.qkv, Ms[si], Ns[si], si ? 0 : Ns[si], sw.qn, sw.kn, q.qk, q.rq, q.rk), s));
     }
     AttnArgs at = attn_args(m, B, SegRows{k.s[0].qk, k.s[1].qk, 2 * d, 2 * d, Nt},
                             SegRows{k.s[0].qkv, k.s[1].qkv, 3 * d, 3 * d, Nt},
@@ -901,25 +952,32 @@ int forward_mmdit(const jagg_model& m, const Saved& S, int B, cudaStream_t s) {
     for (int si = 0; si < 2; ++si) {
       const StreamW& sw = bw.s[si];
       const DitSaved& q = k.s[si];
-      const int Ns = si ? Ni : Nt, Ms = B * Ns;
-      const float* mod = S.mod + sw.mod_col;
-      float* h_out = (l + 1 < Ld) ? S.dbl[l + 1].s[si].h_in : S.hD[si];
-      GemmArgs g = fwd_gemm(m, Ms, d, d, q.o, d, sw.proj_w, sw.proj_b);
-      g.epi = EPI_GATE_RESID; g.C = q.y1; g.ldc = d;
-      g.C2 = q.h_mid; g.ldc2 = d; g.aux = q.h_in; g.ld_aux = d;
-      g.gate = mod + 2 * d; g.gate_stride = Lm; g.rows_per_seq = Ns;
-      JAGG_TRY(gemm(g, s));
-      LnModFwd ln2{q.h_mid, 0, 0, 0, Ms, d, Ns, mod + 3 * d, mod + 4 * d, Lm, q.m, dt, q.st2, q.st2 + Ms};
-      JAGG_TRY(launch_ln_mod_fwd(ln2, s));
-      g = fwd_gemm(m, Ms, dm, d, q.m, d, sw.fc1_w, sw.fc1_b);
-      g.epi = EPI_GELU; g.C = S.keep ? q.gp : nullptr; g.ldc = dm; g.C2 = q.gu; g.ldc2 = dm;
-      JAGG_TRY(gemm(g, s));
-      g = fwd_gemm(m, Ms, d, dm, q.gu, dm, sw.fc2_w, sw.fc2_b);
-      g.epi = EPI_GATE_RESID; g.C = q.y2; g.ldc = d;
-      g.C2 = h_out; g.ldc2 = d; g.aux = q.h_mid; g.ld_aux = d;
-      g.gate = mod + 5 * d; g.gate_stride = Lm; g.rows_per_seq = Ns;
-      JAGG_TRY(gemm(g, s));
+      g[si] = fwd_gemm(m, Ms[si], d, d, q.o, d, sw.proj_w, sw.proj_b);
+      g[si].epi = EPI_GATE_RESID; g[si].C = q.y1; g[si].ldc = d;
+      g[si].C2 = q.h_mid; g[si].ldc2 = d; g[si].aux = q.h_in; g[si].ld_aux = d;
+      g[si].gate = S.mod + sw.mod_col + 2 * d; g[si].gate_stride = Lm; g[si].rows_per_seq = Ns[si];
     }
+    JAGG_TRY(gemm_streams(g, 2, s));
+    for (int si = 0; si < 2; ++si) {
+      const StreamW& sw = bw.s[si];
+      const DitSaved& q = k.s[si];
+      const float* mod = S.mod + sw.mod_col;
+      LnModFwd ln2{q.h_mid, 0, 0, 0, Ms[si], d, Ns[si], mod + 3 * d, mod + 4 * d, Lm, q.m, dt, q.st2, q.st2 + Ms[si]};
+      JAGG_TRY(launch_ln_mod_fwd(ln2, s));
+      g[si] = fwd_gemm(m, Ms[si], dm, d, q.m, d, sw.fc1_w, sw.fc1_b);
+      g[si].epi = EPI_GELU; g[si].C = S.keep ? q.gp : nullptr; g[si].ldc = dm; g[si].C2 = q.gu; g[si].ldc2 = dm;
+    }
+    JAGG_TRY(gemm_streams(g, 2, s));
+    for (int si = 0; si < 2; ++si) {
+      const StreamW& sw = bw.s[si];
+      const DitSaved& q = k.s[si];
+      float* h_out = (l + 1 < Ld) ? S.dbl[l + 1].s[si].h_in : S.hD[si];
+      g[si] = fwd_gemm(m, Ms[si], d, dm, q.gu, dm, sw.fc2_w, sw.fc2_b);
+      g[si].epi = EPI_GATE_RESID; g[si].C = q.y2; g[si].ldc = d;
+      g[si].C2 = h_out; g[si].ldc2 = d; g[si].aux = q.h_mid; g[si].ld_aux = d;
+      g[si].gate = S.mod + sw.mod_col + 5 * d; g[si].gate_stride = Lm; g[si].rows_per_seq = Ns[si];
+    }
+    JAGG_TRY(gemm_streams(g, 2, s));
   }
   float* hj = Ls > 0 ? S.sgl[0].h_in : S.h_fin;
   if (Ld > 0) {  // the two streams join into the [txt; img] layout
@@ -1001,8 +1059,8 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
     JAGG_TRY(launch_qk_norm_rope_bwd(qb, s));
     LnGateBwd prev{};
     if (l > 0) prev = single_gate(l - 1);
-    JAGG_TRY(qkv_and_ln1_bwd(m, M, N, w.dqkv, ld1, (int)ld1, sw.lin1_w, sw.lin1_b, k.a, k.h_in, k.st1, mod, dmod,
-                             w.dh, l > 0 ? &prev : nullptr, w, grad, s));
+    const QkvBwd l1{M, N, w.dqkv, k.a, k.h_in, k.st1, sw.lin1_w, sw.lin1_b, mod, dmod, w.dh, w.dx32, prev};
+    JAGG_TRY(qkv_and_ln1_bwd(m, &l1, 1, ld1, (int)ld1, grad, s));
   }
   if (Ld == 0) return JAGG_OK;
   // the joint gradient splits into the two streams
@@ -1012,6 +1070,8 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
   void* dy_s[2] = {w.dy, at_byte(w.dy, (size_t)Mt * d * e)};
   void* dO_s[2] = {w.dO, at_byte(w.dO, (size_t)Mt * d * e)};
   void* dqkv_s[2] = {w.dqkv, at_byte(w.dqkv, (size_t)Mt * 3 * d * e)};
+  void* du_s[2] = {w.du, at_byte(w.du, (size_t)Mt * dm * e)};
+  float* dx32_s[2] = {w.dx32, w.dx32 + (size_t)Mt * d};
   auto mlp_gate = [&](int l, int si) {
     const StreamW& sw = m.T.doubles[l].s[si];
     const int Ns = si ? Ni : Nt;
@@ -1022,11 +1082,14 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
   for (int l = Ld - 1; l >= 0; --l) {
     const DoubleW& bw = m.T.doubles[l];
     const DoubleSaved& k = S.dbl[l];
+    StreamBwd st[2];
     for (int si = 0; si < 2; ++si) {
       const int Ns = si ? Ni : Nt;
-      JAGG_TRY(mlp_and_proj_bwd(m, B * Ns, Ns, k.s[si], branch_of(bw.s[si]), S.mod + bw.s[si].mod_col,
-                                w.dmod + bw.s[si].mod_col, w.dhs[si], dy_s[si], dO_s[si], w, grad, s));
+      const int64_t mc = bw.s[si].mod_col;
+      st[si] = {B * Ns, Ns, &k.s[si], branch_of(bw.s[si]), S.mod + mc, w.dmod + mc, w.dhs[si], dy_s[si], dO_s[si],
+                du_s[si], dx32_s[si]};
     }
+    JAGG_TRY(mlp_and_proj_bwd(m, st, 2, grad, s));
     AttnBwdArgs ab;
     ab.f = attn_args(m, B, SegRows{k.s[0].qk, k.s[1].qk, 2 * d, 2 * d, Nt},
                      SegRows{k.s[0].qkv, k.s[1].qkv, 3 * d, 3 * d, Nt}, SegRows{k.s[0].o, k.s[1].o, d, d, Nt}, k.lse);
@@ -1036,6 +1099,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
     ab.dq = ab.dk = ab.dv = SegRows{dqkv_s[0], dqkv_s[1], 3 * d, 3 * d, Nt};
     ab.dq_col0 = 0; ab.dk_col0 = d; ab.dv_col0 = 2 * d;
     JAGG_TRY(attention_bwd(ab, s));
+    QkvBwd qk[2];
     for (int si = 0; si < 2; ++si) {
       const StreamW& sw = bw.s[si];
       const DitSaved& q = k.s[si];
@@ -1048,10 +1112,10 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
       JAGG_TRY(launch_qk_norm_rope_bwd(qb, s));
       LnGateBwd prev{};
       if (l > 0) prev = mlp_gate(l - 1, si);
-      JAGG_TRY(qkv_and_ln1_bwd(m, Ms, Ns, dqkv_s[si], 3 * d, 3 * d, sw.qkv_w, sw.qkv_b, q.a, q.h_in, q.st1,
-                               S.mod + sw.mod_col, w.dmod + sw.mod_col, w.dhs[si], l > 0 ? &prev : nullptr, w, grad,
-                               s));
+      qk[si] = {Ms, Ns, dqkv_s[si], q.a, q.h_in, q.st1, sw.qkv_w, sw.qkv_b, S.mod + sw.mod_col, w.dmod + sw.mod_col,
+                w.dhs[si], dx32_s[si], prev};
     }
+    JAGG_TRY(qkv_and_ln1_bwd(m, qk, 2, 3 * d, 3 * d, grad, s));
   }
   return JAGG_OK;
 }

@@ -8,6 +8,8 @@ import pytest
 import torch
 import torch.nn.functional as F
 
+import synth
+from test_gpu_dit import FLUX, _check
 from test_gpu_kernels import _desc, _rel
 
 pytestmark = pytest.mark.gpu
@@ -40,7 +42,18 @@ def _done(*wide):
 BF16_TOL = 4e-3
 
 
-@pytest.mark.parametrize("M,N,K", [(2601, 1088, 1000), (2560, 1024, 1024)])
+def _f32_tol(K):
+    """The tensor core adds 16 products at a time to the f32 accumulator and may truncate: at most
+    one unit in the last place (2^-23) of the running sum per step, all in one direction."""
+    return 1e-6 + 2.0 ** -23 * K / 16
+
+
+# the widths that the estimate picks for them: 128 .. 256 columns, whole and ragged
+SHAPES = [(2601, 1088, 1000), (2560, 1024, 1024), (700, 768, 768), (1225, 3072, 768), (2048, 3072, 320),
+          (5328, 2304, 136), (150, 192, 64)]
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
 def test_forward_epilogues(M, N, K):
     ops, acc = _operands(M, N, K, 0, 0)
     bias = torch.randn(N, device="cuda").bfloat16()
@@ -68,7 +81,7 @@ def test_forward_epilogues(M, N, K):
     assert _rel(G[:, :N].float(), g.detach()) < BF16_TOL and _rel(D[:, :N].float(), v.grad) < BF16_TOL
 
 
-@pytest.mark.parametrize("M,N,K", [(2601, 1096, 1000), (2560, 1024, 1024)])
+@pytest.mark.parametrize("M,N,K", SHAPES + [(2601, 1096, 1000)])
 def test_input_gradient_epilogues(M, N, K):
     ops, acc = _operands(M, N, K, 0, 1)
     X = torch.rand(M, N + 8, device="cuda").bfloat16()
@@ -80,16 +93,16 @@ def test_input_gradient_epilogues(M, N, K):
     assert _rel(O[:, :N].float(), acc * X[:, :N].float()) < BF16_TOL
 
 
-@pytest.mark.parametrize("M,N,K", [(2500, 3080, 4104), (2560, 3072, 4096)])
+@pytest.mark.parametrize("M,N,K", [(2500, 3080, 4104), (2560, 3072, 4096), (2048, 3072, 9216), (900, 2304, 3072)])
 def test_f32_output(M, N, K):
     ops, acc = _operands(M, N, K, 0, 1)
     C = _out(M, N, 4, torch.float32)
     jg.test_gemm(_desc(M, N, K, *ops, C, N + 4, jg.DTYPE_F32))
     _done((C, N))
-    assert _rel(C[:, :N], acc) < 1e-5
+    assert _rel(C[:, :N], acc) < _f32_tol(K)
 
 
-@pytest.mark.parametrize("M,N,K", [(4100, 3076, 8200), (3072, 12288, 2304)])
+@pytest.mark.parametrize("M,N,K", [(4100, 3076, 8200), (3072, 12288, 2304), (3072, 768, 5328), (768, 768, 21312)])
 def test_accumulation(M, N, K):
     """The weight-gradient layout, added to what is there: f32 sums of bf16 products."""
     ops, acc = _operands(M // 4 * 4, N, K, 1, 1)
@@ -103,4 +116,12 @@ def test_accumulation(M, N, K):
     As, Bs = pad(As).contiguous(), pad(Bs).contiguous()
     jg.test_gemm(_desc(M, N, K, As, As.shape[1], 1, Bs, Bs.shape[1], 1, dt, G, N + 4, jg.DTYPE_F32, epi=4))
     _done((G, N))
-    assert _rel(G[:, :N], G0 + acc) < 1e-5
+    assert _rel(G[:, :N], G0 + acc) < _f32_tol(K)
+
+
+@pytest.mark.parametrize("B,latent,txt_len", [(4, (16, 20), 70), (3, (32, 28), 211), (2, (24, 24), 256)])
+def test_streams_in_one_launch(B, latent, txt_len):
+    """Dual-stream blocks whose text and image products run as one launch: different row counts, the
+    larger stream either one, two blocks, against the oracle."""
+    _check(synth.small_variant(FLUX, name="streams", hidden=512, heads=4, mlp=2048, depth=0, depth_double=2,
+                               latent_h=latent[0], latent_w=latent[1], txt_len=txt_len, txt_dim=256), B, 2e-2, 1e-2)
