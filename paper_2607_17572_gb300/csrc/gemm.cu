@@ -14,6 +14,7 @@
 #include <mutex>
 
 #include "gemm.cuh"
+#include "rows.cuh"
 #include "ptx.cuh"
 #include "tmap.cuh"
 
@@ -1203,6 +1204,7 @@ double gemm_best_cost(const GemmArgs& g) {
 int gemm(const GemmArgs& g, cudaStream_t stream) {
   JAGG_TRY(validate(g));
   if (!gemm_tc_eligible(g)) return gemm_simt(g, stream);
+  if (rank_update_serves(g)) return rank_update(g, stream);
   double cost;
   if (takes_pair(g, &cost)) return gemm_pair(g, stream);
   if (!g.a_mn && !g.b_mn) return dispatch_bn<false, false>(g, stream);

@@ -10,6 +10,7 @@
 #include "attention.cuh"
 #include "elementwise.cuh"
 #include "gemm.cuh"
+#include "rows.cuh"
 
 namespace jagg {
 
@@ -566,6 +567,18 @@ GemmArgs rows_dx(const jagg_model& m, int out, int in, int B, const void* dY, in
   return g;
 }
 
+// C[B, out] = act(x) W^T + b with act(x) in the storage type to x_act; silu_out: f32 scratch for
+// SiLU(x), or null for the identity.
+int rows_product(const jagg_model& m, int out, int in, int B, const float* x, float* silu_out, void* x_act,
+                 int64_t w_off, int64_t b_off, float* C, cudaStream_t s) {
+  const int dt = m.cfg.dtype;
+  const RowsFwd f{B, out, in, silu_out ? 1 : 0, x, x_act, W(m, w_off), W(m, b_off), C};
+  if (dt == JAGG_DTYPE_BF16 && rows_fwd_serves(f)) return launch_rows_fwd(f, s);
+  if (silu_out) JAGG_TRY(launch_silu(x, silu_out, (int64_t)B * in, s));
+  JAGG_TRY(launch_gather_rows(silu_out ? silu_out : x, in, 0, 0, 0, x_act, dt, B, in, s));
+  return gemm(rows_gemm(m, out, in, B, x_act, w_off, b_off, C), s);
+}
+
 // Row map of a token range inside the joint [txt; img] layout of B sequences of N rows:
 // row r of the range is (r / seg) * stride + off + r % seg (seg = 0: the identity).
 struct RowMap {
@@ -598,17 +611,11 @@ int prologue_fwd(const jagg_model& m, const void* z, const float* t, const void*
   // the single-stream DiT adds the fixed 2D sin-cos table; the MMDiT rotates q/k instead
   if (c.arch == JAGG_ARCH_DIT) JAGG_TRY(launch_add_pos_embed(h_img, B, m.N, m.Nt, m.gh, m.gw, d, s));
   // t-embedding MLP and every block's modulation (stacked weights): products with B
-  // per-sequence rows, each run as Y^T = W X^T so that the long dimension is M
+  // per-sequence rows
   JAGG_TRY(launch_timestep_embedding(t, S.phi, B, c.freq_dim, s));
-  JAGG_TRY(launch_gather_rows(S.phi, c.freq_dim, 0, 0, 0, S.phi_b, dt, B, c.freq_dim, s));
-  JAGG_TRY(gemm(rows_gemm(m, d, c.freq_dim, B, S.phi_b, m.T.t_w1, m.T.t_b1, S.e1), s));
-  JAGG_TRY(launch_silu(S.e1, S.se1, (int64_t)B * d, s));
-  JAGG_TRY(launch_gather_rows(S.se1, d, 0, 0, 0, S.se1_b, dt, B, d, s));
-  JAGG_TRY(gemm(rows_gemm(m, d, d, B, S.se1_b, m.T.t_w2, m.T.t_b2, S.c), s));
-  JAGG_TRY(launch_silu(S.c, S.sc, (int64_t)B * d, s));
-  JAGG_TRY(launch_gather_rows(S.sc, d, 0, 0, 0, S.sc_b, dt, B, d, s));
-  JAGG_TRY(gemm(rows_gemm(m, (int)m.T.Lmod, d, B, S.sc_b, m.T.mod_w, m.T.mod_b, S.mod), s));
-  return JAGG_OK;
+  JAGG_TRY(rows_product(m, d, c.freq_dim, B, S.phi, nullptr, S.phi_b, m.T.t_w1, m.T.t_b1, S.e1, s));
+  JAGG_TRY(rows_product(m, d, d, B, S.e1, S.se1, S.se1_b, m.T.t_w2, m.T.t_b2, S.c, s));
+  return rows_product(m, (int)m.T.Lmod, d, B, S.c, S.sc, S.sc_b, m.T.mod_w, m.T.mod_b, S.mod, s);
 }
 
 // Final layer on the image rows of the joint stream S.h_fin, then unpatchify.

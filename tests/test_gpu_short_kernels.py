@@ -82,3 +82,26 @@ def test_colsum_row_blocks(rows, cols):
     db = torch.full((cols,), 0.5, device="cuda")
     jg.test_colsum(X, db)
     assert _rel(db, X.double().sum(0) + 0.5) < 1e-5
+
+
+@pytest.mark.parametrize("B", [1, 2, 3, 5, 8, 9, 16, 17])
+def test_few_row_products(B):
+    """The t-embedding MLP and the modulation (forward, and their gradients of rank B) at every
+    row count of the streaming kernels and one past it, against the oracle."""
+    from test_gpu_dit import DITB, _check
+    _check(synth.small_variant(DITB, name="rows", hidden=512, heads=8, mlp=512, depth=1, latent_h=4, latent_w=6,
+                               txt_len=3, txt_dim=64), B, 2e-2, 1e-2)
+
+
+@pytest.mark.parametrize("M,N,K", [(64, 4, 1), (65, 260, 4), (1000, 3072, 5), (2304, 768, 16), (130, 1028, 9)])
+def test_rank_update(M, N, K):
+    """An accumulated product of rank at most 16: ragged rows and columns, every register width."""
+    torch.manual_seed(M + N + K)
+    pad = lambda n: (n + 7) // 8 * 8
+    Y = torch.randn(K, pad(M), device="cuda").bfloat16()
+    X = torch.randn(K, pad(N), device="cuda").bfloat16()
+    G0 = torch.randn(M, N + 4, device="cuda")
+    G = G0.clone()
+    jg.test_gemm(_desc(M, N, K, Y, Y.shape[1], 1, X, X.shape[1], 1, jg.DTYPE_BF16, G, N + 4, jg.DTYPE_F32, epi=4))
+    ref = G0[:, :N].double() + Y[:, :M].double().t() @ X[:, :N].double()
+    assert _rel(G[:, :N], ref) < 1e-6 and torch.equal(G[:, N:], G0[:, N:])
