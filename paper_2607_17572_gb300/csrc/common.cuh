@@ -35,6 +35,7 @@ static inline int read_unit_status(unsigned* v, int clear) {
 int unit_status_gemm(unsigned* v, int clear);
 int unit_status_gemm_pair(unsigned* v, int clear);
 int unit_status_signals(unsigned* v, int clear);
+int unit_status_elementwise(unsigned* v, int clear);
 int unit_status_attention_tc(unsigned* v, int clear);
 int unit_status_testing(unsigned* v, int clear);
 

@@ -2,8 +2,11 @@
 // (forward and backward fused with the gated-residual backward), bias reductions,
 // QK RMSNorm + 2D RoPE.
 #include "elementwise.cuh"
+#include "ptx.cuh"
 
 namespace jagg {
+
+int unit_status_elementwise(unsigned* v, int clear) { return read_unit_status(v, clear); }
 
 namespace {
 
@@ -543,96 +546,164 @@ __global__ void __launch_bounds__(256, 2) ln_gate_rowreg_kernel(LnGateBwd a) {
   }
 }
 
-// Row-per-CTA variant for d = 1024 NV4 (d = 3072 at the Flux and Qwen widths; bf16 y and
-// dy, dm in f32 when the LayerNorm part is present).  The 256 threads of a block take one row at a time,
-// each holding NV4 float4 column groups of every operand in registers, so every row is read
-// once and written once.  The row statistics are two block reductions: warp shuffles, then
-// the 8 warp partials through a shared slot double-buffered by row parity (one barrier per
-// row).  Each CTA owns a contiguous, equal share of the rows and each thread the same columns
-// for all of them, so the per-sequence column sums (dshift, dscale, dgate, sum dh for the
-// bias gradient) stay in registers and leave by one global atomic per column and quantity
-// at each sequence boundary.
-template <int NV4, bool LN, bool GATE>
-__global__ void __launch_bounds__(256, 2) ln_gate_rowcta_kernel(LnGateBwd a) {
-  pdl_wait();
-  constexpr int d = 1024 * NV4;
-  __shared__ float red[2][2][8];  // [row parity][s1, s2][warp]
-  __shared__ __align__(16) float sc_s[LN ? d : 4], gt_s[GATE ? d : 4];  // 1 + scale, gate of the sequence
+// The bf16 widths (d = 128 NV WPR): WPR warps share a row, 8 / WPR rows in work per CTA.  Bound by
+// DRAM, so the loads never wait for the arithmetic: each row group has a ring of LNR_STAGES
+// rows (dh, dm, h, y) that bulk copies fill ahead of the row being worked on.  The row
+// statistics are warp shuffles plus, for WPR > 1, one named barrier over the group, after
+// which the stage is free for the next copy.  Each CTA owns a contiguous, equal share of the rows and each
+// lane the same columns for all of them, so the per-sequence column sums (dshift, dscale,
+// dgate, sum dh for the bias gradient) stay in registers; at each sequence boundary the
+// CTA's groups add theirs in shared memory and one 16-byte reduction per 4 columns and quantity
+// leaves.
+// The sums leave as 16-byte reductions: as scalar atomics 16 bytes apart, four per thread
+// and column group, they took half of the kernel (5328 x 768 rows in 24.8 us, now 18.3; 1225 rows
+// 17.1 -> 11.7; Flux-512's streams 42.7 -> 30.1 us on average), and loading ahead changed nothing.
+constexpr int LNR_STAGES = 2;
+
+template <int NV, int WPR, bool LN, bool GATE>
+struct LnRing {
+  static constexpr int D = 128 * NV * WPR, GROUPS = 8 / WPR;
+  static constexpr int ROW = D * (4 + (LN ? 8 : 0) + (GATE ? 2 : 0));  // bytes of a row's operands
+  static constexpr int OFF_DM = 4 * D, OFF_H = 8 * D, OFF_Y = D * (LN ? 12 : 4);
+  static constexpr int OFF_VEC = GROUPS * LNR_STAGES * ROW;            // 1 + scale [D], gate [D]
+  static constexpr int OFF_SUM = OFF_VEC + 8 * D;                      // [4][D] when groups share
+  static constexpr int OFF_RED = OFF_SUM + (GROUPS > 1 ? 16 * D : 0);  // [GROUPS][parity][2][WPR]
+  static constexpr int OFF_BAR = OFF_RED + 8 * 2 * 2 * 4;
+  static constexpr int SMEM = OFF_BAR + GROUPS * LNR_STAGES * 8;
+  static_assert(ROW % 16 == 0 && OFF_BAR % 8 == 0, "bulk copies and barriers are aligned");
+};
+
+template <int NV, int WPR, bool LN, bool GATE>
+__global__ void __launch_bounds__(256, 2) ln_gate_ring_kernel(LnGateBwd a) {
+  using C = LnRing<NV, WPR, LN, GATE>;
+  constexpr int d = C::D, GROUPS = C::GROUPS, S = LNR_STAGES;
+  extern __shared__ __align__(128) uint8_t lnr_sm[];
+  float* sc_s = reinterpret_cast<float*>(lnr_sm + C::OFF_VEC);
+  float* gt_s = sc_s + d;
+  float* sum_s = reinterpret_cast<float*>(lnr_sm + C::OFF_SUM);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = warp / WPR, gw = warp % WPR;
+  uint8_t* ring = lnr_sm + grp * S * C::ROW;
+  float* red = reinterpret_cast<float*>(lnr_sm + C::OFF_RED) + grp * 2 * 2 * WPR;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(lnr_sm + C::OFF_BAR) + grp * S;
+  if (tid == 0) {
+    uint64_t* all = reinterpret_cast<uint64_t*>(lnr_sm + C::OFF_BAR);
+    for (int i = 0; i < GROUPS * S; ++i) ptx::mbar_init(&all[i], 1);
+    ptx::fence_mbar_init();
+  }
+  __syncthreads();
+  pdl_wait();
+  auto group_sync = [&]() {
+    if constexpr (WPR == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(32 * WPR) : "memory");
+  };
+  const bool leader = gw == 0 && lane == 0;
+  const int col0 = (gw * NV * 32 + lane) * 4;  // columns col0 + 128 i .. + 3, i < NV
   const int row_begin = (int)((int64_t)a.M * blockIdx.x / gridDim.x);
   const int row_end = (int)((int64_t)a.M * (blockIdx.x + 1) / gridDim.x);
-  int parity = 0;
+  auto issue = [&](int m, int st) {  // the leader: row m into stage st
+    uint8_t* dst = ring + st * C::ROW;
+    const int64_t hr = seg_row(m, a.seg, a.seg_off, a.seg_stride);
+    ptx::mbar_arrive_expect_tx(&bar[st], C::ROW);
+    ptx::bulk_load(dst, a.dh_in + hr * d, 4 * d, &bar[st]);
+    if (LN) {
+      ptx::bulk_load(dst + C::OFF_DM, static_cast<const float*>(a.dm) + (int64_t)m * d, 4 * d, &bar[st]);
+      ptx::bulk_load(dst + C::OFF_H, a.h + hr * d, 4 * d, &bar[st]);
+    }
+    if (GATE) ptx::bulk_load(dst + C::OFF_Y, static_cast<const bf16*>(a.y) + (int64_t)m * d, 2 * d, &bar[st]);
+  };
+  int j = 0, parity = 0;  // rows this group has taken from its ring
+  bool alive = true;      // false after a wait gave up: no more waiting, the status word is set
   for (int seg0 = row_begin; seg0 < row_end;) {
     const int b = seg0 / a.rows_per_seq;
     const int seg1 = min(row_end, (b + 1) * a.rows_per_seq);
-    float4 acc[4][NV4];
-    __syncthreads();  // the previous segment's readers of the vectors are done
-#pragma unroll
-    for (int i = 0; i < NV4; ++i) {
-      const int c = (i * 256 + tid) * 4;
+    if (leader)
+      for (int i = 0; i < S && seg0 + grp + i * GROUPS < seg1; ++i) issue(seg0 + grp + i * GROUPS, (j + i) % S);
+    for (int c = tid * 4; c < d; c += 1024) {
       if (LN) {
         float4 v = *reinterpret_cast<const float4*>(a.scale + (int64_t)b * a.mod_stride + c);
         v.x += 1.f; v.y += 1.f; v.z += 1.f; v.w += 1.f;
         *reinterpret_cast<float4*>(sc_s + c) = v;
       }
       if (GATE) *reinterpret_cast<float4*>(gt_s + c) = *reinterpret_cast<const float4*>(a.gate + (int64_t)b * a.mod_stride + c);
+    }
+    float4 acc[4][NV];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int i = 0; i < NV; ++i) acc[q][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    float mu_next = 0.f, rs_next = 0.f;
+    if (LN && seg0 + grp < seg1) {
+      mu_next = a.mean[seg0 + grp];
+      rs_next = a.rstd[seg0 + grp];
     }
     __syncthreads();
 #pragma unroll 1
-    for (int m = seg0; m < seg1; ++m) {
-      const int64_t hr = seg_row(m, a.seg, a.seg_off, a.seg_stride);
-      float4 dh[NV4], dm[NV4], hv[NV4];
-      uint2 yb[NV4];  // y in bf16
-#pragma unroll
-      for (int i = 0; i < NV4; ++i) {
-        const int c = (i * 256 + tid) * 4;
-        dh[i] = *reinterpret_cast<const float4*>(a.dh_in + hr * d + c);
-        if (LN) {
-          dm[i] = *reinterpret_cast<const float4*>(static_cast<const float*>(a.dm) + (int64_t)m * d + c);
-          hv[i] = *reinterpret_cast<const float4*>(a.h + hr * d + c);
-        }
-        if (GATE) yb[i] = *reinterpret_cast<const uint2*>(static_cast<const bf16*>(a.y) + (int64_t)m * d + c);
+    for (int m = seg0 + grp; m < seg1; m += GROUPS, ++j) {
+      const int st = j % S;
+      const uint8_t* src = ring + st * C::ROW;
+      const float mu = mu_next, rs = rs_next;
+      if (LN && m + GROUPS < seg1) {
+        mu_next = a.mean[m + GROUPS];
+        rs_next = a.rstd[m + GROUPS];
       }
-      if (LN) {
-        const float mu = a.mean[m], rs = a.rstd[m];
-        float s1 = 0.f, s2 = 0.f;
+      if (alive) alive = ptx::mbar_wait(&bar[st], (j / S) & 1);
+      float4 dh[NV], dm[NV], hv[NV];
+      uint2 yb[NV];
 #pragma unroll
-        for (int i = 0; i < NV4; ++i) {
+      for (int i = 0; i < NV; ++i) {
+        const int c = col0 + i * 128;
+        dh[i] = *reinterpret_cast<const float4*>(src + 4 * c);
+        if (LN) {
+          dm[i] = *reinterpret_cast<const float4*>(src + C::OFF_DM + 4 * c);
+          hv[i] = *reinterpret_cast<const float4*>(src + C::OFF_H + 4 * c);
+        }
+        if (GATE) yb[i] = *reinterpret_cast<const uint2*>(src + C::OFF_Y + 2 * c);
+      }
+      float s1 = 0.f, s2 = 0.f;
+      if (LN) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
           hv[i].x = (hv[i].x - mu) * rs; hv[i].y = (hv[i].y - mu) * rs;  // now x-hat
           hv[i].z = (hv[i].z - mu) * rs; hv[i].w = (hv[i].w - mu) * rs;
-          const float4 sv = *reinterpret_cast<const float4*>(sc_s + (i * 256 + tid) * 4);
+          const float4 sv = *reinterpret_cast<const float4*>(sc_s + col0 + i * 128);
           const float e0 = dm[i].x * sv.x, e1 = dm[i].y * sv.y, e2 = dm[i].z * sv.z, e3 = dm[i].w * sv.w;
           s1 += (e0 + e1) + (e2 + e3);
           s2 += (e0 * hv[i].x + e1 * hv[i].y) + (e2 * hv[i].z + e3 * hv[i].w);
         }
         s1 = warp_sum(s1);
         s2 = warp_sum(s2);
-        if (lane == 0) {
-          red[parity][0][warp] = s1;
-          red[parity][1][warp] = s2;
+        if (WPR > 1 && lane == 0) {
+          red[(parity * 2) * WPR + gw] = s1;
+          red[(parity * 2 + 1) * WPR + gw] = s2;
         }
-        __syncthreads();
-        s1 = 0.f;
-        s2 = 0.f;
+      }
+      ptx::fence_proxy_async_smem();
+      group_sync();  // every lane has read the stage: refill it
+      if (leader && m + S * GROUPS < seg1) issue(m + S * GROUPS, st);
+      if (LN) {
+        if (WPR > 1) {
+          s1 = s2 = 0.f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) {
-          s1 += red[parity][0][w];
-          s2 += red[parity][1][w];
+          for (int w = 0; w < WPR; ++w) {
+            s1 += red[(parity * 2) * WPR + w];
+            s2 += red[(parity * 2 + 1) * WPR + w];
+          }
+          parity ^= 1;
         }
         s1 /= d;
         s2 /= d;
-        parity ^= 1;
+        float* out = a.dh_out + seg_row(m, a.seg, a.seg_off, a.seg_stride) * d + col0;
 #pragma unroll
-        for (int i = 0; i < NV4; ++i) {
-          const int c = (i * 256 + tid) * 4;
-          const float4 sv = *reinterpret_cast<const float4*>(sc_s + c);
+        for (int i = 0; i < NV; ++i) {
+          const float4 sv = *reinterpret_cast<const float4*>(sc_s + col0 + i * 128);
           dh[i].x += rs * (dm[i].x * sv.x - s1 - hv[i].x * s2);
           dh[i].y += rs * (dm[i].y * sv.y - s1 - hv[i].y * s2);
           dh[i].z += rs * (dm[i].z * sv.z - s1 - hv[i].z * s2);
           dh[i].w += rs * (dm[i].w * sv.w - s1 - hv[i].w * s2);
-          *reinterpret_cast<float4*>(a.dh_out + hr * d + c) = dh[i];
+          *reinterpret_cast<float4*>(out + i * 128) = dh[i];
           acc[0][i].x += dm[i].x; acc[0][i].y += dm[i].y; acc[0][i].z += dm[i].z; acc[0][i].w += dm[i].w;
           acc[1][i].x += dm[i].x * hv[i].x; acc[1][i].y += dm[i].y * hv[i].y;
           acc[1][i].z += dm[i].z * hv[i].z; acc[1][i].w += dm[i].w * hv[i].w;
@@ -640,8 +711,8 @@ __global__ void __launch_bounds__(256, 2) ln_gate_rowcta_kernel(LnGateBwd a) {
       }
       if (GATE) {
 #pragma unroll
-        for (int i = 0; i < NV4; ++i) {
-          const int c = (i * 256 + tid) * 4;
+        for (int i = 0; i < NV; ++i) {
+          const int c = col0 + i * 128;
           const float4 g4 = *reinterpret_cast<const float4*>(gt_s + c);
           const float dy[4] = {g4.x * dh[i].x, g4.y * dh[i].y, g4.z * dh[i].z, g4.w * dh[i].w};
           store4(a.dy, (int64_t)m * d + c, 0, dy);
@@ -652,50 +723,83 @@ __global__ void __launch_bounds__(256, 2) ln_gate_rowcta_kernel(LnGateBwd a) {
         }
       }
     }
+    // the segment's column sums: the groups in turn into shared memory, the last one (or the
+    // only one) out to global memory
 #pragma unroll
-    for (int i = 0; i < NV4; ++i) {
-      const int c = (i * 256 + tid) * 4;
-      const float* q0 = &acc[0][i].x;
-      const float* q1 = &acc[1][i].x;
-      const float* q2 = &acc[2][i].x;
-      const float* q3 = &acc[3][i].x;
-      const float* g4 = gt_s + c;
+    for (int gi = 0; gi < GROUPS; ++gi) {
+      if (grp == gi) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (LN) {
-          atomicAdd(a.dshift + (int64_t)b * a.dmod_stride + c + e, q0[e]);
-          atomicAdd(a.dscale + (int64_t)b * a.dmod_stride + c + e, q1[e]);
-        }
-        if (GATE) {
-          atomicAdd(a.dgate + (int64_t)b * a.dmod_stride + c + e, q2[e]);
-          if (a.dbias) atomicAdd(a.dbias + c + e, g4[e] * q3[e]);
+        for (int i = 0; i < NV; ++i) {
+          const int c = col0 + i * 128;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (q < 2 ? !LN : !GATE) continue;
+            float4 v = acc[q][i];
+            if (GROUPS > 1) {
+              float4* at = reinterpret_cast<float4*>(sum_s + q * d + c);
+              if (gi > 0) {
+                const float4 w = *at;
+                v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+              }
+              if (gi < GROUPS - 1) {
+                *at = v;
+                continue;
+              }
+            }
+            if (q == 3 && !a.dbias) continue;
+            float* dst = q == 0   ? a.dshift + (int64_t)b * a.dmod_stride + c
+                         : q == 1 ? a.dscale + (int64_t)b * a.dmod_stride + c
+                         : q == 2 ? a.dgate + (int64_t)b * a.dmod_stride + c
+                                  : a.dbias + c;
+            if (q == 3) {
+              const float4 g4 = *reinterpret_cast<const float4*>(gt_s + c);
+              v.x *= g4.x; v.y *= g4.y; v.z *= g4.z; v.w *= g4.w;
+            }
+            ptx::red_add_v4(dst, v.x, v.y, v.z, v.w);
+          }
         }
       }
+      if (GROUPS > 1) __syncthreads();
     }
+    if (GROUPS == 1) __syncthreads();  // the vectors are rewritten for the next segment
     seg0 = seg1;
   }
+  // after a give-up, copies may still be landing: wait (bounded) for the last of every stage
+  if (!alive && leader)
+    for (int i = 1; i <= S && j - i >= 0; ++i) ptx::mbar_wait(&bar[(j - i) % S], ((j - i) / S) & 1);
 }
 
-template <int NV4, bool LN, bool GATE>
-int launch_ln_gate_rowcta_t(const LnGateBwd& a, cudaStream_t s) {
+template <int NV, int WPR, bool LN, bool GATE>
+int launch_ln_gate_ring_t(const LnGateBwd& a, cudaStream_t s) {
+  using C = LnRing<NV, WPR, LN, GATE>;
+  auto kernel = ln_gate_ring_kernel<NV, WPR, LN, GATE>;
   static int per_sm = 0;
   if (!per_sm) {
-    JAGG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ln_gate_rowcta_kernel<NV4, LN, GATE>, 256, 0));
+    JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    JAGG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, C::SMEM));
     if (per_sm < 1) per_sm = 1;
   }
-  // equal row shares of at least 8 rows per CTA, at most one wave of resident CTAs
+  // equal row shares of at least two rows per group, at most one wave of resident CTAs
   const int cap = per_sm * sm_count();
-  const int want = ceil_div(a.M, 8);
-  JAGG_CUDA_TRY(launch(ln_gate_rowcta_kernel<NV4, LN, GATE>, want < cap ? want : cap, 256, 0, s, a));
+  const int want = ceil_div(a.M, 2 * C::GROUPS);
+  JAGG_CUDA_TRY(launch(kernel, want < cap ? want : cap, 256, C::SMEM, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 
-template <int NV4>
-int launch_ln_gate_rowcta(const LnGateBwd& a, cudaStream_t s) {
-  if (a.do_ln) return a.do_gate ? launch_ln_gate_rowcta_t<NV4, true, true>(a, s)
-                                : launch_ln_gate_rowcta_t<NV4, true, false>(a, s);
-  return launch_ln_gate_rowcta_t<NV4, false, true>(a, s);
+template <int NV, int WPR>
+int launch_ln_gate_ring(const LnGateBwd& a, cudaStream_t s) {
+  if (a.do_ln) return a.do_gate ? launch_ln_gate_ring_t<NV, WPR, true, true>(a, s)
+                                : launch_ln_gate_ring_t<NV, WPR, true, false>(a, s);
+  return launch_ln_gate_ring_t<NV, WPR, false, true>(a, s);
+}
+
+// What the ring kernel takes: bf16 y and dy, dm in f32, 16-byte aligned rows and sums.
+bool ln_gate_ring_serves(const LnGateBwd& a) {
+  auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  if (!al(a.dh_in) || a.dmod_stride % 4) return false;
+  if (a.do_ln && (!a.dm_f32 || !al(a.dm) || !al(a.h) || !al(a.dshift) || !al(a.dscale))) return false;
+  return !a.do_gate || (a.dtype == JAGG_DTYPE_BF16 && al(a.y) && al(a.dgate) && (!a.dbias || al(a.dbias)));
 }
 
 template <int NV, bool GATE, bool YBF>
@@ -1283,17 +1387,16 @@ int launch_ln_gate_bwd(const LnGateBwd& a, cudaStream_t s) {
   if (!a.do_ln && !a.do_gate) return JAGG_OK;
   const int smem = 4 * a.d * (int)sizeof(float);
   const int tok = prof_start(s);
-  int st;
+  int st = JAGG_ERR_UNSUPPORTED;
+  const bool ring = ln_gate_ring_serves(a);
   switch (a.d % 128 == 0 ? a.d / 128 : 0) {
     case 3: st = launch_ln_gate_rowreg<3>(a, smem, s); break;
-    case 4: st = launch_ln_gate_rowreg<4>(a, smem, s); break;
-    case 6: st = launch_ln_gate_rowreg<6>(a, smem, s); break;
-    case 8: st = launch_ln_gate_nv<8>(a, smem, s); break;
+    case 4: st = ring ? launch_ln_gate_ring<2, 2>(a, s) : launch_ln_gate_rowreg<4>(a, smem, s); break;
+    case 6: st = ring ? launch_ln_gate_ring<3, 2>(a, s) : launch_ln_gate_rowreg<6>(a, smem, s); break;
+    case 8: st = ring ? launch_ln_gate_ring<2, 4>(a, s) : launch_ln_gate_nv<8>(a, smem, s); break;
     case 12: st = launch_ln_gate_nv<12>(a, smem, s); break;
-    case 24:
-      st = (!a.do_ln || a.dm_f32) && a.dtype == JAGG_DTYPE_BF16 ? launch_ln_gate_rowcta<3>(a, s)
-                                                                  : launch_ln_gate_nv<24>(a, smem, s);
-      break;
+    case 16: st = ring ? launch_ln_gate_ring<2, 8>(a, s) : launch_ln_gate_nv<0>(a, smem, s); break;
+    case 24: st = ring ? launch_ln_gate_ring<3, 8>(a, s) : launch_ln_gate_nv<24>(a, smem, s); break;
     default: st = launch_ln_gate_nv<0>(a, smem, s); break;
   }
   JAGG_TRY(st);

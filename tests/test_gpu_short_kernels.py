@@ -105,3 +105,41 @@ def test_rank_update(M, N, K):
     jg.test_gemm(_desc(M, N, K, Y, Y.shape[1], 1, X, X.shape[1], 1, jg.DTYPE_BF16, G, N + 4, jg.DTYPE_F32, epi=4))
     ref = G0[:, :N].double() + Y[:, :M].double().t() @ X[:, :N].double()
     assert _rel(G[:, :N], ref) < 1e-6 and torch.equal(G[:, N:], G0[:, N:])
+
+
+@pytest.mark.parametrize("ln,gate", [(1, 1), (1, 0), (0, 1)])
+@pytest.mark.parametrize("d", [512, 768, 1024, 2048, 3072])
+@pytest.mark.parametrize("seqs,rps", [(1, 1), (3, 5), (7, 333), (2, 1024)])
+def test_ln_gate_backward_rings(d, seqs, rps, ln, gate):
+    """Fewer rows than the ring holds, CTAs whose share spans sequences, long shares, against float64
+    formulas.  bf16 y and dy: dy is rounded once (2^-9)."""
+    torch.manual_seed(d + seqs + rps)
+    M = seqs * rps
+    r = lambda *s: torch.randn(*s, device="cuda")
+    dh, h, dm, sc, gt = r(M, d), r(M, d) * 2 + 0.3, r(M, d), r(seqs, d) * 0.3, r(seqs, d)
+    y = r(M, d).bfloat16()
+    mean, var = h.mean(1), h.var(1, unbiased=False)
+    rstd = torch.rsqrt(var + 1e-6)
+    out = torch.full_like(dh, float("nan"))
+    ds, dc, dg, db = (torch.full((n, d), 0.5, device="cuda") for n in (seqs, seqs, seqs, 1))
+    dy = torch.full((M, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    kw = dict(dm=dm, h=h, mean=mean, rstd=rstd, scale=sc, dshift=ds, dscale=dc) if ln else {}
+    if gate:
+        kw.update(y=y, gate=gt, dgate=dg, dy=dy, dbias=db)
+    jg.test_ln_gate_bwd(M, d, rps, dh, out, **kw)
+    torch.cuda.synchronize()
+    assert jg.device_status() == 0
+    seq = torch.arange(M, device="cuda") // rps
+    g = dh.double()
+    if ln:
+        xh = (h.double() - mean.double()[:, None]) * rstd.double()[:, None]
+        e = dm.double() * (1 + sc.double()[seq])
+        g = g + rstd.double()[:, None] * (e - e.mean(1, keepdim=True) - xh * (e * xh).mean(1, keepdim=True))
+        assert _rel(out, g) < 1e-5
+        seqsum = lambda x: 0.5 + torch.zeros(seqs, d, device="cuda", dtype=torch.float64).index_add(0, seq, x)
+        assert _rel(ds, seqsum(dm.double())) < 1e-5 and _rel(dc, seqsum(dm.double() * xh)) < 1e-5
+    if gate:
+        seqsum = lambda x: 0.5 + torch.zeros(seqs, d, device="cuda", dtype=torch.float64).index_add(0, seq, x)
+        assert _rel(dy.float(), gt.double()[seq] * g) < 4e-3
+        assert _rel(dg, seqsum(g * y.double())) < 1e-5
+        assert _rel(db[0], 0.5 + (gt.double()[seq] * g).sum(0)) < 1e-5
