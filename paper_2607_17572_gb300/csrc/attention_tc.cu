@@ -2,7 +2,7 @@
 // shared-memory operands), bf16: the backward (appendix, Eqs. bwd_V .. bwd_QK, with the
 // softmax recomputed from the saved log-sum-exp) for head dims 128 and 64
 // (fa_bwd_tc128_kernel, fa_bwd_tc64_kernel), and the forward, one pass with an online
-// softmax at head dim 128 (fa_fwd_tc128_kernel), two passes at 64 (fa_fwd_tc_kernel<64>).
+// softmax (fa_fwd_tc_kernel).
 // Ragged ends and the MMDiT text / image split: 3D tensor maps [sequence][token][column]
 // per stream buffer make TMA read zeros past the last token and drop dQ rows past it.
 #include <cuda.h>
@@ -551,39 +551,7 @@ __global__ void __launch_bounds__(FB2_THREADS, 1) fa_bwd_tc64_kernel(const __gri
   fa_bwd_v3<64>(maps, p, smem_fb2);
 }
 
-// ================================================================== forward, head dim 64
-// Persistent over (128-query tile, sequence, head) units, two passes over the sequence's
-// 128-key tiles per unit:
-//   pass 1   S = Q K^T (TMEM), the exact row maximum m of the scaled scores;
-//   pass 2   S again, P = exp(scale (S - m)) (f32 row sums l; bf16 P to shared memory),
-//            O += P V (TMEM, never rescaled);
-//   then     O / l -> bf16 output, lse = scale m + ln l.
-// The extra S product (half the forward's tensor work again) buys a softmax with no running
-// rescale of O.  Warp roles: 0 TMA producer (Q once per unit, K in pass 1, K and V in pass 2),
-// 1 MMA issuer, 2-9 softmax and output (two warps per TMEM lane quarter = 32 query rows,
-// 64 key columns each; they exchange row maxima and sums through shared memory).
-constexpr int FF_THREADS = 320;  // 10 warps
-
-template <int D>
-struct FfCfg {
-  static_assert(D == 64, "head dim 128 has fa_fwd_tc128_kernel");
-  static constexpr int BQ = 128, BK = 128;
-  static constexpr int NS = 3;  // K (pass 1) / K, V (pass 2) stages
-  static constexpr int NP = 2;  // P buffers
-  static constexpr int Q_BYTES = BQ * D * 2;
-  static constexpr int KV_BYTES = BK * D * 2;
-  static constexpr int P_BYTES = BQ * BK * 2;
-  static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + Q_BYTES;
-  static constexpr int OFF_V = OFF_K + NS * KV_BYTES;
-  static constexpr int OFF_P = OFF_V + NS * KV_BYTES;
-  static constexpr int OFF_RED = OFF_P + NP * P_BYTES;  // [2: max, sum][2 halves][128 rows] f32
-  static constexpr int OFF_BAR = OFF_RED + 2 * 2 * 128 * 4;
-  static constexpr int SMEM = OFF_BAR + 256 + 1024;
-  static constexpr int T_O = 256;  // TMEM: S buffers at columns 0 and 128, O at 256
-  static_assert(SMEM <= 232448, "shared memory budget");
-};
-
+// ================================================================== forward, head dims 128 and 64
 struct FfMaps {
   CUtensorMap q[2], k[2], v[2];
 };
@@ -596,308 +564,6 @@ struct FfParams {
   float* lse;
 };
 
-__device__ __forceinline__ void named_bar(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-template <int D>
-__global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_constant__ FfMaps maps, FfParams p) {
-  using C = FfCfg<D>;
-  constexpr int BQ = C::BQ, BK = C::BK, NS = C::NS, NP = C::NP;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sQ = sm + C::OFF_Q;
-  uint8_t* sK = sm + C::OFF_K;
-  uint8_t* sV = sm + C::OFF_V;
-  uint8_t* sP = sm + C::OFF_P;
-  float* red = reinterpret_cast<float*>(sm + C::OFF_RED);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + C::OFF_BAR);
-  uint64_t* full = bar;              // [NS] a K (and V) stage landed
-  uint64_t* empty = full + NS;       // [NS] its products are done
-  uint64_t* qfull = empty + NS;      // the unit's Q landed
-  uint64_t* qfree = qfull + 1;       // the unit's last S product is done
-  uint64_t* bar_s = qfree + 1;       // [2] S in TMEM buffer b
-  uint64_t* sfree = bar_s + 2;       // [2] the 8 warps have read it
-  uint64_t* pready = sfree + 2;      // [NP] P written by the 8 warps
-  uint64_t* pfree = pready + NP;     // [NP] the product reading P is done
-  uint64_t* bar_o = pfree + NP;      // the unit's O is complete
-  uint64_t* ofree = bar_o + 1;       // the 8 warps have read O
-  uint64_t* bar_drain = ofree + 1;   // the MMA thread's drain after a give-up
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_drain + 1);
-  __shared__ volatile int abort_flag;
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int N = p.N;
-  const int nk = tok_tiles(N, p.n0, BK);
-  const int nq = tok_tiles(N, p.n0, BQ);
-  const int units = nq * p.B * p.heads;
-  // unit u: query tile u % nq of sequence-head u / nq
-  auto unit_of = [&](int u, TokTile& qt, int& b, int& h) {
-    const int bh = u / nq;
-    qt = tok_tile(u % nq, N, p.n0, BQ);
-    b = bh / p.heads;
-    h = bh % p.heads;
-  };
-
-  if (threadIdx.x == 0) {
-    abort_flag = 0;
-    for (int i = 0; i < NS; ++i) {
-      ptx::mbar_init(&full[i], 1);
-      ptx::mbar_init(&empty[i], 1);
-    }
-    ptx::mbar_init(qfull, 1);
-    ptx::mbar_init(qfree, 1);
-    for (int i = 0; i < 2; ++i) {
-      ptx::mbar_init(&bar_s[i], 1);
-      ptx::mbar_init(&sfree[i], 8);
-    }
-    for (int i = 0; i < NP; ++i) {
-      ptx::mbar_init(&pready[i], 8);
-      ptx::mbar_init(&pfree[i], 1);
-    }
-    ptx::mbar_init(bar_o, 1);
-    ptx::mbar_init(ofree, 8);
-    ptx::mbar_init(bar_drain, 1);
-    ptx::fence_mbar_init();
-    for (int sg = 0; sg < 2; ++sg) {
-      ptx::prefetch_tmap(&maps.q[sg]);
-      ptx::prefetch_tmap(&maps.k[sg]);
-      ptx::prefetch_tmap(&maps.v[sg]);
-    }
-  }
-  if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, 512);
-    ptx::tmem_relinquish();
-  }
-  ptx::tc_fence_before();
-  __syncthreads();
-  ptx::tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  pdl_wait();
-
-  if (warp == 0) {
-    // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      int g = 0, i = 0, iq_last = -1;  // g: K / V tiles issued; iq_last: the last unit whose Q was issued
-      bool ok = true;
-      for (int u = blockIdx.x; u < units && ok && !abort_flag; u += gridDim.x, ++i) {
-        TokTile qt;
-        int b, h;
-        unit_of(u, qt, b, h);
-        if (i > 0 && !ptx::mbar_wait(qfree, (i - 1) & 1)) { ok = false; break; }
-        iq_last = i;
-        ptx::mbar_arrive_expect_tx(qfull, C::Q_BYTES);
-#pragma unroll
-        for (int c = 0; c < D / 64; ++c)
-          ptx::tma_load_3d(sQ + c * BQ * 128, &maps.q[qt.seg], qfull, (int)(p.q_col0 + h * D + c * 64), qt.row, b);
-        for (int pass = 0; pass < 2 && ok; ++pass) {
-          for (int j = 0; j < nk; ++j, ++g) {
-            const int st = g % NS;
-            if (g >= NS && !ptx::mbar_wait(&empty[st], ((g / NS) & 1) ^ 1)) { ok = false; break; }
-            const TokTile kt = tok_tile(j, N, p.n0, BK);
-            const int sg = kt.seg, r = kt.row;
-            ptx::mbar_arrive_expect_tx(&full[st], (pass + 1) * C::KV_BYTES);
-#pragma unroll
-            for (int c = 0; c < D / 64; ++c) {
-              ptx::tma_load_3d(sK + st * C::KV_BYTES + c * BK * 128, &maps.k[sg], &full[st],
-                               (int)(p.k_col0 + h * D + c * 64), r, b);
-              if (pass == 1)
-                ptx::tma_load_3d(sV + st * C::KV_BYTES + c * BK * 128, &maps.v[sg], &full[st],
-                                 (int)(p.v_col0 + h * D + c * 64), r, b);
-            }
-          }
-        }
-      }
-      if (!ok) abort_flag = 1;
-      // after a give-up: wait (bounded) for the copies still landing before exiting
-      if (abort_flag) {
-        if (iq_last >= 0) ptx::mbar_wait(qfull, iq_last & 1);
-        for (int k = 0; k < NS && g - 1 - k >= 0; ++k) ptx::mbar_wait(&full[(g - 1 - k) % NS], ((g - 1 - k) / NS) & 1);
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------------------------------------------------------- MMA issuer
-    if (ptx::elect_one()) {
-      constexpr uint32_t id_s = ptx::idesc_bf16(128, BK, false, false);
-      constexpr uint32_t id_o = ptx::idesc_bf16(128, D, false, true);
-      const uint32_t aQ = ptx::smem_u32(sQ);
-      bool ok = true;
-      int g = 0, sc = 0, pc = 0, i = 0;
-      auto issue_s = [&](int st) {  // S of the stage's key tile into TMEM buffer sc % 2
-        const int sb = sc & 1;
-        if (sc >= 2 && !ptx::mbar_wait(&sfree[sb], ((sc >> 1) & 1) ^ 1)) return false;
-        ptx::tc_fence_after();
-        const uint32_t aK = ptx::smem_u32(sK + st * C::KV_BYTES);
-#pragma unroll
-        for (int k = 0; k < D / 16; ++k)
-          ptx::umma_bf16(tmem + sb * 128, kmajor_desc(aQ, BQ, k), kmajor_desc(aK, BK, k), id_s, k > 0);
-        ptx::umma_commit(&bar_s[sb]);
-        ++sc;
-        return true;
-      };
-      auto issue_pv = [&](int st, bool first) {  // O += P V of the stage's value tile
-        const int pb = pc % NP;
-        if (!ptx::mbar_wait(&pready[pb], (pc / NP) & 1)) return false;
-        ptx::tc_fence_after();
-        const uint32_t aP = ptx::smem_u32(sP + pb * C::P_BYTES);
-        const uint32_t aV = ptx::smem_u32(sV + st * C::KV_BYTES);
-#pragma unroll
-        for (int k = 0; k < BK / 16; ++k)
-          ptx::umma_bf16(tmem + C::T_O, kmajor_desc(aP, BQ, k), mnmajor_desc(aV, BK * 128, k), id_o,
-                         (!first || k > 0) ? 1u : 0u);
-        ptx::umma_commit(&pfree[pb]);
-        ptx::umma_commit(&empty[st]);
-        ++pc;
-        return true;
-      };
-      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++i) {
-        if (!ptx::mbar_wait(qfull, i & 1)) { ok = false; break; }
-        // pass 1
-        for (int j = 0; j < nk && ok; ++j, ++g) {
-          const int st = g % NS;
-          if (!ptx::mbar_wait(&full[st], (g / NS) & 1)) { ok = false; break; }
-          ok = issue_s(st);
-          ptx::umma_commit(&empty[st]);
-        }
-        // pass 2: S of tile j, then P V of tile j - 1
-        int prev_st = -1;
-        for (int j = 0; j < nk && ok; ++j, ++g) {
-          const int st = g % NS;
-          if (!ptx::mbar_wait(&full[st], (g / NS) & 1)) { ok = false; break; }
-          if (!issue_s(st)) { ok = false; break; }
-          if (j == nk - 1) ptx::umma_commit(qfree);
-          if (j > 0) {
-            if (j == 1 && i > 0 && !ptx::mbar_wait(ofree, (i - 1) & 1)) { ok = false; break; }
-            if (!issue_pv(prev_st, j == 1)) { ok = false; break; }
-          }
-          prev_st = st;
-        }
-        if (!ok) break;
-        if (nk == 1 && i > 0 && !ptx::mbar_wait(ofree, (i - 1) & 1)) { ok = false; break; }
-        if (!issue_pv(prev_st, nk == 1)) { ok = false; break; }
-        ptx::umma_commit(bar_o);
-      }
-      if (!ok) abort_flag = 1;
-      if (abort_flag) {  // MMAs of this thread may still run: drain them before TMEM is freed
-        ptx::umma_commit(bar_drain);
-        ptx::mbar_wait(bar_drain, 0);
-      }
-    }
-  } else {
-    // ---------------------------------------------------------------- softmax, output
-    // The two warps of a lane quarter meet at named barriers, so neither leaves the unit
-    // loop early: after a failed (timed-out) wait a warp runs on without waiting.
-    const int quarter = warp & 3, half = (warp - 2) >> 2;
-    const int r = quarter * 32 + lane;  // query row of the tile = TMEM lane
-    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    const float c2 = p.scale * kLog2eTc;
-    float* red_m = red;
-    float* red_l = red + 2 * 128;
-    bool ok = true;
-    auto wait = [&](uint64_t* b, uint32_t phase) {
-      if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait(b, phase));
-      if (!ok) abort_flag = 1;
-    };
-    int sc = 0, pc = 0, i = 0;
-    for (int u = blockIdx.x; u < units; u += gridDim.x, ++i) {
-      TokTile qt;
-      int b, h;
-      unit_of(u, qt, b, h);
-      // pass 1: the row maximum over the valid keys
-      float m = -INFINITY;
-      for (int j = 0; j < nk; ++j, ++sc) {
-        const int sb = sc & 1;
-        wait(&bar_s[sb], (sc >> 1) & 1);
-        ptx::tc_fence_after();
-        uint32_t rs[64];
-        ptx::tmem_ld_32x32b_x32(trow + sb * 128 + half * 64, *reinterpret_cast<uint32_t(*)[32]>(rs));
-        ptx::tmem_ld_32x32b_x32(trow + sb * 128 + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(rs + 32));
-        ptx::tmem_ld_wait();
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0 && ok) ptx::mbar_arrive(&sfree[sb]);
-        const int kv = tok_tile(j, N, p.n0, BK).valid - half * 64;  // valid keys among this warp's 64
-#pragma unroll
-        for (int c = 0; c < 64; ++c)
-          if (c < kv) m = fmaxf(m, __uint_as_float(rs[c]));
-      }
-      red_m[half * 128 + r] = m;
-      named_bar(1 + quarter, 64);
-      m = fmaxf(m, red_m[(1 - half) * 128 + r]);
-      // pass 2: P, its row sums, O += P V
-      float l = 0.f;
-      for (int j = 0; j < nk; ++j, ++sc, ++pc) {
-        const int sb = sc & 1, pb = pc % NP;
-        wait(&bar_s[sb], (sc >> 1) & 1);
-        ptx::tc_fence_after();
-        uint32_t hp[32];
-        const int kv = tok_tile(j, N, p.n0, BK).valid - half * 64;
-#pragma unroll
-        for (int cc = 0; cc < 2; ++cc) {
-          uint32_t rs[32];
-          ptx::tmem_ld_32x32b_x32(trow + sb * 128 + half * 64 + cc * 32, rs);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float p0 = cc * 32 + c < kv ? ptx::ex2_approx((__uint_as_float(rs[c]) - m) * c2) : 0.f;
-            const float p1 = cc * 32 + c + 1 < kv ? ptx::ex2_approx((__uint_as_float(rs[c + 1]) - m) * c2) : 0.f;
-            l += p0 + p1;
-            hp[cc * 16 + c / 2] = pack2_bf16(p0, p1);
-          }
-        }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0 && ok) ptx::mbar_arrive(&sfree[sb]);
-        if (pc >= NP) wait(&pfree[pb], ((pc - NP) / NP) & 1);
-        uint8_t* tile = sP + pb * C::P_BYTES;
-        st_row32_packed(tile, BQ, r, half * 64, hp);
-        st_row32_packed(tile, BQ, r, half * 64 + 32, hp + 16);
-        ptx::fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0 && ok) ptx::mbar_arrive(&pready[pb]);
-      }
-      red_l[half * 128 + r] = l;
-      named_bar(1 + quarter, 64);
-      l += red_l[(1 - half) * 128 + r];
-      // the unit's output: O / l, and the log-sum-exp
-      wait(bar_o, i & 1);
-      ptx::tc_fence_after();
-      const int q = qt.tok + r;
-      const bool q_live = r < qt.valid;
-      const float inv = 1.f / l;
-#pragma unroll
-      for (int cc = 0; cc < D / 64; ++cc) {
-        uint32_t ro[32];
-        ptx::tmem_ld_32x32b_x32(trow + C::T_O + half * (D / 2) + cc * 32, ro);
-        ptx::tmem_ld_wait();
-        if (q_live && ok) {
-          bf16* o = static_cast<bf16*>(p.o.base(q)) + p.o.off(b, q, N, (int64_t)h * D + half * (D / 2) + cc * 32);
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            uint4 w;
-            w.x = pack2_bf16(__uint_as_float(ro[8 * v]) * inv, __uint_as_float(ro[8 * v + 1]) * inv);
-            w.y = pack2_bf16(__uint_as_float(ro[8 * v + 2]) * inv, __uint_as_float(ro[8 * v + 3]) * inv);
-            w.z = pack2_bf16(__uint_as_float(ro[8 * v + 4]) * inv, __uint_as_float(ro[8 * v + 5]) * inv);
-            w.w = pack2_bf16(__uint_as_float(ro[8 * v + 6]) * inv, __uint_as_float(ro[8 * v + 7]) * inv);
-            *reinterpret_cast<uint4*>(o + 8 * v) = w;
-          }
-        }
-      }
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0 && ok) ptx::mbar_arrive(ofree);
-      if (half == 0 && q_live && ok) p.lse[((int64_t)b * p.heads + h) * N + q] = p.scale * m + logf(l);
-    }
-  }
-  ptx::tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, 512);
-  }
-}
-
-// ================================================================== forward, head dim 128
 // One pass over the keys with an online softmax.  Persistent over (pair of 128-query tiles A
 // and B, sequence, head) units; per unit the sequence's 128-key tiles stream through a K ring
 // and a V ring, each K and V tile serving both query tiles.  Tensor memory (512 columns):
@@ -912,19 +578,26 @@ __global__ void __launch_bounds__(FF_THREADS, 1) fa_fwd_tc_kernel(const __grid_c
 // into registers first) and is the A operand of P V, whose key blocks follow that placement.
 // Row maxima take the three-input max, the scale-shift and the row sums the paired f32 forms.
 // At the end O / l leaves in bf16 and lse = scale m + ln l.
-constexpr int FF2_THREADS = 320;  // 10 warps
-
+// Head dim 128 takes pairs of query tiles (NX = 2), which share every K and V tile and overlap in
+// one CTA.  Head dim 64 (DiT-B's few hundred tokens) takes single tiles (NX = 1) in half of the
+// tensor memory and two CTAs per SM: a unit of three key tiles is a chain of latencies, and 8
+// sequences of 333 tokens are 288 such units on 152 SMs.  16 rows
+// 25 -> 17 us, 8 rows 15 -> 10; pairs of tiles, one CTA per SM, took 24 and 17 us, and the earlier kernel with two
+// passes over the keys (the exact maximum first) 25 and 15.
+template <int D_>
 struct Ff2 {
-  static constexpr int D = 128, BQ = 128, BK = 128, NKS = 2, NVS = 3;
-  static constexpr int TILE = 128 * 128 * 2;  // 32 KB: 128 rows x 128 bf16, two 64-column chunks
-  static constexpr int OFF_Q = 0;             // Q_A, Q_B
-  static constexpr int OFF_K = OFF_Q + 2 * TILE;
+  static constexpr int D = D_, NX = D == 128 ? 2 : 1, BQ = 128, BK = 128, NKS = 2, NVS = D == 128 ? 3 : 2;
+  static constexpr int THREADS = 64 + 128 * NX, CTAS = D == 128 ? 1 : 2;  // CTAs per SM
+  static constexpr int TILE = 128 * D * 2;  // 128 rows in 64-column chunks: 32 KB at D = 128, 16 KB at 64
+  static constexpr int OFF_Q = 0;           // Q_A, Q_B
+  static constexpr int OFF_K = OFF_Q + NX * TILE;
   static constexpr int OFF_V = OFF_K + NKS * TILE;
   static constexpr int OFF_BAR = OFF_V + NVS * TILE;
   static constexpr int NBAR = 24;
   static constexpr int SMEM = OFF_BAR + NBAR * 8 + 16 + 1024;  // + alignment of the base to 1024 bytes
-  static_assert(SMEM <= 232448, "shared memory budget");
-  static constexpr uint32_t T_S = 0, T_O = 256;  // S_X at 128 X, O_X at 256 + 128 X
+  static_assert(CTAS * (SMEM + 1024) <= 233472, "shared memory budget");
+  static constexpr uint32_t T_S = 0, T_O = 128 * NX;  // S_X at 128 X, O_X (D columns) at T_O + 128 X
+  static constexpr uint32_t TMEM = 256 * NX;
   // Column (within S_X) of P of keys 16 kb .. 16 kb + 15, two bf16 per column: key blocks 4-7
   // at 64-95, 0-3 at 96-127.
   static __host__ __device__ constexpr uint32_t p_col(int kb) { return 64 + 8 * ((kb + 4) & 7); }
@@ -965,10 +638,10 @@ __device__ __forceinline__ void exp_pack(uint32_t (&r)[n], float2 vc2, float2 vm
   }
 }
 
-__global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __grid_constant__ FfMaps maps,
-                                                                      FfParams p) {
-  using C = Ff2;
-  constexpr int BQ = C::BQ, BK = C::BK, D = C::D, NKS = C::NKS, NVS = C::NVS;
+template <int D>
+__global__ void __launch_bounds__(Ff2<D>::THREADS, Ff2<D>::CTAS) fa_fwd_tc_kernel(const __grid_constant__ FfMaps maps, FfParams p) {
+  using C = Ff2<D>;
+  constexpr int BQ = C::BQ, BK = C::BK, NKS = C::NKS, NVS = C::NVS, NX = C::NX;
   extern __shared__ uint8_t smem_ff2[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_ff2) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = sm + C::OFF_Q;
@@ -993,12 +666,12 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
   const int N = p.N;
   const int nk = tok_tiles(N, p.n0, BK);
   const int nq = tok_tiles(N, p.n0, BQ);
-  const int npair = (nq + 1) / 2;
-  const int units = npair * p.B * p.heads;
-  // unit u: query tiles j0 = 2 (u % npair) and j0 + 1 of sequence-head u / npair
+  const int nu = (nq + NX - 1) / NX;
+  const int units = nu * p.B * p.heads;
+  // unit u: query tiles j0 = NX (u % nu) .. j0 + NX - 1 of sequence-head u / nu
   auto unit_of = [&](int u, int& j0, int& b, int& h) {
-    const int bh = u / npair;
-    j0 = (u % npair) * 2;
+    const int bh = u / nu;
+    j0 = (u % nu) * NX;
     b = bh / p.heads;
     h = bh % p.heads;
   };
@@ -1030,7 +703,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
     }
   }
   if (warp == 1) {
-    ptx::tmem_alloc(tmem_slot, 512);
+    ptx::tmem_alloc(tmem_slot, C::TMEM);
     ptx::tmem_relinquish();
   }
   ptx::tc_fence_before();
@@ -1049,10 +722,10 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
         unit_of(u, j0, b, h);
         if (!ptx::mbar_wait(qfree, (i & 1) ^ 1)) { ok = false; break; }
         iq_last = i;
-        ptx::mbar_arrive_expect_tx(qfull, 2 * C::TILE);
-        for (int x = 0; x < 2; ++x) {
-          // query tile B past the last tile (odd tile count): tile A again, not written
-          const TokTile qx = tok_tile(j0 + x < nq ? j0 + x : j0, N, p.n0, BQ);
+        const int nx = min(NX, nq - j0);  // an odd tile count leaves the last unit without a tile B
+        ptx::mbar_arrive_expect_tx(qfull, nx * C::TILE);
+        for (int x = 0; x < nx; ++x) {
+          const TokTile qx = tok_tile(j0 + x, N, p.n0, BQ);
 #pragma unroll
           for (int c = 0; c < D / 64; ++c)
             ptx::tma_load_3d(sQ + x * C::TILE + c * BQ * 128, &maps.q[qx.seg], qfull,
@@ -1094,6 +767,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
       bool ok = true;
       int gk = 0, gv = 0, i = 0;
       uint32_t pr_phase[2] = {0u, 0u};  // pready[X] phases consumed
+      int done[2] = {0, 0};             // units in which tile X has taken part
       auto issue_s = [&](int x, int ks) {  // S_X = Q_X K^T of K stage ks
         const uint32_t aQ = ptx::smem_u32(sQ + x * C::TILE), aK = ptx::smem_u32(sK + ks * C::TILE);
 #pragma unroll
@@ -1111,23 +785,24 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
       };
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++i) {
         if (!ptx::mbar_wait(qfull, i & 1)) { ok = false; break; }
+        const int nx = min(NX, nq - (u % nu) * NX);
         // key tile 0: S_A, S_B
         if (!ptx::mbar_wait(&kfull[gk % NKS], (gk / NKS) & 1)) { ok = false; break; }
         ptx::tc_fence_after();
-        issue_s(0, gk % NKS);
-        issue_s(1, gk % NKS);
+        for (int x = 0; x < nx; ++x) issue_s(x, gk % NKS);
         ptx::umma_commit(&kempty[gk % NKS]);
         if (nk == 1) ptx::umma_commit(qfree);
         ++gk;
         for (int j = 1; j <= nk && ok; ++j) {
           const int vs = gv % NVS;
-          for (int x = 0; x < 2 && ok; ++x) {
+          for (int x = 0; x < nx && ok; ++x) {
             // P_X of key tile j - 1, then (j < nk) S_X of key tile j over it
             if (!ptx::mbar_wait(&pready[x], pr_phase[x])) { ok = false; break; }
             pr_phase[x] ^= 1u;
             ptx::tc_fence_after();
-            if (j == 1 && i > 0) {  // O_X of the previous unit has been read
-              if (!ptx::mbar_wait(&ofree[x], (i - 1) & 1)) { ok = false; break; }
+            if (j == 1) {  // O_X of tile X's previous unit has been read
+              if (done[x] > 0 && !ptx::mbar_wait(&ofree[x], (done[x] - 1) & 1)) { ok = false; break; }
+              ++done[x];
               ptx::tc_fence_after();
             }
             if (x == 0 && !ptx::mbar_wait(&vfull[vs], (gv / NVS) & 1)) { ok = false; break; }
@@ -1157,7 +832,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
     }
   } else {
     // ---------------------------------------------------------------- softmax, output
-    const int x = (warp - 2) >> 2;       // query tile A (warps 2-5) or B (6-9)
+    const int x = (warp - 2) >> 2;       // query tile A (warps 2-5) or, NX = 2, B (6-9)
     const int quarter = warp & 3;
     const int r = quarter * 32 + lane;   // query row of the tile = TMEM lane
     const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -1170,6 +845,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++i) {
       int j0, b, h;
       unit_of(u, j0, b, h);
+      if (j0 + x >= nq) continue;
       float m = -INFINITY, l = 0.f;
       for (int j = 0; j < nk; ++j) {
         ok = __all_sync(0xffffffffu, ptx::mbar_wait(&bar_s[x], s_phase));
@@ -1215,7 +891,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
           l *= f;
           m = mn;
         }
-        // P = exp(scale (S - m)) (at most 2^8) in bf16 at the columns Ff2::p_col gives: keys 64-127 over the
+        // P = exp(scale (S - m)) (at most 2^8) in bf16 at the columns Ff2<D>::p_col gives: keys 64-127 over the
         // S columns 64-95 (already in registers), keys 0-63 over 96-127, so keys 0-63 can be
         // read again while keys 64-127 are exponentiated
         const float mc = m * c2;
@@ -1254,7 +930,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
       ptx::tc_fence_after();
       const TokTile qt = tok_tile(j0 + x, N, p.n0, BQ);
       const int q = qt.tok + r;
-      const bool q_live = j0 + x < nq && r < qt.valid;
+      const bool q_live = r < qt.valid;
       const float inv = 1.f / l;
 #pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
@@ -1284,7 +960,7 @@ __global__ void __launch_bounds__(FF2_THREADS, 1) fa_fwd_tc128_kernel(const __gr
   __syncthreads();
   if (warp == 1) {
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, 512);
+    ptx::tmem_dealloc(tmem, C::TMEM);
   }
 }
 
@@ -1347,9 +1023,27 @@ int launch_v3(const AttnBwdArgs& a, cudaStream_t s) {
   return JAGG_OK;
 }
 
+}  // namespace
+
+// Whether the tensor-core forward serves the call: bf16, head dim 64 / 128, 16-byte aligned
+// operands and output rows.
+bool attention_fwd_tc_eligible(const AttnArgs& f) {
+  if (f.dtype != JAGG_DTYPE_BF16 || (f.dh != 64 && f.dh != 128) || !f.lse) return false;
+  const int n0 = f.q.n0;
+  const bool single = n0 >= f.N;
+  if (!single && n0 <= 0) return false;
+  const SegRows* views[4] = {&f.q, &f.k, &f.v, &f.o};
+  for (const SegRows* v : views) {
+    if (v->n0 != n0) return false;
+    if (!aligned16(v->p0) || v->ld0 % 8) return false;
+    if (!single && (!aligned16(v->p1) || v->ld1 % 8)) return false;
+  }
+  return f.q_col0 % 8 == 0 && f.k_col0 % 8 == 0 && f.v_col0 % 8 == 0;
+}
+
 template <int D>
-int launch_fwd(const AttnArgs& f, cudaStream_t s) {
-  using C = FfCfg<D>;
+static int launch_fwd(const AttnArgs& f, cudaStream_t s) {
+  using C = Ff2<D>;
   const int n0 = f.q.n0, N = f.N;
   const int n1 = N - n0;
   FfMaps maps;
@@ -1376,69 +1070,15 @@ int launch_fwd(const AttnArgs& f, cudaStream_t s) {
     JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_fwd_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     attr = true;
   }
-  const int units = tok_tiles(N, p.n0, C::BQ) * f.B * f.heads;
-  const int nsm = sm_count();
-  JAGG_CUDA_TRY(launch(fa_fwd_tc_kernel<D>, units < nsm ? units : nsm, FF_THREADS, C::SMEM, s, maps, p));
-  JAGG_LAUNCHED();
-  return JAGG_OK;
-}
-
-}  // namespace
-
-// Whether the tensor-core forward serves the call: bf16, head dim 64 / 128, 16-byte aligned
-// operands and output rows.
-bool attention_fwd_tc_eligible(const AttnArgs& f) {
-  if (f.dtype != JAGG_DTYPE_BF16 || (f.dh != 64 && f.dh != 128) || !f.lse) return false;
-  const int n0 = f.q.n0;
-  const bool single = n0 >= f.N;
-  if (!single && n0 <= 0) return false;
-  const SegRows* views[4] = {&f.q, &f.k, &f.v, &f.o};
-  for (const SegRows* v : views) {
-    if (v->n0 != n0) return false;
-    if (!aligned16(v->p0) || v->ld0 % 8) return false;
-    if (!single && (!aligned16(v->p1) || v->ld1 % 8)) return false;
-  }
-  return f.q_col0 % 8 == 0 && f.k_col0 % 8 == 0 && f.v_col0 % 8 == 0;
-}
-
-// The head-dim-128 forward (fa_fwd_tc128_kernel).
-int launch_fwd128(const AttnArgs& f, cudaStream_t s) {
-  using C = Ff2;
-  const int n0 = f.q.n0, N = f.N;
-  const int n1 = N - n0;
-  FfMaps maps;
-  for (int sg = 0; sg < 2; ++sg) {
-    const int nt = sg == 0 ? n0 : n1;
-    if (nt <= 0) {  // single stream: the second views are unused copies
-      maps.q[1] = maps.q[0];
-      maps.k[1] = maps.k[0];
-      maps.v[1] = maps.v[0];
-      break;
-    }
-    JAGG_TRY(seg_map(&maps.q[sg], sg ? f.q.p1 : f.q.p0, sg ? f.q.ld1 : f.q.ld0, nt, f.B, C::BQ));
-    JAGG_TRY(seg_map(&maps.k[sg], sg ? f.k.p1 : f.k.p0, sg ? f.k.ld1 : f.k.ld0, nt, f.B, C::BK));
-    JAGG_TRY(seg_map(&maps.v[sg], sg ? f.v.p1 : f.v.p0, sg ? f.v.ld1 : f.v.ld0, nt, f.B, C::BK));
-  }
-  FfParams p;
-  p.B = f.B; p.N = N; p.heads = f.heads; p.n0 = n0 > 0 && n0 < N ? n0 : N;
-  p.scale = f.scale;
-  p.q_col0 = f.q_col0; p.k_col0 = f.k_col0; p.v_col0 = f.v_col0;
-  p.o = f.o;
-  p.lse = f.lse;
-  static bool attr = false;
-  if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_fwd_tc128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr = true;
-  }
-  const int units = ceil_div(tok_tiles(N, p.n0, C::BQ), 2) * f.B * f.heads;
-  const int nsm = sm_count();
-  JAGG_CUDA_TRY(launch(fa_fwd_tc128_kernel, units < nsm ? units : nsm, FF2_THREADS, C::SMEM, s, maps, p));
+  const int units = ceil_div(tok_tiles(N, p.n0, C::BQ), C::NX) * f.B * f.heads;
+  const int slots = C::CTAS * sm_count();
+  JAGG_CUDA_TRY(launch(fa_fwd_tc_kernel<D>, units < slots ? units : slots, C::THREADS, C::SMEM, s, maps, p));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 
 int attention_fwd_tc(const AttnArgs& f, cudaStream_t s) {
-  return f.dh == 64 ? launch_fwd<64>(f, s) : launch_fwd128(f, s);
+  return f.dh == 64 ? launch_fwd<64>(f, s) : launch_fwd<128>(f, s);
 }
 
 // Whether the tensor-core backward serves the call: bf16, head dim 64 / 128, 16-byte aligned
