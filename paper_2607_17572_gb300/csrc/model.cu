@@ -720,13 +720,17 @@ struct StreamBwd {
   void* du;     // [Ms, dm] scratch
   float* dx32;  // [Ms, d] scratch
 };
-int mlp_and_proj_bwd(const jagg_model& m, const StreamBwd* st, int n, float* grad, cudaStream_t s) {
+// With one stream the weight gradients run two to a launch (fc2 with fc1 here, the output
+// projection's, returned in *proj_dw, with qkv's in qkv_and_ln1_bwd: their operands stay intact
+// until then): each of them alone fills the machine badly.
+int mlp_and_proj_bwd(const jagg_model& m, const StreamBwd* st, int n, float* grad, GemmArgs* proj_dw,
+                     cudaStream_t s) {
   const int dt = m.cfg.dtype, d = m.d, dmw = m.dm;
   const int64_t Lm = m.T.Lmod;
-  GemmArgs g[2];
+  GemmArgs g[2], fc2[2];
   for (int i = 0; i < n; ++i)
-    g[i] = dw_gemm(m, st[i].Ms, d, dmw, st[i].dy, d, st[i].k->gu, dmw, grad, st[i].bw.fc2_w);
-  JAGG_TRY(gemm_streams(g, n, s));
+    fc2[i] = dw_gemm(m, st[i].Ms, d, dmw, st[i].dy, d, st[i].k->gu, dmw, grad, st[i].bw.fc2_w);
+  if (n == 2) JAGG_TRY(gemm_streams(fc2, n, s));
   for (int i = 0; i < n; ++i) {
     g[i] = dx_gemm(m, st[i].Ms, d, dmw, st[i].dy, d, st[i].bw.fc2_w);
     g[i].epi = EPI_MUL_AUX; g[i].C = st[i].du; g[i].ldc = dmw; g[i].aux = st[i].k->gp; g[i].ld_aux = dmw;
@@ -736,7 +740,7 @@ int mlp_and_proj_bwd(const jagg_model& m, const StreamBwd* st, int n, float* gra
     JAGG_TRY(launch_colsum(st[i].du, dt == JAGG_DTYPE_F32, dt, st[i].Ms, dmw, dmw, grad + st[i].bw.fc1_b, s));
   for (int i = 0; i < n; ++i)
     g[i] = dw_gemm(m, st[i].Ms, dmw, d, st[i].du, dmw, st[i].k->m, d, grad, st[i].bw.fc1_w);
-  JAGG_TRY(gemm_streams(g, n, s));
+  JAGG_TRY(n == 2 ? gemm_streams(g, n, s) : gemm_two(fc2[0], g[0], s));
   for (int i = 0; i < n; ++i) {
     g[i] = dx_gemm(m, st[i].Ms, dmw, d, st[i].du, dmw, st[i].bw.fc1_w);
     g[i].C = st[i].dx32; g[i].ldc = d; g[i].c_dtype = JAGG_DTYPE_F32;
@@ -754,7 +758,10 @@ int mlp_and_proj_bwd(const jagg_model& m, const StreamBwd* st, int n, float* gra
     JAGG_TRY(launch_ln_gate_bwd(a, s));
   }
   for (int i = 0; i < n; ++i) g[i] = dw_gemm(m, st[i].Ms, d, d, st[i].dy, d, st[i].k->o, d, grad, st[i].bw.proj_w);
-  JAGG_TRY(gemm_streams(g, n, s));
+  if (n == 2)
+    JAGG_TRY(gemm_streams(g, n, s));
+  else
+    *proj_dw = g[0];
   for (int i = 0; i < n; ++i) {
     g[i] = dx_gemm(m, st[i].Ms, d, d, st[i].dy, d, st[i].bw.proj_w);
     g[i].C = st[i].dO; g[i].ldc = d;
@@ -778,8 +785,9 @@ struct QkvBwd {
   float* dx32;  // [Ms, d] scratch
   LnGateBwd gate;
 };
+// `out_dw`, with one stream: the weight gradient of the block's output projection.
 int qkv_and_ln1_bwd(const jagg_model& m, const QkvBwd* st, int n, int64_t ld_dqkv, int n_out, float* grad,
-                    cudaStream_t s) {
+                    const GemmArgs* out_dw, cudaStream_t s) {
   const int dt = m.cfg.dtype, d = m.d;
   const int64_t Lm = m.T.Lmod;
   GemmArgs g[2];
@@ -787,7 +795,7 @@ int qkv_and_ln1_bwd(const jagg_model& m, const QkvBwd* st, int n, int64_t ld_dqk
     JAGG_TRY(launch_colsum(st[i].dqkv, dt == JAGG_DTYPE_F32, dt, st[i].Ms, n_out, ld_dqkv, grad + st[i].b_off, s));
     g[i] = dw_gemm(m, st[i].Ms, n_out, d, st[i].dqkv, ld_dqkv, st[i].a_in, d, grad, st[i].w_off);
   }
-  JAGG_TRY(gemm_streams(g, n, s));
+  JAGG_TRY(n == 2 ? gemm_streams(g, n, s) : gemm_two(*out_dw, g[0], s));
   for (int i = 0; i < n; ++i) {
     g[i] = dx_gemm(m, st[i].Ms, n_out, d, st[i].dqkv, ld_dqkv, st[i].w_off);
     g[i].C = st[i].dx32; g[i].ldc = d; g[i].c_dtype = JAGG_DTYPE_F32;
@@ -903,7 +911,8 @@ int vjp_dit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float* g
     const float* mod = S.mod + bw.mod_col;
     float* dmod = w.dmod + bw.mod_col;
     const StreamBwd st{M, N, &k, branch_of(bw), mod, dmod, w.dh, w.dy, w.dO, w.du, w.dx32};
-    JAGG_TRY(mlp_and_proj_bwd(m, &st, 1, grad, s));
+    GemmArgs proj_dw;
+    JAGG_TRY(mlp_and_proj_bwd(m, &st, 1, grad, &proj_dw, s));
     AttnBwdArgs ab;
     ab.f = attn_args(m, B, seg_single(k.qkv, 3 * d, N), seg_single(k.qkv, 3 * d, N), seg_single(k.o, d, N), k.lse);
     ab.f.q_col0 = 0; ab.f.k_col0 = d; ab.f.v_col0 = 2 * d;
@@ -915,7 +924,7 @@ int vjp_dit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float* g
     LnGateBwd prev{};
     if (l > 0) prev = mlp_gate(l - 1);
     const QkvBwd qb{M, N, w.dqkv, k.a, k.h_in, k.st1, bw.qkv_w, bw.qkv_b, mod, dmod, w.dh, w.dx32, prev};
-    JAGG_TRY(qkv_and_ln1_bwd(m, &qb, 1, 3 * d, 3 * d, grad, s));
+    JAGG_TRY(qkv_and_ln1_bwd(m, &qb, 1, 3 * d, 3 * d, grad, &proj_dw, s));
   }
   return JAGG_OK;
 }
@@ -1040,7 +1049,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
     const SingleSaved& k = S.sgl[l];
     const float* mod = S.mod + sw.mod_col;
     float* dmod = w.dmod + sw.mod_col;
-    JAGG_TRY(gemm(dw_gemm(m, M, d, d + dm, w.dy, d, k.cat, d + dm, grad, sw.lin2_w), s));
+    const GemmArgs lin2_dw = dw_gemm(m, M, d, d + dm, w.dy, d, k.cat, d + dm, grad, sw.lin2_w);  // with lin1's
     {  // d(cat) = dy Wlin2: the attention-output columns, then GELU's columns times GELU'
       GemmArgs g = dx_gemm(m, M, d, d, w.dy, d, sw.lin2_w, d + dm);
       g.C = w.dO; g.ldc = d;
@@ -1067,7 +1076,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
     LnGateBwd prev{};
     if (l > 0) prev = single_gate(l - 1);
     const QkvBwd l1{M, N, w.dqkv, k.a, k.h_in, k.st1, sw.lin1_w, sw.lin1_b, mod, dmod, w.dh, w.dx32, prev};
-    JAGG_TRY(qkv_and_ln1_bwd(m, &l1, 1, ld1, (int)ld1, grad, s));
+    JAGG_TRY(qkv_and_ln1_bwd(m, &l1, 1, ld1, (int)ld1, grad, &lin2_dw, s));
   }
   if (Ld == 0) return JAGG_OK;
   // the joint gradient splits into the two streams
@@ -1096,7 +1105,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
       st[si] = {B * Ns, Ns, &k.s[si], branch_of(bw.s[si]), S.mod + mc, w.dmod + mc, w.dhs[si], dy_s[si], dO_s[si],
                 du_s[si], dx32_s[si]};
     }
-    JAGG_TRY(mlp_and_proj_bwd(m, st, 2, grad, s));
+    JAGG_TRY(mlp_and_proj_bwd(m, st, 2, grad, nullptr, s));
     AttnBwdArgs ab;
     ab.f = attn_args(m, B, SegRows{k.s[0].qk, k.s[1].qk, 2 * d, 2 * d, Nt},
                      SegRows{k.s[0].qkv, k.s[1].qkv, 3 * d, 3 * d, Nt}, SegRows{k.s[0].o, k.s[1].o, d, d, Nt}, k.lse);
@@ -1122,7 +1131,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
       qk[si] = {Ms, Ns, dqkv_s[si], q.a, q.h_in, q.st1, sw.qkv_w, sw.qkv_b, S.mod + sw.mod_col, w.dmod + sw.mod_col,
                 w.dhs[si], dx32_s[si], prev};
     }
-    JAGG_TRY(qkv_and_ln1_bwd(m, qk, 2, 3 * d, 3 * d, grad, s));
+    JAGG_TRY(qkv_and_ln1_bwd(m, qk, 2, 3 * d, 3 * d, grad, nullptr, s));
   }
   return JAGG_OK;
 }
