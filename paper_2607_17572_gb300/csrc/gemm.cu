@@ -13,6 +13,7 @@
 #include <cuda.h>
 #include <mutex>
 
+#include "elementwise.cuh"
 #include "gemm.cuh"
 #include "rows.cuh"
 #include "ptx.cuh"
@@ -1018,6 +1019,7 @@ int validate(const GemmArgs& g) {
   JAGG_CHECK_ARG(g.epi != EPI_GELU || g.C2, "gemm: GELU epilogue needs C2");
   JAGG_CHECK_ARG(g.epi != EPI_GATE_RESID || (g.C2 && g.aux && g.gate), "gemm: gate epilogue needs C2/aux/gate");
   JAGG_CHECK_ARG(g.epi != EPI_MUL_AUX || g.aux, "gemm: multiply epilogue needs aux");
+  JAGG_CHECK_ARG(!g.col_sum || g.epi == EPI_MUL_AUX, "gemm: column sums need the multiply epilogue");
   return JAGG_OK;
 }
 
@@ -1203,6 +1205,14 @@ double gemm_best_cost(const GemmArgs& g) {
 
 int gemm(const GemmArgs& g, cudaStream_t stream) {
   JAGG_TRY(validate(g));
+  if (g.col_sum) {  // the pair kernel sums in its epilogue; after the others, a pass over the output
+    double cost;
+    if (gemm_tc_eligible(g) && takes_pair(g, &cost)) return gemm_pair(g, stream);
+    GemmArgs plain = g;
+    plain.col_sum = nullptr;
+    JAGG_TRY(gemm(plain, stream));
+    return launch_colsum(g.C, g.c_dtype == JAGG_DTYPE_F32, g.c_dtype, g.M, g.N, g.ldc, g.col_sum, stream);
+  }
   if (!gemm_tc_eligible(g)) return gemm_simt(g, stream);
   if (rank_update_serves(g)) return rank_update(g, stream);
   double cost;

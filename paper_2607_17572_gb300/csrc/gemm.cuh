@@ -50,6 +50,9 @@ struct GemmArgs {
   // indexed by m instead of n.
   bool c_trans = false;
   bool bias_m = false;
+  // EPI_MUL_AUX: when given, col_sum[n] += sum over m of the C just written (in its storage type):
+  // the bias gradient of the layer before, without a pass of its own where the kernel can.
+  float* col_sum = nullptr;
   int tile_n = 0;  // tensor-core tile width (64 / 128 / 256); 0 = chosen by the cost model
 };
 

@@ -67,6 +67,7 @@ struct PairParams {
   int64_t gate_stride;
   int rows_per_seq;
   int gelu_d;           // PE_GELU: also write GELU'(u)
+  float* col_sum;       // PE_MUL: column sums of the output, added, or null
   bf16* y;              // PE_GATE: the branch output before the gate, row pitch ldy
   int64_t ldy;
 };
@@ -471,6 +472,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
           }
           ptx::bulk_commit();
         }
+        if constexpr (EPI == PE_MUL) {
+          // column sums of the box just written (rows past M are zeros): a lane sums a column pair over
+          // every other row, so a step of the warp reads two whole rows
+          if (p.col_sum) {
+            const int cp = lane & 15, odd = lane >> 4;
+            float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              const int rr = 2 * k + odd;
+              sum = ptx::add2(sum, unpack2(*reinterpret_cast<const uint32_t*>(
+                                       slot + rr * 64 + (((cp >> 2) ^ (k & 3)) << 4) + (cp & 3) * 4)));
+            }
+            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, 16);
+            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, 16);
+            if (!odd && n0 + 2 * cp < p.N) ptx::red_add_v2(p.col_sum + n0 + 2 * cp, sum.x, sum.y);
+          }
+        }
         sb = (sb + (EPI == PE_GELU ? 2 : 1)) % Cfg::BOXES;
       }
       ptx::tc_fence_before();
@@ -516,7 +534,8 @@ int pair_epi(const GemmArgs& g) {
     case EPI_ACCUM:
       return c_f32 ? PE_ACCUM : -1;
     case EPI_MUL_AUX:
-      return !c_f32 && al16(g.aux) && g.ld_aux % 8 == 0 ? PE_MUL : -1;
+      return !c_f32 && al16(g.aux) && g.ld_aux % 8 == 0 && (!g.col_sum || (al16(g.col_sum) && g.N % 2 == 0)) ? PE_MUL
+                                                                                                             : -1;
     case EPI_GELU:
       return !c_f32 && g.C2 && al16(g.C2) && g.ldc2 % 8 == 0 ? PE_GELU : -1;
     case EPI_GATE_RESID:
@@ -556,6 +575,7 @@ int fill_pair(const GemmArgs& g, int bn, int splits, PairMaps& maps, PairParams&
   p.gate_stride = g.gate_stride;
   p.rows_per_seq = g.rows_per_seq > 0 ? g.rows_per_seq : 1;
   p.gelu_d = EPI == PE_GELU && g.C ? 1 : 0;
+  p.col_sum = g.col_sum;
   p.y = static_cast<bf16*>(g.C);
   p.ldy = g.ldc;
   return JAGG_OK;

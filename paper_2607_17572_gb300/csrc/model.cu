@@ -734,10 +734,9 @@ int mlp_and_proj_bwd(const jagg_model& m, const StreamBwd* st, int n, float* gra
   for (int i = 0; i < n; ++i) {
     g[i] = dx_gemm(m, st[i].Ms, d, dmw, st[i].dy, d, st[i].bw.fc2_w);
     g[i].epi = EPI_MUL_AUX; g[i].C = st[i].du; g[i].ldc = dmw; g[i].aux = st[i].k->gp; g[i].ld_aux = dmw;
+    g[i].col_sum = grad + st[i].bw.fc1_b;
   }
   JAGG_TRY(gemm_streams(g, n, s));
-  for (int i = 0; i < n; ++i)
-    JAGG_TRY(launch_colsum(st[i].du, dt == JAGG_DTYPE_F32, dt, st[i].Ms, dmw, dmw, grad + st[i].bw.fc1_b, s));
   for (int i = 0; i < n; ++i)
     g[i] = dw_gemm(m, st[i].Ms, dmw, d, st[i].du, dmw, st[i].k->m, d, grad, st[i].bw.fc1_w);
   JAGG_TRY(n == 2 ? gemm_streams(g, n, s) : gemm_two(fc2[0], g[0], s));
@@ -785,14 +784,15 @@ struct QkvBwd {
   float* dx32;  // [Ms, d] scratch
   LnGateBwd gate;
 };
-// `out_dw`, with one stream: the weight gradient of the block's output projection.
+// `out_dw`, with one stream: the weight gradient of the block's output projection.  Of the n_out
+// columns of dqkv the first 3 d still need their bias gradient.
 int qkv_and_ln1_bwd(const jagg_model& m, const QkvBwd* st, int n, int64_t ld_dqkv, int n_out, float* grad,
                     const GemmArgs* out_dw, cudaStream_t s) {
   const int dt = m.cfg.dtype, d = m.d;
   const int64_t Lm = m.T.Lmod;
   GemmArgs g[2];
   for (int i = 0; i < n; ++i) {
-    JAGG_TRY(launch_colsum(st[i].dqkv, dt == JAGG_DTYPE_F32, dt, st[i].Ms, n_out, ld_dqkv, grad + st[i].b_off, s));
+    JAGG_TRY(launch_colsum(st[i].dqkv, dt == JAGG_DTYPE_F32, dt, st[i].Ms, 3 * d, ld_dqkv, grad + st[i].b_off, s));
     g[i] = dw_gemm(m, st[i].Ms, n_out, d, st[i].dqkv, ld_dqkv, st[i].a_in, d, grad, st[i].w_off);
   }
   JAGG_TRY(n == 2 ? gemm_streams(g, n, s) : gemm_two(*out_dw, g[0], s));
@@ -1056,6 +1056,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
       JAGG_TRY(gemm(g, s));
       g = dx_gemm(m, M, d, dm, w.dy, d, sw.lin2_w + d, d + dm);
       g.epi = EPI_MUL_AUX; g.C = at_byte(w.dqkv, (size_t)3 * d * e); g.ldc = ld1; g.aux = k.gp; g.ld_aux = dm;
+      g.col_sum = grad + sw.lin1_b + 3 * d;
       JAGG_TRY(gemm(g, s));
     }
     AttnBwdArgs ab;
