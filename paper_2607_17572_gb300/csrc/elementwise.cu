@@ -71,8 +71,10 @@ __global__ void temb_kernel(const float* t, float* phi, int B, int dim) {
     // w_k = 10000^(-k/half) evaluated in double so the argument 1000 t w_k is accurate
     const double w = exp(-log(10000.0) * (double)k / (double)half);
     const double a = 1000.0 * (double)t[b] * w;
-    phi[(int64_t)b * dim + k] = (float)cos(a);
-    phi[(int64_t)b * dim + half + k] = (float)sin(a);
+    double sn, cs;
+    sincos(a, &sn, &cs);  // one argument reduction for both
+    phi[(int64_t)b * dim + k] = (float)cs;
+    phi[(int64_t)b * dim + half + k] = (float)sn;
   }
 }
 
@@ -81,10 +83,14 @@ __global__ void silu_kernel(const float* in, float* out, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = silu_f(in[i]);
 }
-__global__ void mul_silu_grad_kernel(float* g, const float* x, int64_t n) {
+// g *= SiLU'(x), and its copy in the storage type (an operand of the next products).
+__global__ void mul_silu_grad_kernel(float* g, const float* x, void* copy, int copy_f32, int64_t n) {
   pdl_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    g[i] *= silu_grad_f(x[i]);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const float v = g[i] * silu_grad_f(x[i]);
+    g[i] = v;
+    stx(copy, i, copy_f32, v);
+  }
 }
 
 // One thread per 4 columns of one image token, added to that token of every sequence: each sine
@@ -802,6 +808,149 @@ bool ln_gate_ring_serves(const LnGateBwd& a) {
   return !a.do_gate || (a.dtype == JAGG_DTYPE_BF16 && al(a.y) && al(a.dgate) && (!a.dbias || al(a.dbias)));
 }
 
+// Narrow rows, d = 4 L NV <= 256 (the f32 configuration): L lanes per row, so a warp works on 32 / L
+// rows at once, every operand loaded once into registers.  Bound by latency: a few hundred
+// rows are one or two rounds of loads.  The column sums of a lane's rows stay in registers, meet
+// in shared memory and leave as 16-byte reductions, one per 4 columns, quantity and CTA.
+// 192 rows of 64 columns: 10.8 us in the general kernel (two passes over the operands, shared-memory and
+// scalar global atomics); a tiny f32 training pass, with seven of them, 350 -> 323 us together with the
+// launches saved around it.
+template <int L, int NV>
+__global__ void __launch_bounds__(256) ln_gate_narrow_kernel(LnGateBwd a, int rows_per_cta, int chunks) {
+  pdl_wait();
+  constexpr int d = 4 * L * NV, TEAMS = 256 / L;
+  __shared__ __align__(16) float part[TEAMS][4 * L * NV];
+  const int team = threadIdx.x / L, lane = threadIdx.x % L;
+  const int is_f32 = a.dtype == JAGG_DTYPE_F32;
+  const int b = blockIdx.x / chunks, r0 = (blockIdx.x % chunks) * rows_per_cta;
+  const int r1 = min(r0 + rows_per_cta, a.rows_per_seq);
+  auto vec = [&](const float* p, int i) {
+    return p ? *reinterpret_cast<const float4*>(p + (int64_t)b * a.mod_stride + (i * L + lane) * 4)
+             : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  float4 sc[NV], gt[NV], acc[4][NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    sc[i] = vec(a.do_ln ? a.scale : nullptr, i);
+    gt[i] = vec(a.do_gate ? a.gate : nullptr, i);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[q][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  auto team_sum = [&](float v) {
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  // every team makes the same number of rounds (the sums are warp-wide)
+  for (int base = r0; base < r1; base += TEAMS) {
+    const bool live = base + team < r1;
+    const int m = b * a.rows_per_seq + (live ? base + team : r0);
+    const int64_t hr = seg_row(m, a.seg, a.seg_off, a.seg_stride) * d, mr = (int64_t)m * d;
+    float dh[NV][4], dm[NV][4], xh[NV][4], y[NV][4];
+    const float mu = a.do_ln ? a.mean[m] : 0.f, rs = a.do_ln ? a.rstd[m] : 0.f;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = (i * L + lane) * 4;
+      load4(a.dh_in, hr + c, 1, dh[i]);
+      if (a.do_ln) {
+        load4(a.dm, mr + c, a.dm_f32, dm[i]);
+        load4(a.h, hr + c, 1, xh[i]);
+      }
+      if (a.do_gate) load4(a.y, mr + c, is_f32, y[i]);
+    }
+    if (a.do_ln) {
+      float s1 = 0.f, s2 = 0.f;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const float sv[4] = {1.f + sc[i].x, 1.f + sc[i].y, 1.f + sc[i].z, 1.f + sc[i].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          xh[i][e] = (xh[i][e] - mu) * rs;
+          s1 += dm[i][e] * sv[e];
+          s2 += dm[i][e] * sv[e] * xh[i][e];
+        }
+      }
+      s1 = team_sum(s1) / d;
+      s2 = team_sum(s2) / d;
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const float sv[4] = {1.f + sc[i].x, 1.f + sc[i].y, 1.f + sc[i].z, 1.f + sc[i].w};
+        float* q0 = &acc[0][i].x;
+        float* q1 = &acc[1][i].x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          dh[i][e] += rs * (dm[i][e] * sv[e] - s1 - xh[i][e] * s2);
+          if (live) {
+            q0[e] += dm[i][e];
+            q1[e] += dm[i][e] * xh[i][e];
+          }
+        }
+        if (live) store4(a.dh_out, hr + (i * L + lane) * 4, 1, dh[i]);
+      }
+    }
+    if (a.do_gate && live) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const float gv[4] = {gt[i].x, gt[i].y, gt[i].z, gt[i].w};
+        float dy[4];
+        float* q2 = &acc[2][i].x;
+        float* q3 = &acc[3][i].x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          dy[e] = gv[e] * dh[i][e];
+          q2[e] += dh[i][e] * y[i][e];
+          q3[e] += dh[i][e];
+        }
+        store4(a.dy, mr + (i * L + lane) * 4, is_f32, dy);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (q < 2 ? !a.do_ln : !a.do_gate) continue;
+    if (q == 3 && !a.dbias) continue;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NV; ++i) *reinterpret_cast<float4*>(&part[team][(i * L + lane) * 4]) = acc[q][i];
+    __syncthreads();
+    if (threadIdx.x < d / 4) {
+      const int c = threadIdx.x * 4;
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < TEAMS; ++w) {
+        const float4 v = *reinterpret_cast<const float4*>(&part[w][c]);
+        t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+      }
+      float* dst = q == 0   ? a.dshift + (int64_t)b * a.dmod_stride + c
+                   : q == 1 ? a.dscale + (int64_t)b * a.dmod_stride + c
+                   : q == 2 ? a.dgate + (int64_t)b * a.dmod_stride + c
+                            : a.dbias + c;
+      if (q == 3) {
+        const float4 g4 = *reinterpret_cast<const float4*>(a.gate + (int64_t)b * a.mod_stride + c);
+        t.x *= g4.x; t.y *= g4.y; t.z *= g4.z; t.w *= g4.w;
+      }
+      ptx::red_add_v4(dst, t.x, t.y, t.z, t.w);
+    }
+  }
+}
+
+template <int L, int NV>
+int launch_ln_gate_narrow(const LnGateBwd& a, cudaStream_t s) {
+  // two rounds of rows per CTA
+  const int rows = 2 * 256 / L, chunks = ceil_div(a.rows_per_seq, rows);
+  JAGG_CUDA_TRY(launch(ln_gate_narrow_kernel<L, NV>, (a.M / a.rows_per_seq) * chunks, 256, 0, s, a, rows, chunks));
+  JAGG_LAUNCHED();
+  return JAGG_OK;
+}
+
+// The narrow kernel's 16-byte accesses: every row, vector and sum aligned.
+bool ln_gate_narrow_serves(const LnGateBwd& a) {
+  auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  if (!al(a.dh_in) || a.mod_stride % 4 || a.dmod_stride % 4) return false;
+  if (a.do_ln && !(al(a.dm) && al(a.h) && al(a.dh_out) && al(a.scale) && al(a.dshift) && al(a.dscale))) return false;
+  return !a.do_gate || (al(a.y) && al(a.dy) && al(a.gate) && al(a.dgate) && (!a.dbias || al(a.dbias)));
+}
+
 template <int NV, bool GATE, bool YBF>
 int launch_ln_gate_rowreg_t(const LnGateBwd& a, cudaStream_t s) {
   const int smem = (8 * 4 + 2) * 128 * NV * (int)sizeof(float);
@@ -1340,8 +1489,8 @@ int launch_silu(const float* in, float* out, int64_t n, cudaStream_t s) {
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
-int launch_mul_silu_grad(float* g, const float* x, int64_t n, cudaStream_t s) {
-  JAGG_CUDA_TRY(launch(mul_silu_grad_kernel, grid_for(n, 256), 256, 0, s, g, x, n));
+int launch_mul_silu_grad(float* g, const float* x, void* copy, int dtype, int64_t n, cudaStream_t s) {
+  JAGG_CUDA_TRY(launch(mul_silu_grad_kernel, grid_for(n, 256), 256, 0, s, g, x, copy, dtype == JAGG_DTYPE_F32, n));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
@@ -1389,7 +1538,10 @@ int launch_ln_gate_bwd(const LnGateBwd& a, cudaStream_t s) {
   const int tok = prof_start(s);
   int st = JAGG_ERR_UNSUPPORTED;
   const bool ring = ln_gate_ring_serves(a);
-  switch (a.d % 128 == 0 ? a.d / 128 : 0) {
+  if ((a.d == 64 || a.d == 128 || a.d == 256) && ln_gate_narrow_serves(a))
+    st = a.d == 64 ? launch_ln_gate_narrow<16, 1>(a, s)
+                   : a.d == 128 ? launch_ln_gate_narrow<32, 1>(a, s) : launch_ln_gate_narrow<32, 2>(a, s);
+  else switch (a.d % 128 == 0 ? a.d / 128 : 0) {
     case 3: st = launch_ln_gate_rowreg<3>(a, smem, s); break;
     case 4: st = ring ? launch_ln_gate_ring<2, 2>(a, s) : launch_ln_gate_rowreg<4>(a, smem, s); break;
     case 6: st = ring ? launch_ln_gate_ring<3, 2>(a, s) : launch_ln_gate_rowreg<6>(a, smem, s); break;

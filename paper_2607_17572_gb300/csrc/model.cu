@@ -574,8 +574,12 @@ int rows_product(const jagg_model& m, int out, int in, int B, const float* x, fl
   const int dt = m.cfg.dtype;
   const RowsFwd f{B, out, in, silu_out ? 1 : 0, x, x_act, W(m, w_off), W(m, b_off), C};
   if (dt == JAGG_DTYPE_BF16 && rows_fwd_serves(f)) return launch_rows_fwd(f, s);
-  if (silu_out) JAGG_TRY(launch_silu(x, silu_out, (int64_t)B * in, s));
-  JAGG_TRY(launch_gather_rows(silu_out ? silu_out : x, in, 0, 0, 0, x_act, dt, B, in, s));
+  if (silu_out && dt == JAGG_DTYPE_F32) {
+    JAGG_TRY(launch_silu(x, static_cast<float*>(x_act), (int64_t)B * in, s));
+  } else {
+    if (silu_out) JAGG_TRY(launch_silu(x, silu_out, (int64_t)B * in, s));
+    JAGG_TRY(launch_gather_rows(silu_out ? silu_out : x, in, 0, 0, 0, x_act, dt, B, in, s));
+  }
   return gemm(rows_gemm(m, out, in, B, x_act, w_off, b_off, C), s);
 }
 
@@ -673,18 +677,20 @@ int epilogue_bwd(const jagg_model& m, int B, const Saved& S, const VjpWs& w, con
   JAGG_TRY(gemm(dw_gemm(m, Mt, d, c.txt_dim, w.dxe, d, S.txt, c.txt_dim, grad, m.T.txt_w), s));
   // stacked modulation: dW += dmod^T silu(c), db += sum_b dmod, d silu(c) = dmod W
   JAGG_TRY(launch_colsum(w.dmod, 1, dt, B, (int)Lm, Lm, grad + m.T.mod_b, s));
-  JAGG_TRY(launch_gather_rows(w.dmod, Lm, 0, 0, 0, w.dmod_b, dt, B, (int)Lm, s));
-  JAGG_TRY(gemm(rows_dw(m, (int)Lm, d, B, w.dmod_b, S.sc_b, grad, m.T.mod_w), s));
-  JAGG_TRY(gemm(rows_dx(m, (int)Lm, d, B, w.dmod_b, m.T.mod_w, w.dsc), s));  // d silu(c)
+  const void* dmod_op = w.dmod;  // the products' operand: in f32 models the accumulator itself
+  if (dt != JAGG_DTYPE_F32) {
+    JAGG_TRY(launch_gather_rows(w.dmod, Lm, 0, 0, 0, w.dmod_b, dt, B, (int)Lm, s));
+    dmod_op = w.dmod_b;
+  }
+  JAGG_TRY(gemm(rows_dw(m, (int)Lm, d, B, dmod_op, S.sc_b, grad, m.T.mod_w), s));
+  JAGG_TRY(gemm(rows_dx(m, (int)Lm, d, B, dmod_op, m.T.mod_w, w.dsc), s));  // d silu(c)
   // t-embedding MLP
-  JAGG_TRY(launch_mul_silu_grad(w.dsc, S.c, (int64_t)B * d, s));  // dc
+  JAGG_TRY(launch_mul_silu_grad(w.dsc, S.c, w.dc_b, dt, (int64_t)B * d, s));  // dc
   JAGG_TRY(launch_colsum(w.dsc, 1, dt, B, d, d, grad + m.T.t_b2, s));
-  JAGG_TRY(launch_gather_rows(w.dsc, d, 0, 0, 0, w.dc_b, dt, B, d, s));
   JAGG_TRY(gemm(rows_dw(m, d, d, B, w.dc_b, S.se1_b, grad, m.T.t_w2), s));
   JAGG_TRY(gemm(rows_dx(m, d, d, B, w.dc_b, m.T.t_w2, w.de1), s));  // d silu(e1)
-  JAGG_TRY(launch_mul_silu_grad(w.de1, S.e1, (int64_t)B * d, s));
+  JAGG_TRY(launch_mul_silu_grad(w.de1, S.e1, w.dc_b, dt, (int64_t)B * d, s));
   JAGG_TRY(launch_colsum(w.de1, 1, dt, B, d, d, grad + m.T.t_b1, s));
-  JAGG_TRY(launch_gather_rows(w.de1, d, 0, 0, 0, w.dc_b, dt, B, d, s));
   JAGG_TRY(gemm(rows_dw(m, d, c.freq_dim, B, w.dc_b, S.phi_b, grad, m.T.t_w1), s));
   return JAGG_OK;
 }

@@ -111,18 +111,31 @@ def test_rank_update(M, N, K):
 @pytest.mark.parametrize("d", [512, 768, 1024, 2048, 3072])
 @pytest.mark.parametrize("seqs,rps", [(1, 1), (3, 5), (7, 333), (2, 1024)])
 def test_ln_gate_backward_rings(d, seqs, rps, ln, gate):
-    """Fewer rows than the ring holds, CTAs whose share spans sequences, long shares, against float64
-    formulas.  bf16 y and dy: dy is rounded once (2^-9)."""
+    """Fewer rows than the ring holds, CTAs whose share spans sequences, long shares."""
+    _check_ln_gate(d, seqs, rps, ln, gate, torch.bfloat16)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("ln,gate", [(1, 1), (1, 0), (0, 1)])
+@pytest.mark.parametrize("d", [64, 128, 256])
+@pytest.mark.parametrize("seqs,rps", [(1, 1), (8, 24), (3, 33), (2, 150)])
+def test_ln_gate_backward_narrow(d, seqs, rps, ln, gate, dtype):
+    """Less than one round of rows, a remainder, several CTAs per sequence."""
+    _check_ln_gate(d, seqs, rps, ln, gate, dtype)
+
+
+def _check_ln_gate(d, seqs, rps, ln, gate, dtype):
+    """Against float64 formulas; in bf16 dy is rounded once (2^-9)."""
     torch.manual_seed(d + seqs + rps)
     M = seqs * rps
     r = lambda *s: torch.randn(*s, device="cuda")
     dh, h, dm, sc, gt = r(M, d), r(M, d) * 2 + 0.3, r(M, d), r(seqs, d) * 0.3, r(seqs, d)
-    y = r(M, d).bfloat16()
+    y = r(M, d).to(dtype)
     mean, var = h.mean(1), h.var(1, unbiased=False)
     rstd = torch.rsqrt(var + 1e-6)
     out = torch.full_like(dh, float("nan"))
     ds, dc, dg, db = (torch.full((n, d), 0.5, device="cuda") for n in (seqs, seqs, seqs, 1))
-    dy = torch.full((M, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    dy = torch.full((M, d), float("nan"), device="cuda", dtype=dtype)
     kw = dict(dm=dm, h=h, mean=mean, rstd=rstd, scale=sc, dshift=ds, dscale=dc) if ln else {}
     if gate:
         kw.update(y=y, gate=gt, dgate=dg, dy=dy, dbias=db)
@@ -140,6 +153,6 @@ def test_ln_gate_backward_rings(d, seqs, rps, ln, gate):
         assert _rel(ds, seqsum(dm.double())) < 1e-5 and _rel(dc, seqsum(dm.double() * xh)) < 1e-5
     if gate:
         seqsum = lambda x: 0.5 + torch.zeros(seqs, d, device="cuda", dtype=torch.float64).index_add(0, seq, x)
-        assert _rel(dy.float(), gt.double()[seq] * g) < 4e-3
+        assert _rel(dy.float(), gt.double()[seq] * g) < (4e-3 if dtype == torch.bfloat16 else 1e-5)
         assert _rel(dg, seqsum(g * y.double())) < 1e-5
         assert _rel(db[0], 0.5 + (gt.double()[seq] * g).sum(0)) < 1e-5
