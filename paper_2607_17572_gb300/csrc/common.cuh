@@ -153,11 +153,13 @@ enum ProfFamily : int {
 // touches global memory, so completion stays transitive along the stream.  Measured against
 // plain launches: a DiT-B window 6.53 -> 5.81 ms (305 launches), 3.82 -> 3.08 ms at 5 short
 // rows, a tiny f32 window 1.06 -> 0.87 ms, no change where kernels run for milliseconds.  An
-// explicit early trigger (griddepcontrol.launch_dependents at the start of a kernel, or when
-// a persistent kernel issues its last loads) was slower in every case (5.86 and 5.86 ms on
-// DiT-B, 308 instead of 296 ms on Flux-1024 with both): the early CTAs share the SMs
-// with the CTAs still working.
+// early trigger (griddepcontrol.launch_dependents at the start of a kernel, or when a persistent
+// kernel issues its last loads) was slower in every case (5.86 and 5.86 ms on DiT-B, 308 instead
+// of 296 ms on Flux-1024 with both): the early CTAs share the SMs with the CTAs still working.
+// Only the CTA-pair products trigger, once nothing but their last stores is left (a DiT-B window
+// 4.41 -> 4.39 ms).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
 inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchAttribute attr{};

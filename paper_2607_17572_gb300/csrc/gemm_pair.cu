@@ -498,6 +498,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
       if (!ok) { abort_flag = 1; break; }
       if (++acc == 2) { acc = 0; acc_phase ^= 1; }
     }
+    pdl_trigger();  // only the stores in flight are left: the next kernel's small CTAs may come
     if (lane == 0) ptx::bulk_wait<0>();
     __syncwarp();
   }
