@@ -67,6 +67,10 @@ int jagg_test_attention_fwd(const void* qkv, int B, int N, int heads, int dh, in
 int64_t jagg_test_attention_scratch_bytes(int B, int N, int heads, int dh);
 int jagg_test_attention_bwd(const void* qkv, const void* o, const float* lse, const void* dO, int B, int N,
                             int heads, int dh, int dtype, void* dqkv, void* scratch, cudaStream_t stream);
+/* The same, and db [3 heads dh] += the column sums of dqkv (the qkv bias gradient). */
+int jagg_test_attention_bwd_bias(const void* qkv, const void* o, const float* lse, const void* dO, int B, int N,
+                                 int heads, int dh, int dtype, void* dqkv, float* db, void* scratch,
+                                 cudaStream_t stream);
 /* The backward over two-stream views, as the MMDiT double blocks use it: the first n0
  * tokens of every sequence live in qkv0 / o0 / dO0 / dqkv0 ([B*n0, 3d], [B*n0, d], ...),
  * the remaining N - n0 in qkv1 / o1 / dO1 / dqkv1 (n0 = N: one buffer, the *1 pointers

@@ -116,6 +116,7 @@ _SIGNATURES = {
     "jagg_test_attention_fwd": (_I, [_P, _I, _I, _I, _I, _I, _P, _P, _P]),
     "jagg_test_attention_scratch_bytes": (_I64, [_I, _I, _I, _I]),
     "jagg_test_attention_bwd": (_I, [_P, _P, _P, _P, _I, _I, _I, _I, _I, _P, _P, _P]),
+    "jagg_test_attention_bwd_bias": (_I, [_P, _P, _P, _P, _I, _I, _I, _I, _I, _P, _P, _P, _P]),
     "jagg_test_attention_fwd_streams": (_I, [_P, _P, _P, _P, _P, _I, _I, _I, _I, _I, _I, _I, _P]),
     "jagg_test_ln_gate_bwd": (_I, [_I, _I, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
                                    _I, _P]),
@@ -435,6 +436,14 @@ def test_attention_bwd(qkv, o, lse, dO, B, N, heads, dh, dqkv, stream=None):
     scratch = alloc_bytes(lib().jagg_test_attention_scratch_bytes(B, N, heads, dh), qkv.device)
     _check(lib().jagg_test_attention_bwd(_ptr(qkv), _ptr(o), _ptr(lse), _ptr(dO), B, N, heads, dh, dt, _ptr(dqkv),
                                          _ptr(scratch), _stream(stream)), "jagg_test_attention_bwd")
+
+
+def test_attention_bwd_bias(qkv, o, lse, dO, B, N, heads, dh, dqkv, db, stream=None):
+    dt = DTYPE_BF16 if qkv.dtype == torch.bfloat16 else DTYPE_F32
+    scratch = alloc_bytes(lib().jagg_test_attention_scratch_bytes(B, N, heads, dh), qkv.device)
+    _check(lib().jagg_test_attention_bwd_bias(_ptr(qkv), _ptr(o), _ptr(lse), _ptr(dO), B, N, heads, dh, dt, _ptr(dqkv),
+                                              _ptr(db), _ptr(scratch), _stream(stream)),
+           "jagg_test_attention_bwd_bias")
 
 
 def test_attention_fwd_streams(qkv, o, lse, B, N, n0, heads, dh, impl=0, stream=None):

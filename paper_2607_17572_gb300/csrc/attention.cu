@@ -656,6 +656,124 @@ __global__ void dq_store_kernel(AttnBwdArgs a) {
   }
 }
 
+// dq_store_kernel and the column sums of [dq | dk | dv] (the qkv bias gradient) in one pass: bound by
+// launches and latency, since at DiT widths both were passes of a few us over data that is in L2
+// (a training pass as one launch less per block: 192 rows of 64 columns in f32 318 -> 313 us, 12 blocks of 1225
+// rows 2362 -> 2346 us, of 5328 rows 4389 -> 4372 us).
+// A block takes 256 columns and rows_per_block rows; a thread 8 columns of every eighth row; the
+// 8 row slices meet in shared memory and a column leaves as one add per block.  dq's columns are
+// rounded and stored on the way, and what is summed is the rounded value, as in a pass over the
+// stored matrix.
+template <bool F32>
+__global__ void __launch_bounds__(256) dq_store_colsum_kernel(AttnBwdArgs a, int rows_per_block) {
+  pdl_wait();
+  __shared__ float part[8][257];
+  const AttnArgs& f = a.f;
+  const int d = f.heads * f.dh, rows = f.B * f.N;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int c0 = (blockIdx.x * 32 + tx) * 8;
+  const int r0 = blockIdx.y * rows_per_block, r1 = min(r0 + rows_per_block, rows);
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  constexpr int U = 4;  // rows in flight per thread
+  if (c0 < d) {
+    for (int r = r0 + ty; r < r1; r += 8 * U) {
+      float4 v[U][2];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float4* src = reinterpret_cast<const float4*>(a.dq_acc + (int64_t)(r + 8 * u) * d + c0);
+        const bool in = r + 8 * u < r1;
+        v[u][0] = in ? src[0] : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[u][1] = in ? src[1] : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t at = (int64_t)(r + 8 * u) * a.dq.ld0 + c0;
+        float* e = reinterpret_cast<float*>(&v[u][0]);
+        if (!F32) {
+          uint4 raw;
+          __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&raw);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            h[i] = __floats2bfloat162_rn(e[2 * i], e[2 * i + 1]);
+            const float2 f2 = __bfloat1622float2(h[i]);
+            e[2 * i] = f2.x;
+            e[2 * i + 1] = f2.y;
+          }
+          if (r + 8 * u < r1) *reinterpret_cast<uint4*>(static_cast<bf16*>(a.dq.p0) + at) = raw;
+        } else if (r + 8 * u < r1) {
+          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(a.dq.p0) + at);
+          dst[0] = v[u][0];
+          dst[1] = v[u][1];
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i] += e[i];
+      }
+    }
+  } else if (c0 < 3 * d) {
+    for (int r = r0 + ty; r < r1; r += 8 * U) {
+      uint4 raw[U][F32 ? 2 : 1];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t at = (int64_t)(r + 8 * u) * a.dq.ld0 + c0;
+        const bool in = r + 8 * u < r1;
+        const uint4* src = reinterpret_cast<const uint4*>(static_cast<const char*>(a.dq.p0) + at * (F32 ? 4 : 2));
+#pragma unroll
+        for (int j = 0; j < (F32 ? 2 : 1); ++j) raw[u][j] = in ? src[j] : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (F32) {
+          const float* e = reinterpret_cast<const float*>(&raw[u][0]);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) acc[i] += e[i];
+        } else {
+          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw[u][0]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 f2 = __bfloat1622float2(h[i]);
+            acc[2 * i] += f2.x;
+            acc[2 * i + 1] += f2.y;
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) part[ty][tx * 8 + i] = acc[i];
+  __syncthreads();
+  const int c = blockIdx.x * 256 + threadIdx.x;
+  if (c < 3 * d) {
+    float t = 0.f;
+#pragma unroll
+    for (int y = 0; y < 8; ++y) t += part[y][threadIdx.x];
+    atomicAdd(a.db + c, t);
+  }
+}
+
+// dq out of its accumulator, and the column sums of [dq | dk | dv] where they are asked for.
+int store_dq(const AttnBwdArgs& a, int64_t chunks, cudaStream_t s) {
+  const AttnArgs& f = a.f;
+  const int rows = f.B * f.N, d = f.heads * f.dh;
+  const int tok = prof_start(s);
+  if (!a.db) {
+    JAGG_CUDA_TRY(launch(dq_store_kernel, (int)((chunks + 255) / 256), 256, 0, s, a));
+    JAGG_LAUNCHED();
+    prof_stop(tok, s, PROF_ATTN_AUX, 0.0, 6.0 * rows * d);
+    return JAGG_OK;
+  }
+  // about six blocks per SM, at most 256 rows each
+  const int cb = ceil_div(3 * d, 256), want = ceil_div((int64_t)6 * sm_count(), cb);
+  int rpb = (ceil_div(rows, want) + 7) / 8 * 8;
+  rpb = rpb > 256 ? 256 : rpb;
+  if (ceil_div(rows, rpb) > 65535) rpb = (ceil_div(rows, 65535) + 7) / 8 * 8;
+  const bool f32 = f.dtype == JAGG_DTYPE_F32;
+  JAGG_CUDA_TRY(launch(f32 ? dq_store_colsum_kernel<true> : dq_store_colsum_kernel<false>,
+                       dim3(cb, ceil_div(rows, rpb)), 256, 0, s, a, rpb));
+  JAGG_LAUNCHED();
+  prof_stop(tok, s, PROF_ATTN_AUX, 0.0, (f32 ? 16.0 : 10.0) * rows * d);
+  return JAGG_OK;
+}
+
 template <int D>
 int fwd_tc(const AttnArgs& a, cudaStream_t s) {
   const int smem = 3 * TILE * (D + 8) * 2;
@@ -771,6 +889,11 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
   JAGG_CHECK_ARG(f.dh % 8 == 0 && f.dh <= 256, "attention: head dim %d unsupported", f.dh);
   const int64_t chunks = (int64_t)f.B * f.N * f.heads * f.dh / 8;
   JAGG_CHECK_ARG(chunks < (1ll << 31), "attention: too many rows");
+  const int d = f.heads * f.dh, per16 = f.dtype == JAGG_DTYPE_F32 ? 4 : 8;
+  JAGG_CHECK_ARG(!a.db || (a.dq.n0 >= f.N && a.dk.p0 == a.dq.p0 && a.dv.p0 == a.dq.p0 && a.dk.ld0 == a.dq.ld0 &&
+                           a.dv.ld0 == a.dq.ld0 && a.dq_col0 == 0 && a.dk_col0 == d && a.dv_col0 == 2 * d &&
+                           a.dq.ld0 % per16 == 0 && (reinterpret_cast<uintptr_t>(a.dq.p0) & 15) == 0),
+                 "attention: column sums need [dq | dk | dv] in one 16-byte aligned buffer");
   int tok = prof_start(s);
   JAGG_CUDA_TRY(launch(rowdot_zero_kernel, (int)((chunks + 255) / 256), 256, 0, s, a));
   JAGG_LAUNCHED();
@@ -800,12 +923,7 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
     if (st == JAGG_ERR_UNSUPPORTED) set_last_error("attention: head dim %d unsupported", f.dh);
     return st;
   }
-  const int64_t total = (int64_t)f.B * f.N * f.heads * f.dh;
-  tok = prof_start(s);
-  JAGG_CUDA_TRY(launch(dq_store_kernel, (int)((chunks + 255) / 256), 256, 0, s, a));
-  JAGG_LAUNCHED();
-  prof_stop(tok, s, PROF_ATTN_AUX, 0.0, 6.0 * total);
-  return JAGG_OK;
+  return store_dq(a, chunks, s);
 }
 
 }  // namespace jagg

@@ -41,6 +41,9 @@ struct AttnBwdArgs {
   SegRows dq, dk, dv;  // outputs (dtype), columns dq_col0 + h * dh etc.
   int64_t dq_col0, dk_col0, dv_col0;
   int impl = 0;  // 0: the library's choice; 1: warp-level MMA kernel; 2: tcgen05 kernel
+  // One stream with [dq | dk | dv] side by side in one buffer from column 0: add the column sums
+  // (the qkv bias gradient, 3 heads dh floats) here, or nullptr.
+  float* db = nullptr;
 };
 
 int attention_fwd(const AttnArgs& a, cudaStream_t s);

@@ -783,7 +783,7 @@ struct QkvBwd {
   const void* a_in;
   const float* h_in;
   const float* st1;
-  int64_t w_off, b_off;
+  int64_t w_off, b_off;  // b_off < 0: the bias gradient is already summed
   const float* mod;
   float* dmod;
   float* dh;
@@ -798,7 +798,8 @@ int qkv_and_ln1_bwd(const jagg_model& m, const QkvBwd* st, int n, int64_t ld_dqk
   const int64_t Lm = m.T.Lmod;
   GemmArgs g[2];
   for (int i = 0; i < n; ++i) {
-    JAGG_TRY(launch_colsum(st[i].dqkv, dt == JAGG_DTYPE_F32, dt, st[i].Ms, 3 * d, ld_dqkv, grad + st[i].b_off, s));
+    if (st[i].b_off >= 0)
+      JAGG_TRY(launch_colsum(st[i].dqkv, dt == JAGG_DTYPE_F32, dt, st[i].Ms, 3 * d, ld_dqkv, grad + st[i].b_off, s));
     g[i] = dw_gemm(m, st[i].Ms, n_out, d, st[i].dqkv, ld_dqkv, st[i].a_in, d, grad, st[i].w_off);
   }
   JAGG_TRY(n == 2 ? gemm_streams(g, n, s) : gemm_two(*out_dw, g[0], s));
@@ -926,10 +927,11 @@ int vjp_dit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float* g
     attention_bwd_scratch(w.attn, B, N, m.heads, &ab.Dv, &ab.dq_acc);
     ab.dq = ab.dk = ab.dv = seg_single(w.dqkv, 3 * d, N);
     ab.dq_col0 = 0; ab.dk_col0 = d; ab.dv_col0 = 2 * d;
+    ab.db = grad + bw.qkv_b;
     JAGG_TRY(attention_bwd(ab, s));
     LnGateBwd prev{};
     if (l > 0) prev = mlp_gate(l - 1);
-    const QkvBwd qb{M, N, w.dqkv, k.a, k.h_in, k.st1, bw.qkv_w, bw.qkv_b, mod, dmod, w.dh, w.dx32, prev};
+    const QkvBwd qb{M, N, w.dqkv, k.a, k.h_in, k.st1, bw.qkv_w, -1, mod, dmod, w.dh, w.dx32, prev};
     JAGG_TRY(qkv_and_ln1_bwd(m, &qb, 1, 3 * d, 3 * d, grad, &proj_dw, s));
   }
   return JAGG_OK;

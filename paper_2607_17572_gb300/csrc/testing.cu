@@ -77,10 +77,8 @@ extern "C" int64_t jagg_test_attention_scratch_bytes(int B, int N, int heads, in
   return attention_bwd_scratch_floats(B, N, heads, dh) * 4;
 }
 
-extern "C" int jagg_test_attention_bwd(const void* qkv, const void* o, const float* lse, const void* dO, int B, int N,
-                                       int heads, int dh, int dtype, void* dqkv, void* scratch,
-                                       cudaStream_t stream) {
-  JAGG_CHECK_ARG(qkv && o && lse && dO && dqkv && scratch, "jagg_test_attention_bwd: null pointer");
+static int test_attention_bwd(const void* qkv, const void* o, const float* lse, const void* dO, int B, int N, int heads,
+                              int dh, int dtype, void* dqkv, float* db, void* scratch, cudaStream_t stream) {
   AttnBwdArgs ab;
   ab.f = make_args(qkv, B, N, heads, dh, dtype, const_cast<void*>(o), const_cast<float*>(lse));
   const int d = heads * dh;
@@ -88,7 +86,22 @@ extern "C" int jagg_test_attention_bwd(const void* qkv, const void* o, const flo
   attention_bwd_scratch(static_cast<float*>(scratch), B, N, heads, &ab.Dv, &ab.dq_acc);
   ab.dq = ab.dk = ab.dv = seg_single(dqkv, 3 * d, N);
   ab.dq_col0 = 0; ab.dk_col0 = d; ab.dv_col0 = 2 * d;
+  ab.db = db;
   return attention_bwd(ab, stream);
+}
+
+extern "C" int jagg_test_attention_bwd(const void* qkv, const void* o, const float* lse, const void* dO, int B, int N,
+                                       int heads, int dh, int dtype, void* dqkv, void* scratch,
+                                       cudaStream_t stream) {
+  JAGG_CHECK_ARG(qkv && o && lse && dO && dqkv && scratch, "jagg_test_attention_bwd: null pointer");
+  return test_attention_bwd(qkv, o, lse, dO, B, N, heads, dh, dtype, dqkv, nullptr, scratch, stream);
+}
+
+extern "C" int jagg_test_attention_bwd_bias(const void* qkv, const void* o, const float* lse, const void* dO, int B,
+                                            int N, int heads, int dh, int dtype, void* dqkv, float* db, void* scratch,
+                                            cudaStream_t stream) {
+  JAGG_CHECK_ARG(qkv && o && lse && dO && dqkv && db && scratch, "jagg_test_attention_bwd_bias: null pointer");
+  return test_attention_bwd(qkv, o, lse, dO, B, N, heads, dh, dtype, dqkv, db, scratch, stream);
 }
 
 extern "C" int jagg_test_attention_fwd_streams(const void* qkv0, const void* qkv1, void* o0, void* o1, float* lse,

@@ -156,3 +156,25 @@ def _check_ln_gate(d, seqs, rps, ln, gate, dtype):
         assert _rel(dy.float(), gt.double()[seq] * g) < (4e-3 if dtype == torch.bfloat16 else 1e-5)
         assert _rel(dg, seqsum(g * y.double())) < 1e-5
         assert _rel(db[0], 0.5 + (gt.double()[seq] * g).sum(0)) < 1e-5
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B,N,H,dh", [(1, 1, 1, 64), (1, 7, 5, 128), (2, 33, 3, 64), (1, 130, 4, 64), (3, 333, 2, 64)])
+def test_attention_backward_with_bias_sums(B, N, H, dh, dtype):
+    """The bias gradient summed where dQ leaves its accumulator: one row, ragged row blocks and
+    column blocks.  A column's sum takes at most rows + 8 additions of f32 (2^-24 each, relative
+    to the sum of magnitudes), on top of what is there."""
+    torch.manual_seed(N + H)
+    d = H * dh
+    qkv = (torch.randn(B * N, 3 * d, device="cuda") * 1.5).to(dtype)
+    dO = torch.randn(B * N, d, device="cuda").to(dtype)
+    o, lse = torch.empty_like(dO), torch.empty(B, H, N, device="cuda")
+    jg.test_attention_fwd(qkv, B, N, H, dh, o, lse)
+    plain, got = torch.full_like(qkv, float("nan")), torch.full_like(qkv, float("nan"))
+    db = torch.ones(3 * d, device="cuda")
+    jg.test_attention_bwd(qkv, o, lse, dO, B, N, H, dh, plain)
+    jg.test_attention_bwd_bias(qkv, o, lse, dO, B, N, H, dh, got, db)
+    # the key tiles' parts of dQ meet in any order; rounded to the type
+    assert _rel(got, plain) < (1e-5 if dtype == torch.float32 else 2e-3)
+    bound = (B * N + 8) * 2.0 ** -24 * (got.double().abs().sum(0) + 1)
+    assert ((db.double() - 1 - got.double().sum(0)).abs() <= bound).all()
