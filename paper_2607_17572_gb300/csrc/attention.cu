@@ -894,6 +894,7 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
                            a.dv.ld0 == a.dq.ld0 && a.dq_col0 == 0 && a.dk_col0 == d && a.dv_col0 == 2 * d &&
                            a.dq.ld0 % per16 == 0 && (reinterpret_cast<uintptr_t>(a.dq.p0) & 15) == 0),
                  "attention: column sums need [dq | dk | dv] in one 16-byte aligned buffer");
+  JAGG_CHECK_ARG(!a.db || !a.keep_dq32, "attention: no column sums of a dq that is not stored");
   int tok = prof_start(s);
   JAGG_CUDA_TRY(launch(rowdot_zero_kernel, (int)((chunks + 255) / 256), 256, 0, s, a));
   JAGG_LAUNCHED();
@@ -923,7 +924,7 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
     if (st == JAGG_ERR_UNSUPPORTED) set_last_error("attention: head dim %d unsupported", f.dh);
     return st;
   }
-  return store_dq(a, chunks, s);
+  return a.keep_dq32 ? JAGG_OK : store_dq(a, chunks, s);
 }
 
 }  // namespace jagg

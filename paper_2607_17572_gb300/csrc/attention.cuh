@@ -44,6 +44,7 @@ struct AttnBwdArgs {
   // One stream with [dq | dk | dv] side by side in one buffer from column 0: add the column sums
   // (the qkv bias gradient, 3 heads dh floats) here, or nullptr.
   float* db = nullptr;
+  bool keep_dq32 = false;  // leave dq in dq_acc for a caller that reads it there; the dq view is not written
 };
 
 int attention_fwd(const AttnArgs& a, cudaStream_t s);

@@ -1092,28 +1092,6 @@ __global__ void copy_rows_v16_kernel(const uint8_t* in, int64_t ld_in_b, int is,
   }
 }
 
-__global__ void attn_rowdot_kernel(const void* dO, const void* O, int64_t ld, float* Dv, int B, int N, int heads,
-                                   int dh, int is_f32) {
-  pdl_wait();
-  // one warp per (row, head)
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
-  const int lane = threadIdx.x & 31;
-  const int64_t total = (int64_t)B * N * heads;
-  if (w >= total) return;
-  const int hd = (int)(w % heads);
-  const int64_t row = w / heads;  // b * N + n
-  float s = 0.f;
-  for (int c = lane; c < dh; c += 32) {
-    const int64_t i = row * ld + (int64_t)hd * dh + c;
-    s += ldx(dO, i, is_f32) * ldx(O, i, is_f32);
-  }
-  s = warp_sum(s);
-  if (lane == 0) {
-    const int64_t b = row / N, n = row % N;
-    Dv[(b * heads + hd) * N + n] = s;
-  }
-}
-
 // ------------------------------------------------------------------ QK RMSNorm + RoPE
 // One warp per (row, head) handles q and k; dh <= 128 -> up to 4 elements per lane as
 // two rotated pairs.
@@ -1201,6 +1179,7 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_bwd_kernel(QkNormRop
     const int m = (int)(w / a.heads);
     const int n = m % a.N;
     const bool txt = n < a.n_txt;
+    const float* q32 = b.dq32 ? b.dq32 + ((int64_t)(m / a.N) * b.dq32_seq + b.dq32_row0 + n) * a.d + hd * dh : nullptr;
 #pragma unroll
     for (int which = 0; which < 2; ++which) {
       const void* scl = which == 0 ? (txt ? a.qscale_txt : a.qscale_img) : (txt ? a.kscale_txt : a.kscale_img);
@@ -1214,7 +1193,9 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_bwd_kernel(QkNormRop
         const int pair = lane + 32 * j;
         if (2 * pair < dh) {
           // undo the rotation of the incoming gradient (rotate by -angle)
-          const float g0 = ldx(b.dqk, gb + 2 * pair, is_f32), g1 = ldx(b.dqk, gb + 2 * pair + 1, is_f32);
+          const bool wide = which == 0 && q32;
+          const float g0 = wide ? q32[2 * pair] : ldx(b.dqk, gb + 2 * pair, is_f32);
+          const float g1 = wide ? q32[2 * pair + 1] : ldx(b.dqk, gb + 2 * pair + 1, is_f32);
           float cs = 1.f, sn = 0.f;
           if (a.rope) rope_angle(n, a.n_txt, a.gw, dh, pair, cs, sn);
           const float dy0 = g0 * cs + g1 * sn;
@@ -1270,8 +1251,12 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_bwd_kernel(QkNormRop
 // [4l, 4l + 4) of q and of k, i.e. the rotated pairs 2l and 2l + 1, so every operand moves
 // in 8-byte vectors and each lane's RMSNorm scales and RoPE frequencies are fixed for the
 // whole kernel.  The angles are the ones rope_angle forms (same expressions), so the forward
-// rotation and its inverse in the backward agree bit for bit.  A warp walks rows, each row's
-// heads two (backward) or four (forward) at a time: 2 KB of loads in flight per warp.
+// rotation and its inverse in the backward agree bit for bit.  A warp walks units, rows or parts
+// of their heads, two (backward) or four (forward) heads at a time: 2 KB of loads in flight per
+// warp.  Bound by HBM on many rows, by latency on a few thousand: with whole rows only, 4096
+// rows of 24 heads were 1.1 rounds of the resident warps (text + image of 6144 rows at d = 3072:
+// backward 72 -> 65 us with dq read from attention's f32 accumulator, a pass over it less;
+// forward 49 -> 45; 2973 rows 49 -> 41 and 33 -> 28).
 constexpr int QKV_ITEMS = 2;      // heads per warp iteration of the backward
 constexpr int QKV_ITEMS_FWD = 4;  // and of the forward (fewer live registers)
 
@@ -1320,10 +1305,10 @@ __device__ __forceinline__ void rope_lane(const QkNormRope& a, const float2* tab
   cs[0] = v.x; sn[0] = v.y; cs[1] = v.z; sn[1] = v.w;
 }
 
-__global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_v_kernel(QkNormRope a) {
-  pdl_wait();
+__global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_v_kernel(QkNormRope a, int heads_per_unit) {
   extern __shared__ __align__(16) float2 rope_tab[];  // [side][32] when a.rope
   if (a.rope) rope_table_fill(a, rope_tab);
+  pdl_wait();
   __syncthreads();
   const int lane = threadIdx.x & 31;
   float scl[4][4];  // q txt, q img, k txt, k img: this lane's 4 elements
@@ -1331,26 +1316,29 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_v_kernel(QkNormR
   bf16x4_load(static_cast<const bf16*>(a.qscale_img) + 4 * lane, scl[1]);
   bf16x4_load(static_cast<const bf16*>(a.kscale_txt) + 4 * lane, scl[2]);
   bf16x4_load(static_cast<const bf16*>(a.kscale_img) + 4 * lane, scl[3]);
-  // one row per warp, its heads two at a time: the token's stream and angles once per row
-  for (int m = blockIdx.x * QKN_WARPS + threadIdx.x / 32; m < a.M; m += gridDim.x * QKN_WARPS) {
+  // one unit per warp, its heads four at a time: the token's stream and angles once per unit
+  const int upr = (a.heads + heads_per_unit - 1) / heads_per_unit;
+  for (int unit = blockIdx.x * QKN_WARPS + threadIdx.x / 32; unit < a.M * upr; unit += gridDim.x * QKN_WARPS) {
+    const int m = unit / upr, h_lo = (unit - m * upr) * heads_per_unit;
+    const int h_hi = min(h_lo + heads_per_unit, a.heads);
     const int n = m % a.N;
     const bool txt = n < a.n_txt;
     float cs[2], sn[2];
     rope_lane(a, rope_tab, n, lane, cs, sn);
     const bf16* row = static_cast<const bf16*>(a.qkv) + (int64_t)m * a.ld_qkv + 4 * lane;
     bf16* out = static_cast<bf16*>(a.qk_out) + (int64_t)m * 2 * a.d + 4 * lane;
-    for (int h0 = 0; h0 < a.heads; h0 += QKV_ITEMS_FWD) {
+    for (int h0 = h_lo; h0 < h_hi; h0 += QKV_ITEMS_FWD) {
       float x[QKV_ITEMS_FWD][2][4];
 #pragma unroll
       for (int it = 0; it < QKV_ITEMS_FWD; ++it) {
-        const int hd = h0 + it < a.heads ? h0 + it : h0;
+        const int hd = h0 + it < h_hi ? h0 + it : h0;
 #pragma unroll
         for (int which = 0; which < 2; ++which) bf16x4_load(row + which * a.d + hd * 128, x[it][which]);
       }
 #pragma unroll
       for (int it = 0; it < QKV_ITEMS_FWD; ++it) {
         const int hd = h0 + it;
-        if (hd >= a.heads) break;
+        if (hd >= h_hi) break;
 #pragma unroll
         for (int which = 0; which < 2; ++which) {
           float sc[4];  // selected per element: the array index stays a compile-time constant
@@ -1374,54 +1362,67 @@ __global__ void __launch_bounds__(QKN_THREADS) qk_norm_rope_fwd_v_kernel(QkNormR
   }
 }
 
-__global__ void __launch_bounds__(QKN_THREADS, 3) qk_norm_rope_bwd_v_kernel(QkNormRopeBwd b) {
-  pdl_wait();
+template <bool DQ32>
+__global__ void __launch_bounds__(QKN_THREADS, 3) qk_norm_rope_bwd_v_kernel(QkNormRopeBwd b, int heads_per_unit) {
   const QkNormRope& a = b.f;
   __shared__ float part[QKN_WARPS][4][128];
   extern __shared__ __align__(16) float2 rope_tab[];  // [side][32] when a.rope
   if (a.rope) rope_table_fill(a, rope_tab);
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
   __shared__ __align__(16) float scl[4][128];  // q txt, q img, k txt, k img
   for (int t = threadIdx.x; t < 4 * 128; t += QKN_THREADS) {
     const void* p = t < 128 ? a.qscale_txt : t < 256 ? a.qscale_img : t < 384 ? a.kscale_txt : a.kscale_img;
     scl[t / 128][t % 128] = __bfloat162float(static_cast<const bf16*>(p)[t % 128]);
   }
-  // scale gradients of the warp's rows, [which * 2 + stream][element]: one read-modify-write
-  // of the lane's 4 elements per row
+  // scale gradients of the warp's units, [which * 2 + stream][element]: one read-modify-write
+  // of the lane's 4 elements per unit
   float4* wpart = reinterpret_cast<float4*>(&part[warp][0][0]);
 #pragma unroll
   for (int i = 0; i < 4; ++i) wpart[i * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
-  // one row per warp, its heads two at a time: the token's stream and angles once per row
-  for (int m = blockIdx.x * QKN_WARPS + warp; m < a.M; m += gridDim.x * QKN_WARPS) {
+  // one unit per warp, its heads two at a time: the token's stream and angles once per unit
+  const int upr = (a.heads + heads_per_unit - 1) / heads_per_unit;
+  for (int unit = blockIdx.x * QKN_WARPS + warp; unit < a.M * upr; unit += gridDim.x * QKN_WARPS) {
+    const int m = unit / upr, h_lo = (unit - m * upr) * heads_per_unit;
+    const int h_hi = min(h_lo + heads_per_unit, a.heads);
     const int n = m % a.N;
     const bool txt = n < a.n_txt;
     float cs[2], sn[2];
     rope_lane(a, rope_tab, n, lane, cs, sn);
     const bf16* xrow = static_cast<const bf16*>(a.qkv) + (int64_t)m * a.ld_qkv + 4 * lane;
     bf16* grow = static_cast<bf16*>(b.dqk) + (int64_t)m * b.ld_dqk + 4 * lane;
-    float rowacc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};  // q, k scale gradients of the row
-    for (int h0 = 0; h0 < a.heads; h0 += QKV_ITEMS) {
-      float x[QKV_ITEMS][2][4], g[QKV_ITEMS][2][4];
+    const float* q32 = nullptr;
+    if (DQ32) q32 = b.dq32 + ((int64_t)(m / a.N) * b.dq32_seq + b.dq32_row0 + n) * a.d + 4 * lane;
+    float rowacc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};  // q, k scale gradients of the unit
+    for (int h0 = h_lo; h0 < h_hi; h0 += QKV_ITEMS) {
+      float x[QKV_ITEMS][2][4], g[QKV_ITEMS][2][4], rms[QKV_ITEMS][2];
 #pragma unroll
       for (int it = 0; it < QKV_ITEMS; ++it) {
-        const int hd = h0 + it < a.heads ? h0 + it : h0;
+        const int hd = h0 + it < h_hi ? h0 + it : h0;
 #pragma unroll
         for (int which = 0; which < 2; ++which) {
           bf16x4_load(xrow + which * a.d + hd * 128, x[it][which]);
-          bf16x4_load(grow + which * a.d + hd * 128, g[it][which]);
+          if (DQ32 && which == 0) {
+            const float4 q = *reinterpret_cast<const float4*>(q32 + hd * 128);
+            g[it][0][0] = q.x; g[it][0][1] = q.y; g[it][0][2] = q.z; g[it][0][3] = q.w;
+          } else {
+            bf16x4_load(grow + which * a.d + hd * 128, g[it][which]);
+          }
+          // with the rows: behind the first store to dqk it would be a load of its own per head
+          rms[it][which] = (which == 0 ? a.rq : a.rk)[(int64_t)m * a.heads + hd];
         }
       }
 #pragma unroll
       for (int it = 0; it < QKV_ITEMS; ++it) {
         const int hd = h0 + it;
-        if (hd >= a.heads) break;
+        if (hd >= h_hi) break;
 #pragma unroll
         for (int which = 0; which < 2; ++which) {
           const float4 sc4 = *reinterpret_cast<const float4*>(&scl[which * 2 + (txt ? 0 : 1)][4 * lane]);
           const float sc[4] = {sc4.x, sc4.y, sc4.z, sc4.w};
           const float* xv = x[it][which];
-          const float r = (which == 0 ? a.rq : a.rk)[(int64_t)m * a.heads + hd];
+          const float r = rms[it][which];
           float u[4], dy[4];
 #pragma unroll
           for (int e = 0; e < 2; ++e) {  // undo the rotation of the incoming gradient
@@ -1622,14 +1623,6 @@ int launch_copy_rows(const void* in, int64_t ld_in, int in_seg, int in_seg_off, 
   prof_stop(tok, s, PROF_COPY, 0.0, 2.0 * rows * cols * elem_bytes);
   return JAGG_OK;
 }
-int launch_attn_rowdot(const void* dO, const void* O, int64_t ld, float* Dv, int B, int N, int heads, int dh,
-                       int dtype, cudaStream_t s) {
-  const int64_t warps = (int64_t)B * N * heads;
-  JAGG_CUDA_TRY(launch(attn_rowdot_kernel, grid_for(warps * 32, 256), 256, 0, s, dO, O, ld, Dv, B, N, heads, dh,
-                                                              dtype == JAGG_DTYPE_F32));
-  JAGG_LAUNCHED();
-  return JAGG_OK;
-}
 // The vectorised kernels serve head dim 128 in bf16 with 8-byte aligned rows and scales.
 static bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7) == 0; }
 static int qkn_table_bytes(const QkNormRope& a) {
@@ -1642,8 +1635,26 @@ static bool qkn_vector(const QkNormRope& a) {
                  a.gw > QKN_TABLE_MAX))
     return false;
   return a.dtype == JAGG_DTYPE_BF16 && a.heads > 0 && a.d == 128 * a.heads && a.ld_qkv % 4 == 0 &&
+         (int64_t)a.M * a.heads < (1ll << 30) &&
          aligned8(a.qkv) && aligned8(a.qk_out) && aligned8(a.qscale_txt) && aligned8(a.qscale_img) &&
          aligned8(a.kscale_txt) && aligned8(a.kscale_img);
+}
+// Heads per unit of the vectorised kernels (a multiple of `items`): whole rows where there are many,
+// parts of a row where whole rows would leave the last round of the resident warps nearly empty.
+// A unit costs its batches of heads plus about half a batch (stream, angles, scale sums).
+static int qkn_heads_per_unit(const QkNormRope& a, int items, int warps) {
+  int best = a.heads;
+  double best_cost = 0.0;
+  for (int parts = 1; parts <= ceil_div(a.heads, items); ++parts) {
+    const int hu = ceil_div(ceil_div(a.heads, parts), items) * items;
+    const int64_t units = (int64_t)a.M * ceil_div(a.heads, hu);
+    const double cost = (double)ceil_div(units, (int64_t)warps) * (hu / items + 0.5);
+    if (parts == 1 || cost < 0.97 * best_cost) {
+      best_cost = cost;
+      best = hu;
+    }
+  }
+  return best;
 }
 int launch_qk_norm_rope_fwd(const QkNormRope& a, cudaStream_t s) {
   JAGG_CHECK_ARG(a.heads > 0 && a.d % a.heads == 0 && a.d / a.heads <= 128 && (a.d / a.heads) % 2 == 0,
@@ -1652,10 +1663,11 @@ int launch_qk_norm_rope_fwd(const QkNormRope& a, cudaStream_t s) {
   const int64_t blocks = ((int64_t)a.M * a.heads + QKN_WARPS - 1) / QKN_WARPS;
   const int tok = prof_start(s);
   if (qkn_vector(a)) {
-    const int64_t vb = ceil_div((int64_t)a.M, (int64_t)QKN_WARPS);
     const int cap = 3 * sm_count();  // the resident blocks (77 registers, 3 per SM)
+    const int hu = qkn_heads_per_unit(a, QKV_ITEMS_FWD, cap * QKN_WARPS);
+    const int64_t vb = ceil_div((int64_t)a.M * ceil_div(a.heads, hu), (int64_t)QKN_WARPS);
     JAGG_CUDA_TRY(launch(qk_norm_rope_fwd_v_kernel, (int)(vb < cap ? vb : cap), QKN_THREADS, qkn_table_bytes(a), s,
-                         a));
+                         a, hu));
   } else {
     JAGG_CUDA_TRY(launch(qk_norm_rope_fwd_kernel, (int)(blocks < 65536 ? blocks : 65536), QKN_THREADS, 0, s, a));
   }
@@ -1675,19 +1687,21 @@ int launch_qk_norm_rope_bwd(const QkNormRopeBwd& a, cudaStream_t s) {
   const int64_t blocks = ((int64_t)f.M * f.heads + QKN_WARPS - 1) / QKN_WARPS;
   const int cap = 4 * sm_count();
   const int tok = prof_start(s);
-  if (qkn_vector(f) && a.ld_dqk % 4 == 0 && aligned8(a.dqk)) {
+  if (qkn_vector(f) && a.ld_dqk % 4 == 0 && aligned8(a.dqk) && (reinterpret_cast<uintptr_t>(a.dq32) & 15) == 0) {
     // a few blocks per SM: each block ends in 4 x 128 scale-gradient atomics
-    const int64_t vb = ceil_div((int64_t)f.M, (int64_t)QKN_WARPS);
     const int vcap = 3 * sm_count();  // the resident blocks (80 registers, 3 per SM)
-    JAGG_CUDA_TRY(launch(qk_norm_rope_bwd_v_kernel, (int)(vb < vcap ? vb : vcap), QKN_THREADS, qkn_table_bytes(f), s,
-                         a));
+    const int hu = qkn_heads_per_unit(f, QKV_ITEMS, vcap * QKN_WARPS);
+    const int64_t vb = ceil_div((int64_t)f.M * ceil_div(f.heads, hu), (int64_t)QKN_WARPS);
+    JAGG_CUDA_TRY(launch(a.dq32 ? qk_norm_rope_bwd_v_kernel<true> : qk_norm_rope_bwd_v_kernel<false>,
+                         (int)(vb < vcap ? vb : vcap), QKN_THREADS, qkn_table_bytes(f), s, a, hu));
   } else {
     JAGG_CUDA_TRY(launch(qk_norm_rope_bwd_kernel, (int)(blocks < cap ? blocks : cap), QKN_THREADS, 0, s, a));
   }
   JAGG_LAUNCHED();
-  // algorithmic bytes: dq, dk read and rewritten in place, raw q, k read (storage type), 1/rms
+  // algorithmic bytes: dq, dk read and written, raw q, k read (storage type, dq in f32 if so given), 1/rms
   const double esz = f.dtype == JAGG_DTYPE_F32 ? 4.0 : 2.0;
-  prof_stop(tok, s, PROF_QKN_BWD, 0.0, (double)f.M * (6.0 * f.d * esz + 8.0 * f.heads));
+  const double dq = a.dq32 ? 4.0 : esz;
+  prof_stop(tok, s, PROF_QKN_BWD, 0.0, (double)f.M * (f.d * (dq + 5.0 * esz) + 8.0 * f.heads));
   return JAGG_OK;
 }
 

@@ -92,10 +92,6 @@ int launch_copy_rows(const void* in, int64_t ld_in, int in_seg, int in_seg_off, 
                      int64_t ld_out, int out_seg, int out_seg_off, int64_t out_seg_stride, int rows, int cols,
                      int elem_bytes, cudaStream_t s);
 
-// Attention helper: Dv[b, head, n] = sum_c dO[row, head*dh + c] * O[row, head*dh + c].
-int launch_attn_rowdot(const void* dO, const void* O, int64_t ld, float* Dv, int B, int N, int heads, int dh,
-                       int dtype, cudaStream_t s);
-
 // Per-head RMSNorm (learned scale, eps 1e-6) followed by 2D RoPE on q and k of a qkv buffer,
 // writing the transformed q/k into qk_out [M, 2d] (dtype); saves 1/rms for q and k.
 struct QkNormRope {
@@ -120,6 +116,10 @@ struct QkNormRopeBwd {
   QkNormRope f;
   void* dqk;  // [M, ld_dqk] dtype, in place
   int64_t ld_dqk;
+  // The incoming dq in f32, 16-byte aligned rows of d (attention's accumulator), or nullptr: in dqk.
+  // Its row of (sequence b, token n) is b dq32_seq + dq32_row0 + n.
+  const float* dq32;
+  int dq32_seq, dq32_row0;
   float* dqs_txt;
   float* dks_txt;
   float* dqs_img;

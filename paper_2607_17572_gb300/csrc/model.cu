@@ -1075,10 +1075,12 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
     attention_bwd_scratch(w.attn, B, N, m.heads, &ab.Dv, &ab.dq_acc);
     ab.dq = ab.dk = ab.dv = seg_single(w.dqkv, ld1, N);
     ab.dq_col0 = 0; ab.dk_col0 = d; ab.dv_col0 = 2 * d;
+    ab.keep_dq32 = true;  // QK-norm's backward reads it
     JAGG_TRY(attention_bwd(ab, s));
     QkNormRopeBwd qb;
     qb.f = qk_args(m, k.qkv, M, N, Nt, sw.qn, sw.kn, k.qk, k.rq, k.rk);
     qb.dqk = w.dqkv; qb.ld_dqk = ld1;
+    qb.dq32 = ab.dq_acc; qb.dq32_seq = N; qb.dq32_row0 = 0;
     qb.dqs_txt = qb.dqs_img = grad + sw.qn;
     qb.dks_txt = qb.dks_img = grad + sw.kn;
     JAGG_TRY(launch_qk_norm_rope_bwd(qb, s));
@@ -1123,6 +1125,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
     attention_bwd_scratch(w.attn, B, N, m.heads, &ab.Dv, &ab.dq_acc);
     ab.dq = ab.dk = ab.dv = SegRows{dqkv_s[0], dqkv_s[1], 3 * d, 3 * d, Nt};
     ab.dq_col0 = 0; ab.dk_col0 = d; ab.dv_col0 = 2 * d;
+    ab.keep_dq32 = true;
     JAGG_TRY(attention_bwd(ab, s));
     QkvBwd qk[2];
     for (int si = 0; si < 2; ++si) {
@@ -1132,6 +1135,7 @@ int vjp_mmdit(const jagg_model& m, const Saved& S, int B, const VjpWs& w, float*
       QkNormRopeBwd qb;
       qb.f = qk_args(m, q.qkv, Ms, Ns, si ? 0 : Ns, sw.qn, sw.kn, q.qk, q.rq, q.rk);
       qb.dqk = dqkv_s[si]; qb.ld_dqk = 3 * d;
+      qb.dq32 = ab.dq_acc; qb.dq32_seq = N; qb.dq32_row0 = si ? Nt : 0;
       qb.dqs_txt = qb.dqs_img = grad + sw.qn;
       qb.dks_txt = qb.dks_img = grad + sw.kn;
       JAGG_TRY(launch_qk_norm_rope_bwd(qb, s));

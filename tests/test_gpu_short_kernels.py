@@ -9,7 +9,7 @@ import torch
 import synth
 from gpu_cases import GpuModel, model_inputs, rel_l2
 from oracle import dit
-from test_gpu_kernels import _desc, _rel
+from test_gpu_kernels import _desc, _qkn_reference, _rel
 
 pytestmark = pytest.mark.gpu
 
@@ -178,3 +178,31 @@ def test_attention_backward_with_bias_sums(B, N, H, dh, dtype):
     assert _rel(got, plain) < (1e-5 if dtype == torch.float32 else 2e-3)
     bound = (B * N + 8) * 2.0 ** -24 * (got.double().abs().sum(0) + 1)
     assert ((db.double() - 1 - got.double().sum(0)).abs() <= bound).all()
+
+
+@pytest.mark.parametrize("H", [1, 5, 24])
+@pytest.mark.parametrize("N,n_txt,gw", [(1, 1, 1), (13, 4, 3), (780, 0, 26), (2048, 0, 64), (3660, 12, 57)])
+def test_qk_norm_in_parts_of_a_row(N, n_txt, gw, H):
+    """Head dim 128 in bf16: from one row to just above the resident warps, where a warp takes a
+    whole row or some of its heads, with a ragged last part.  Tolerances as for the kernels' other
+    parity test: bf16 outputs 2^-8 relative (twice that through the backward), f32 sums 1e-4."""
+    torch.manual_seed(N + H)
+    d = 128 * H
+    qkv = (torch.randn(N, 3 * d, device="cuda") * 2).bfloat16()
+    qs, ks = ((1 + 0.1 * torch.randn(128, device="cuda")).bfloat16() for _ in range(2))
+    qk = torch.full((N, 2 * d), float("nan"), device="cuda", dtype=torch.bfloat16)
+    rq, rk = torch.empty(N, H, device="cuda"), torch.empty(N, H, device="cuda")
+    jg.test_qk_norm_rope_fwd(qkv, N, N, H, n_txt, gw, qs, ks, qk, rq, rk, rope=True)
+    g_up = torch.randn(N, 3 * d, device="cuda").bfloat16()
+    dqk, dscale = g_up.clone(), [torch.zeros(128, device="cuda") for _ in range(2)]
+    jg.test_qk_norm_rope_bwd(qkv, N, N, H, n_txt, gw, qs, ks, rq, rk, dqk, *dscale, rope=True)
+    for i, (s, r, ds) in enumerate(zip((qs, ks), (rq, rk), dscale)):
+        x = qkv[:, i * d:(i + 1) * d].float().view(N, H, 128).requires_grad_()
+        s = s.float().requires_grad_()
+        y = _qkn_reference(x, N, n_txt, gw, 128, s, True).reshape(N, d)
+        assert _rel(qk[:, i * d:(i + 1) * d].float(), y) < 1e-2
+        assert _rel(r, torch.rsqrt((x.detach() ** 2).mean(-1) + 1e-6)) < 1e-5
+        (y * g_up[:, i * d:(i + 1) * d].float()).sum().backward()
+        assert _rel(dqk[:, i * d:(i + 1) * d].float(), x.grad.reshape(N, d)) < 2e-2
+        assert _rel(ds, s.grad) < 1e-4
+    assert torch.equal(dqk[:, 2 * d:], g_up[:, 2 * d:])
