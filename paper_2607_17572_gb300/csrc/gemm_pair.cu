@@ -39,23 +39,26 @@ constexpr int PK = 64;        // k-block
 constexpr int P_EW = 8;       // epilogue warps
 constexpr int P_THREADS = 64 + 32 * P_EW;
 constexpr int P_HALF = 128 * PK * 2;      // bytes of a CTA's half of an operand tile
-constexpr int P_STAGE = 2 * P_HALF;
+constexpr int P_SMEM = 232448 - 512;      // dynamic shared memory of a block
+constexpr int P_FIXED = 1024 /*align*/ + 512 /*barriers*/;
+constexpr int P_MAX_STAGES = 8;
 
 template <int EPI>
 struct PairCfg {
   // Staging boxes of 32 rows x 32 columns per epilogue warp: 8 KB where inputs or a second output
-  // share them, 4 KB otherwise.  The rest of shared memory is operand stages (five or six): with
-  // four the products are 7 % slower (18432 x 3072 x 12288: 805 us against 748), since the
-  // loads of 4 x 0.27 us of tensor work no longer cover the L2 latency under load.
+  // share them, 4 KB otherwise.  The rest of shared memory is operand stages, as many as fit at
+  // the launch's tile width: five or six of 256 columns, six to eight of 128.  With four at 256
+  // columns the products are 7 % slower (18432 x 3072 x 12288: 805 us against 748), since the
+  // loads of 4 x 0.27 us of tensor work no longer cover the L2 latency under load.  At 128 columns six
+  // stages cover less time, and a product of fewer units than pairs has nothing else to do: stages as
+  // narrow as the tile took the pass over 5 x 245 rows (d = 768) from 2351 to 2306 us, the
+  // forward of 8 x 333 rows from 1028 to 1018; wider tiles keep the ring they had.
   static constexpr bool OUT_BF16 = EPI == PE_STORE_BF16 || EPI == PE_MUL || EPI == PE_GELU;
   static constexpr int BOX = OUT_BF16 ? 2048 : 4096;
   static constexpr int BOXES = EPI == PE_STORE_BF16 ? 2 : EPI <= PE_ACCUM ? 1 : EPI == PE_GATE ? 2 : 4;
   static constexpr int WARP_BYTES = BOXES * BOX;
   static constexpr int EPI_BYTES = P_EW * WARP_BYTES;
-  static constexpr int FIXED = 1024 /*align*/ + 512 /*barriers*/;
-  static constexpr int STAGES = (232448 - FIXED - EPI_BYTES) / P_STAGE;
-  static constexpr int SMEM = STAGES * P_STAGE + EPI_BYTES + FIXED;
-  static_assert(SMEM <= 232448, "shared memory budget");
+  static_assert((2 * P_MAX_STAGES + 6 + BOXES * P_EW) * 8 + 4 <= 512, "barriers");
 };
 
 struct PairParams {
@@ -85,6 +88,7 @@ struct PairGroup {
   PairMaps maps[2];
   PairParams p[2];
   int total0, total;  // units of the first product, and of both
+  int stages, stage_bytes;  // the operand ring: a stage holds 128 rows of A and half of the widest tile's columns of B
 };
 
 // Tiles walk groups of P_GROUP row tiles, the row tile fastest inside a group: the 76 pairs at work
@@ -133,13 +137,13 @@ template <bool A_MN, bool B_MN, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ PairGroup g) {
   using Cfg = PairCfg<EPI>;
-  constexpr int STAGES = Cfg::STAGES;
+  const int stages = g.stages, ring_stage = g.stage_bytes;
   extern __shared__ uint8_t smem_pair[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_pair) + 1023) & ~uintptr_t(1023));
-  uint8_t* epi_smem = smem + STAGES * P_STAGE;
+  uint8_t* epi_smem = smem + stages * ring_stage;
   uint64_t* full = reinterpret_cast<uint64_t*>(epi_smem + Cfg::EPI_BYTES);  // leader's: a stage landed in both CTAs
-  uint64_t* empty = full + STAGES;     // per CTA: the products reading the stage are done
-  uint64_t* tfull = empty + STAGES;    // [2] per CTA: an accumulator is complete
+  uint64_t* empty = full + P_MAX_STAGES;     // per CTA: the products reading the stage are done
+  uint64_t* tfull = empty + P_MAX_STAGES;    // [2] per CTA: an accumulator is complete
   uint64_t* tempty = tfull + 2;        // [2] leader's: both CTAs' epilogue warps have drained it
   uint64_t* auxbar = tempty + 2;       // [BOXES per epilogue warp] an epilogue input box landed
   uint64_t* drainbar = auxbar + Cfg::BOXES * P_EW;
@@ -152,7 +156,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       ptx::mbar_init(&full[s], 1);
       ptx::mbar_init(&empty[s], 1);
     }
@@ -195,6 +199,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
     if (ptx::elect_one()) {
       // ---------------- TMA producer: this CTA's halves of A and B
       int stage = 0;
+      uint8_t* sA = smem;
       uint32_t phase = 0;
       uint32_t issued = 0, issued_parity = 0;
       for (int t = blockIdx.x >> 1; t < total && !abort_flag; t += npairs) {
@@ -209,7 +214,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
         const uint32_t stage_bytes = 2u * (P_HALF + (B_MN ? (two_chunks ? P_HALF : P_HALF / 2) : half_n * PK * 2));
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!ptx::mbar_wait(&empty[stage], phase ^ 1)) { abort_flag = 1; break; }
-          uint8_t* sA = smem + stage * P_STAGE;
           uint8_t* sB = sA + P_HALF;
           if (rank == 0) ptx::mbar_arrive_expect_tx(&full[stage], stage_bytes);
           const uint32_t bar = ptx::mapa(ptx::smem_u32(&full[stage]), 0);
@@ -227,7 +231,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
           }
           issued |= 1u << stage;
           issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
+          sA += ring_stage;
+          if (++stage == stages) { stage = 0; phase ^= 1; sA = smem; }
         }
       }
       // After a give-up, loads already issued may still be landing: the leader waits (bounded)
@@ -235,7 +240,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
       // barriers, for the length of one bounded wait.
       if (abort_flag) {
         if (rank == 0) {
-          for (int s = 0; s < STAGES; ++s)
+          for (int s = 0; s < stages; ++s)
             if (issued & (1u << s)) ptx::mbar_wait(&full[s], (issued_parity >> s) & 1u);
         } else if (issued) {
           ptx::mbar_wait(never, 0);
@@ -246,6 +251,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
     if (rank == 0 && ptx::elect_one()) {
       // ---------------- MMA issuer for both CTAs
       int stage = 0, acc = 0;
+      const uint32_t a_first = ptx::smem_u32(smem);
+      uint32_t a_addr = a_first;
       uint32_t phase = 0, acc_phase = 0;
       for (int t = blockIdx.x >> 1; t < total && !abort_flag; t += npairs) {
         int pr, tm, tn, ks, kb0, kb1;
@@ -259,7 +266,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!ptx::mbar_wait(&full[stage], phase)) { ok = false; break; }
           ptx::tc_fence_after();
-          const uint32_t a_addr = ptx::smem_u32(smem + stage * P_STAGE);
           const uint32_t b_addr = a_addr + P_HALF;
           // K-major: a step of 16 elements is 32 bytes inside the swizzled 128-byte row;
           // MN-major: two 1024-byte atoms.  (The start-address field counts 16 bytes and never
@@ -271,7 +277,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
             ptx::umma_bf16_pair(d, ad + (uint64_t)(k * (A_MN ? 128 : 2)), bd + (uint64_t)(k * (B_MN ? 128 : 2)), idesc,
                                 (kb > kb0 || k > 0) ? 1u : 0u);
           ptx::umma_commit_pair(&empty[stage]);
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
+          a_addr += ring_stage;
+          if (++stage == stages) { stage = 0; phase ^= 1; a_addr = a_first; }
         }
         if (!ok) { abort_flag = 1; break; }
         ptx::umma_commit_pair(&tfull[acc]);
@@ -603,14 +610,20 @@ int launch_pair(const GemmArgs& a, const GemmArgs* b, const PairPlan (&plan)[2],
   auto units = [](const PairParams& p) { return p.tiles_m * p.tiles_n * p.splits; };
   grp.total0 = units(grp.p[0]);
   grp.total = grp.total0 + (b ? units(grp.p[1]) : 0);
+  // B arrives K-major in bn / 2 rows of 128 bytes, MN-major in whole chunks of 64 columns
+  const int bn = b && plan[1].bn > plan[0].bn ? plan[1].bn : plan[0].bn;
+  grp.stage_bytes = P_HALF + (B_MN ? (bn > 128 ? P_HALF : P_HALF / 2) : bn / 2 * PK * 2);
+  const int fit = (P_SMEM - P_FIXED - Cfg::EPI_BYTES) / grp.stage_bytes;
+  grp.stages = fit < P_MAX_STAGES ? fit : P_MAX_STAGES;
+  const int smem = grp.stages * grp.stage_bytes + Cfg::EPI_BYTES + P_FIXED;
   auto kernel = gemm_pair_kernel<A_MN, B_MN, EPI>;
   static bool attr = false;
   if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM));
+    JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM));
     attr = true;
   }
   const int tok = prof_start(s);
-  JAGG_CUDA_TRY(launch(kernel, 2 * (grp.total < npairs ? grp.total : npairs), P_THREADS, Cfg::SMEM, s, grp));
+  JAGG_CUDA_TRY(launch(kernel, 2 * (grp.total < npairs ? grp.total : npairs), P_THREADS, smem, s, grp));
   JAGG_LAUNCHED();
   double flops = 0.0, bytes = 0.0;
   for (const GemmArgs* g : {&a, b}) {
