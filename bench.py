@@ -96,7 +96,7 @@ def describe(wl) -> str:
 # bytes, from one ncu capture of the kernel alone (`--kernel gemm`) on the workload's
 # backward products at the step's rows; the roofline's `traffic` is this ratio times the
 # step's algorithmic bytes per launch.  Absent: no capture of the current kernel.
-TRAFFIC_RATIO = {"mmdit_flux1024_bf16": 3.01}
+TRAFFIC_RATIO = {"mmdit_flux1024_bf16": 3.42}
 
 
 def peaks():
@@ -714,7 +714,7 @@ def run_gpu(args, ws, rank):
     # the products and attention run back to back for the seconds of a step: sustained peak
     psrc = f"bf16_tflops_sustained of {src} peaks"
     roofline = family_roofline(fam, "gemm_tcgen05", sustained, psrc,
-                               "gemm_tc_kernel (all dense products of the joint VJP)")
+                               "gemm_pair_kernel, gemm_tc_kernel (all dense products of the joint VJP)")
     ratio = TRAFFIC_RATIO.get(wl.name)
     roofline["traffic"] = ratio * roofline["algorithmic_bytes_per_launch"] if ratio else None
     roofline["frac_of_burst"] = roofline["achieved"] / burst
