@@ -862,7 +862,7 @@ int attention_fwd(const AttnArgs& a, cudaStream_t s) {
   if (tc && a.impl != 1) {
     const int tok = prof_start(s);
     JAGG_TRY(attention_fwd_tc(a, s));
-    // QK^T and PV: 2 N^2 d multiply-adds per (sequence, head); the second S pass is not counted
+    // QK^T and PV: 2 N^2 d multiply-adds per (sequence, head)
     prof_stop(tok, s, PROF_ATTN_FWD, 4.0 * a.B * a.heads * (double)a.N * a.N * a.dh,
               2.0 * a.B * (double)a.N * a.heads * a.dh * 4);
     return JAGG_OK;
