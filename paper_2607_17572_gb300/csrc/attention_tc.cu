@@ -22,7 +22,7 @@ constexpr float kLog2eTc = 1.4426950408889634f;
 // in the second: each stream is cut into tiles of its own, the first stream's last tile
 // partly filled when n0 is not a multiple of the tile.  The order of the keys does not matter
 // to a softmax, so a partly filled tile in the middle of the sequence is masked like the one at
-// its end, and a stream boundary may lie on any token.
+// its end (the forward's scores to -inf, the backward's P to 0), and a stream boundary may lie on any token.
 struct TokTile {
   int seg, row, valid, tok;  // stream, first row in it, tokens of the tile, first token of the sequence
 };
@@ -384,6 +384,12 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
     bool ok = true;
     int i = 0;
     for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++i) {
+      TokTile kt;
+      int b, h;
+      unit_of(u, kt, b, h);
+      // A key row past the tile's last key was read as zeros: its logit 0 against an lse far below 0
+      // gives exp(-lse), infinite below about -88, and 0 * inf in dQ.  Its P is set to 0 (and so dS).
+      const bool ragged = kt.valid < BK;
       for (int j = 0; j < nq; ++j) {
         const int g = i * nq + j;
         const int st = g % NS, bb = g & 1;
@@ -407,6 +413,10 @@ __device__ __forceinline__ void fa_bwd_v3(const FbMaps& maps, const FbParams& p,
             const float p3 = ptx::ex2_approx(fmaf(__uint_as_float(rs[e + 3]), c1, -l4.w * kLog2eTc));
             hp[e / 2] = pack2_bf16(p0, p1);
             hp[e / 2 + 1] = pack2_bf16(p2, p3);
+          }
+          if (ragged) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) hp[e] = r < kt.valid ? hp[e] : 0u;
           }
         }
         // over this warp's own S^T columns, read already
