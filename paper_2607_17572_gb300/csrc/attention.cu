@@ -262,6 +262,8 @@ __global__ void __launch_bounds__(128) fa_bwd_kernel(AttnBwdArgs a) {
     dv[i][0] = dv[i][1] = dv[i][2] = dv[i][3] = 0.f;
   }
   const int nqt = (N + TILE - 1) / TILE;
+  const int k0 = kt * TILE + warp * 16 + g, k1 = k0 + 8;  // this lane's keys
+  const bool live0 = k0 < N, live1 = k1 < N;
   if (NBUF == 2) fetch_queries(0);
   for (int qt = 0; qt < nqt; ++qt) {
     __syncthreads();  // every warp is done with the buffer about to be refilled
@@ -305,13 +307,14 @@ __global__ void __launch_bounds__(128) fa_bwd_kernel(AttnBwdArgs a) {
         mma16816(dpt[2 * np + 1], va, ob[2], ob[3]);
       }
     }
-    // P^T and dS^T
+    // P^T and dS^T.  Keys past the last one were read as zeros: their logit 0 against an lse far
+    // below 0 gives exp(-lse), infinite below about -88, and 0 * inf in dQ, so their P is 0.
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int q = nt * 8 + 2 * tig + (e & 1);
-        const float p = exp2f(st[nt][e] * sl2 - sL[q]);
+        const float p = (e < 2 ? live0 : live1) ? exp2f(st[nt][e] * sl2 - sL[q]) : 0.f;
         st[nt][e] = p;
         dpt[nt][e] = p * (dpt[nt][e] - sDv[q]);
       }
@@ -387,17 +390,16 @@ __global__ void __launch_bounds__(128) fa_bwd_kernel(AttnBwdArgs a) {
     }
   }
   // dK (times the softmax scale) and dV for this CTA's keys
-  const int k0 = kt * TILE + warp * 16 + g, k1 = k0 + 8;
 #pragma unroll
   for (int dt = 0; dt < D / 8; ++dt) {
     const int64_t c = (int64_t)h * D + dt * 8 + 2 * tig;
-    if (k0 < N) {
+    if (live0) {
       *reinterpret_cast<uint32_t*>(static_cast<bf16*>(a.dk.base(k0)) + a.dk.off(b, k0, N, a.dk_col0 + c)) =
           pack_bf16(dk[dt][0] * f.scale, dk[dt][1] * f.scale);
       *reinterpret_cast<uint32_t*>(static_cast<bf16*>(a.dv.base(k0)) + a.dv.off(b, k0, N, a.dv_col0 + c)) =
           pack_bf16(dv[dt][0], dv[dt][1]);
     }
-    if (k1 < N) {
+    if (live1) {
       *reinterpret_cast<uint32_t*>(static_cast<bf16*>(a.dk.base(k1)) + a.dk.off(b, k1, N, a.dk_col0 + c)) =
           pack_bf16(dk[dt][2] * f.scale, dk[dt][3] * f.scale);
       *reinterpret_cast<uint32_t*>(static_cast<bf16*>(a.dv.base(k1)) + a.dv.off(b, k1, N, a.dv_col0 + c)) =
