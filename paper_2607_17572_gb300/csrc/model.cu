@@ -25,6 +25,7 @@ void set_last_error(const char* fmt, ...) {
   va_end(ap);
 }
 int cuda_status(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here: a later call's launch check must not find it again
   set_last_error("CUDA error %d (%s) at %s", (int)e, cudaGetErrorString(e), where);
   return JAGG_ERR_CUDA;
 }

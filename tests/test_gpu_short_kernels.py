@@ -206,3 +206,16 @@ def test_qk_norm_in_parts_of_a_row(N, n_txt, gw, H):
         assert _rel(dqk[:, i * d:(i + 1) * d].float(), x.grad.reshape(N, d)) < 2e-2
         assert _rel(ds, s.grad) < 1e-4
     assert torch.equal(dqk[:, 2 * d:], g_up[:, 2 * d:])
+
+
+def test_a_refused_launch_does_not_reach_the_next_call():
+    """The grid of the f32 attention holds at most 65535 (sequence, head) pairs; the runtime refuses
+    more on the host and nothing runs.  The error belongs to that call alone."""
+    B = 65536
+    qkv, o, lse = (torch.zeros(B, n, device="cuda") for n in (48, 16, 1))
+    for _ in range(2):
+        with pytest.raises(jg.JaggError, match="invalid"):
+            jg.test_attention_fwd(qkv, B, 1, 1, 16, o, lse)
+        jg.test_attention_fwd(qkv, 3, 1, 1, 16, o, lse)
+    torch.cuda.synchronize()
+    assert jg.device_status() == 0
