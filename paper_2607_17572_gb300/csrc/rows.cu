@@ -84,11 +84,14 @@ __global__ void __launch_bounds__(32 * RF_MAX_WARPS, 1) rows_fwd_kernel(RowsFwd 
 
 // ------------------------------------------------------------------ G += Y^T X, few rows
 // G [M, N] f32, Y [K, M] and X [K, N] bf16 with K <= KMAX: an update of rank K.  Bound by reading and
-// writing G: a thread keeps its 4 columns of every X row in registers and walks rows of G, four
-// at a time; Y's values, uniform over the CTA, are broadcast from shared memory.  43008 x 3072 of rank 4:
-// 213 -> 173 us (6.1 TB/s read and written), 56832 x 768 of rank 5 81 -> 63, 3072 x 3072 20 -> 14,
-// against reduce-adds of nearly empty tensor-core tiles.
-constexpr int RU_THREADS = 256, RU_ROWS = 4, RU_CHUNK = 64;
+// writing G, which the L2 does: a thread keeps its 4 columns of every X row in registers, walks rows of G and
+// sends each row's 4 sums as one 16-byte reduction; Y's values, uniform over the CTA, are broadcast
+// from shared memory.  The reductions are atomic as in every other accumulated product, so passes
+// on several streams may add into one gradient.  43008 x 3072 of rank 4: 213 -> 188 us (5.6 TB/s
+// read and written), 56832 x 768 of rank 5 81 -> 68, of rank 16 68, 3072 x 3072 20 -> 19, against reduce-adds of
+// nearly empty tensor-core tiles; a plain read, add and write of G, not safe beside another pass,
+// takes 175, 65, 85 and 20.
+constexpr int RU_THREADS = 256, RU_CHUNK = 64;
 
 template <int KMAX>
 __global__ void __launch_bounds__(RU_THREADS) rank_update_kernel(RankUpdate a) {
@@ -117,28 +120,20 @@ __global__ void __launch_bounds__(RU_THREADS) rank_update_kernel(RankUpdate a) {
     __syncthreads();
     if (!live) continue;
     float* gp = a.g + (int64_t)c0 * a.ldg + n;
-    for (int r0 = 0; r0 < rows; r0 += RU_ROWS) {
-      float4 g[RU_ROWS];
+#pragma unroll 4
+    for (int r = 0; r < rows; ++r) {
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int r = 0; r < RU_ROWS; ++r)
-        if (r0 + r < rows) g[r] = __ldcs(reinterpret_cast<const float4*>(gp + (int64_t)(r0 + r) * a.ldg));
+      for (int k = 0; k < KMAX; k += 4) {
+        const float4 y4 = *reinterpret_cast<const float4*>(&ys[r][k]);
+        const float y[4] = {y4.x, y4.y, y4.z, y4.w};
 #pragma unroll
-      for (int r = 0; r < RU_ROWS; ++r) {
-        if (r0 + r >= rows) break;
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < KMAX; k += 4) {
-          const float4 y4 = *reinterpret_cast<const float4*>(&ys[r0 + r][k]);
-          const float y[4] = {y4.x, y4.y, y4.z, y4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            t.x = fmaf(y[e], x[k + e].x, t.x); t.y = fmaf(y[e], x[k + e].y, t.y);
-            t.z = fmaf(y[e], x[k + e].z, t.z); t.w = fmaf(y[e], x[k + e].w, t.w);
-          }
+        for (int e = 0; e < 4; ++e) {
+          t.x = fmaf(y[e], x[k + e].x, t.x); t.y = fmaf(y[e], x[k + e].y, t.y);
+          t.z = fmaf(y[e], x[k + e].z, t.z); t.w = fmaf(y[e], x[k + e].w, t.w);
         }
-        g[r].x += t.x; g[r].y += t.y; g[r].z += t.z; g[r].w += t.w;
-        __stcs(reinterpret_cast<float4*>(gp + (int64_t)(r0 + r) * a.ldg), g[r]);
       }
+      ptx::red_add_v4(gp + (int64_t)r * a.ldg, t.x, t.y, t.z, t.w);
     }
   }
 }

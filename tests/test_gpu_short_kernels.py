@@ -107,6 +107,24 @@ def test_rank_update(M, N, K):
     assert _rel(G[:, :N], ref) < 1e-6 and torch.equal(G[:, N:], G0[:, N:])
 
 
+@pytest.mark.parametrize("M,N,K", [(768, 768, 1), (2304, 768, 5), (3072, 256, 16)])
+def test_rank_updates_of_two_streams_into_one_gradient(M, N, K):
+    """Accumulation is atomic, as in the other products: updates issued on two streams all arrive.
+    Whole numbers below 2^24, so every order of the sums is exact."""
+    torch.manual_seed(M + K)
+    Y, X = (torch.randint(-3, 4, (2, K, n), device="cuda").bfloat16() for n in (M, N))
+    G = torch.zeros(M, N, device="cuda")
+    n = 100
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(n):
+        for i, s in enumerate(streams):
+            jg.test_gemm(_desc(M, N, K, Y[i], M, 1, X[i], N, 1, jg.DTYPE_BF16, G, N, jg.DTYPE_F32, epi=4), stream=s)
+    torch.cuda.synchronize()
+    ref = sum(Y[i].double().t() @ X[i].double() for i in range(2)) * n
+    assert ref.abs().max().item() < 2 ** 24 and torch.equal(G.double(), ref)
+
+
 @pytest.mark.parametrize("ln,gate", [(1, 1), (1, 0), (0, 1)])
 @pytest.mark.parametrize("d", [512, 768, 1024, 2048, 3072])
 @pytest.mark.parametrize("seqs,rps", [(1, 1), (3, 5), (7, 333), (2, 1024)])
