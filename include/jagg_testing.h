@@ -102,6 +102,12 @@ int jagg_test_ln_gate_bwd(int M, int d, int rows_per_seq, int do_ln, int do_gate
                           const float* dh_in, float* dh_out, const void* y, const float* gate, float* dgate,
                           void* dy, float* dbias, int dtype, cudaStream_t stream);
 
+/* The kernel that a LayerNorm / gate backward of width d would take (host only, nothing is read
+ * or launched): 0 the general one, 1 rows in registers, 2 row rings, 3 narrow rows.  at [12]:
+ * the addresses of dh_in, dh_out, dm, h, scale, dshift, dscale, y, gate, dgate, dy, dbias. */
+int jagg_test_ln_gate_route(int d, int do_ln, int do_gate, const uint64_t* at, int64_t mod_stride,
+                            int64_t dmod_stride, int dtype);
+
 /* Per-head RMSNorm of q and k (learned scale [dh], eps 1e-6) followed by 2D RoPE (the MMDiT
  * blocks' QK normalisation; the backbone reading of the paper's Flux / Qwen-Image models), on
  * M rows of N tokens per sequence whose first n_txt tokens are text (not rotated) and whose

@@ -118,6 +118,7 @@ _SIGNATURES = {
     "jagg_test_attention_bwd": (_I, [_P, _P, _P, _P, _I, _I, _I, _I, _I, _P, _P, _P]),
     "jagg_test_attention_bwd_bias": (_I, [_P, _P, _P, _P, _I, _I, _I, _I, _I, _P, _P, _P, _P]),
     "jagg_test_attention_fwd_streams": (_I, [_P, _P, _P, _P, _P, _I, _I, _I, _I, _I, _I, _I, _P]),
+    "jagg_test_ln_gate_route": (_I, [_I, _I, _I, ctypes.POINTER(ctypes.c_uint64), _I64, _I64, _I]),
     "jagg_test_ln_gate_bwd": (_I, [_I, _I, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
                                    _I, _P]),
     "jagg_test_qk_norm_rope_fwd": (_I, [_P, _I64, _I, _I, _I, _I, _I, _I, _P, _P, _I, _P, _P, _P, _I, _P]),
@@ -477,6 +478,12 @@ def test_ln_gate_bwd(M, d, rows_per_seq, dh_in, dh_out, dm=None, h=None, mean=No
                                        _ptr(rstd), _ptr(scale), _ptr(dshift), _ptr(dscale), _ptr(dh_in),
                                        _ptr(dh_out), _ptr(y), _ptr(gate), _ptr(dgate), _ptr(dy), _ptr(dbias), dt,
                                        _stream(stream)), "jagg_test_ln_gate_bwd")
+
+
+def test_ln_gate_route(d, do_ln, do_gate, at, mod_stride, dmod_stride, dtype) -> int:
+    """The kernel a LayerNorm / gate backward would take (jagg_test_ln_gate_route); at: 12 addresses."""
+    return lib().jagg_test_ln_gate_route(d, int(do_ln), int(do_gate), (ctypes.c_uint64 * 12)(*at), mod_stride,
+                                         dmod_stride, dtype)
 
 
 def test_qk_norm_rope_fwd(qkv, M, N, heads, n_txt, gw, qscale, kscale, qk_out, rq, rk, rope=True, stream=None):

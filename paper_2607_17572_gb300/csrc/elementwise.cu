@@ -800,12 +800,15 @@ int launch_ln_gate_ring(const LnGateBwd& a, cudaStream_t s) {
   return launch_ln_gate_ring_t<NV, WPR, false, true>(a, s);
 }
 
-// What the ring kernel takes: bf16 y and dy, dm in f32, 16-byte aligned rows and sums.
+// What the ring kernel takes: bf16 y and dy, dm in f32, and its 16-byte accesses (8-byte stores of
+// dy): every row, vector and sum aligned.
 bool ln_gate_ring_serves(const LnGateBwd& a) {
   auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  if (!al(a.dh_in) || a.dmod_stride % 4) return false;
-  if (a.do_ln && (!a.dm_f32 || !al(a.dm) || !al(a.h) || !al(a.dshift) || !al(a.dscale))) return false;
-  return !a.do_gate || (a.dtype == JAGG_DTYPE_BF16 && al(a.y) && al(a.dgate) && (!a.dbias || al(a.dbias)));
+  if (!al(a.dh_in) || a.mod_stride % 4 || a.dmod_stride % 4) return false;
+  if (a.do_ln && !(a.dm_f32 && al(a.dm) && al(a.h) && al(a.dh_out) && al(a.scale) && al(a.dshift) && al(a.dscale)))
+    return false;
+  return !a.do_gate || (a.dtype == JAGG_DTYPE_BF16 && al(a.y) && al(a.dy) && al(a.gate) && al(a.dgate) &&
+                        (!a.dbias || al(a.dbias)));
 }
 
 // Narrow rows, d = 4 L NV <= 256 (the f32 configuration): L lanes per row, so a warp works on 32 / L
@@ -1521,16 +1524,23 @@ int launch_ln_mod_fwd(const LnModFwd& a, cudaStream_t s) {
             (double)a.M * (a.d * (4.0 + (a.dtype == JAGG_DTYPE_F32 ? 4.0 : 2.0)) + 8.0));
   return JAGG_OK;
 }
-// The row-in-registers kernel serves LayerNorm backwards with an f32 dm (with or without the
-// gate); the rest go to the persistent kernel.
+// The row-in-registers kernel: LayerNorm backwards with an f32 dm, with or without the gate.
 template <int NV>
-int launch_ln_gate_rowreg(const LnGateBwd& a, int smem_fused, cudaStream_t s) {
-  if (!a.do_ln || !a.dm_f32) return launch_ln_gate_nv<0>(a, smem_fused, s);
+int launch_ln_gate_rowreg(const LnGateBwd& a, cudaStream_t s) {
   if (!a.do_gate) return launch_ln_gate_rowreg_t<NV, false, false>(a, s);
   return a.dtype == JAGG_DTYPE_F32 ? launch_ln_gate_rowreg_t<NV, true, false>(a, s)
                                    : launch_ln_gate_rowreg_t<NV, true, true>(a, s);
 }
 
+int ln_gate_route(const LnGateBwd& a) {
+  switch (a.d) {
+    case 64: case 128: case 256: return ln_gate_narrow_serves(a) ? LNG_NARROW : LNG_GENERAL;
+    case 384: return a.do_ln && a.dm_f32 ? LNG_ROWREG : LNG_GENERAL;
+    case 512: case 768: return ln_gate_ring_serves(a) ? LNG_RING : a.do_ln && a.dm_f32 ? LNG_ROWREG : LNG_GENERAL;
+    case 1024: case 2048: case 3072: return ln_gate_ring_serves(a) ? LNG_RING : LNG_GENERAL;
+  }
+  return LNG_GENERAL;
+}
 int launch_ln_gate_bwd(const LnGateBwd& a, cudaStream_t s) {
   JAGG_CHECK_ARG(a.d % 4 == 0 && a.d <= 3072, "ln_gate_bwd: hidden %d unsupported", a.d);
   JAGG_CHECK_ARG(a.M % a.rows_per_seq == 0, "ln_gate_bwd: rows not a whole number of sequences");
@@ -1538,19 +1548,25 @@ int launch_ln_gate_bwd(const LnGateBwd& a, cudaStream_t s) {
   const int smem = 4 * a.d * (int)sizeof(float);
   const int tok = prof_start(s);
   int st = JAGG_ERR_UNSUPPORTED;
-  const bool ring = ln_gate_ring_serves(a);
-  if ((a.d == 64 || a.d == 128 || a.d == 256) && ln_gate_narrow_serves(a))
-    st = a.d == 64 ? launch_ln_gate_narrow<16, 1>(a, s)
-                   : a.d == 128 ? launch_ln_gate_narrow<32, 1>(a, s) : launch_ln_gate_narrow<32, 2>(a, s);
-  else switch (a.d % 128 == 0 ? a.d / 128 : 0) {
-    case 3: st = launch_ln_gate_rowreg<3>(a, smem, s); break;
-    case 4: st = ring ? launch_ln_gate_ring<2, 2>(a, s) : launch_ln_gate_rowreg<4>(a, smem, s); break;
-    case 6: st = ring ? launch_ln_gate_ring<3, 2>(a, s) : launch_ln_gate_rowreg<6>(a, smem, s); break;
-    case 8: st = ring ? launch_ln_gate_ring<2, 4>(a, s) : launch_ln_gate_nv<8>(a, smem, s); break;
-    case 12: st = launch_ln_gate_nv<12>(a, smem, s); break;
-    case 16: st = ring ? launch_ln_gate_ring<2, 8>(a, s) : launch_ln_gate_nv<0>(a, smem, s); break;
-    case 24: st = ring ? launch_ln_gate_ring<3, 8>(a, s) : launch_ln_gate_nv<24>(a, smem, s); break;
-    default: st = launch_ln_gate_nv<0>(a, smem, s); break;
+  switch (ln_gate_route(a)) {
+    case LNG_NARROW:
+      st = a.d == 64 ? launch_ln_gate_narrow<16, 1>(a, s)
+                     : a.d == 128 ? launch_ln_gate_narrow<32, 1>(a, s) : launch_ln_gate_narrow<32, 2>(a, s);
+      break;
+    case LNG_RING:
+      st = a.d == 512    ? launch_ln_gate_ring<2, 2>(a, s)
+           : a.d == 768  ? launch_ln_gate_ring<3, 2>(a, s)
+           : a.d == 1024 ? launch_ln_gate_ring<2, 4>(a, s)
+           : a.d == 2048 ? launch_ln_gate_ring<2, 8>(a, s) : launch_ln_gate_ring<3, 8>(a, s);
+      break;
+    case LNG_ROWREG:
+      st = a.d == 384 ? launch_ln_gate_rowreg<3>(a, s)
+                      : a.d == 512 ? launch_ln_gate_rowreg<4>(a, s) : launch_ln_gate_rowreg<6>(a, s);
+      break;
+    default:
+      st = a.d == 1024   ? launch_ln_gate_nv<8>(a, smem, s)
+           : a.d == 1536 ? launch_ln_gate_nv<12>(a, smem, s)
+           : a.d == 3072 ? launch_ln_gate_nv<24>(a, smem, s) : launch_ln_gate_nv<0>(a, smem, s);
   }
   JAGG_TRY(st);
   // algorithmic bytes: dh read + write (f32), dm (f32), h (f32), y and dy (storage type)

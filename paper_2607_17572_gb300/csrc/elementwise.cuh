@@ -78,6 +78,9 @@ struct LnGateBwd {
   int dtype;
 };
 int launch_ln_gate_bwd(const LnGateBwd& a, cudaStream_t s);
+// The kernel that serves the call: by width, types and alignment.
+enum LnGateRoute : int { LNG_GENERAL = 0, LNG_ROWREG, LNG_RING, LNG_NARROW };
+int ln_gate_route(const LnGateBwd& a);
 
 // db[n] += sum_r X[r * ld + n], r < rows, n < cols (X f32 or dtype).
 int launch_colsum(const void* X, int x_f32, int dtype, int rows, int cols, int64_t ld, float* db, cudaStream_t s);

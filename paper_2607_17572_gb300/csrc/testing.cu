@@ -175,6 +175,20 @@ extern "C" int jagg_test_ln_gate_bwd(int M, int d, int rows_per_seq, int do_ln, 
   return launch_ln_gate_bwd(a, stream);
 }
 
+extern "C" int jagg_test_ln_gate_route(int d, int do_ln, int do_gate, const uint64_t* at, int64_t mod_stride,
+                                       int64_t dmod_stride, int dtype) {
+  JAGG_CHECK_ARG(at, "jagg_test_ln_gate_route: null addresses");
+  auto f = [&](int i) { return reinterpret_cast<float*>(static_cast<uintptr_t>(at[i])); };
+  LnGateBwd a{};
+  a.M = a.rows_per_seq = 1; a.d = d;
+  a.do_ln = do_ln; a.dm = f(2); a.dm_f32 = 1; a.h = f(3);
+  a.scale = f(4); a.mod_stride = mod_stride; a.dshift = f(5); a.dscale = f(6); a.dmod_stride = dmod_stride;
+  a.dh_in = f(0); a.dh_out = f(1);
+  a.do_gate = do_gate; a.y = f(7); a.gate = f(8); a.dgate = f(9); a.dy = f(10); a.dbias = f(11);
+  a.dtype = dtype;
+  return ln_gate_route(a);
+}
+
 static QkNormRope qkn_args(const void* qkv, int64_t ld_qkv, int M, int N, int d, int heads, int n_txt, int gw,
                            const void* qscale, const void* kscale, int rope, int dtype) {
   QkNormRope q{};

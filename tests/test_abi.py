@@ -132,3 +132,28 @@ def test_wait_timeout_rejects_limits_outside_its_range(jg):
     for bad in (0, 2_000_000_001):
         assert L.jagg_test_wait_timeout(bad, ctypes.c_void_p(16), None) == -1
         assert "limit" in L.jagg_last_error().decode()
+
+
+LN_GATE_BUFFERS = ["dh_in", "dh_out", "dm", "h", "scale", "dshift", "dscale", "y", "gate", "dgate", "dy", "dbias"]
+
+
+@pytest.mark.parametrize("ln,gate", [(1, 1), (1, 0), (0, 1)])
+@pytest.mark.parametrize("d,best,unaligned", [(64, 3, 0), (256, 3, 0), (512, 2, 1), (768, 2, 1), (1024, 2, 0),
+                                              (2048, 2, 0), (3072, 2, 0)])
+def test_ln_gate_backward_route_by_alignment(jg, d, best, unaligned, ln, gate):
+    """The kernels with 16-byte accesses serve a call only when every buffer that it uses and both
+    strides allow them; one 4-byte offset anywhere takes it to the kernel it had without them
+    (rows in registers at 512 and 768 for a LayerNorm part, else the general one)."""
+    base = [4096 * (i + 1) for i in range(12)]
+    route = lambda at, ms=d, ds=d, dt=jg.DTYPE_BF16: jg.test_ln_gate_route(d, ln, gate, at, ms, ds, dt)
+    other = unaligned if ln else 0
+    assert route(base) == best
+    used = {"dh_in"} | ({"dh_out", "dm", "h", "scale", "dshift", "dscale"} if ln else set())
+    used |= {"y", "gate", "dgate", "dy", "dbias"} if gate else set()
+    for i, name in enumerate(LN_GATE_BUFFERS):
+        at = list(base)
+        at[i] += 4
+        assert route(at) == (other if name in used else best), name
+    assert route(base, ms=d + 1) == other and route(base, ds=d + 2) == other
+    # f32 rows go through the rings only without a gate part (y and dy are bf16 there)
+    assert route(base, dt=jg.DTYPE_F32) == (other if gate and best == 2 else best)
