@@ -779,11 +779,8 @@ int store_dq(const AttnBwdArgs& a, int64_t chunks, cudaStream_t s) {
 template <int D>
 int fwd_tc(const AttnArgs& a, cudaStream_t s) {
   const int smem = 3 * TILE * (D + 8) * 2;
-  static bool set = false;
-  if (!set) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    set = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, fa_fwd_kernel<D>, smem));
   dim3 grid(ceil_div(a.N, TILE), a.B * a.heads);
   const int tok = prof_start(s);
   JAGG_CUDA_TRY(launch(fa_fwd_kernel<D>, grid, 128, smem, s, a));
@@ -796,11 +793,8 @@ int fwd_tc(const AttnArgs& a, cudaStream_t s) {
 template <int D>
 int bwd_tc(const AttnBwdArgs& a, cudaStream_t s) {
   const int smem = BwdCfg<D>::SMEM;
-  static bool set = false;
-  if (!set) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_bwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    set = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, fa_bwd_kernel<D>, smem));
   dim3 grid(ceil_div(a.f.N, TILE), a.f.B * a.f.heads);
   const int tok = prof_start(s);
   JAGG_CUDA_TRY(launch(fa_bwd_kernel<D>, grid, 128, smem, s, a));
@@ -815,11 +809,8 @@ int bwd_tc(const AttnBwdArgs& a, cudaStream_t s) {
 template <int D>
 int fwd_simt(const AttnArgs& a, cudaStream_t s) {
   constexpr int smem = 3 * ST * (D + 1) * (int)sizeof(float);
-  static bool set = false;
-  if (!set) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(attn_fwd_simt<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    set = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, attn_fwd_simt<D>, smem));
   dim3 grid(ceil_div(a.N, ST), a.B * a.heads);
   JAGG_CUDA_TRY(launch(attn_fwd_simt<D>, grid, 256, smem, s, a));
   JAGG_LAUNCHED();
@@ -828,11 +819,8 @@ int fwd_simt(const AttnArgs& a, cudaStream_t s) {
 template <int D>
 int bwd_simt(const AttnBwdArgs& a, cudaStream_t s) {
   constexpr int smem = (4 * ST * (D + 1) + 2 * ST * (ST + 1)) * (int)sizeof(float);
-  static bool set = false;
-  if (!set) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(attn_bwd_simt<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    set = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, attn_bwd_simt<D>, smem));
   dim3 grid(ceil_div(a.f.N, ST), a.f.B * a.f.heads);
   JAGG_CUDA_TRY(launch(attn_bwd_simt<D>, grid, 256, smem, s, a));
   JAGG_LAUNCHED();

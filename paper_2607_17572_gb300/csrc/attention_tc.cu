@@ -1021,11 +1021,8 @@ int launch_v3(const AttnBwdArgs& a, cudaStream_t s) {
   p.dk_col0 = a.dk_col0; p.dv_col0 = a.dv_col0;
   p.lse = f.lse; p.Dv = a.Dv;
   p.dk = a.dk; p.dv = a.dv;
-  static bool attr = false;
-  if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, kernel, C::SMEM));
   const int units = tok_tiles(N, p.n0, C::BK) * f.B * f.heads;
   const int nsm = sm_count();
   JAGG_CUDA_TRY(launch(kernel, units < nsm ? units : nsm, FB2_THREADS, C::SMEM, s, maps, p));
@@ -1075,11 +1072,8 @@ static int launch_fwd(const AttnArgs& f, cudaStream_t s) {
   p.q_col0 = f.q_col0; p.k_col0 = f.k_col0; p.v_col0 = f.v_col0;
   p.o = f.o;
   p.lse = f.lse;
-  static bool attr = false;
-  if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(fa_fwd_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, fa_fwd_tc_kernel<D>, C::SMEM));
   const int units = ceil_div(tok_tiles(N, p.n0, C::BQ), C::NX) * f.B * f.heads;
   const int slots = C::CTAS * sm_count();
   JAGG_CUDA_TRY(launch(fa_fwd_tc_kernel<D>, units < slots ? units : slots, C::THREADS, C::SMEM, s, maps, p));

@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "../../include/jagg.h"
+#include "per_device.cuh"
 
 namespace jagg {
 
@@ -173,6 +174,27 @@ inline cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+// Lets `kernel` be launched with up to `bytes` of dynamic shared memory.  A function attribute
+// belongs to one device, so it is set once on each device that a launch is made on.
+template <class... P>
+inline cudaError_t allow_smem(OncePerDevice& once, void (*kernel)(P...), int bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once.run(dev, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+}
+// The CTAs of `threads` threads and `smem` bytes that an SM holds (at least 1), asked once.
+template <class... P>
+inline cudaError_t resident_ctas(std::atomic<int>& known, void (*kernel)(P...), int threads, size_t smem, int* n) {
+  *n = known.load(std::memory_order_relaxed);
+  if (*n > 0) return cudaSuccess;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, threads, smem);
+  if (e != cudaSuccess) return e;
+  if (*n < 1) *n = 1;
+  known.store(*n, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 int prof_start(cudaStream_t s);  // returns a token, or -1 when profiling is off

@@ -779,12 +779,11 @@ template <int NV, int WPR, bool LN, bool GATE>
 int launch_ln_gate_ring_t(const LnGateBwd& a, cudaStream_t s) {
   using C = LnRing<NV, WPR, LN, GATE>;
   auto kernel = ln_gate_ring_kernel<NV, WPR, LN, GATE>;
-  static int per_sm = 0;
-  if (!per_sm) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    JAGG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, C::SMEM));
-    if (per_sm < 1) per_sm = 1;
-  }
+  static OncePerDevice once;
+  static std::atomic<int> ctas{0};
+  int per_sm = 0;
+  JAGG_CUDA_TRY(allow_smem(once, kernel, C::SMEM));
+  JAGG_CUDA_TRY(resident_ctas(ctas, kernel, 256, C::SMEM, &per_sm));
   // equal row shares of at least two rows per group, at most one wave of resident CTAs
   const int cap = per_sm * sm_count();
   const int want = ceil_div(a.M, 2 * C::GROUPS);
@@ -957,40 +956,28 @@ bool ln_gate_narrow_serves(const LnGateBwd& a) {
 template <int NV, bool GATE, bool YBF>
 int launch_ln_gate_rowreg_t(const LnGateBwd& a, cudaStream_t s) {
   const int smem = (8 * 4 + 2) * 128 * NV * (int)sizeof(float);
-  static bool attr = false;
-  if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(ln_gate_rowreg_kernel<NV, GATE, YBF>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    attr = true;
-  }
-  static int per_sm = 0;
-  if (!per_sm) {
-    JAGG_CUDA_TRY(
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ln_gate_rowreg_kernel<NV, GATE, YBF>, 256, smem));
-    if (per_sm < 1) per_sm = 1;
-  }
+  auto kernel = ln_gate_rowreg_kernel<NV, GATE, YBF>;
+  static OncePerDevice once;
+  static std::atomic<int> ctas{0};
+  int per_sm = 0;
+  JAGG_CUDA_TRY(allow_smem(once, kernel, smem));
+  JAGG_CUDA_TRY(resident_ctas(ctas, kernel, 256, smem, &per_sm));
   // equal row shares of at least 16 rows per CTA, at most one wave of resident CTAs
   const int cap = per_sm * sm_count();
   const int want = ceil_div(a.M, 16);
-  JAGG_CUDA_TRY(launch(ln_gate_rowreg_kernel<NV, GATE, YBF>, want < cap ? want : cap, 256, smem, s, a));
+  JAGG_CUDA_TRY(launch(kernel, want < cap ? want : cap, 256, smem, s, a));
   JAGG_LAUNCHED();
   return JAGG_OK;
 }
 
 template <int NVT>
 int launch_ln_gate_nv(const LnGateBwd& a, int smem, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(ln_gate_fused_kernel<NVT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       4 * 3072 * (int)sizeof(float)));
-    attr = true;
-  }
-  static int per_sm = 0;
-  if (!per_sm) {
-    JAGG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ln_gate_fused_kernel<NVT>, 256,
-                                                                4 * 3072 * (int)sizeof(float)));
-    if (per_sm < 1) per_sm = 1;
-  }
+  constexpr int most = 4 * 3072 * (int)sizeof(float);
+  static OncePerDevice once;
+  static std::atomic<int> ctas{0};
+  int per_sm = 0;
+  JAGG_CUDA_TRY(allow_smem(once, ln_gate_fused_kernel<NVT>, most));
+  JAGG_CUDA_TRY(resident_ctas(ctas, ln_gate_fused_kernel<NVT>, 256, most, &per_sm));
   const int units = (a.M / a.rows_per_seq) * ceil_div(a.rows_per_seq, LNF_ROWS);
   const int cap = per_sm * sm_count();
   JAGG_CUDA_TRY(launch(ln_gate_fused_kernel<NVT>, units < cap ? units : cap, 256, smem, s, a));

@@ -1060,12 +1060,8 @@ int launch_tc(const GemmArgs& g, cudaStream_t stream) {
   p.e = make_epi(g);
   const int total = p.tiles_m * p.tiles_n * p.splits;
   const int grid = total < nsm ? total : nsm;
-  static bool attr_set = false;  // one per template instance
-  if (!attr_set) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<BN, A_MN, B_MN, AUX, EW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       Cfg::SMEM_BYTES));
-    attr_set = true;
-  }
+  static OncePerDevice once;  // one per template instance
+  JAGG_CUDA_TRY(allow_smem(once, gemm_tc_kernel<BN, A_MN, B_MN, AUX, EW>, Cfg::SMEM_BYTES));
   const int tok = prof_start(stream);
   JAGG_CUDA_TRY(launch(gemm_tc_kernel<BN, A_MN, B_MN, AUX, EW>, grid, tc_threads(EW), Cfg::SMEM_BYTES, stream, ta,
                        tb, tc, tx, p));

@@ -617,11 +617,8 @@ int launch_pair(const GemmArgs& a, const GemmArgs* b, const PairPlan (&plan)[2],
   grp.stages = fit < P_MAX_STAGES ? fit : P_MAX_STAGES;
   const int smem = grp.stages * grp.stage_bytes + Cfg::EPI_BYTES + P_FIXED;
   auto kernel = gemm_pair_kernel<A_MN, B_MN, EPI>;
-  static bool attr = false;
-  if (!attr) {
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM));
-    attr = true;
-  }
+  static OncePerDevice once;
+  JAGG_CUDA_TRY(allow_smem(once, kernel, P_SMEM));
   const int tok = prof_start(s);
   JAGG_CUDA_TRY(launch(kernel, 2 * (grp.total < npairs ? grp.total : npairs), P_THREADS, smem, s, grp));
   JAGG_LAUNCHED();

@@ -149,13 +149,10 @@ bool rows_fwd_serves(const RowsFwd& a) {
 
 int launch_rows_fwd(const RowsFwd& a, cudaStream_t s) {
   const int smem = 16 * (a.in * 2 + 64);
-  static bool attr = false;
-  if (!attr) {
-    constexpr int most = 16 * (3072 * 2 + 64);
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(rows_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    JAGG_CUDA_TRY(cudaFuncSetAttribute(rows_fwd_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-    attr = true;
-  }
+  constexpr int most = 16 * (3072 * 2 + 64);
+  static OncePerDevice once1, once4;
+  JAGG_CUDA_TRY(allow_smem(once1, rows_fwd_kernel<1>, most));
+  JAGG_CUDA_TRY(allow_smem(once4, rows_fwd_kernel<4>, most));
   const int nsm = sm_count(), groups = a.out / 8;
   const int tok = prof_start(s);
   if (groups < 8 * nsm) {  // four warps per 8 rows
