@@ -1486,7 +1486,7 @@ int launch_mul_silu_grad(float* g, const float* x, void* copy, int dtype, int64_
   return JAGG_OK;
 }
 int launch_add_pos_embed(float* h, int B, int rows_per_seq, int row0, int gh, int gw, int d, cudaStream_t s) {
-  JAGG_CUDA_TRY(launch(pos_embed_kernel, grid_for((int64_t)B * gh * gw * d, 256), 256, 0, s, h, B, rows_per_seq,
+  JAGG_CUDA_TRY(launch(pos_embed_kernel, ceil_div((int64_t)gh * gw * (d / 4), 256), 256, 0, s, h, B, rows_per_seq,
                        row0, gh, gw, d));
   JAGG_LAUNCHED();
   return JAGG_OK;
