@@ -55,9 +55,16 @@ typedef struct jagg_gemm_desc {
   int32_t c_trans;
   int32_t bias_m;
   int32_t tile_n;
+  float* col_sum; /* epi mul: col_sum[n] += sum over m of the stored C, or NULL */
 } jagg_gemm_desc;
 
 int jagg_test_gemm(const jagg_gemm_desc* desc, cudaStream_t stream);
+/* The CTA-pair kernel and no other: the product x, or x and y (nullable) of one layout and epilogue in
+ * one launch, in tiles of bn columns (128 to 256 in steps of 32; 0 = the library's choice, of
+ * the splits too) and, for accum, K splits of at most one per 64 of K (else 1).  JAGG_ERR_ARG
+ * where the kernel does not serve the product. */
+int jagg_test_gemm_pair(const jagg_gemm_desc* x, const jagg_gemm_desc* y, int bn_x, int splits_x, int bn_y,
+                        int splits_y, cudaStream_t stream);
 
 /* Joint softmax attention over qkv [B*N, 3*heads*dh] (q, k, v at column offsets 0, d, 2d;
  * dtype JAGG_DTYPE_*): o [B*N, d], lse [B, heads, N] f32.  The backward takes dO [B*N, d]
@@ -75,7 +82,8 @@ int jagg_test_attention_bwd_bias(const void* qkv, const void* o, const float* ls
  * tokens of every sequence live in qkv0 / o0 / dO0 / dqkv0 ([B*n0, 3d], [B*n0, d], ...),
  * the remaining N - n0 in qkv1 / o1 / dO1 / dqkv1 (n0 = N: one buffer, the *1 pointers
  * ignored).  impl: 0 the library's choice, 1 the warp-level MMA kernel, 2 the tcgen05
- * kernel (JAGG_ERR_ARG when it does not serve the call). */
+ * kernel with n0 on a multiple of 128 tokens, 3 the tcgen05 kernel with any n0 (JAGG_ERR_ARG when it does
+ * not serve the call). */
 /* The forward over two-stream views (same layout and impl codes as the backward below):
  * o0 / o1 receive the output rows of each stream, lse [B, heads, N]. */
 int jagg_test_attention_fwd_streams(const void* qkv0, const void* qkv1, void* o0, void* o1, float* lse, int B,
@@ -120,11 +128,13 @@ int jagg_test_qk_norm_rope_fwd(const void* qkv, int64_t ld_qkv, int M, int N, in
                                int dtype, cudaStream_t stream);
 /* Backward of the above: dqk [M, ld_dqk] (dtype) holds the gradient of the rotated q at column
  * 0 and of k at column d on entry and the gradient of the raw q, k on exit; dqscale,
- * dkscale [dh] f32 accumulate the scale gradients.  rq, rk from the forward. */
+ * dkscale [dh] f32 accumulate the scale gradients.  rq, rk from the forward.  dq32 (nullable): q's
+ * gradient comes in f32 from rows of d floats instead, that of token n of sequence b in row
+ * b * dq32_seq + dq32_row0 + n. */
 int jagg_test_qk_norm_rope_bwd(const void* qkv, int64_t ld_qkv, int M, int N, int d, int heads, int n_txt, int gw,
                                const void* qscale, const void* kscale, int rope, const float* rq, const float* rk,
-                               void* dqk, int64_t ld_dqk, float* dqscale, float* dkscale, int dtype,
-                               cudaStream_t stream);
+                               void* dqk, int64_t ld_dqk, const float* dq32, int dq32_seq, int dq32_row0,
+                               float* dqscale, float* dkscale, int dtype, cudaStream_t stream);
 /* Column sums db[c] += sum_r X[r * ld + c] (r < rows, c < cols; X f32 when x_f32 else bf16):
  * the bias gradients of the joint VJP. */
 int jagg_test_colsum(const void* X, int x_f32, int rows, int cols, int64_t ld, float* db, cudaStream_t stream);

@@ -58,7 +58,7 @@ class GemmDesc(ctypes.Structure):
                 ("gate", ctypes.c_void_p), ("gate_stride", ctypes.c_int64),
                 ("rows_per_seq", ctypes.c_int32), ("split_k", ctypes.c_int32),
                 ("force_simt", ctypes.c_int32), ("c_trans", ctypes.c_int32), ("bias_m", ctypes.c_int32),
-                ("tile_n", ctypes.c_int32)]
+                ("tile_n", ctypes.c_int32), ("col_sum", ctypes.c_void_p)]
 
 
 class ProfileStat(ctypes.Structure):
@@ -112,6 +112,7 @@ _SIGNATURES = {
     "jagg_grad_reduce_workspace_bytes": (_I64, [_I64]),
     "grad_reduce": (_I, [_P, _P, _I64, ctypes.c_float, _P, _P, _P, _SZ, _P]),
     "jagg_test_gemm": (_I, [ctypes.POINTER(GemmDesc), _P]),
+    "jagg_test_gemm_pair": (_I, [ctypes.POINTER(GemmDesc), ctypes.POINTER(GemmDesc), _I, _I, _I, _I, _P]),
     "jagg_test_wait_timeout": (_I, [ctypes.c_ulonglong, _P, _P]),
     "jagg_test_attention_fwd": (_I, [_P, _I, _I, _I, _I, _I, _P, _P, _P]),
     "jagg_test_attention_scratch_bytes": (_I64, [_I, _I, _I, _I]),
@@ -122,8 +123,8 @@ _SIGNATURES = {
     "jagg_test_ln_gate_bwd": (_I, [_I, _I, _I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
                                    _I, _P]),
     "jagg_test_qk_norm_rope_fwd": (_I, [_P, _I64, _I, _I, _I, _I, _I, _I, _P, _P, _I, _P, _P, _P, _I, _P]),
-    "jagg_test_qk_norm_rope_bwd": (_I, [_P, _I64, _I, _I, _I, _I, _I, _I, _P, _P, _I, _P, _P, _P, _I64, _P, _P, _I,
-                                        _P]),
+    "jagg_test_qk_norm_rope_bwd": (_I, [_P, _I64, _I, _I, _I, _I, _I, _I, _P, _P, _I, _P, _P, _P, _I64, _P, _I, _I,
+                                        _P, _P, _I, _P]),
     "jagg_test_colsum": (_I, [_P, _I, _I, _I, _I64, _P, _P]),
     "jagg_test_attention_bwd_streams": (_I, [_P, _P, _P, _P, _P, _P, _P, _I, _I, _I, _I, _I, _I, _P, _P, _P, _I,
                                              _P]),
@@ -426,6 +427,12 @@ def test_gemm(desc: GemmDesc, stream=None):
     _check(lib().jagg_test_gemm(ctypes.byref(desc), _stream(stream)), "jagg_test_gemm")
 
 
+def test_gemm_pair(x: GemmDesc, y=None, bn=(0, 0), splits=(1, 1), stream=None):
+    """The CTA-pair kernel on x, or on x and y in one launch (jagg_test_gemm_pair)."""
+    _check(lib().jagg_test_gemm_pair(ctypes.byref(x), ctypes.byref(y) if y is not None else None, bn[0], splits[0],
+                                     bn[1], splits[1], _stream(stream)), "jagg_test_gemm_pair")
+
+
 def test_attention_fwd(qkv, B, N, heads, dh, o, lse, stream=None):
     dt = DTYPE_BF16 if qkv.dtype == torch.bfloat16 else DTYPE_F32
     _check(lib().jagg_test_attention_fwd(_ptr(qkv), B, N, heads, dh, dt, _ptr(o), _ptr(lse), _stream(stream)),
@@ -496,13 +503,13 @@ def test_qk_norm_rope_fwd(qkv, M, N, heads, n_txt, gw, qscale, kscale, qk_out, r
 
 
 def test_qk_norm_rope_bwd(qkv, M, N, heads, n_txt, gw, qscale, kscale, rq, rk, dqk, dqscale, dkscale, rope=True,
-                          stream=None):
+                          dq32=None, dq32_seq=0, dq32_row0=0, stream=None):
     """Its backward in place on dqk [M, >= 2d] (jagg_test_qk_norm_rope_bwd)."""
     d = qscale.numel() * heads
     dt = DTYPE_BF16 if qkv.dtype == torch.bfloat16 else DTYPE_F32
     _check(lib().jagg_test_qk_norm_rope_bwd(_ptr(qkv), qkv.stride(0), M, N, d, heads, n_txt, gw, _ptr(qscale),
                                             _ptr(kscale), int(rope), _ptr(rq), _ptr(rk), _ptr(dqk), dqk.stride(0),
-                                            _ptr(dqscale), _ptr(dkscale), dt, _stream(stream)),
+                                            _ptr(dq32), dq32_seq, dq32_row0, _ptr(dqscale), _ptr(dkscale), dt, _stream(stream)),
            "jagg_test_qk_norm_rope_bwd")
 
 

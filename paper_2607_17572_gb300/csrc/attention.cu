@@ -840,15 +840,17 @@ void attention_bwd_scratch(float* scratch, int B, int N, int heads, float** Dv, 
   *dq_acc = scratch + dv_floats_padded(B, N, heads);
 }
 
-// The stream boundary on a 128-token multiple: what an explicit request for the tcgen05 kernels
-// (impl = 2) has to meet; the library's own choice takes any boundary to them.
-static bool whole_tiles(const AttnArgs& a) { return a.q.n0 >= a.N || a.q.n0 % 128 == 0; }
+// Whether the call meets an explicit request: impl = 2 asks for the tcgen05 kernels and a stream boundary
+// on a 128-token multiple, impl = 3 for the tcgen05 kernels; the library's own choice takes any boundary to them.
+static bool impl_serves(int impl, bool tc, const AttnArgs& a) {
+  return impl < 2 || (tc && (impl == 3 || a.q.n0 >= a.N || a.q.n0 % 128 == 0));
+}
 
 int attention_fwd(const AttnArgs& a, cudaStream_t s) {
   JAGG_CHECK_ARG(a.B > 0 && a.N > 0 && a.heads > 0, "attention: empty shape");
-  JAGG_CHECK_ARG(a.impl >= 0 && a.impl <= 2, "attention: bad implementation %d", a.impl);
+  JAGG_CHECK_ARG(a.impl >= 0 && a.impl <= 3, "attention: bad implementation %d", a.impl);
   const bool tc = attention_fwd_tc_eligible(a);
-  JAGG_CHECK_ARG(a.impl != 2 || (tc && whole_tiles(a)), "attention: the tcgen05 forward does not serve this call");
+  JAGG_CHECK_ARG(impl_serves(a.impl, tc, a), "attention: the tcgen05 forward does not serve this call");
   if (tc && a.impl != 1) {
     const int tok = prof_start(s);
     JAGG_TRY(attention_fwd_tc(a, s));
@@ -890,9 +892,9 @@ int attention_bwd(const AttnBwdArgs& a, cudaStream_t s) {
   JAGG_LAUNCHED();
   prof_stop(tok, s, PROF_ATTN_AUX, 0.0, 4.0 * f.B * f.N * f.heads * f.dh * 1.5);
   int st = JAGG_ERR_UNSUPPORTED;
-  JAGG_CHECK_ARG(a.impl >= 0 && a.impl <= 2, "attention: bad implementation %d", a.impl);
+  JAGG_CHECK_ARG(a.impl >= 0 && a.impl <= 3, "attention: bad implementation %d", a.impl);
   const bool tc = attention_bwd_tc_eligible(a);
-  JAGG_CHECK_ARG(a.impl != 2 || (tc && whole_tiles(f)), "attention: the tcgen05 backward does not serve this call");
+  JAGG_CHECK_ARG(impl_serves(a.impl, tc, f), "attention: the tcgen05 backward does not serve this call");
   if (tc && a.impl != 1) {
     tok = prof_start(s);
     st = attention_bwd_tc(a, s);

@@ -30,7 +30,9 @@ struct AttnArgs {
   SegRows o;  // output, col h * dh
   float* lse;  // [B, heads, N] natural-log log-sum-exp of the scaled scores
   int dtype;
-  int impl = 0;  // forward: 0 the library's choice; 1 warp-level MMA kernel; 2 tcgen05 kernel
+  // 0: the library's choice; 1: warp-level MMA kernel; tcgen05 kernel: 2 with whole tiles of the
+  // first stream, 3 with any stream boundary
+  int impl = 0;
 };
 
 struct AttnBwdArgs {
@@ -40,7 +42,7 @@ struct AttnBwdArgs {
   float* dq_acc;  // f32 [B*N, heads*dh] scratch, zeroed by the launcher
   SegRows dq, dk, dv;  // outputs (dtype), columns dq_col0 + h * dh etc.
   int64_t dq_col0, dk_col0, dv_col0;
-  int impl = 0;  // 0: the library's choice; 1: warp-level MMA kernel; 2: tcgen05 kernel
+  int impl = 0;  // as above
   // One stream with [dq | dk | dv] side by side in one buffer from column 0: add the column sums
   // (the qkv bias gradient, 3 heads dh floats) here, or nullptr.
   float* db = nullptr;

@@ -1011,7 +1011,9 @@ int staged_mode(const GemmArgs& g) {
   return STAGED_NONE;
 }
 
-int validate(const GemmArgs& g) {
+}  // namespace
+
+int gemm_validate(const GemmArgs& g) {
   JAGG_CHECK_ARG(g.M > 0 && g.N > 0 && g.K > 0, "gemm: empty shape %dx%dx%d", g.M, g.N, g.K);
   JAGG_CHECK_ARG(g.A && g.B && (g.C || (g.epi == EPI_GELU && g.C2)), "gemm: null operand");
   JAGG_CHECK_ARG(g.epi >= EPI_STORE && g.epi <= EPI_ACCUM, "gemm: bad epilogue %d", g.epi);
@@ -1022,6 +1024,8 @@ int validate(const GemmArgs& g) {
   JAGG_CHECK_ARG(!g.col_sum || g.epi == EPI_MUL_AUX, "gemm: column sums need the multiply epilogue");
   return JAGG_OK;
 }
+
+namespace {
 
 template <int BN, bool A_MN, bool B_MN, int AUX, int EW = 4>
 int launch_tc(const GemmArgs& g, cudaStream_t stream) {
@@ -1148,7 +1152,7 @@ int encode_tmap(CUtensorMap* m, bool f32, int rank, const void* base, const uint
 }
 
 int gemm_simt(const GemmArgs& g, cudaStream_t stream) {
-  JAGG_TRY(validate(g));
+  JAGG_TRY(gemm_validate(g));
   SimtParams p;
   p.M = g.M; p.N = g.N; p.K = g.K;
   p.A = g.A; p.lda = g.lda; p.a_mn = g.a_mn; p.a_bf16 = g.a_dtype == JAGG_DTYPE_BF16;
@@ -1200,7 +1204,7 @@ double gemm_best_cost(const GemmArgs& g) {
 }
 
 int gemm(const GemmArgs& g, cudaStream_t stream) {
-  JAGG_TRY(validate(g));
+  JAGG_TRY(gemm_validate(g));
   if (g.col_sum) {  // the pair kernel sums in its epilogue; after the others, a pass over the output
     double cost;
     if (gemm_tc_eligible(g) && takes_pair(g, &cost)) return gemm_pair(g, stream);

@@ -65,6 +65,10 @@ int gemm(const GemmArgs& g, cudaStream_t stream);
 bool gemm_pair_serves(const GemmArgs& g, double* cost);
 int gemm_pair(const GemmArgs& g, cudaStream_t stream);
 
+// The pair kernel and nothing else (tests): one product, or two in one launch, in tiles of bn columns
+// (0: the estimate's plan) and K splits; an error where it has no instance.
+int gemm_pair_as(const GemmArgs& x, const GemmArgs* y, const int (&bn)[2], const int (&splits)[2], cudaStream_t stream);
+
 // Two independent products of the same layout and epilogue (the text and image streams of a
 // dual-stream block), in one launch where the CTA-pair kernel serves both.
 int gemm_two(const GemmArgs& x, const GemmArgs& y, cudaStream_t stream);
@@ -73,6 +77,9 @@ int gemm_two(const GemmArgs& x, const GemmArgs& y, cudaStream_t stream);
 double gemm_best_cost(const GemmArgs& g);
 // bf16 operands that the tensor-core kernels can address.
 bool gemm_tc_eligible(const GemmArgs& g);
+
+// Operands present, shapes and epilogue consistent.
+int gemm_validate(const GemmArgs& g);
 
 // Forces the SIMT kernel (tests of the tensor-core path compare against it).
 int gemm_simt(const GemmArgs& g, cudaStream_t stream);

@@ -724,6 +724,24 @@ int gemm_pair(const GemmArgs& g, cudaStream_t s) {
   return dispatch_pair(g, nullptr, plan, s);
 }
 
+int gemm_pair_as(const GemmArgs& x, const GemmArgs* y, const int (&bn)[2], const int (&splits)[2], cudaStream_t s) {
+  PairPlan plan[2] = {};
+  for (int i = 0; i < (y ? 2 : 1); ++i) {
+    const GemmArgs& g = i ? *y : x;
+    JAGG_TRY(gemm_validate(g));
+    JAGG_CHECK_ARG(gemm_tc_eligible(g) && pair_instance(g), "gemm: the pair kernel does not serve this product");
+    pair_plan(g, sm_count() / 2, &plan[i]);
+    if (!bn[i]) continue;
+    JAGG_CHECK_ARG(bn[i] % 32 == 0 && bn[i] >= 128 && bn[i] <= PT, "gemm: pair tiles of %d columns", bn[i]);
+    JAGG_CHECK_ARG(splits[i] >= 1 && splits[i] <= (g.epi == EPI_ACCUM ? ceil_div(g.K, PK) : 1), "gemm: %d K splits",
+                   splits[i]);
+    plan[i] = {bn[i], splits[i]};
+  }
+  JAGG_CHECK_ARG(!y || (x.a_mn == y->a_mn && x.b_mn == y->b_mn && pair_epi(x) == pair_epi(*y)),
+                 "gemm: a grouped launch needs one layout and epilogue");
+  return dispatch_pair(x, y, plan, s);
+}
+
 int gemm_two(const GemmArgs& x, const GemmArgs& y, cudaStream_t s) {
   const bool same = x.a_mn == y.a_mn && x.b_mn == y.b_mn && x.epi == y.epi && gemm_tc_eligible(x) &&
                     gemm_tc_eligible(y) && pair_instance(x) && pair_instance(y) && pair_epi(x) == pair_epi(y);
@@ -732,7 +750,7 @@ int gemm_two(const GemmArgs& x, const GemmArgs& y, cudaStream_t s) {
     const GemmArgs& a = x.K > y.K || (x.K == y.K && x.M >= y.M) ? x : y;
     const GemmArgs& b = &a == &x ? y : x;
     const int np = sm_count() / 2;
-    PairPlan plan[2] = {}, alone;
+    PairPlan plan[2] = {};
     double best = 0.0;
     const int sa_max = most_splits(a) < 8 ? most_splits(a) : 8, sb_max = most_splits(b) < 4 ? most_splits(b) : 4;
     for (int wa = 0; wa < 5; ++wa)

@@ -36,8 +36,7 @@ extern "C" int jagg_test_wait_timeout(unsigned long long limit_ns, unsigned long
   return JAGG_OK;
 }
 
-extern "C" int jagg_test_gemm(const jagg_gemm_desc* d, cudaStream_t stream) {
-  JAGG_CHECK_ARG(d, "jagg_test_gemm: null descriptor");
+static GemmArgs gemm_args(const jagg_gemm_desc* d) {
   GemmArgs g;
   g.M = d->M; g.N = d->N; g.K = d->K;
   g.A = d->A; g.lda = d->lda; g.a_mn = d->a_mn != 0; g.a_dtype = d->a_dtype;
@@ -52,7 +51,23 @@ extern "C" int jagg_test_gemm(const jagg_gemm_desc* d, cudaStream_t stream) {
   g.c_trans = d->c_trans != 0;
   g.bias_m = d->bias_m != 0;
   g.tile_n = d->tile_n;
+  g.col_sum = d->col_sum;
+  return g;
+}
+
+extern "C" int jagg_test_gemm(const jagg_gemm_desc* d, cudaStream_t stream) {
+  JAGG_CHECK_ARG(d, "jagg_test_gemm: null descriptor");
+  const GemmArgs g = gemm_args(d);
   return d->force_simt ? gemm_simt(g, stream) : gemm(g, stream);
+}
+
+extern "C" int jagg_test_gemm_pair(const jagg_gemm_desc* x, const jagg_gemm_desc* y, int bn_x, int splits_x, int bn_y,
+                                   int splits_y, cudaStream_t stream) {
+  JAGG_CHECK_ARG(x, "jagg_test_gemm_pair: null descriptor");
+  const GemmArgs a = gemm_args(x);
+  GemmArgs b;
+  if (y) b = gemm_args(y);
+  return gemm_pair_as(a, y ? &b : nullptr, {bn_x, bn_y}, {splits_x, splits_y}, stream);
 }
 
 static AttnArgs make_args(const void* qkv, int B, int N, int heads, int dh, int dtype, void* o, float* lse) {
@@ -223,15 +238,18 @@ extern "C" int jagg_test_qk_norm_rope_fwd(const void* qkv, int64_t ld_qkv, int M
 
 extern "C" int jagg_test_qk_norm_rope_bwd(const void* qkv, int64_t ld_qkv, int M, int N, int d, int heads, int n_txt,
                                           int gw, const void* qscale, const void* kscale, int rope, const float* rq,
-                                          const float* rk, void* dqk, int64_t ld_dqk, float* dqscale, float* dkscale,
-                                          int dtype, cudaStream_t stream) {
+                                          const float* rk, void* dqk, int64_t ld_dqk, const float* dq32,
+                                          int dq32_seq, int dq32_row0, float* dqscale, float* dkscale, int dtype,
+                                          cudaStream_t stream) {
   JAGG_TRY(qkn_check("jagg_test_qk_norm_rope_bwd", M, N, d, heads, n_txt, gw, rope, dtype));
+  JAGG_CHECK_ARG(!dq32 || (dq32_row0 >= 0 && dq32_seq >= dq32_row0 + N), "jagg_test_qk_norm_rope_bwd: bad dq32 rows");
   JAGG_CHECK_ARG(qkv && qscale && kscale && rq && rk && dqk && dqscale && dkscale,
                  "jagg_test_qk_norm_rope_bwd: null pointer");
   QkNormRopeBwd b{};
   b.f = qkn_args(qkv, ld_qkv, M, N, d, heads, n_txt, gw, qscale, kscale, rope, dtype);
   b.f.rq = const_cast<float*>(rq); b.f.rk = const_cast<float*>(rk);
   b.dqk = dqk; b.ld_dqk = ld_dqk;
+  b.dq32 = dq32; b.dq32_seq = dq32_seq; b.dq32_row0 = dq32_row0;
   b.dqs_txt = b.dqs_img = dqscale;
   b.dks_txt = b.dks_img = dkscale;
   return launch_qk_norm_rope_bwd(b, stream);

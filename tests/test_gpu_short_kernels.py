@@ -237,3 +237,35 @@ def test_a_refused_launch_does_not_reach_the_next_call():
         jg.test_attention_fwd(qkv, 3, 1, 1, 16, o, lse)
     torch.cuda.synchronize()
     assert jg.device_status() == 0
+
+
+@pytest.mark.parametrize("dh,H,dtype", [(128, 3, torch.bfloat16), (64, 2, torch.bfloat16), (32, 4, torch.float32)])
+@pytest.mark.parametrize("N,n_txt,row0,rest", [(65, 5, 0, 0), (60, 0, 77, 0), (33, 33, 0, 91)])
+def test_qk_norm_backward_from_the_f32_accumulator(N, n_txt, row0, rest, dh, H, dtype):
+    """dQ read in f32 from attention's accumulator, whose sequences hold both streams: the stream's
+    rows start at row0 and `rest` rows follow.  Nothing else of the accumulator and none of q's columns of the
+    gradient buffer is read (NaN there).  Tolerances as for the other forms of these kernels."""
+    torch.manual_seed(N + dh)
+    B, gw, d = 3, 5, H * dh
+    M, seq = B * N, row0 + N + rest
+    qkv = (torch.randn(M, 3 * d, device="cuda") * 2).to(dtype)
+    qs, ks = ((1 + 0.1 * torch.randn(dh, device="cuda")).to(dtype) for _ in range(2))
+    qk, rq, rk = torch.empty(M, 2 * d, device="cuda", dtype=dtype), *(torch.empty(M, H, device="cuda") for _ in "qk")
+    jg.test_qk_norm_rope_fwd(qkv, M, N, H, n_txt, gw, qs, ks, qk, rq, rk, rope=True)
+    acc = torch.full((B, seq, d), float("nan"), device="cuda")
+    acc[:, row0:row0 + N] = torch.randn(B, N, d, device="cuda")
+    dqk = torch.randn(M, 3 * d, device="cuda").to(dtype)
+    up = [acc[:, row0:row0 + N].reshape(M, d), dqk[:, d:2 * d].clone().float()]
+    dqk[:, :d] = float("nan")
+    dscale = [torch.zeros(dh, device="cuda") for _ in range(2)]
+    jg.test_qk_norm_rope_bwd(qkv, M, N, H, n_txt, gw, qs, ks, rq, rk, dqk, *dscale, rope=True, dq32=acc, dq32_seq=seq,
+                             dq32_row0=row0)
+    torch.cuda.synchronize()
+    tol = 1e-2 if dtype == torch.bfloat16 else 1e-5
+    for i, (s, ds) in enumerate(zip((qs, ks), dscale)):
+        x = qkv[:, i * d:(i + 1) * d].float().view(M, H, dh).requires_grad_()
+        s = s.float().requires_grad_()
+        y = _qkn_reference(x, N, n_txt, gw, dh, s, True).reshape(M, d)
+        (y * up[i]).sum().backward()
+        assert _rel(dqk[:, i * d:(i + 1) * d].float(), x.grad.reshape(M, d)) < 2 * tol
+        assert _rel(ds, s.grad) < 1e-4
