@@ -461,11 +461,19 @@ constexpr int GR_RUN = GR_THREADS * GR_UNROLL;  // float4 of a vector per CTA an
 
 // HAS_B: a second vector b (else <a, b> = |b|^2 = |a|^2 and b is not read); HAS_ACC: the
 // update acc += alpha a.  A CTA walks runs of GR_RUN consecutive float4 of each vector; each
-// thread issues its GR_UNROLL loads of every input before using any, as streaming accesses
-// (the vectors are read once); f32 sums over 16 terms fold into f64.  Bound by DRAM: with a,
-// b and acc of 130 M elements 305 us (6.8 TB/s, the copy rate); 427 us when a thread's eight
-// loads were a grid apart, 1024 CTAs ran in more than one wave and one thread per sum
-// added the partials.
+// thread issues its GR_UNROLL loads of every input before using any; f32 sums over 16 terms fold
+// into f64.  Bound by DRAM.  CTAs per SM and cache policy by form, each at its best of 2 to 5 CTAs with streaming
+// and with plain accesses (130 M elements; us with the sums' second launch where there are sums):
+//   acc, a, b   4, plain      304   (streaming 315; 3 CTAs 309)
+//   acc, a      4, plain      232   (streaming, 3 CTAs: 248)
+//   a, b        5, streaming  175   (3 CTAs 220; plain 185)
+//   a           3, streaming   91   (plain 107)
+// 435, 236, 265 and 166 when a thread's eight loads were a grid apart, 1024 CTAs ran in more than one
+// wave and one thread per sum added the partials.
+constexpr int gr_ctas_per_sm(bool has_b, bool has_acc) { return has_acc ? 4 : has_b ? 5 : 3; }
+template <bool PLAIN>
+__device__ __forceinline__ float4 gr_load(const float4* p) { return PLAIN ? *p : __ldcs(p); }
+
 template <bool HAS_B, bool HAS_ACC>
 __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a, const float* b, int64_t P,
                                                                  float alpha, float* acc, double* partial) {
@@ -482,9 +490,9 @@ __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a,
     for (int r = 0; r < GR_UNROLL; ++r) {
       const int64_t q = i0 + r * GR_THREADS;
       const bool in = q < nvec;
-      x[r] = in ? __ldcs(a4 + q) : zero;
-      if constexpr (HAS_B) y[r] = in ? __ldcs(b4 + q) : zero;
-      if constexpr (HAS_ACC) c[r] = in ? __ldcs(c4 + q) : zero;
+      x[r] = in ? gr_load<HAS_ACC>(a4 + q) : zero;
+      if constexpr (HAS_B) y[r] = in ? gr_load<HAS_ACC>(b4 + q) : zero;
+      if constexpr (HAS_ACC) c[r] = in ? c4[q] : zero;
     }
     float fab = 0.f, faa = 0.f, fbb = 0.f;
 #pragma unroll
@@ -497,7 +505,7 @@ __global__ void __launch_bounds__(GR_THREADS) grad_reduce_kernel(const float* a,
       if constexpr (HAS_ACC) {
         const int64_t q = i0 + r * GR_THREADS;
         c[r].x += alpha * x[r].x; c[r].y += alpha * x[r].y; c[r].z += alpha * x[r].z; c[r].w += alpha * x[r].w;
-        if (q < nvec) __stcs(c4 + q, c[r]);
+        if (q < nvec) c4[q] = c[r];
       }
     }
     if constexpr (!HAS_B) fab = fbb = faa;
@@ -749,9 +757,10 @@ extern "C" int grad_reduce(const float* a, const float* b, int64_t P, float alph
   }
   const int tok = prof_start(stream);
   double* part = out3 ? static_cast<double*>(ws) : nullptr;
-  // as many CTAs as stay resident at 3 per SM, fewer for a short vector
+  // one wave of resident CTAs, fewer for a short vector
   const int64_t runs = (P / 4 + GR_RUN - 1) / GR_RUN;
-  const int most = 3 * sm_count() < GR_BLOCKS ? 3 * sm_count() : GR_BLOCKS;
+  const int wave = gr_ctas_per_sm(b != nullptr, acc != nullptr) * sm_count();
+  const int most = wave < GR_BLOCKS ? wave : GR_BLOCKS;
   const int blocks = runs < 1 ? 1 : (runs < most ? (int)runs : most);
   if (b && acc)
     JAGG_CUDA_TRY(launch(grad_reduce_kernel<true, true>, blocks, GR_THREADS, 0, stream, a, b, P, alpha, acc, part));
