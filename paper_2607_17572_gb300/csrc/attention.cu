@@ -8,8 +8,8 @@
 // dS^T = P^T (dP^T - rowsum(dO O)), dV += P^T dO, dK += dS^T Q, and dQ += dS K through
 // shared memory and f32 atomics (appendix, Eqs. bwd_V .. bwd_QK).
 //
-// f32 (and any head dim): straightforward SIMT kernels, one thread per query (forward)
-// or per key (backward).
+// f32 (and head dims 16, 32): SIMT kernels on 32 x 32 tiles in shared memory, a CTA per 32 queries
+// (forward) or per 32 keys (backward).
 #include <algorithm>
 
 #include "attention.cuh"

@@ -591,9 +591,9 @@ struct FfParams {
 // Head dim 128 takes pairs of query tiles (NX = 2), which share every K and V tile and overlap in
 // one CTA.  Head dim 64 (DiT-B's few hundred tokens) takes single tiles (NX = 1) in half of the
 // tensor memory and two CTAs per SM: a unit of three key tiles is a chain of latencies, and 8
-// sequences of 333 tokens are 288 such units on 152 SMs.  16 rows
-// 25 -> 17 us, 8 rows 15 -> 10; pairs of tiles, one CTA per SM, took 24 and 17 us, and the earlier kernel with two
-// passes over the keys (the exact maximum first) 25 and 15.
+// sequences of 333 tokens are 288 such units on 152 SMs.  Device time of a launch, before (two
+// passes over the keys, the exact maximum first) and now: 16 rows 25.4 -> 17.3 us, 8 rows
+// 14.8 -> 11.0 (28.8 -> 20.6 and 18.6 -> 14.3 by events around it); pairs of tiles, one CTA per SM, gained nothing.
 template <int D_>
 struct Ff2 {
   static constexpr int D = D_, NX = D == 128 ? 2 : 1, BQ = 128, BK = 128, NKS = 2, NVS = D == 128 ? 3 : 2;

@@ -95,7 +95,7 @@ __global__ void mul_silu_grad_kernel(float* g, const float* x, void* copy, int c
 
 // One thread per 4 columns of one image token, added to that token of every sequence: each sine
 // is evaluated once, not once per sequence (16 sequences of 256 tokens, d = 768:
-// 28 -> under 9 us).
+// 27.2 -> 7.8 us).
 __global__ void pos_embed_kernel(float* h, int B, int rows_per_seq, int row0, int gh, int gw, int d) {
   pdl_wait();
   const int q = d / 4, groups = d / 4;  // d is a multiple of 64: a group never crosses a quarter

@@ -16,7 +16,7 @@ int launch_timestep_embedding(const float* t, float* phi, int B, int dim, cudaSt
 
 // out = silu(in) (f32 -> f32), n elements.
 int launch_silu(const float* in, float* out, int64_t n, cudaStream_t s);
-// g[i] *= silu'(x[i]) (f32).
+// g[i] *= silu'(x[i]) (f32); copy[i] = g[i] in `dtype`, the operand of the products after it.
 int launch_mul_silu_grad(float* g, const float* x, void* copy, int dtype, int64_t n, cudaStream_t s);
 
 // h[b, row0 + n, :] += 2D sin-cos position table of patch n (gh x gw grid), f32.

@@ -532,10 +532,10 @@ GemmArgs dw_gemm(const jagg_model& m, int M, int N, int K, const void* dY, int64
   return g;
 }
 
-// Products over the B per-sequence rows (t-embedding MLP, stacked modulation).  B is small
-// (a few dozen rows: one 128-row tile, the rest of it zero-filled by TMA), and the products
-// are bound by reading W, so they keep the plain row-major output with the staged
-// epilogues:
+// Products over the B per-sequence rows (t-embedding MLP, stacked modulation), bound by reading W
+// (or its gradient).  In bf16 with B <= 16 the forward and the weight gradient are streaming
+// kernels (rows.cu); more rows, and the input gradient, take one 128-row tensor-core tile, the
+// rest of it zero-filled by TMA; f32 takes the SIMT tiles:
 //   rows_gemm: C[B, out] (f32) = X[B, in] W[out, in]^T + b
 //   rows_dw:   grad[out, in] += dY[B, out]^T X[B, in]        (K = B)
 //   rows_dx:   dX[B, in] += dY[B, out] W[out, in]             (split over out)

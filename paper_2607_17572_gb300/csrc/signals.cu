@@ -21,8 +21,8 @@
 // coefficients by one thread per CTA, a chunk's sum by four warps): a window of 4 x 4 steps
 // of 262144 bf16 elements took 80 us with an f64 coefficient set and butterfly in every thread
 // and five launches, 67 us with the log-prob part repeated by every CTA of the elementwise
-// pass (two launches), and takes 35 us like this (29 us replayed from a CUDA graph; reading
-// and writing its 38 MB once is 5.6 us); 8 x 4 steps of 16384 elements 37 -> 25 us.
+// pass (two launches), and takes 28 to 32 us like this (reading and writing its 38 MB once is
+// 5.6 us; the kernels alone take 11.8, 6.2 and 7.7); 8 x 4 steps of 16384 elements 37 -> 25 to 27 us.
 #include <mutex>
 
 #include "common.cuh"
@@ -568,6 +568,8 @@ using namespace jagg;
 extern "C" int64_t jagg_signals_workspace_bytes(int G, int W, int64_t D) {
   if (G <= 0 || W <= 0 || D <= 0) return 0;
   const int64_t chunks = (D + SIG_CHUNK - 1) / SIG_CHUNK;
+  // the mean coefficients, the partial sums, and G W floats that no kernel uses any more: the
+  // size stays what callers, and the bound of the static variant, have been given
   return mean_coef_bytes(W) + (int64_t)G * W * chunks * 8 + (int64_t)G * W * 4 + 64;
 }
 
