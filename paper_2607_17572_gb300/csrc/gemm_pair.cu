@@ -121,9 +121,9 @@ __device__ __forceinline__ void gelu2(float2 u, float2& g, float2& dg) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(t.y) : "f"(in.y));
   const float2 h = ptx::mul2(u, both(0.5f));
   g = ptx::fma2(h, t, h);
-  const float2 om = ptx::fma2(ptx::mul2(t, both(-1.f)), t, both(1.f));  // 1 - t^2
-  const float2 w = ptx::mul2(h, ptx::fma2(u2, both(3.f * a * c), both(c)));
-  dg = ptx::fma2(w, om, ptx::fma2(t, both(0.5f), both(0.5f)));
+  // h (1 - t^2) first: it is 0 where t has reached +-1, while h times the polynomial overflows from |u| = 1.4e13 on
+  const float2 ho = ptx::mul2(h, ptx::fma2(ptx::mul2(t, both(-1.f)), t, both(1.f)));
+  dg = ptx::fma2(ho, ptx::fma2(u2, both(3.f * a * c), both(c)), ptx::fma2(t, both(0.5f), both(0.5f)));
 }
 __device__ __forceinline__ uint32_t pack2(float x, float y) {
   __nv_bfloat162 v = __floats2bfloat162_rn(x, y);

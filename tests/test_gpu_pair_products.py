@@ -182,6 +182,29 @@ def test_every_width(M, N, K, bn):
         assert _rel(G[:, :N] - 5.0, acc) < _f32_tol(K) + 1e-5, splits  # 5 + x - 5 in f32
 
 
+def test_gelu_of_large_pre_activations():
+    """GELU and its derivative stay finite as long as u^2 does: u or 0, and 1 or 0."""
+    M, N, K = 256, 128, 64
+    ops, acc = _operands(M, N, K, 0, 0)
+    bias = torch.zeros(N, device="cuda")
+    big = torch.tensor([6.0, 1e3, 1e9, 1e13, 2e13, 1e15, 1e18, -6.0, -1e3, -1e9, -1e13, -2e13, -1e15, -1e18], device="cuda")
+    bias[:len(big)] = big
+    bias = bias.bfloat16()
+    D, G = _out(M, N, 8, torch.bfloat16), _out(M, N, 8, torch.bfloat16)
+    jg.test_gemm_pair(_desc(M, N, K, *ops, D, N + 8, jg.DTYPE_BF16, epi=1, bias=bias, C2=G, ldc2=N + 8))
+    _done((D, N), (G, N))
+    u = (acc + bias.float()).double().requires_grad_()
+    g = F.gelu(u, approximate="tanh")
+    g.sum().backward()
+    for c in range(len(big) + 1):  # a column at a time: the sizes differ by 18 orders
+        # bf16 rounding (2^-9), and tanh's absolute error below 2^-10 times |u| (or |u| + 1) where it has not reached 1
+        near = u[:, c].detach().abs() < 30
+        slack = torch.where(near, 2.0 ** -10 * (u[:, c].detach().abs() + 1), torch.zeros_like(u[:, c]))
+        for x, ref in ((G, g.detach()), (D, u.grad)):
+            x, ref = x[:, c].double(), ref[:, c]
+            assert ((x - ref).abs() <= 2.0 ** -8 * ref.abs() + slack).all(), c
+
+
 @pytest.mark.parametrize("bn", [(256, 128), (160, 224), (128, 256), (0, 0)])
 @pytest.mark.parametrize("splits", [(1, 1), (3, 2), (2, 8)])
 def test_two_accumulated_products_in_one_launch(bn, splits):
